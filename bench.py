@@ -652,7 +652,8 @@ def run_large_grid(dev, steps):
         sfx = "" if prec == "fp64" else "_f32"
         hb = {}
         for stage, kerns in (("asy_spread", ["k_asy_spread" + sfx]), ("asy_interp", ["k_asy_interp" + sfx]),
-                             ("asy_fft", ["k_asy_fft_pass_a", "k_asy_fft_pass_b"])):
+                             ("asy_fft", ["k_asy_fft"] if prec == "fp64" else
+                              ["k_asy_fft_pass_a_f32", "k_asy_fft_pass_b_f32"])):
             got = [stored_traffic(k, wl) for k in kerns]
             if all(tr for tr, _ in got):
                 tr = sum(t for t, _ in got)
@@ -870,7 +871,7 @@ def run_ours(a):
     flops, units = _dominant_flops(dom, info, blocks, tab)
     kernel_of = {"asy_spread": "k_asy_spread", "asy_interp": "k_asy_interp",
                  "local_moments": "k_local_moments", "local_eval": "k_local_eval",
-                 "direct": "k_direct", "asy_fft": "k_asy_fft_small"}
+                 "direct": "k_direct", "asy_fft": "k_asy_fft"}
     roof = None
     hbm_peak, hbm_src = measured_hbm_peak()
     if flops is not None:

@@ -25,13 +25,14 @@
 // come from 64-bit fixed-point products with per-block constants (integer
 // instructions); kernel taps, weighted values, the per-bin moments and sums
 // and the FFT run in double-float (df64.cuh, ~48 bits, on the FP32 pipes);
-// the spreading grids accumulate in FP64 atomics.  The FFT output is stored
-// split into (hi, lo) floats so that the interpolation reads it as
+// the spreading grids accumulate in FP64 atomics.  The FFT (k_fft.cu) stores
+// its output split into (hi, lo) floats so that the interpolation reads it as
 // double-float without FP64 work.  Mixed precision (the _f32 kernels and the
-// LOWP FFT instances) keeps the fixed-point positions and phases and runs the
+// FP32 FFTs) keeps the fixed-point positions and phases and runs the
 // taps, sums and butterflies in FP32.
 #include <cstdint>
 
+#include "asy_dev.cuh"
 #include "device_math.cuh"
 #include "df64.cuh"
 #include "nuht_internal.h"
@@ -125,21 +126,6 @@ __device__ __forceinline__ int interp_cell_sv(const AsyBlock& B, int w, double w
     const long long t0 = (A + ((1LL << 40) - 1)) >> 40;                     // ceil
     *svo = 2 * ((t0 << 40) - A) - (1LL << 40);
     return (int)t0;
-}
-
-// psi^(xi) for xi >= 0 given as double-float, double-float throughout: with
-// t = xi times the table's pieces per unit, piece floor(t) (clamped to the
-// table) and v = 2 (t - piece) - 1 in [-1, 1], the compensated Horner sum of
-// that piece's polynomial.
-__device__ __forceinline__ df psihat_of(const Tables& T, df xi)
-{
-    const df t = df_mul(xi, df{T.ph_scale2.x, T.ph_scale2.y});
-    int piece = (int)t.h;
-    if ((float)piece == t.h && t.l < 0.f && piece > 0) --piece;
-    if (piece > T.ph_pieces - 1) piece = T.ph_pieces - 1;
-    const df u = df_add(t, df{-(float)piece, 0.f});
-    const df v = df_add(df{2.f * u.h, 2.f * u.l}, df{-1.f, 0.f});
-    return horner_comp(T.ph2 + piece * (T.ph_deg + 1), T.ph_deg, v.h, v.l, T.ph_comp);
 }
 
 // psi^(xi) for xi = alpha s (s from the fixed-point offset S).
@@ -1042,435 +1028,6 @@ __global__ void k_asy_spread(const ProbParams* __restrict__ probs, const AsyBloc
     }
     else
         spread_taps<MULTI>(B, Q, t, tab, r_s, r2, c2, c_stride, V, moff, gb, smem4);
-}
-
-// -------------------------------------------------------------------- FFT
-// Complex double-float values are float4 (re.h, re.l, im.h, im.l); the FFTs
-// run in double-float on the FP32 pipes (FP64 is 1/64 of the FP32 rate).
-__device__ __forceinline__ float4 cdf(df re, df im) { return make_float4(re.h, re.l, im.h, im.l); }
-
-__device__ __forceinline__ float4 cdf_mul(float4 a, float4 b)
-{
-    const df ar{a.x, a.y}, ai{a.z, a.w}, br{b.x, b.y}, bi{b.z, b.w};
-    return cdf(df_add(df_mul(ar, br), df_negate(df_mul(ai, bi))), df_add(df_mul(ar, bi), df_mul(ai, br)));
-}
-
-__device__ __forceinline__ float4 cdf_scale(float4 a, df s)
-{
-    return cdf(df_mul(df{a.x, a.y}, s), df_mul(df{a.z, a.w}, s));
-}
-
-// u + v w and u - v w
-__device__ __forceinline__ void cdf_butterfly(float4& u, float4& v, float4 w)
-{
-    const float4 vw = cdf_mul(v, w);
-    const df ur{u.x, u.y}, ui{u.z, u.w}, vr{vw.x, vw.y}, vi{vw.z, vw.w};
-    u = cdf(df_add(ur, vr), df_add(ui, vi));
-    v = cdf(df_add(ur, df_negate(vr)), df_add(ui, df_negate(vi)));
-}
-
-// The same on the FP32 parts (x, z) alone (mixed-precision FFTs): the low
-// parts of the results are zero.
-__device__ __forceinline__ float4 cf_mul(float4 a, float4 b)
-{
-    return make_float4(a.x * b.x - a.z * b.z, 0.f, a.x * b.z + a.z * b.x, 0.f);
-}
-
-__device__ __forceinline__ void cf_butterfly(float4& u, float4& v, float4 w)
-{
-    const float4 vw = cf_mul(v, w);
-    const float ur = u.x, ui = u.z;
-    u = make_float4(ur + vw.x, 0.f, ui + vw.z, 0.f);
-    v = make_float4(ur - vw.x, 0.f, ui - vw.z, 0.f);
-}
-
-// A finite double as double-float from its bits (integer and FP32
-// instructions only; FP64 runs at 1/64 of the FP32 rate): the top 24 bits of
-// the significand exactly, the next 29 rounded; zero and subnormals give 0.
-__device__ __forceinline__ df df_from_bits(double x)
-{
-    const long long b = __double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff);
-    if (e == 0) return df{0.f, 0.f};
-    const long long m = (b & 0xFFFFFFFFFFFFFLL) | (1LL << 52);   // x = +-m 2^(e - 1075)
-    float h = ldexpf((float)(int)(m >> 29), e - 1075 + 29);
-    float l = ldexpf((float)(int)(m & 0x1FFFFFFF), e - 1075);
-    if (b < 0) {
-        h = -h;
-        l = -l;
-    }
-    return fast_two_sum(h, l);
-}
-
-// FP64 complex as double-float
-__device__ __forceinline__ float4 cdf_from(double2 v)
-{
-    return cdf(df_from_bits(v.x), df_from_bits(v.y));
-}
-
-// nlines independent FFTs (e^{+2 pi i k n / N}) of N = 2^logN points stored
-// one after the other in shared memory, each in bit-reversed order, sharing
-// every butterfly stage.  tw2[k] = e^{2 pi i k / 2^tw_log2} as double-float.
-// LOWP: the butterflies in FP32 on the values' FP32 parts (mixed precision).
-// The decimation-in-time stages run two at a time (radix 4): a thread loads
-// the four values a group of stages st, st + 1 combines (offsets 0, len,
-// 2 len, 3 len), applies both stages' butterflies in registers and stores them
-// back, so each value crosses shared memory once per two stages and the CTA
-// synchronises half as often.  An odd stage count starts with one radix-2
-// stage (twiddle 1).
-template <bool LOWP>
-__device__ __forceinline__ void fft_bfly(float4& u, float4& v, float4 w)
-{
-    if (LOWP) cf_butterfly(u, v, w);
-    else cdf_butterfly(u, v, w);
-}
-
-template <bool LOWP>
-__device__ void smem_fft_lines(float4* X, int logN, int nlines, const float4* __restrict__ tw2, int tw_log2)
-{
-    const int N = 1 << logN;
-    int st = 0;
-    if (logN & 1) {
-        const int half = N >> 1;
-        const float4 one = tw2[0];
-        for (int b = threadIdx.x; b < nlines * half; b += blockDim.x) {
-            const int i0 = 2 * b;   // stage 0: pairs (2b, 2b + 1), twiddle 1
-            float4 u = X[i0], v = X[i0 + 1];
-            fft_bfly<LOWP>(u, v, one);
-            X[i0] = u;
-            X[i0 + 1] = v;
-        }
-        __syncthreads();
-        st = 1;
-    }
-    const int quarter = N >> 2;
-    for (; st < logN; st += 2) {
-        const int len = 1 << st;
-        const int sh1 = tw_log2 - (st + 1), sh2 = tw_log2 - (st + 2);
-        for (int b = threadIdx.x; b < nlines * quarter; b += blockDim.x) {
-            const int line = b >> (logN - 2);
-            const int bb = b & (quarter - 1);
-            const int pos = bb & (len - 1);
-            const int i0 = line * N + ((bb >> st) << (st + 2)) + pos;
-            float4 a = X[i0], c1 = X[i0 + len], c2 = X[i0 + 2 * len], c3 = X[i0 + 3 * len];
-            const float4 t1 = tw2[pos << sh1];
-            fft_bfly<LOWP>(a, c1, t1);                       // stage st: (0, len), (2 len, 3 len)
-            fft_bfly<LOWP>(c2, c3, t1);
-            fft_bfly<LOWP>(a, c2, tw2[pos << sh2]);          // stage st + 1: (0, 2 len), (len, 3 len)
-            fft_bfly<LOWP>(c1, c3, tw2[(pos + len) << sh2]);
-            X[i0] = a;
-            X[i0 + len] = c1;
-            X[i0 + 2 * len] = c2;
-            X[i0 + 3 * len] = c3;
-        }
-        __syncthreads();
-    }
-}
-
-// The mixed-precision FFT on FP32 complex values (float2: re, im) in shared
-// memory: the stages of smem_fft_lines on half the bytes per value, with the
-// twiddles' FP32 parts.
-__device__ __forceinline__ void cf2_bfly(float2& u, float2& v, float4 w)
-{
-    const float vr = v.x * w.x - v.y * w.z, vi = fmaf(v.x, w.z, v.y * w.x);
-    const float ur = u.x, ui = u.y;
-    u = make_float2(ur + vr, ui + vi);
-    v = make_float2(ur - vr, ui - vi);
-}
-
-__device__ void smem_fft_lines_f32(float2* X, int logN, int nlines, const float4* __restrict__ tw2, int tw_log2)
-{
-    const int N = 1 << logN;
-    int st = 0;
-    if (logN & 1) {
-        const int half = N >> 1;
-        for (int b = threadIdx.x; b < nlines * half; b += blockDim.x) {
-            const int i0 = 2 * b;
-            const float2 u = X[i0], v = X[i0 + 1];
-            X[i0] = make_float2(u.x + v.x, u.y + v.y);
-            X[i0 + 1] = make_float2(u.x - v.x, u.y - v.y);
-        }
-        __syncthreads();
-        st = 1;
-    }
-    const int quarter = N >> 2;
-    for (; st < logN; st += 2) {
-        const int len = 1 << st;
-        const int sh1 = tw_log2 - (st + 1), sh2 = tw_log2 - (st + 2);
-        for (int b = threadIdx.x; b < nlines * quarter; b += blockDim.x) {
-            const int line = b >> (logN - 2);
-            const int bb = b & (quarter - 1);
-            const int pos = bb & (len - 1);
-            const int i0 = line * N + ((bb >> st) << (st + 2)) + pos;
-            float2 a = X[i0], c1 = X[i0 + len], c2 = X[i0 + 2 * len], c3 = X[i0 + 3 * len];
-            const float4 t1 = tw2[pos << sh1];
-            cf2_bfly(a, c1, t1);
-            cf2_bfly(c2, c3, t1);
-            cf2_bfly(a, c2, tw2[pos << sh2]);
-            cf2_bfly(c1, c3, tw2[(pos + len) << sh2]);
-            X[i0] = a;
-            X[i0 + len] = c1;
-            X[i0 + 2 * len] = c2;
-            X[i0 + 3 * len] = c3;
-        }
-        __syncthreads();
-    }
-}
-
-__device__ __forceinline__ float2 cf2_of(float4 v) { return make_float2(v.x, v.z); }
-__device__ __forceinline__ float4 cf4_of(float2 v) { return make_float4(v.x, 0.f, v.y, 0.f); }
-
-// e^{2 pi i m / N} for 0 <= m < N = 2^logN as double-float: the table entry for
-// the top bits of m / N times the rotation by the rest, an angle below
-// 2 pi / 2^tw_log2, from its Taylor series (five terms, truncation < 1e-19).
-__device__ __forceinline__ float4 cdf_twiddle(const Tables& tab, int logN, long long m)
-{
-    const int sh = logN - tab.tw_log2;
-    const int hi = sh > 0 ? (int)(m >> sh) : (int)(m << -sh);   // table index, < 2^tw_log2
-    const int half = 1 << (tab.tw_log2 - 1);
-    float4 t = tab.tw2[hi & (half - 1)];
-    if (hi >= half) t = make_float4(-t.x, -t.y, -t.z, -t.w);
-    const int lo = sh > 0 ? (int)(m & ((1LL << sh) - 1)) : 0;
-    if (lo == 0) return t;
-    // angle 2 pi lo / N: lo / N is exact in FP32 (lo < 2^sh <= 2^11, N a power of two)
-    const df twopi{6.2831854820251465f, -1.7484555314695172e-07f};
-    const df a = df_mul(twopi, df{ldexpf((float)lo, -logN), 0.f});
-    const df a2 = df_mul(a, a);
-    // sin a = a (1 - a^2/6 (1 - a^2/20 (1 - a^2/42))), cos a = 1 - a^2/2 (1 - a^2/12 (1 - a^2/30))
-    df sn = df_add(df{1.f, 0.f}, df_negate(df_mul(a2, df{1.f / 42.f, 0.f})));
-    sn = df_add(df{1.f, 0.f}, df_negate(df_mul(df_mul(a2, df{0.05f, -7.450580707946131e-10f}), sn)));
-    sn = df_add(df{1.f, 0.f}, df_negate(df_mul(df_mul(a2, df{0.1666666716337204f, -4.967053879312289e-09f}), sn)));
-    sn = df_mul(a, sn);
-    df cs = df_add(df{1.f, 0.f}, df_negate(df_mul(a2, df{0.03333333507180214f, -1.7384682293e-09f})));
-    cs = df_add(df{1.f, 0.f}, df_negate(df_mul(df_mul(a2, df{0.0833333358168602f, -2.4835269e-09f}), cs)));
-    cs = df_add(df{1.f, 0.f}, df_negate(df_mul(df_mul(a2, df{0.5f, 0.f}), cs)));
-    return cdf_mul(t, cdf(cs, sn));
-}
-
-// Split of a two-pass FFT of 2^LN points into lines: N2 = 2^ceil(LN/2)
-// points per pass-A line, N1 = 2^floor(LN/2) per pass-B line; each CTA takes
-// as many lines as fit kFftLineBatch points.
-struct FourStep {
-    int logN1, logN2, N1, N2, lpcA, lpcB, groupsA, groupsB;
-};
-__host__ __device__ __forceinline__ FourStep four_step(int LN)
-{
-    FourStep f;
-    f.logN2 = (LN + 1) >> 1;
-    f.logN1 = LN - f.logN2;
-    f.N1 = 1 << f.logN1;
-    f.N2 = 1 << f.logN2;
-    f.lpcA = kFftLineBatch >> f.logN2; if (f.lpcA < 1) f.lpcA = 1;
-    f.lpcB = kFftLineBatch >> f.logN1; if (f.lpcB < 1) f.lpcB = 1;
-    f.groupsA = (f.N1 + f.lpcA - 1) / f.lpcA;
-    f.groupsB = (f.N2 + f.lpcB - 1) / f.lpcB;
-    return f;
-}
-
-// 1 / psi^(alpha2 l): the correction of mode l of the inner FFT, in
-// double-float (|l| <= N1 < 2^24 is exact in FP32).
-__device__ __forceinline__ df mode_correction(const AsyBlock& B, const Tables& tab, int l)
-{
-    const df a2 = df_from_bits(B.alpha2);
-    return df_recip(psihat_of(tab, df_mul(a2, df{(float)(l < 0 ? -l : l), 0.f})));
-}
-
-// FFT input / output of the forward (ADJ = false) and the transposed
-// (ADJ = true) type-3 pipelines.  Forward: modes l (|l| <= N1) of the spread
-// grid src (at b_off), corrected by 1/psi^(alpha2 l), transformed to every t
-// and stored at dst + q_off.  Transposed: the target grid src (at q_off,
-// every t) is transformed (the DFT matrix e^{2 pi i l t / nf2} is symmetric),
-// and only the modes |l| <= N1 are kept, corrected, and stored at dst + b_off.
-template <bool ADJ>
-__device__ __forceinline__ float4 fft_in(const AsyBlock& B, const Tables& tab, const double2* __restrict__ src,
-                                         int Q, int q, int tt)
-{
-    if (ADJ) return cdf_from(src[B.q_off + (int64_t)tt * Q + q]);
-    const int l = (tt < (B.nf2 >> 1)) ? tt : tt - B.nf2;
-    if (l < -B.N1 || l > B.N1) return make_float4(0.f, 0.f, 0.f, 0.f);
-    return cdf_scale(cdf_from(src[B.b_off + (int64_t)(l + B.N1) * Q + q]), mode_correction(B, tab, l));
-}
-
-template <bool ADJ>
-__device__ __forceinline__ void fft_out(const AsyBlock& B, const Tables& tab, float4* __restrict__ dst, int Q,
-                                        int q, int tt, float4 v)
-{
-    if (!ADJ) {
-        dst[B.q_off + (int64_t)tt * Q + q] = v;
-        return;
-    }
-    const int l = (tt < (B.nf2 >> 1)) ? tt : tt - B.nf2;
-    if (l < -B.N1 || l > B.N1) return;
-    dst[B.b_off + (int64_t)(l + B.N1) * Q + q] = cdf_scale(v, mode_correction(B, tab, l));
-}
-
-template <bool ADJ, bool LOWP>
-__global__ void k_asy_fft_small(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                                const Tile* __restrict__ items, Tables tab,
-                                const double2* __restrict__ src, float4* __restrict__ dst, int64_t src_stride,
-                                int64_t dst_stride)
-{
-    extern __shared__ float4 Xs[];
-    src += blockIdx.y * src_stride;   // member blockIdx.y of a batch of real components
-    dst += blockIdx.y * dst_stride;
-    const Tile it = items[blockIdx.x];
-    const AsyBlock B = blks[it.blk];
-    const int Q = probs[B.prob].Q;
-    const int q = (int)it.start;
-    const int N = B.nf2, logN = B.log2nf2;
-    float2* Xf = reinterpret_cast<float2*>(Xs);   // LOWP: FP32 values
-    for (int tt = threadIdx.x; tt < N; tt += blockDim.x) {
-        const float4 v = fft_in<ADJ>(B, tab, src, Q, q, tt);
-        if (LOWP) Xf[__brev(tt) >> (32 - logN)] = cf2_of(v);
-        else Xs[__brev(tt) >> (32 - logN)] = v;
-    }
-    __syncthreads();
-    if (LOWP) smem_fft_lines_f32(Xf, logN, 1, tab.tw2, tab.tw_log2);
-    else smem_fft_lines<false>(Xs, logN, 1, tab.tw2, tab.tw_log2);
-    for (int tt = threadIdx.x; tt < N; tt += blockDim.x)
-        fft_out<ADJ>(B, tab, dst, Q, q, tt, LOWP ? cf4_of(Xf[tt]) : Xs[tt]);
-}
-
-// All Q grids of one small block (nf2 * Q <= kFftSmemMax) in one CTA: the
-// deconvolution factor of each mode is computed once and used for every q;
-// the Q transforms share every butterfly stage.  A launch takes the blocks
-// with pts_lo < nf2 * Q <= pts_hi (the others return at once), so that small
-// blocks run in CTAs sized for them.
-template <bool ADJ, bool LOWP>
-__global__ void k_asy_fft_block(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                                const Tile* __restrict__ items, Tables tab,
-                                const double2* __restrict__ src, float4* __restrict__ dst, int pts_lo, int pts_hi,
-                                int64_t src_stride, int64_t dst_stride)
-{
-    extern __shared__ float4 Xs[];   // [Q][N], each grid bit-reversed
-    src += blockIdx.y * src_stride;   // member blockIdx.y of a batch of real components
-    dst += blockIdx.y * dst_stride;
-    const Tile it = items[blockIdx.x];
-    const AsyBlock B = blks[it.blk];
-    const int Q = probs[B.prob].Q;
-    const int pts = B.nf2 * Q;
-    if (pts <= pts_lo || pts > pts_hi) return;
-    const int N = B.nf2, logN = B.log2nf2, half = N >> 1;
-    float2* Xf = reinterpret_cast<float2*>(Xs);   // LOWP: FP32 values
-    auto put = [&](int i, float4 v) {
-        if (LOWP) Xf[i] = cf2_of(v);
-        else Xs[i] = v;
-    };
-    for (int tt = threadIdx.x; tt < N; tt += blockDim.x) {
-        const int l = (tt < half) ? tt : tt - N;
-        const int dst_i = __brev(tt) >> (32 - logN);
-        if (ADJ) {
-            const double2* row = src + B.q_off + (int64_t)tt * Q;
-            for (int q = 0; q < Q; ++q) put(q * N + dst_i, cdf_from(row[q]));
-        } else if (l < -B.N1 || l > B.N1) {
-            for (int q = 0; q < Q; ++q) put(q * N + dst_i, make_float4(0.f, 0.f, 0.f, 0.f));
-        } else {
-            const df sc = mode_correction(B, tab, l);
-            const double2* row = src + B.b_off + (int64_t)(l + B.N1) * Q;
-            for (int q = 0; q < Q; ++q) put(q * N + dst_i, cdf_scale(cdf_from(row[q]), sc));
-        }
-    }
-    __syncthreads();
-    if (LOWP) smem_fft_lines_f32(Xf, logN, Q, tab.tw2, tab.tw_log2);
-    else smem_fft_lines<false>(Xs, logN, Q, tab.tw2, tab.tw_log2);
-    auto get = [&](int i) { return LOWP ? cf4_of(Xf[i]) : Xs[i]; };
-    if (!ADJ) {
-        float4* gq = dst + B.q_off;
-        for (int idx = threadIdx.x; idx < N * Q; idx += blockDim.x) {
-            const int tt = idx / Q, q = idx - tt * Q;
-            gq[idx] = get(q * N + tt);
-        }
-    } else {
-        const int nf1 = 2 * B.N1 + 1;
-        float4* gb = dst + B.b_off;
-        for (int li = threadIdx.x; li < nf1; li += blockDim.x) {
-            const int l = li - B.N1;
-            const df sc = mode_correction(B, tab, l);
-            for (int q = 0; q < Q; ++q) gb[(int64_t)li * Q + q] = cdf_scale(get(q * N + (l & (N - 1))), sc);
-        }
-    }
-}
-
-// Two-pass (four-step) FFT for nf2 = N1 * N2 > kFftSingleMax.
-// Pass A: for each n1, FFT over n2 of x[n1 + N1 n2], times e^{2 pi i n1 k2 / N},
-// stored at tmp[n1 + N1 k2].  Pass B: for each k2, FFT over n1 of
-// tmp[n1 + N1 k2], which is X[k2 + N2 k1].  Work item ordinal = g * Q + q,
-// g a group of lines handled by one CTA: the Q CTAs of a group run side by
-// side and read and write the same rows of the [point][Q] grids (one row is
-// all Q values of a point), so a row moves through HBM once, not once per q.
-template <bool ADJ, bool LOWP>
-__global__ void k_asy_fft_pass_a(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                                 const Tile* __restrict__ items, Tables tab,
-                                 const double2* __restrict__ src, float4* __restrict__ tmp)
-{
-    extern __shared__ float4 Xs[];
-    const Tile it = items[blockIdx.x];
-    const AsyBlock B = blks[it.blk];
-    const int Q = probs[B.prob].Q;
-    const int N = B.nf2;
-    const FourStep f = four_step(B.log2nf2);
-    const int g = (int)(it.start / Q);
-    const int iq = (int)(it.start - (int64_t)g * Q);
-    const int l0 = g * f.lpcA;
-    const int nl = (f.N1 - l0) < f.lpcA ? (f.N1 - l0) : f.lpcA;
-    float2* Xf = reinterpret_cast<float2*>(Xs);   // LOWP: FP32 values
-    for (int idx = threadIdx.x; idx < nl * f.N2; idx += blockDim.x) {
-        const int li = idx >> f.logN2, n2 = idx & (f.N2 - 1);
-        const int i = li * f.N2 + (__brev(n2) >> (32 - f.logN2));
-        const float4 v = fft_in<ADJ>(B, tab, src, Q, iq, (l0 + li) + f.N1 * n2);
-        if (LOWP) Xf[i] = cf2_of(v);
-        else Xs[i] = v;
-    }
-    __syncthreads();
-    if (LOWP) smem_fft_lines_f32(Xf, f.logN2, nl, tab.tw2, tab.tw_log2);
-    else smem_fft_lines<false>(Xs, f.logN2, nl, tab.tw2, tab.tw_log2);
-    for (int idx = threadIdx.x; idx < nl * f.N2; idx += blockDim.x) {
-        const int li = idx >> f.logN2, k2 = idx & (f.N2 - 1);
-        const int n1 = l0 + li;
-        const long long m = ((long long)n1 * k2) & (N - 1);   // e^{2 pi i n1 k2 / N}
-        const int64_t o = B.q_off + (int64_t)(n1 + f.N1 * k2) * Q + iq;
-        if (LOWP) {
-            // FP32 twiddle (m / N is exact in FP32, N <= 2^24); the pass
-            // temporary holds FP32 complex values (float2, half the bytes)
-            float sn, cs;
-            sincospif(ldexpf(2.f * (float)m, -B.log2nf2), &sn, &cs);
-            const float2 x = Xf[idx];
-            reinterpret_cast<float2*>(tmp)[o] = make_float2(x.x * cs - x.y * sn, fmaf(x.x, sn, x.y * cs));
-        } else {
-            tmp[o] = cdf_mul(Xs[idx], cdf_twiddle(tab, B.log2nf2, m));
-        }
-    }
-}
-
-template <bool ADJ, bool LOWP>
-__global__ void k_asy_fft_pass_b(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                                 const Tile* __restrict__ items, Tables tab,
-                                 const float4* __restrict__ tmp, float4* __restrict__ dst)
-{
-    extern __shared__ float4 Xs[];
-    const Tile it = items[blockIdx.x];
-    const AsyBlock B = blks[it.blk];
-    const int Q = probs[B.prob].Q;
-    const FourStep f = four_step(B.log2nf2);
-    const int g = (int)(it.start / Q);
-    const int iq = (int)(it.start - (int64_t)g * Q);
-    const int k20 = g * f.lpcB;
-    const int nl = (f.N2 - k20) < f.lpcB ? (f.N2 - k20) : f.lpcB;
-    float2* Xf = reinterpret_cast<float2*>(Xs);   // LOWP: FP32 values
-    for (int idx = threadIdx.x; idx < nl * f.N1; idx += blockDim.x) {
-        const int li = idx >> f.logN1, n1 = idx & (f.N1 - 1);
-        const int i = li * f.N1 + (f.logN1 > 0 ? (__brev(n1) >> (32 - f.logN1)) : 0);
-        const int64_t o = B.q_off + (int64_t)(n1 + f.N1 * (k20 + li)) * Q + iq;
-        if (LOWP) Xf[i] = reinterpret_cast<const float2*>(tmp)[o];
-        else Xs[i] = tmp[o];
-    }
-    __syncthreads();
-    if (LOWP) smem_fft_lines_f32(Xf, f.logN1, nl, tab.tw2, tab.tw_log2);
-    else smem_fft_lines<false>(Xs, f.logN1, nl, tab.tw2, tab.tw_log2);
-    for (int idx = threadIdx.x; idx < nl * f.N1; idx += blockDim.x) {
-        const int li = idx >> f.logN1, k1 = idx & (f.N1 - 1);
-        fft_out<ADJ>(B, tab, dst, Q, iq, (k20 + li) + f.N2 * k1, LOWP ? cf4_of(Xf[idx]) : Xs[idx]);
-    }
 }
 
 // ------------------------------------------------------------ interpolate
@@ -2639,85 +2196,6 @@ cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, con
     kern<<<ntiles, nt, smem, s>>>(probs, blks, tiles, modes, tab, r_s, r2, c2, c_stride, members, grid_b,
                                   gb_stride);
     count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_asy_fft_small(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
-                                 int nitems, int max_nf2, Tables tab, const double2* src,
-                                 float4* dst, cudaStream_t s, bool adj, bool lowp, int members,
-                                 int64_t src_stride, int64_t dst_stride)
-{
-    if (nitems <= 0) return cudaSuccess;
-    if (members < 1 || members > 65535) return cudaErrorInvalidValue;
-    size_t smem = (lowp ? sizeof(float2) : sizeof(float4)) * (size_t)max_nf2;
-    auto kern = adj ? (lowp ? k_asy_fft_small<true, true> : k_asy_fft_small<true, false>)
-                    : (lowp ? k_asy_fft_small<false, true> : k_asy_fft_small<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int nt = max_nf2 / 2;
-    if (nt > 256) nt = 256;
-    if (nt < 32) nt = 32;
-    kern<<<dim3(nitems, members), nt, smem, s>>>(probs, blks, items, tab, src, dst, src_stride, dst_stride);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_asy_fft_block(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
-                                 int nitems, int max_pts, Tables tab, const double2* src, float4* dst,
-                                 cudaStream_t s, bool adj, bool lowp, int members, int64_t src_stride,
-                                 int64_t dst_stride)
-{
-    if (nitems <= 0) return cudaSuccess;
-    if (members < 1 || members > 65535) return cudaErrorInvalidValue;
-    if (max_pts < 1 || max_pts > kFftSmemMax) max_pts = kFftSmemMax;
-    auto kern = adj ? (lowp ? k_asy_fft_block<true, true> : k_asy_fft_block<true, false>)
-                    : (lowp ? k_asy_fft_block<false, true> : k_asy_fft_block<false, false>);
-    // blocks of up to kFftSmallPts points in small CTAs (16 KiB, many per SM),
-    // the larger ones in CTAs sized for the largest; each launch skips the
-    // other size class at once
-    constexpr int kFftSmallPts = 1024;
-    const int ranges[2][2] = {{0, max_pts < kFftSmallPts ? max_pts : kFftSmallPts}, {kFftSmallPts, max_pts}};
-    int launched = 0;
-    for (int r = 0; r < 2; ++r) {
-        const int lo = ranges[r][0], hi = ranges[r][1];
-        if (hi <= lo) continue;
-        const size_t smem = (lowp ? sizeof(float2) : sizeof(float4)) * (size_t)hi;
-        int nt = ((hi / 2 + 31) / 32) * 32;
-        if (r == 0 && nt > 128) nt = 128;
-        if (nt > 256) nt = 256;
-        if (nt < 32) nt = 32;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<dim3(nitems, members), nt, smem, s>>>(probs, blks, items, tab, src, dst, lo, hi, src_stride,
-                                                     dst_stride);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        ++launched;
-    }
-    count_launches(launched);
-    return cudaSuccess;
-}
-
-cudaError_t launch_asy_fft_large(const ProbParams* probs, const AsyBlock* blks, const Tile* items_a,
-                                 int nitems_a, const Tile* items_b, int nitems_b, Tables tab,
-                                 const double2* src, float4* tmp, float4* dst,
-                                 cudaStream_t s, bool adj, bool lowp)
-{
-    if (nitems_a <= 0) return cudaSuccess;
-    size_t smem = (lowp ? sizeof(float2) : sizeof(float4)) * (size_t)kFftLineBatch;
-    auto ka = adj ? (lowp ? k_asy_fft_pass_a<true, true> : k_asy_fft_pass_a<true, false>)
-                  : (lowp ? k_asy_fft_pass_a<false, true> : k_asy_fft_pass_a<false, false>);
-    auto kb = adj ? (lowp ? k_asy_fft_pass_b<true, true> : k_asy_fft_pass_b<true, false>)
-                  : (lowp ? k_asy_fft_pass_b<false, true> : k_asy_fft_pass_b<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    ka<<<nitems_a, 256, smem, s>>>(probs, blks, items_a, tab, src, tmp);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    kb<<<nitems_b, 256, smem, s>>>(probs, blks, items_b, tab, tmp, dst);
-    count_launches(2);
     return cudaGetLastError();
 }
 

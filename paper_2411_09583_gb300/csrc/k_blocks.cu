@@ -151,6 +151,11 @@ __global__ void k_block_sizes(BlockBuild bb)
                     continue;
                 }
             }
+            {
+                // the largest FFT-grid position of a frequency, and w cells around it
+                const double te = ceil(fmax(e.w - ab.wc, ab.wc - e.z) * ab.hd) + bb.w + 2.0;
+                ab.tmax = te < (double)ab.nf2 ? (int32_t)te : ab.nf2;
+            }
             ab.rho_h = (float)ab.rho;
             ab.rho_l = (float)(ab.rho - (double)ab.rho_h);
             bb.asy[a] = ab;
@@ -159,7 +164,18 @@ __global__ void k_block_sizes(BlockBuild bb)
             c[AC_GQ] = (int64_t)ab.nf2 * Q;
             c[AC_TSPREAD] = ceil_div(cols, bb.spread_tile);
             c[AC_TINTERP] = ceil_div(rows, bb.interp_tile);
-            if ((int64_t)ab.nf2 * Q <= kFftSmemMax) {             // all Q grids in one CTA
+            atomic_max64(&bb.maxv[MX_LOG2], lg);
+            {
+                const int np = fft_split(lg).np;
+                c[AC_IP0] = fft_tile(lg, 0, Q).ntiles;
+                c[AC_NP1] = np > 1;
+                c[AC_NP2] = np > 2;
+                if (np > 1) c[AC_IP1] = fft_tile(lg, 1, Q).ntiles;
+                if (np > 2) c[AC_IP2] = fft_tile(lg, 2, Q).ntiles;
+            }
+            if (!bb.lowp) {
+                // double-float FFTs only
+            } else if ((int64_t)ab.nf2 * Q <= kFftSmemMax) {      // all Q grids in one CTA
                 bb.fcls[a] = 0;
                 c[AC_NFK] = 1;
                 c[AC_IFK] = 1;
@@ -177,7 +193,6 @@ __global__ void k_block_sizes(BlockBuild bb)
                 const int lpcB = (kFftLineBatch >> logN1) > 0 ? (kFftLineBatch >> logN1) : 1;
                 c[AC_IFA] = (int64_t)Q * (((1 << logN1) + lpcA - 1) / lpcA);
                 c[AC_IFB] = (int64_t)Q * (((1 << logN2) + lpcB - 1) / lpcB);
-                atomic_max64(&bb.maxv[MX_LARGE], 1);
             }
             c[AC_RC] = rows + cols;
             c[AC_NF2] = ab.nf2;
@@ -317,6 +332,9 @@ __global__ void k_block_fill(BlockBuild bb, BuildLists L)
         L.pre[LIST_FSMALL][ta[AC_NFS]] = (int32_t)ta[AC_IFS];
         L.pre[LIST_FA][ta[AC_NFL]] = (int32_t)ta[AC_IFA];
         L.pre[LIST_FB][ta[AC_NFL]] = (int32_t)ta[AC_IFB];
+        L.pre[LIST_P0][na] = (int32_t)ta[AC_IP0];
+        L.pre[LIST_P1][ta[AC_NP1]] = (int32_t)ta[AC_IP1];
+        L.pre[LIST_P2][ta[AC_NP2]] = (int32_t)ta[AC_IP2];
     }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl + na + nd;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -338,7 +356,15 @@ __global__ void k_block_fill(BlockBuild bb, BuildLists L)
             put_seg(L, LIST_SPREAD, a, (int32_t)a, bb.spread_tile, ab.j0, ab.j1, c[AC_TSPREAD]);
             put_seg(L, LIST_INTERP, a, (int32_t)a, bb.interp_tile, ab.k0, ab.k1, c[AC_TINTERP]);
             const int Q = bb.probs[ab.prob].Q;
-            if (bb.fcls[a] == 0) {
+            const int np = fft_split(ab.log2nf2).np;
+            put_seg(L, LIST_P0, a, (int32_t)a, 1, 0, fft_tile(ab.log2nf2, 0, Q).ntiles - 1, c[AC_IP0]);
+            if (np > 1)
+                put_seg(L, LIST_P1, c[AC_NP1], (int32_t)a, 1, 0, fft_tile(ab.log2nf2, 1, Q).ntiles - 1, c[AC_IP1]);
+            if (np > 2)
+                put_seg(L, LIST_P2, c[AC_NP2], (int32_t)a, 1, 0, fft_tile(ab.log2nf2, 2, Q).ntiles - 1, c[AC_IP2]);
+            if (bb.fcls[a] < 0) {
+                // no FP32 FFT
+            } else if (bb.fcls[a] == 0) {
                 put_seg(L, LIST_FBLOCK, c[AC_NFK], (int32_t)a, 1, 0, 0, c[AC_IFK]);
             } else if (bb.fcls[a] == 1) {
                 put_seg(L, LIST_FSMALL, c[AC_NFS], (int32_t)a, 1, 0, Q - 1, c[AC_IFS]);

@@ -25,10 +25,55 @@ constexpr double kAsyMaxXS = 3.2e6;
 constexpr int kMomFold = 32;        // FP32 partial sums of the spreading moments span at most this many points
 constexpr int kMaxNtop = 400;       // largest Bessel index kept by the local evaluation
                                     // (the transposed moments then stay within 205 KB of shared memory)
+constexpr int kFftMaxLog2 = 24;     // largest FFT
+// Double-float FFT (k_asy_fft): tiles of up to kFftTileVals values (32 KiB)
+// and kFftTilePts points, at most kFftQMax Hankel terms each.
+constexpr int kFftThreads = 128;
+constexpr int kFftTileVals = 2048;
+constexpr int kFftTilePts = 512;
+constexpr int kFftQMax = 12;
+// Mixed-precision FFT (FP32 butterflies)
 constexpr int kFftSmemMax = 4096;   // points of all Q grids of a block FFT'd by one CTA
-constexpr int kFftSingleMax = 8192; // largest single-grid FFT done by one CTA (128 KiB)
+constexpr int kFftSingleMax = 8192; // largest single-grid FFT done by one CTA (64 KiB)
 constexpr int kFftLineBatch = 4096; // points per CTA in the passes of a two-pass FFT
-constexpr int kFftMaxLog2 = 24;     // largest FFT (two passes of <= 4096-point lines)
+
+// Passes of a double-float FFT of 2^LN points, 5 <= LN <= 24: lines of 2^lg
+// points, 5 <= lg <= 9, pass 0 the slowest digit; a line's points lie 2^lgst
+// rows apart in pass p.
+struct FftSplit {
+    int np, lg0, lg1, lg2, LN;
+    __host__ __device__ int lg(int p) const { return p == 0 ? lg0 : (p == 1 ? lg1 : lg2); }
+    __host__ __device__ int lgst(int p) const { return LN - lg0 - (p > 0 ? lg1 : 0) - (p > 1 ? lg2 : 0); }
+};
+__host__ __device__ inline FftSplit fft_split(int LN)
+{
+    if (LN <= 9) return FftSplit{1, LN, 0, 0, LN};
+    if (LN <= 18) return FftSplit{2, (LN + 1) >> 1, LN >> 1, 0, LN};
+    const int a = (LN + 2) / 3, b = (LN - a + 1) >> 1;
+    return FftSplit{3, a, b, LN - a - b, LN};
+}
+
+// The tiles of a pass: 2^lgl lines of 2^lg points, qc of the Q terms (nqc
+// chunks cover them), ntiles in all.
+struct FftTile {
+    int lg, lgl, qc, nqc;
+    int64_t ntiles;
+};
+__host__ __device__ inline FftTile fft_tile(int LN, int pass, int Q)
+{
+    FftTile T;
+    T.lg = fft_split(LN).lg(pass);
+    const int lines = LN - T.lg;   // log2
+    int qm = kFftTileVals >> T.lg;
+    if (qm > kFftQMax) qm = kFftQMax;
+    T.nqc = (Q + qm - 1) / qm;
+    T.qc = (Q + T.nqc - 1) / T.nqc;
+    T.lgl = 0;
+    while (T.lgl < lines && (T.qc << (T.lg + T.lgl + 1)) <= kFftTileVals && (2 << (T.lg + T.lgl)) <= kFftTilePts)
+        ++T.lgl;
+    T.ntiles = ((int64_t)1 << (lines - T.lgl)) * T.nqc;
+    return T;
+}
 
 // Per-problem constants.
 struct ProbParams {
@@ -95,7 +140,7 @@ struct AsyBlock {
     int64_t Wc_fx, KD, KRc;
     int32_t fw, sD, sR;
     float alpha_h, alpha_l;   // alpha as double-float
-    int32_t pad_fx2;
+    int32_t tmax;             // the interpolation reads FFT rows |t| <= tmax only
 };
 
 struct DirectBlock {
@@ -128,12 +173,13 @@ struct SubBlk {
 // (columns), their exclusive prefix sums and totals, maxima, and the tile lists.
 enum { LC_MOM, LC_TMOM, LC_TEVAL, LC_RC, kLocalCols };
 enum { AC_GB, AC_GQ, AC_TSPREAD, AC_TINTERP, AC_NFK, AC_NFS, AC_NFL, AC_IFK, AC_IFS, AC_IFA, AC_IFB,
-       AC_RC, AC_NF2, kAsyCols };
+       AC_RC, AC_NF2, AC_IP0, AC_IP1, AC_IP2, AC_NP1, AC_NP2, kAsyCols };
 enum { DC_ENTRIES, kDirCols };
 enum { TOT_LOCAL = 0, TOT_ASY = kLocalCols, TOT_DIR = kLocalCols + kAsyCols,
        kTotals = kLocalCols + kAsyCols + kDirCols };
-enum { MX_DIR_ROWS, MX_DIR_COLS, MX_DIR_AREA, MX_NF2_SMALL, MX_LARGE, MX_ERR, MX_FBLOCK_PTS, kMaxv };
-enum { LIST_MOM, LIST_EVAL, LIST_SPREAD, LIST_INTERP, LIST_FSMALL, LIST_FA, LIST_FB, LIST_FBLOCK, kLists };
+enum { MX_DIR_ROWS, MX_DIR_COLS, MX_DIR_AREA, MX_NF2_SMALL, MX_LOG2, MX_ERR, MX_FBLOCK_PTS, kMaxv };
+enum { LIST_MOM, LIST_EVAL, LIST_SPREAD, LIST_INTERP, LIST_FSMALL, LIST_FA, LIST_FB, LIST_FBLOCK,
+       LIST_P0, LIST_P1, LIST_P2, kLists };
 
 struct BlockBuild {
     const int64_t* res;       // counts of local, asymptotic, direct blocks (device)
@@ -143,10 +189,11 @@ struct BlockBuild {
     const double4* ba;        // [na] (r_j0, r_j1, omega_k0, omega_k1) of each asymptotic block
     const ProbParams* probs;
     int w, mom_tile, eval_tile, spread_tile, interp_tile;
+    int lowp;                 // mixed precision: the FP32 FFT's lists are built too
     LocalBlock* loc;          // descriptors before their offsets are known
     AsyBlock* asy;
     DirectBlock* dir;
-    int8_t* fcls;             // FFT class of each asymptotic block (0 one CTA, 1 per grid, 2 two passes)
+    int8_t* fcls;             // FP32 FFT class of each asymptotic block (0 one CTA, 1 per grid, 2 two passes; -1 none)
     int64_t* lcnt;            // [nl][kLocalCols] counters, then exclusive prefix sums
     int64_t* acnt;            // [na][kAsyCols]
     int64_t* dcnt;            // [nd][kDirCols]
@@ -339,22 +386,26 @@ cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks,
                                   int ntiles, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
                                   const float4* grid_q, int64_t gq_stride, int members, double* g_s,
                                   int64_t g_stride, cudaStream_t s);
-// lowp: FP32 butterflies on the FP32 parts of the values (mixed precision).
-// members: a batch of real components (grids src + v src_stride -> dst + v
-// dst_stride) in one launch.
-cudaError_t launch_asy_fft_small(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
-                                 int nitems, int max_nf2, Tables tab, const double2* src,
-                                 float4* dst, cudaStream_t s, bool adj = false, bool lowp = false,
-                                 int members = 1, int64_t src_stride = 0, int64_t dst_stride = 0);
+// One pass of the double-float FFTs (pass 0 reads src, the last one of a block
+// writes dst, tmp between); adj: the transposed transform.  smem: the largest
+// fft_smem_bytes over the plan's Q.  members: a batch of real components (grids
+// src + v src_stride -> dst + v dst_stride) in one launch.
+size_t fft_smem_bytes(int max_log2, int pass, int Q);
+cudaError_t launch_asy_fft(const ProbParams* probs, const AsyBlock* blks, const Tile* items, int nitems,
+                           size_t smem, int pass, Tables tab, const double2* src, float4* tmp, float4* dst,
+                           cudaStream_t s, bool adj, int members, int64_t src_stride, int64_t tmp_stride,
+                           int64_t dst_stride);
+// Mixed-precision forward FFTs (FP32 butterflies).
+cudaError_t launch_asy_fft_small_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
+                                     int nitems, int max_nf2, Tables tab, const double2* src, float4* dst,
+                                     cudaStream_t s, int members, int64_t src_stride, int64_t dst_stride);
 // max_pts: the largest nf2 * Q among the blocks of the list (sizes the CTA).
-cudaError_t launch_asy_fft_block(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
-                                 int nitems, int max_pts, Tables tab, const double2* src, float4* dst,
-                                 cudaStream_t s, bool adj = false, bool lowp = false, int members = 1,
-                                 int64_t src_stride = 0, int64_t dst_stride = 0);
-cudaError_t launch_asy_fft_large(const ProbParams* probs, const AsyBlock* blks, const Tile* items_a,
-                                 int nitems_a, const Tile* items_b, int nitems_b, Tables tab,
-                                 const double2* src, float4* tmp, float4* dst,
-                                 cudaStream_t s, bool adj = false, bool lowp = false);
+cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* items,
+                                     int nitems, int max_pts, Tables tab, const double2* src, float4* dst,
+                                     cudaStream_t s, int members, int64_t src_stride, int64_t dst_stride);
+cudaError_t launch_asy_fft_large_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* items_a,
+                                     int nitems_a, const Tile* items_b, int nitems_b, Tables tab,
+                                     const double2* src, float2* tmp, float4* dst, cudaStream_t s);
 // members: real components interpolated by one launch (FFT outputs grid_q + v
 // gq_stride, sums into g_s + v g_stride).
 cudaError_t launch_asy_interp(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,

@@ -47,26 +47,6 @@ struct Arena {
     }
 };
 
-// Segments of a tile list plus their exclusive prefix of tile counts; the
-// tiles themselves are expanded on the device.
-struct SegList {
-    std::vector<Seg> segs;
-    std::vector<int32_t> prefix{0};
-    void add(int32_t blk, int64_t first, int64_t last, int len)
-    {
-        const int64_t cnt = (last - first + len) / len;
-        segs.push_back(Seg{blk, len, first, last});
-        prefix.push_back(prefix.back() + (int32_t)cnt);
-    }
-    void reserve(size_t k)
-    {
-        segs.reserve(k);
-        prefix.reserve(k + 1);
-    }
-    int nseg() const { return (int)segs.size(); }
-    int total() const { return prefix.back(); }
-};
-
 }  // namespace
 
 struct nuht_plan_s {
@@ -95,13 +75,14 @@ struct nuht_plan_s {
     AsyBlock* d_asy = nullptr;
     Tile *d_tspread = nullptr, *d_tinterp = nullptr;
     int32_t* d_smode = nullptr;   // path of each spreading tile (k_spread_modes)
-    Tile *d_fblock = nullptr, *d_fsmall = nullptr, *d_fa = nullptr, *d_fb = nullptr;
+    Tile *d_fblock = nullptr, *d_fsmall = nullptr, *d_fa = nullptr, *d_fb = nullptr;   // FP32 FFTs
+    Tile* d_fpass[3] = {nullptr, nullptr, nullptr};   // passes of the double-float FFTs
     DirectBlock* d_dir = nullptr;
     double* d_mom = nullptr;
     double2* d_gb = nullptr;
-    float4* d_gtmp = nullptr;   // two-pass FFT intermediate (double-float)
     float4* d_gq = nullptr;   // FFT output, complex values as double-float parts
-    double2* d_tg = nullptr;  // adjoint: frequencies spread onto the FFT grid
+    double2* d_tg = nullptr;  // adjoint: frequencies spread onto the FFT grid; the forward FFT's intermediate
+                              // (and d_gq the adjoint's)
     float4* d_bq = nullptr;   // adjoint: corrected modes, double-float parts
     double *d_cs = nullptr, *d_gs = nullptr;
     float2 *d_r2 = nullptr, *d_w2 = nullptr, *d_cs2 = nullptr;   // double-float copies
@@ -136,7 +117,8 @@ struct nuht_plan_s {
     // interpolation, FP64 path): grids for that many are allocated
     int asy_members = 1;
     int interp_threads = kInterpTileMax;   // frequencies per interpolation tile (one thread each)
-    bool has_large_fft = false;
+    int n_fpass[3] = {0, 0, 0};
+    size_t fft_smem[3] = {0, 0, 0};
     Tables tab{};
     SubBlk* d_blk = nullptr;          // every block (local, asymptotic, direct), global sorted indices
     int64_t direct_entries = 0, local_rc = 0, asy_rc = 0, fft_points = 0;
@@ -721,6 +703,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     bb.ba = d_ba;
     bb.probs = d_prb;
     bb.w = P->w;
+    bb.lowp = P->opt.precision == NUHT_PREC_MIXED;
     bb.mom_tile = kMomentTile;
     bb.eval_tile = P->eval_threads;
     bb.spread_tile = sp_tile;
@@ -844,10 +827,20 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     P->max_dir_area = (int)hmax[MX_DIR_AREA];
     P->max_nf2_small = (int)hmax[MX_NF2_SMALL];
     P->max_fblock_pts = (int)hmax[MX_FBLOCK_PTS];
-    P->has_large_fft = hmax[MX_LARGE] != 0;
-    const int64_t nseg[kLists] = {nl, nl, na, na, ta_[AC_NFS], ta_[AC_NFL], ta_[AC_NFL], ta_[AC_NFK]};
+    P->n_fpass[0] = (int)ta_[AC_IP0]; P->n_fpass[1] = (int)ta_[AC_IP1]; P->n_fpass[2] = (int)ta_[AC_IP2];
+    {
+        // the largest tile of each FFT pass, over the problems' distinct Q
+        bool seen[kMaxQ + 1] = {};
+        for (const ProbParams& q : probs) seen[q.Q] = true;
+        for (int q = 1; q <= kMaxQ; ++q)
+            for (int ps = 0; seen[q] && ps < 3; ++ps)
+                P->fft_smem[ps] = std::max(P->fft_smem[ps], fft_smem_bytes((int)hmax[MX_LOG2], ps, q));
+    }
+    const int64_t nseg[kLists] = {nl, nl, na, na, ta_[AC_NFS], ta_[AC_NFL], ta_[AC_NFL], ta_[AC_NFK],
+                                  na, ta_[AC_NP1], ta_[AC_NP2]};
     const int64_t ntile[kLists] = {tl[LC_TMOM], tl[LC_TEVAL], ta_[AC_TSPREAD], ta_[AC_TINTERP],
-                                   ta_[AC_IFS], ta_[AC_IFA], ta_[AC_IFB], ta_[AC_IFK]};
+                                   ta_[AC_IFS], ta_[AC_IFA], ta_[AC_IFB], ta_[AC_IFK],
+                                   ta_[AC_IP0], ta_[AC_IP1], ta_[AC_IP2]};
     P->plan_ms[1] = ms_since(clk);
 
     // ---- one device arena for everything the plan keeps -------------------
@@ -887,7 +880,6 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     size_t a_gb = A.reserve<double2>((size_t)P->asy_members * (size_t)P->gb_len);
     size_t a_gq = A.reserve<float4>((size_t)P->asy_members * (size_t)P->gq_len);
-    size_t a_gt = A.reserve<float4>(P->has_large_fft ? (size_t)P->gq_len : 1);
     size_t a_cs = A.reserve<double>(gcopies * (size_t)n), a_gs = A.reserve<double>(gcopies * (size_t)m);
     size_t a_r2 = A.reserve<float2>(n), a_w2 = A.reserve<float2>(m);
     size_t a_cs2 = A.reserve<float2>(gcopies * (size_t)n);
@@ -981,6 +973,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     P->d_tspread = tiles[LIST_SPREAD]; P->d_tinterp = tiles[LIST_INTERP];
     P->d_fsmall = tiles[LIST_FSMALL]; P->d_fa = tiles[LIST_FA]; P->d_fb = tiles[LIST_FB];
     P->d_fblock = tiles[LIST_FBLOCK];
+    for (int ps = 0; ps < 3; ++ps) P->d_fpass[ps] = tiles[LIST_P0 + ps];
     P->d_pre_mom = bl.pre[LIST_MOM];
     P->d_blk = bl.blk;
     // sorted arrays and permutations stay on the device
@@ -1000,7 +993,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     P->d_dir = bl.dir;
     P->d_es = (double*)(D + a_es); P->d_ph = (double*)(D + a_ph); P->d_tw = (double2*)(D + a_tw);
     P->d_mom = (double*)(D + a_mom); P->d_momb = P->d_mom + P->mom_len;
-    P->d_gb = (double2*)(D + a_gb); P->d_gq = (float4*)(D + a_gq); P->d_gtmp = (float4*)(D + a_gt);
+    P->d_gb = (double2*)(D + a_gb); P->d_gq = (float4*)(D + a_gq);
     P->d_cs = (double*)(D + a_cs); P->d_gs = (double*)(D + a_gs);
     P->d_r2 = (float2*)(D + a_r2); P->d_w2 = (float2*)(D + a_w2); P->d_cs2 = (float2*)(D + a_cs2);
     P->d_csb = P->d_cs + n; P->d_gsb = P->d_gs + m; P->d_cs2b = P->d_cs2 + n;
@@ -1367,16 +1360,22 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         if (P->det) NUHT_CK(launch_fx_decode(P->f_gb, (double*)P->d_gb, 2 * P->gb_len, P->d_prob, as));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_SPREAD, as));
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_FFT, as));
-        // the members' FFTs of whole blocks in one launch each; the two-pass
-        // FFTs of large blocks per member (one temporary)
-        NUHT_CK(launch_asy_fft_block(P->d_prob, P->d_asy, P->d_fblock, P->n_fblock, P->max_fblock_pts, P->tab,
-                                     P->d_gb, P->d_gq, as, false, lowp, nv, P->gb_len, P->gq_len));
-        NUHT_CK(launch_asy_fft_small(P->d_prob, P->d_asy, P->d_fsmall, P->n_fsmall, P->max_nf2_small,
-                                     P->tab, P->d_gb, P->d_gq, as, false, lowp, nv, P->gb_len, P->gq_len));
-        for (int u = 0; P->has_large_fft && u < nv; ++u)
-            NUHT_CK(launch_asy_fft_large(P->d_prob, P->d_asy, P->d_fa, P->n_fa, P->d_fb, P->n_fb, P->tab,
-                                         P->d_gb + (int64_t)u * P->gb_len, P->d_gtmp,
-                                         P->d_gq + (int64_t)u * P->gq_len, as, false, lowp));
+        if (lowp) {
+            // the members' FFTs of whole blocks in one launch each; the two-pass
+            // FFTs of large blocks per member (one temporary)
+            NUHT_CK(launch_asy_fft_block_f32(P->d_prob, P->d_asy, P->d_fblock, P->n_fblock, P->max_fblock_pts,
+                                             P->tab, P->d_gb, P->d_gq, as, nv, P->gb_len, P->gq_len));
+            NUHT_CK(launch_asy_fft_small_f32(P->d_prob, P->d_asy, P->d_fsmall, P->n_fsmall, P->max_nf2_small,
+                                             P->tab, P->d_gb, P->d_gq, as, nv, P->gb_len, P->gq_len));
+            for (int u = 0; P->n_fa && u < nv; ++u)
+                NUHT_CK(launch_asy_fft_large_f32(P->d_prob, P->d_asy, P->d_fa, P->n_fa, P->d_fb, P->n_fb, P->tab,
+                                                 P->d_gb + (int64_t)u * P->gb_len, (float2*)P->d_tg,
+                                                 P->d_gq + (int64_t)u * P->gq_len, as));
+        }
+        for (int ps = 0; !lowp && ps < 3; ++ps)
+            NUHT_CK(launch_asy_fft(P->d_prob, P->d_asy, P->d_fpass[ps], P->n_fpass[ps], P->fft_smem[ps], ps, P->tab,
+                                   P->d_gb, (float4*)P->d_tg, P->d_gq, as, false, nv, P->gb_len, P->gq_len,
+                                   P->gq_len));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_FFT, as));
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_INTERP, as));
         if (lowp)
@@ -1537,14 +1536,9 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
         if (P->det) NUHT_CK(launch_fx_decode(P->f_tg, (double*)P->d_tg, 2 * P->gq_len, P->d_prob, as));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_SPREAD, as));
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_FFT, as));
-        NUHT_CK(launch_asy_fft_block(P->d_prob, P->d_asy, P->d_fblock, P->n_fblock, P->max_fblock_pts, P->tab,
-                                     P->d_tg, P->d_bq, as, true, false, nv, P->gq_len, P->gb_len));
-        NUHT_CK(launch_asy_fft_small(P->d_prob, P->d_asy, P->d_fsmall, P->n_fsmall, P->max_nf2_small, P->tab,
-                                     P->d_tg, P->d_bq, as, true, false, nv, P->gq_len, P->gb_len));
-        for (int u = 0; P->has_large_fft && u < nv; ++u)
-            NUHT_CK(launch_asy_fft_large(P->d_prob, P->d_asy, P->d_fa, P->n_fa, P->d_fb, P->n_fb, P->tab,
-                                         P->d_tg + (int64_t)u * P->gq_len, P->d_gtmp,
-                                         P->d_bq + (int64_t)u * P->gb_len, as, true));
+        for (int ps = 0; ps < 3; ++ps)
+            NUHT_CK(launch_asy_fft(P->d_prob, P->d_asy, P->d_fpass[ps], P->n_fpass[ps], P->fft_smem[ps], ps, P->tab,
+                                   P->d_tg, P->d_gq, P->d_bq, as, true, nv, P->gq_len, P->gq_len, P->gb_len));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_FFT, as));
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_INTERP, as));
         NUHT_CK(launch_asy_adj_interp(P->d_prob, P->d_asy, P->d_tspread, P->n_tspread, P->qmax, P->tab, P->d_r,
