@@ -944,33 +944,50 @@ __device__ void spread_taps(const AsyBlock& B, int Q, const Tile& t, const Table
 // Path of a spreading tile, packed: bits 0-1 the path (0 taps, 1 plain
 // moments, 2 q-folded moments), bits 2-5 the fold's K, bits 6-11 its E,
 // bits 12-17 its Edf.  The path depends only on the sorted points and the
-// block, so it is decided once per plan (k_spread_modes).
+// block, so it is decided once per plan (k_expand_lists).
 __device__ __forceinline__ FoldPlan fold_unpack(int mode)
 {
     return FoldPlan{(mode >> 2) & 15, (mode >> 6) & 63, (mode >> 12) & 63};
 }
 
-__global__ void k_spread_modes(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                               const Tile* __restrict__ tiles, int ntiles, Tables tab,
-                               const double* __restrict__ r_s, int32_t* __restrict__ modes)
+__device__ int spread_mode(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks, const Tile& t,
+                           const Tables& tab, const double* __restrict__ r_s)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ntiles; i += gridDim.x * blockDim.x) {
-        const Tile t = tiles[i];
-        int mode = 0;
-        if (t.count > 0) {
-            const AsyBlock B = blks[t.blk];
-            long long X;
-            df vd;
-            const int lfirst = spread_cell_fx(B, tab.w, r_s[t.start], &X, &vd);
-            const int nbins = spread_cell_fx(B, tab.w, r_s[t.start + t.count - 1], &X, &vd) - lfirst + 1;
-            if (nbins <= kMaxTileBins && t.count >= kMomMinPerBin * nbins) {
-                mode = 1;
-                FoldPlan fp;
-                if (fold_plan(B, tab, probs[B.prob].Q, lfirst, &fp))
-                    mode = 2 | (fp.K << 2) | (fp.E << 6) | (fp.Edf << 12);
-            }
+    if (t.count <= 0) return 0;
+    const AsyBlock& B = blks[t.blk];
+    long long X;
+    df vd;
+    const int lfirst = spread_cell_fx(B, tab.w, r_s[t.start], &X, &vd);
+    const int nbins = spread_cell_fx(B, tab.w, r_s[t.start + t.count - 1], &X, &vd) - lfirst + 1;
+    if (nbins > kMaxTileBins || t.count < kMomMinPerBin * nbins) return 0;
+    FoldPlan fp;
+    if (fold_plan(B, tab, probs[B.prob].Q, lfirst, &fp)) return 2 | (fp.K << 2) | (fp.E << 6) | (fp.Edf << 12);
+    return 1;
+}
+
+// Every tile of every list (one launch for all lists; eleven launches of a
+// few microseconds each before): tile i of a list lies in the segment b with
+// prefix[b] <= i < prefix[b + 1] (binary search), then its start and count
+// inside the segment's index range; spreading tiles also get their path.
+__global__ void k_expand_lists(ExpandLists E, int total, const ProbParams* __restrict__ probs,
+                               const AsyBlock* __restrict__ blks, Tables tab, const double* __restrict__ r_s,
+                               int32_t* __restrict__ modes)
+{
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < total; x += gridDim.x * blockDim.x) {
+        int i = x, l = 0;
+        while (i >= E.ntile[l]) i -= E.ntile[l++];
+        const int32_t* prefix = E.pre[l];
+        int lo = 0, hi = E.nseg[l];   // last b with prefix[b] <= i
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (prefix[mid] <= i) lo = mid; else hi = mid;
         }
-        modes[i] = mode;
+        const Seg sg = E.seg[l][lo];
+        const int64_t start = sg.first + (int64_t)(i - prefix[lo]) * sg.len;
+        const int64_t rem = sg.last - start + 1;
+        const Tile t{sg.blk, (int32_t)(rem < sg.len ? rem : sg.len), start};
+        E.tiles[l][i] = t;
+        if (l == LIST_SPREAD) modes[i] = spread_mode(probs, blks, t, tab, r_s);
     }
 }
 
@@ -2166,12 +2183,15 @@ cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks,
     return cudaGetLastError();
 }
 
-cudaError_t launch_spread_modes(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles, int ntiles,
-                                Tables tab, const double* r_s, int32_t* modes, cudaStream_t s)
+cudaError_t launch_expand_lists(const ExpandLists& E, const ProbParams* probs, const AsyBlock* blks, Tables tab,
+                                const double* r_s, int32_t* modes, cudaStream_t s)
 {
-    if (ntiles <= 0) return cudaSuccess;
-    const int nb = (ntiles + 255) / 256, cap = device_sm_count() * 16;
-    k_spread_modes<<<nb < cap ? nb : cap, 256, 0, s>>>(probs, blks, tiles, ntiles, tab, r_s, modes);
+    int64_t total = 0;
+    for (int i = 0; i < kLists; ++i) total += E.ntile[i];
+    if (total <= 0) return cudaSuccess;
+    if (total > 0x7fffffff) return cudaErrorInvalidValue;
+    const int64_t nb = (total + 127) / 128, cap = (int64_t)device_sm_count() * 32;
+    k_expand_lists<<<(unsigned)(nb < cap ? nb : cap), 128, 0, s>>>(E, (int)total, probs, blks, tab, r_s, modes);
     count_launches(1);
     return cudaGetLastError();
 }

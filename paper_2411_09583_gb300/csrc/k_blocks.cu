@@ -2,18 +2,16 @@
 // subdivision (Algorithm 1): per-block descriptors (local expansion, Sec. 3.1;
 // type-3 geometry of the asymptotic blocks, Sec. 3.2 / 4.2; direct blocks),
 // the offsets of their moments and grids, and the tile segments of every
-// kernel.  Three kernels: sizes (one thread per block), column-wise exclusive
-// prefix sums (one CTA), fill (one thread per block).  The block counts are
-// read from device memory, so nothing here waits for the host.
+// kernel.  Two kernels: sizes (one thread per block; the CTA that finishes last
+// also forms the column-wise prefix over the CTAs' sums) and fill (one thread
+// per block).  The block counts are read from device memory, so nothing here
+// waits for the host.
 #include <cmath>
 #include <cstdint>
 
 #include "nuht_internal.h"
 
 namespace nuht {
-
-// streaming multiprocessors of the current device, cached per device (k_det.cu)
-int device_sm_count();
 
 namespace {
 
@@ -26,20 +24,25 @@ __device__ __forceinline__ void atomic_max64(int64_t* p, int64_t v)
 
 __device__ __forceinline__ int64_t clamp_count(int64_t c, int64_t cap) { return c < cap ? c : cap; }
 
-__global__ void k_block_sizes(BlockBuild bb)
+// Rows of class y (0 local, 1 asymptotic, 2 direct), its counter columns and
+// the place of their totals.
+__device__ __forceinline__ int64_t class_rows(const BlockBuild& bb, int y) { return clamp_count(bb.res[y], bb.ocap); }
+__device__ __forceinline__ int class_cols(int y) { return y == 0 ? kLocalCols : (y == 1 ? kAsyCols : kDirCols); }
+__device__ __forceinline__ int class_total(int y) { return y == 0 ? TOT_LOCAL : (y == 1 ? TOT_ASY : TOT_DIR); }
+
+// Descriptor and counters of one block; maxima into smax (shared).
+__device__ __forceinline__ void block_size_one(const BlockBuild& bb, int y, int64_t i, unsigned long long* smax)
 {
-    const int64_t nl = clamp_count(bb.res[0], bb.ocap), na = clamp_count(bb.res[1], bb.ocap),
-                  nd = clamp_count(bb.res[2], bb.ocap);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl + na + nd;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < nl) {
+    auto maxv = [&](int k, int64_t v) { atomicMax(&smax[k], (unsigned long long)v); };
+    {
+        if (y == 0) {
             const SubBlk b = bb.sub[i];
             const ProbParams& P = bb.probs[b.prob];
             LocalBlock lb{};
             lb.prob = b.prob;
             lb.k0 = (int32_t)(b.k0 + P.w_off); lb.k1 = (int32_t)(b.k1 + P.w_off);
             lb.j0 = (int32_t)(b.j0 + P.r_off); lb.j1 = (int32_t)(b.j1 + P.r_off);
-            lb.R = bb.bl[i];
+            lb.R = bb.r_s[lb.j1];
             lb.R_h = (float)lb.R;
             lb.R_l = (float)(lb.R - (double)lb.R_h);
             const double iR = lb.R > 0.0 ? 1.0 / lb.R : 0.0;
@@ -52,11 +55,13 @@ __global__ void k_block_sizes(BlockBuild bb)
             c[LC_TMOM] = ceil_div(cols, bb.mom_tile);
             c[LC_TEVAL] = ceil_div(rows, bb.eval_tile);
             c[LC_RC] = rows + cols;
-        } else if (i < nl + na) {
-            const int64_t a = i - nl;
+        } else if (y == 1) {
+            const int64_t a = i;
             const SubBlk b = bb.sub[bb.ocap + a];
             const ProbParams& P = bb.probs[b.prob];
-            const double4 e = bb.ba[a];   // r_j0, r_j1, omega_k0, omega_k1
+            struct { double x, y, z, w; } e;   // r_j0, r_j1, omega_k0, omega_k1
+            e.x = bb.r_s[P.r_off + b.j0]; e.y = bb.r_s[P.r_off + b.j1];
+            e.z = bb.w_s[P.w_off + b.k0]; e.w = bb.w_s[P.w_off + b.k1];
             const int Q = P.Q;
             AsyBlock ab{};
             ab.prob = b.prob;
@@ -109,16 +114,16 @@ __global__ void k_block_sizes(BlockBuild bb)
             for (int k = 0; k < kAsyCols; ++k) c[k] = 0;
             bb.fcls[a] = -1;
             if (fx_bad || !(n1f <= (double)(1 << 22))) {
-                atomic_max64(&bb.maxv[MX_ERR], 1);
-                continue;
+                maxv(MX_ERR, 1);
+                return;
             }
             ab.N1 = (int32_t)n1f;
             const int64_t nf1 = 2 * (int64_t)ab.N1 + 1;
             int lg = 64 - __clzll((long long)(2 * nf1 - 1));   // smallest 2^lg >= 2 nf1
             if (lg < 5) lg = 5;
             if (lg > kFftMaxLog2) {
-                atomic_max64(&bb.maxv[MX_ERR], 1);
-                continue;
+                maxv(MX_ERR, 1);
+                return;
             }
             ab.log2nf2 = lg;
             ab.nf2 = 1 << lg;
@@ -147,8 +152,8 @@ __global__ void k_block_sizes(BlockBuild bb)
                 ab.KRc = kr;
                 ab.sR = sr;
                 if (ab.sD < 1 || ab.sD > 127 || sr < 0) {
-                    atomic_max64(&bb.maxv[MX_ERR], 1);
-                    continue;
+                    maxv(MX_ERR, 1);
+                    return;
                 }
             }
             {
@@ -164,7 +169,7 @@ __global__ void k_block_sizes(BlockBuild bb)
             c[AC_GQ] = (int64_t)ab.nf2 * Q;
             c[AC_TSPREAD] = ceil_div(cols, bb.spread_tile);
             c[AC_TINTERP] = ceil_div(rows, bb.interp_tile);
-            atomic_max64(&bb.maxv[MX_LOG2], lg);
+            maxv(MX_LOG2, lg);
             {
                 const int np = fft_split(lg).np;
                 c[AC_IP0] = fft_tile(lg, 0, Q).ntiles;
@@ -179,12 +184,12 @@ __global__ void k_block_sizes(BlockBuild bb)
                 bb.fcls[a] = 0;
                 c[AC_NFK] = 1;
                 c[AC_IFK] = 1;
-                atomic_max64(&bb.maxv[MX_FBLOCK_PTS], (int64_t)ab.nf2 * Q);
+                maxv(MX_FBLOCK_PTS, (int64_t)ab.nf2 * Q);
             } else if (ab.nf2 <= kFftSingleMax) {                 // one CTA per grid
                 bb.fcls[a] = 1;
                 c[AC_NFS] = 1;
                 c[AC_IFS] = Q;
-                atomic_max64(&bb.maxv[MX_NF2_SMALL], ab.nf2);
+                maxv(MX_NF2_SMALL, ab.nf2);
             } else {                                              // two passes, groups of lines
                 bb.fcls[a] = 2;
                 c[AC_NFL] = 1;
@@ -197,115 +202,105 @@ __global__ void k_block_sizes(BlockBuild bb)
             c[AC_RC] = rows + cols;
             c[AC_NF2] = ab.nf2;
         } else {
-            const int64_t d = i - nl - na;
+            const int64_t d = i;
             const SubBlk b = bb.sub[2 * bb.ocap + d];
             const ProbParams& P = bb.probs[b.prob];
             bb.dir[d] = DirectBlock{b.prob, (int32_t)(b.k0 + P.w_off), (int32_t)(b.k1 + P.w_off),
                                     (int32_t)(b.j0 + P.r_off), (int32_t)(b.j1 + P.r_off), 0};
             const int64_t rows = b.k1 - b.k0 + 1, cols = b.j1 - b.j0 + 1;
             bb.dcnt[d] = rows * cols;
-            atomic_max64(&bb.maxv[MX_DIR_ROWS], rows);
-            atomic_max64(&bb.maxv[MX_DIR_COLS], cols);
-            atomic_max64(&bb.maxv[MX_DIR_AREA], rows * cols);
+            maxv(MX_DIR_ROWS, rows);
+            maxv(MX_DIR_COLS, cols);
+            maxv(MX_DIR_AREA, rows * cols);
         }
     }
 }
 
-// Exclusive prefix sums of the columns of the three counter matrices
-// (row-major, rows = blocks) in place, and the column totals: tile sums (one
-// CTA per kScanTile rows), one CTA over the tile sums, then each tile again
-// with its offset.  blockIdx.y picks the matrix.
-constexpr int kScanTile = 256;
-
-struct ScanMat {
-    int64_t* mat;
-    int64_t n;
-    int ncol;
-    int64_t* totals;
-};
-
-__device__ __forceinline__ ScanMat scan_mat(const BlockBuild& bb, int which)
+// Sizes, descriptors and counters of every block (CTA = kBlockTile rows of
+// class blockIdx.y), the CTAs' column sums, and by the CTA that finishes last
+// their exclusive prefix and the totals (four launches before: sizes and three
+// of scans).
+__global__ void __launch_bounds__(kBlockTile) k_block_sizes(BlockBuild bb)
 {
-    if (which == 0) return ScanMat{bb.lcnt, clamp_count(bb.res[0], bb.ocap), kLocalCols, bb.totals + TOT_LOCAL};
-    if (which == 1) return ScanMat{bb.acnt, clamp_count(bb.res[1], bb.ocap), kAsyCols, bb.totals + TOT_ASY};
-    return ScanMat{bb.dcnt, clamp_count(bb.res[2], bb.ocap), kDirCols, bb.totals + TOT_DIR};
+    __shared__ unsigned long long smax[kMaxv], ssum[kAsyCols];
+    __shared__ bool is_last;
+    const int y = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t rows = class_rows(bb, y);
+    if ((int64_t)blockIdx.x * kBlockTile >= rows) return;   // whole CTA
+    if (threadIdx.x < kMaxv) smax[threadIdx.x] = 0;
+    if (threadIdx.x < kAsyCols) ssum[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * kBlockTile + threadIdx.x;
+    if (i < rows) block_size_one(bb, y, i, smax);
+    __syncthreads();
+    const int ncol = class_cols(y);
+    const int64_t* mat = y == 0 ? bb.lcnt : (y == 1 ? bb.acnt : bb.dcnt);
+    for (int c = 0; c < ncol; ++c) {
+        int64_t v = i < rows ? mat[i * ncol + c] : 0;   // this thread's own stores
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0 && v) atomicAdd(&ssum[c], (unsigned long long)v);
+    }
+    __syncthreads();
+    if (threadIdx.x < ncol)
+        bb.part[((int64_t)y * bb.ptiles + blockIdx.x) * kAsyCols + threadIdx.x] = (int64_t)ssum[threadIdx.x];
+    if (threadIdx.x < kMaxv && smax[threadIdx.x]) atomic_max64(&bb.maxv[threadIdx.x], (int64_t)smax[threadIdx.x]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned active = 0;
+        for (int k = 0; k < 3; ++k) active += (unsigned)ceil_div(class_rows(bb, k), kBlockTile);
+        is_last = atomicAdd(bb.ticket, 1u) + 1 == active;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    // one warp per column
+    for (int col = warp; col < kTotals; col += kBlockTile / 32) {
+        const int k = col >= TOT_DIR ? 2 : (col >= TOT_ASY ? 1 : 0), c = col - class_total(k);
+        const int64_t nt = ceil_div(class_rows(bb, k), kBlockTile);
+        int64_t carry = 0;
+        for (int64_t t0 = 0; t0 < nt; t0 += 32) {
+            const int64_t t = t0 + lane;
+            int64_t* pp = bb.part + ((int64_t)k * bb.ptiles + t) * kAsyCols + c;
+            const int64_t v = t < nt ? __ldcg((const long long*)pp) : 0;
+            int64_t x = v;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int64_t o = __shfl_up_sync(0xffffffffu, x, off);
+                if (lane >= off) x += o;
+            }
+            if (t < nt) *pp = carry + x - v;   // exclusive offset of the tile
+            carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) bb.totals[col] = carry;
+    }
 }
 
-// block-wide inclusive scan of one value per thread (kScanTile threads)
-__device__ __forceinline__ int64_t block_incl_scan(int64_t v, int64_t* wsum, int64_t* total)
+// Exclusive prefix sums of NCOL counters over all rows of a class: c[] of this
+// thread's row, the tile's offset from part.
+template <int NCOL>
+__device__ __forceinline__ void class_prefix(const BlockBuild& bb, int y, const int64_t* row, bool live, int64_t* c,
+                                             int64_t (*wsum)[kBlockTile / 32])
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int64_t x = v;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int64_t y = __shfl_up_sync(0xffffffffu, x, off);
-        if (lane >= off) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int64_t s = lane < kScanTile / 32 ? wsum[lane] : 0;
+    for (int k = 0; k < NCOL; ++k) {
+        const int64_t v = live ? row[k] : 0;
+        int64_t x = v;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, s, off);
-            if (lane >= off) s += y;
+            const int64_t o = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += o;
         }
-        if (lane < kScanTile / 32) wsum[lane] = s;
+        if (lane == 31) wsum[k][warp] = x;
+        c[k] = x - v;
     }
     __syncthreads();
-    const int64_t r = x + (wid > 0 ? wsum[wid - 1] : 0);
-    *total = wsum[kScanTile / 32 - 1];
-    __syncthreads();
-    return r;
-}
-
-__global__ void __launch_bounds__(kScanTile) k_scan_tiles(BlockBuild bb, int64_t* part, int64_t ptiles)
-{
-    __shared__ int64_t wsum[kScanTile / 32];
-    const ScanMat S = scan_mat(bb, blockIdx.y);
-    const int64_t row = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
-    if ((int64_t)blockIdx.x * kScanTile >= S.n) return;   // whole CTA
-    for (int c = 0; c < S.ncol; ++c) {
-        int64_t tot;
-        block_incl_scan(row < S.n ? S.mat[row * S.ncol + c] : 0, wsum, &tot);
-        if (threadIdx.x == 0) part[((int64_t)blockIdx.y * ptiles + blockIdx.x) * kAsyCols + c] = tot;
-    }
-}
-
-__global__ void __launch_bounds__(kScanTile) k_scan_top(BlockBuild bb, int64_t* part, int64_t ptiles)
-{
-    __shared__ int64_t wsum[kScanTile / 32];
-    for (int which = 0; which < 3; ++which) {
-        const ScanMat S = scan_mat(bb, which);
-        const int64_t nt = (S.n + kScanTile - 1) / kScanTile;
-        for (int c = 0; c < S.ncol; ++c) {
-            int64_t carry = 0;
-            for (int64_t t0 = 0; t0 < nt; t0 += kScanTile) {
-                const int64_t t = t0 + threadIdx.x;
-                int64_t* pp = part + ((int64_t)which * ptiles + t) * kAsyCols + c;
-                const int64_t v = t < nt ? *pp : 0;
-                int64_t tot;
-                const int64_t incl = block_incl_scan(v, wsum, &tot);
-                if (t < nt) *pp = carry + incl - v;   // exclusive offset of the tile
-                carry += tot;
-            }
-            if (threadIdx.x == 0) S.totals[c] = carry;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kScanTile) k_scan_apply(BlockBuild bb, const int64_t* part, int64_t ptiles)
-{
-    __shared__ int64_t wsum[kScanTile / 32];
-    const ScanMat S = scan_mat(bb, blockIdx.y);
-    const int64_t row = blockIdx.x * (int64_t)kScanTile + threadIdx.x;
-    if ((int64_t)blockIdx.x * kScanTile >= S.n) return;
-    for (int c = 0; c < S.ncol; ++c) {
-        const int64_t v = row < S.n ? S.mat[row * S.ncol + c] : 0;
-        int64_t tot;
-        const int64_t incl = block_incl_scan(v, wsum, &tot);
-        if (row < S.n)
-            S.mat[row * S.ncol + c] = part[((int64_t)blockIdx.y * ptiles + blockIdx.x) * kAsyCols + c] + incl - v;
+    const int64_t* part = bb.part + ((int64_t)y * bb.ptiles + blockIdx.x) * kAsyCols;
+#pragma unroll
+    for (int k = 0; k < NCOL; ++k) {
+        int64_t p = part[k];
+        for (int w = 0; w < warp; ++w) p += wsum[k][w];
+        c[k] += p;
     }
 }
 
@@ -316,13 +311,15 @@ __device__ __forceinline__ void put_seg(const BuildLists& L, int list, int64_t i
     L.pre[list][idx] = (int32_t)prefix;
 }
 
-__global__ void k_block_fill(BlockBuild bb, BuildLists L)
+__global__ void __launch_bounds__(kBlockTile) k_block_fill(BlockBuild bb, BuildLists L)
 {
     const int64_t nl = clamp_count(bb.res[0], bb.ocap), na = clamp_count(bb.res[1], bb.ocap),
                   nd = clamp_count(bb.res[2], bb.ocap);
     const int64_t* tl = bb.totals + TOT_LOCAL;
     const int64_t* ta = bb.totals + TOT_ASY;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    __shared__ int64_t wsum[kAsyCols][kBlockTile / 32];
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        *L.status = 0;
         // closing entries of the prefix arrays
         L.pre[LIST_MOM][nl] = (int32_t)tl[LC_TMOM];
         L.pre[LIST_EVAL][nl] = (int32_t)tl[LC_TEVAL];
@@ -336,19 +333,26 @@ __global__ void k_block_fill(BlockBuild bb, BuildLists L)
         L.pre[LIST_P1][ta[AC_NP1]] = (int32_t)ta[AC_IP1];
         L.pre[LIST_P2][ta[AC_NP2]] = (int32_t)ta[AC_IP2];
     }
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl + na + nd;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < nl) {
-            const int64_t* c = bb.lcnt + i * kLocalCols;
+    const int y = blockIdx.y;
+    const int64_t rows = y == 0 ? nl : (y == 1 ? na : nd), i = (int64_t)blockIdx.x * kBlockTile + threadIdx.x;
+    if ((int64_t)blockIdx.x * kBlockTile >= rows) return;   // whole CTA
+    const bool live = i < rows;
+    {
+        if (y == 0) {
+            int64_t c[kLocalCols];
+            class_prefix<kLocalCols>(bb, y, bb.lcnt + i * kLocalCols, live, c, wsum);
+            if (!live) return;
             LocalBlock lb = bb.loc[i];
             lb.mom_off = c[LC_MOM];
             L.loc[i] = lb;
             put_seg(L, LIST_MOM, i, (int32_t)i, bb.mom_tile, lb.j0, lb.j1, c[LC_TMOM]);
             put_seg(L, LIST_EVAL, i, (int32_t)i, bb.eval_tile, lb.k0, lb.k1, c[LC_TEVAL]);
             L.blk[i] = SubBlk{lb.k0, lb.k1, lb.j0, lb.j1, lb.prob};
-        } else if (i < nl + na) {
-            const int64_t a = i - nl;
-            const int64_t* c = bb.acnt + a * kAsyCols;
+        } else if (y == 1) {
+            const int64_t a = i;
+            int64_t c[kAsyCols];
+            class_prefix<kAsyCols>(bb, y, bb.acnt + a * kAsyCols, live, c, wsum);
+            if (!live) return;
             AsyBlock ab = bb.asy[a];
             ab.b_off = c[AC_GB];
             ab.q_off = c[AC_GQ];
@@ -379,8 +383,8 @@ __global__ void k_block_fill(BlockBuild bb, BuildLists L)
                 put_seg(L, LIST_FB, c[AC_NFL], (int32_t)a, 1, 0, ib - 1, c[AC_IFB]);
             }
             L.blk[nl + a] = SubBlk{ab.k0, ab.k1, ab.j0, ab.j1, ab.prob};
-        } else {
-            const int64_t d = i - nl - na;
+        } else if (live) {
+            const int64_t d = i;
             const DirectBlock db = bb.dir[d];
             L.dir[d] = db;
             L.blk[nl + na + d] = SubBlk{db.k0, db.k1, db.j0, db.j1, db.prob};
@@ -390,27 +394,29 @@ __global__ void k_block_fill(BlockBuild bb, BuildLists L)
 
 }  // namespace
 
-int64_t block_scan_scratch(int64_t cap) { return 3 * ((cap + kScanTile - 1) / kScanTile) * kAsyCols; }
-
-cudaError_t launch_block_build(const BlockBuild& bb, int64_t* scratch, cudaStream_t s)
+static cudaError_t block_grid(int64_t tiles, dim3* grid)
 {
-    k_block_sizes<<<device_sm_count() * 8, 256, 0, s>>>(bb);
-    cudaError_t e = cudaGetLastError();
+    if (tiles < 1 || tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    *grid = dim3((unsigned)tiles, 3);
+    return cudaSuccess;
+}
+
+cudaError_t launch_block_build(const BlockBuild& bb, cudaStream_t s)
+{
+    dim3 grid;
+    const cudaError_t e = block_grid(bb.ptiles, &grid);   // the counts are still on the device
     if (e != cudaSuccess) return e;
-    const int64_t ptiles = (bb.ocap + kScanTile - 1) / kScanTile;
-    if (ptiles > 0) {
-        const dim3 grid((unsigned)ptiles, 3);
-        k_scan_tiles<<<grid, kScanTile, 0, s>>>(bb, scratch, ptiles);
-        k_scan_top<<<1, kScanTile, 0, s>>>(bb, scratch, ptiles);
-        k_scan_apply<<<grid, kScanTile, 0, s>>>(bb, scratch, ptiles);
-    }
-    count_launches(4);
+    k_block_sizes<<<grid, kBlockTile, 0, s>>>(bb);
+    count_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_fill(const BlockBuild& bb, const BuildLists& L, cudaStream_t s)
+cudaError_t launch_block_fill(const BlockBuild& bb, const BuildLists& L, int64_t max_rows, cudaStream_t s)
 {
-    k_block_fill<<<device_sm_count() * 8, 256, 0, s>>>(bb, L);
+    dim3 grid;
+    const cudaError_t e = block_grid((max_rows > 0 ? max_rows + kBlockTile - 1 : kBlockTile) / kBlockTile, &grid);
+    if (e != cudaSuccess) return e;
+    k_block_fill<<<grid, kBlockTile, 0, s>>>(bb, L);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -1,17 +1,23 @@
-// Plan-time device kernels: input domain check, LSD radix sort of FP64 keys
-// with their original indices, and the execute-time gather / scatter between
-// user order and sorted order.
+// Plan-time device kernels: input domain check, radix sort of FP64 values
+// with their original indices, the staircase; and the execute-time gather /
+// scatter between user order and sorted order.
 //
 // The subdivision of Algorithm 1 and the complexity theorem of Sec. 4.2 take
 // the points and frequencies sorted ascending; the inputs are unsorted, so the
-// plan sorts them once and keeps the permutations.
+// plan sorts both once and keeps the permutations.
 //
-// Keys are non-negative doubles (checked first), whose IEEE bit patterns
-// compare like unsigned integers, so an 8-pass, 8-bit LSD radix sort on the
-// raw 64-bit patterns sorts them.  Each pass: per-tile digit histogram,
-// one exclusive scan over (digit, tile), then a stable scatter in which each
-// warp ranks its run of the tile (warp match + per-warp digit counts) and one
-// prefix over the warps places the runs, so equal keys keep their input order.
+// Values are non-negative doubles (checked beside), whose IEEE bit patterns
+// compare like unsigned integers.  They are sorted stably by a 32-bit key, the
+// leading 31 bits of (pattern - smallest non-zero pattern) within the range
+// that the input spans (zero has a key of its own), in four 8-bit passes
+// instead of the eight a 64-bit pattern takes and over 8-byte (key, index)
+// pairs instead of 12 bytes; the few values that share a key are then ordered
+// by their full patterns where they lie.  Points and frequencies share every
+// launch, and up to kSmallSort of each are sorted by one CTA in one launch.
+// Measured, both arrays on an idle GPU (sum of the launches): n = m = 1e6
+// 0.45 ms in 52 launches on two streams -> 0.17 in 15; 1e5 0.16 -> 0.05; 2000
+// 0.12 -> 0.02 in one launch.  Bound by the scatters' 8-byte stores (L2) at
+// 1e6 and by launch latency below 1e5.
 #include <cstdint>
 
 #include "nuht_internal.h"
@@ -27,86 +33,151 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 4;                       // elements per thread per tile
 constexpr int kSortTile = kSortThreads * kSortItems; // 1024: ~4 CTAs per SM at n = 1e6 (4096 left the scatter passes latency-bound)
 constexpr int kRadix = 256;
+constexpr int kSortDirectTiles = 128;   // up to this many tiles each scatter CTA sums the tile counts itself
+constexpr int kRunMax = 64;             // longest run of equal keys ordered element by element
 static_assert(kSortThreads == kRadix, "the scatter kernel scans one digit total per thread");
 
-__global__ void k_check_domain(const double* __restrict__ x, int64_t n, int* flag)
+// Bit pattern with -0.0 folded onto +0.0.
+__device__ __forceinline__ uint64_t sort_bits(double v)
 {
+    return v == 0.0 ? 0ull : (uint64_t)__double_as_longlong(v);
+}
+
+// false for negatives, NaN and +-inf; -0.0 is accepted
+__device__ __forceinline__ bool in_domain(double v) { return v >= 0.0 && v <= 1.7976931348623157e308; }
+
+// The 32-bit key: 0 for zero, else 1 + (bits - lo) >> shift, lo the smallest
+// non-zero pattern and shift such that the largest fits 31 bits.
+struct SortQuant {
+    uint64_t lo;
+    int shift;
+    __device__ __forceinline__ uint32_t key(uint64_t b) const { return b == 0 ? 0u : 1u + (uint32_t)((b - lo) >> shift); }
+};
+
+// stats[0] = the largest ~bits over non-zero values, stats[1] = the largest bits
+__device__ __forceinline__ SortQuant sort_quant(const unsigned long long* stats)
+{
+    const uint64_t hi = stats[1], lo = hi ? ~stats[0] : 0ull;
+    const int used = 64 - __clzll((long long)(hi - lo));
+    return SortQuant{lo, used > 31 ? used - 31 : 0};
+}
+
+__device__ __forceinline__ void warp_range(uint64_t& mn, uint64_t& mx)
+{
+    for (int off = 16; off > 0; off >>= 1) {
+        const uint64_t a = __shfl_xor_sync(0xffffffffu, mn, off), c = __shfl_xor_sync(0xffffffffu, mx, off);
+        mn = a > mn ? a : mn;
+        mx = c > mx ? c : mx;
+    }
+}
+
+// Domain check and value range of both arrays (blockIdx.y).
+__global__ void __launch_bounds__(kSortThreads) k_sort_range(SortPair S)
+{
+    const SortArray& A = S.a[blockIdx.y];
+    uint64_t mn = 0, mx = 0;   // of ~bits (non-zero), of bits
     int bad = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double v = x[i];
-        // rejects negatives, NaN and +-inf; -0.0 is accepted
-        if (!(v >= 0.0) || !(v <= 1.7976931348623157e308)) bad = 1;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double v = A.in[i];
+        if (!in_domain(v)) bad = 1;
+        const uint64_t b = sort_bits(v);
+        if (b && ~b > mn) mn = ~b;
+        if (b > mx) mx = b;
     }
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
+    // one pair of global updates per CTA (one per warp cost 80 us at n = m = 1e6)
+    __shared__ unsigned long long cmn, cmx;
+    if (threadIdx.x == 0) cmn = cmx = 0;
+    __syncthreads();
+    warp_range(mn, mx);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&cmn, (unsigned long long)mn);
+        atomicMax(&cmx, (unsigned long long)mx);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (cmn) atomicMax(A.stats, cmn);
+        if (cmx) atomicMax(A.stats + 1, cmx);
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(A.flag, 1);
 }
 
-// keys: bit patterns (with -0.0 folded onto +0.0), values: 0..n-1
-__global__ void k_sort_init(const double* __restrict__ in, int64_t n, uint64_t* __restrict__ keys,
-                            int32_t* __restrict__ vals)
+// Segment of the element at input index x (offsets off[0..nseg]).
+__device__ __forceinline__ uint32_t seg_of(const int64_t* off, int nseg, int64_t x)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double v = in[i];
-        if (v == 0.0) v = 0.0;  // -0.0 -> +0.0
-        keys[i] = (uint64_t)__double_as_longlong(v);
-        vals[i] = (int32_t)i;
+    int lo = 0, hi = nseg;   // last segment with off[seg] <= x
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (off[mid] <= x) lo = mid; else hi = mid;
     }
+    return (uint32_t)lo;
 }
 
-__global__ void k_sort_hist(const uint64_t* __restrict__ keys, int64_t n, int shift, int ntiles,
-                            uint32_t* __restrict__ hist)
+// What a pass sorts by: the keys formed from the input (first pass), the
+// keys of the pairs, or the pairs' segment numbers.
+enum { SORT_FIRST, SORT_KEY, SORT_SEG };
+
+template <int KIND>
+__device__ __forceinline__ uint2 sort_load(const SortArray& A, const SortQuant& q, const uint2* src, int64_t i)
+{
+    if (KIND == SORT_FIRST) return make_uint2(q.key(sort_bits(A.in[i])), (uint32_t)i);
+    return src[i];
+}
+
+template <int KIND>
+__device__ __forceinline__ unsigned sort_digit(const SortArray& A, int nseg, uint2 e, int shift)
+{
+    return ((KIND == SORT_SEG ? seg_of(A.off, nseg, e.y) : e.x) >> shift) & 0xFF;
+}
+
+// the array and tile of a CTA: the tiles of a[0], then those of a[1]
+__device__ __forceinline__ int sort_tile_of(const SortPair& S, int blk, int* tile)
+{
+    const int w = blk >= S.a[0].ntiles;
+    *tile = w ? blk - S.a[0].ntiles : blk;
+    return w;
+}
+
+// Digit counts of every tile: hist[tile * kRadix + d].
+template <int KIND>
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortPair S, int from, int shift)
 {
     __shared__ uint32_t h[kRadix];
-    for (int i = threadIdx.x; i < kRadix; i += blockDim.x) h[i] = 0;
+    int tile;
+    const SortArray& A = S.a[sort_tile_of(S, blockIdx.x, &tile)];
+    const SortQuant q = KIND == SORT_FIRST ? sort_quant(A.stats) : SortQuant{0, 0};
+    const uint2* src = A.e[from];
+    h[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const int64_t base = (int64_t)tile * kSortTile;
+#pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
-        int64_t i = base + it * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 0xFF], 1u);
+        const int64_t i = base + it * kSortThreads + threadIdx.x;
+        if (i < A.n) atomicAdd(&h[sort_digit<KIND>(A, S.nseg, sort_load<KIND>(A, q, src, i), shift)], 1u);
     }
     __syncthreads();
-    // digit-major layout: hist[d * ntiles + tile]
-    for (int d = threadIdx.x; d < kRadix; d += blockDim.x)
-        hist[(int64_t)d * ntiles + blockIdx.x] = h[d];
+    A.hist[(int64_t)tile * kRadix + threadIdx.x] = h[threadIdx.x];
 }
 
-// One CTA per digit: exclusive scan of that digit's per-tile counts (in place,
-// hist[d * ntiles + tile]) and the digit's total in tot[d].
-__global__ void k_sort_rowscan(uint32_t* __restrict__ hist, int ntiles, uint32_t* __restrict__ tot)
+// Per digit (thread), the exclusive prefix of the tile counts in place and the
+// digit's total in tot[d]: CTA = 32 digits x 32 runs of tiles.
+__global__ void __launch_bounds__(1024) k_sort_colscan(SortPair S)
 {
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t carry;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t* a = hist + (int64_t)blockIdx.x * ntiles;
-    if (threadIdx.x == 0) carry = 0;
+    __shared__ uint32_t part[32][33];
+    const SortArray& A = S.a[blockIdx.y];
+    const int d = blockIdx.x * 32 + (threadIdx.x & 31), run = threadIdx.x >> 5;
+    const int per = (A.ntiles + 31) >> 5, t0 = run * per, t1 = t0 + per < A.ntiles ? t0 + per : A.ntiles;
+    uint32_t sum = 0;
+    for (int t = t0; t < t1; ++t) sum += A.hist[(int64_t)t * kRadix + d];
+    part[run][threadIdx.x & 31] = sum;
     __syncthreads();
-    for (int base = 0; base < ntiles; base += 1024) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = (i < ntiles) ? a[i] : 0u;
-        uint32_t x = v;
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += t;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t y = wsum[lane];
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, y, off);
-                if (lane >= off) y += t;
-            }
-            wsum[lane] = y;
-        }
-        __syncthreads();
-        const uint32_t incl = x + (warp > 0 ? wsum[warp - 1] : 0u);
-        if (i < ntiles) a[i] = carry + incl - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += incl;
-        __syncthreads();
+    uint32_t acc = 0;
+    for (int r = 0; r < run; ++r) acc += part[r][threadIdx.x & 31];
+    if (run == 31) A.tot[d] = acc + sum;
+    for (int t = t0; t < t1; ++t) {
+        const uint32_t v = A.hist[(int64_t)t * kRadix + d];
+        A.hist[(int64_t)t * kRadix + d] = acc;
+        acc += v;
     }
-    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
 }
 
 // Stable scatter of one pass.  Warp w of a tile owns its 128 consecutive
@@ -114,21 +185,38 @@ __global__ void k_sort_rowscan(uint32_t* __restrict__ hist, int ntiles, uint32_t
 // warp ranks its elements among equal digits with a per-warp digit count in
 // shared memory (warp-synchronous, no CTA barrier per round), then one
 // exclusive prefix over the warps per digit places every warp's run after
-// the earlier warps' in the tile's part of each digit bucket.
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
-    const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t n, int shift, int ntiles,
-    const uint32_t* __restrict__ offs, const uint32_t* __restrict__ tot, uint64_t* __restrict__ kout,
-    int32_t* __restrict__ vout)
+// the earlier warps' in the tile's part of each digit bucket.  With DIRECT
+// (few tiles) the CTA forms the counts of the tiles before it and the totals
+// itself instead of a scan launch between.
+template <int KIND, bool DIRECT>
+__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(SortPair S, int from, int shift)
 {
     constexpr int kWarps = kSortThreads / 32;
     __shared__ uint32_t wcnt[kWarps][kRadix];   // per-warp digit counts, then the warps' starts
     __shared__ uint32_t wsum[kWarps];
+    int tile;
+    const SortArray& A = S.a[sort_tile_of(S, blockIdx.x, &tile)];
+    const SortQuant q = KIND == SORT_FIRST ? sort_quant(A.stats) : SortQuant{0, 0};
+    const uint2* src = A.e[from];
+    uint2* dst = A.e[from ^ 1];
+    const int64_t n = A.n;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // start of digit threadIdx.x's bucket for this tile: exclusive scan of the
     // 256 digit totals plus this tile's offset inside the bucket
     uint32_t mybase;
     {
-        const uint32_t v = tot[threadIdx.x];     // blockDim.x == kRadix
+        uint32_t v = 0, mine = 0;
+        if (DIRECT) {
+#pragma unroll 8
+            for (int t = 0; t < A.ntiles; ++t) {
+                const uint32_t c = A.hist[(int64_t)t * kRadix + threadIdx.x];
+                mine += t < tile ? c : 0u;
+                v += c;
+            }
+        } else {
+            v = A.tot[threadIdx.x];     // blockDim.x == kRadix
+            mine = A.hist[(int64_t)tile * kRadix + threadIdx.x];
+        }
         uint32_t x = v;
         for (int off = 1; off < 32; off <<= 1) {
             const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
@@ -139,21 +227,22 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
         __syncthreads();
         uint32_t pre = 0;
         for (int w = 0; w < warp; ++w) pre += wsum[w];
-        mybase = pre + x - v + offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+        mybase = pre + x - v + mine;
     }
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t wbase = (int64_t)blockIdx.x * kSortTile + (int64_t)warp * (32 * kSortItems);
-    uint64_t key[kSortItems];
-    int32_t val[kSortItems];
+    const int64_t wbase = (int64_t)tile * kSortTile + (int64_t)warp * (32 * kSortItems);
+    uint2 el[kSortItems];
     unsigned dig[kSortItems];
     uint32_t rk[kSortItems];
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
         const int64_t i = wbase + it * 32 + lane;
-        const bool valid = i < n;
-        key[it] = valid ? kin[i] : 0ull;
-        val[it] = valid ? vin[i] : 0;
-        const unsigned d = valid ? (unsigned)((key[it] >> shift) & 0xFF) : 0x100u;
+        el[it] = i < n ? sort_load<KIND>(A, q, src, i) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int it = 0; it < kSortItems; ++it) {
+        const bool valid = wbase + it * 32 + lane < n;
+        const unsigned d = valid ? sort_digit<KIND>(A, S.nseg, el[it], shift) : 0x100u;
         dig[it] = d;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const uint32_t prior = valid ? wcnt[warp][d] : 0u;
@@ -174,20 +263,286 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
     }
     __syncthreads();
 #pragma unroll
-    for (int it = 0; it < kSortItems; ++it) {
-        if (dig[it] < 0x100u) {
-            const uint32_t pos = wcnt[warp][dig[it]] + rk[it];
-            kout[pos] = key[it];
-            vout[pos] = val[it];
+    for (int it = 0; it < kSortItems; ++it)
+        if (dig[it] < 0x100u) dst[wcnt[warp][dig[it]] + rk[it]] = el[it];
+}
+
+__device__ __forceinline__ void sort_put(const SortArray& A, int64_t pos, uint64_t bits, uint32_t idx)
+{
+    const double v = __longlong_as_double((long long)bits);
+    A.out[pos] = v;
+    A.perm[pos] = (int32_t)idx;
+    const float h = (float)v;
+    A.split[pos] = make_float2(h, (float)(v - (double)h));
+}
+
+// Writes the sorted values, their indices and their double-float parts.  An
+// element of a run of equal keys (and segments) goes to its rank by full
+// pattern within the run; equal patterns keep their order.  Runs of more than
+// kRunMax stay as they are, are listed, and set runh[1] when two neighbours
+// of one are out of order (k_sort_runs then sorts them).
+__global__ void __launch_bounds__(kSortThreads) k_sort_finish(SortPair S, int from)
+{
+    const SortArray& A = S.a[blockIdx.y];
+    const uint2* e = A.e[from];
+    const SortQuant q = sort_quant(A.stats);
+    auto bits_of = [&](int64_t i) { return sort_bits(A.in[e[i].y]); };
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint2 el = e[i];
+        const uint64_t b = sort_bits(A.in[el.y]);
+        auto same = [&](int64_t k) {
+            if (k < 0 || k >= A.n) return false;
+            const uint2 o = e[k];
+            return o.x == el.x && (S.nseg <= 1 || seg_of(A.off, S.nseg, o.y) == seg_of(A.off, S.nseg, el.y));
+        };
+        int64_t pos = i;
+        if (q.shift > 0 && el.x != 0) {
+            int left = 0, right = 0;
+            while (left < kRunMax && same(i - left - 1)) ++left;
+            while (right < kRunMax && same(i + right + 1)) ++right;
+            if (left + right + 1 <= kRunMax) {
+                int rank = 0;
+                for (int k = 1; k <= left; ++k) rank += bits_of(i - k) <= b;
+                for (int k = 1; k <= right; ++k) rank += bits_of(i + k) < b;
+                pos = i - left + rank;
+            } else {
+                if (left == 0) {
+                    const uint32_t slot = atomicAdd(A.runh, 1u);
+                    A.runs[slot] = (uint32_t)i;   // at most n / kRunMax long runs
+                }
+                if (left > 0 && bits_of(i - 1) > b) A.runh[1] = 1u;
+            }
         }
+        sort_put(A, pos, b, el.y);
     }
 }
 
-__global__ void k_sort_finish(const uint64_t* __restrict__ keys, int64_t n, double* __restrict__ out)
+// Runs of more than kRunMax equal keys that are out of order: one CTA per run,
+// a stable radix sort of the remaining low bits of the patterns, ping-pong
+// between the two pair arrays' parts of the run (which other runs' searches
+// may read: every pair there has this run's key and segment).  Inputs need values packed
+// more densely than 1 / kRunMax of a 2^-31 step of their range for it; it
+// returns at once otherwise.
+__global__ void __launch_bounds__(1024) k_sort_runs(SortPair S, int from)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = __longlong_as_double((long long)keys[i]);
+    __shared__ uint32_t cnt[32][kRadix];
+    __shared__ uint32_t base[kRadix], wtot[kRadix / 32];
+    const SortArray& A = S.a[blockIdx.y];
+    if (A.runh[1] == 0) return;
+    const uint32_t nruns = A.runh[0];
+    const SortQuant q = sort_quant(A.stats);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (uint32_t rr = blockIdx.x; rr < nruns; rr += gridDim.x) {
+        const int64_t s = A.runs[rr];
+        const uint2 first = A.e[from][s];
+        const uint32_t seg = S.nseg > 1 ? seg_of(A.off, S.nseg, first.y) : 0u;
+        // end of the run: first later pair with another segment or key
+        int64_t lo = s + 1, hi = A.n;
+        while (lo < hi) {
+            const int64_t mid = lo + ((hi - lo) >> 1);
+            const uint2 o = A.e[from][mid];
+            const bool in = o.x == first.x && (S.nseg <= 1 || seg_of(A.off, S.nseg, o.y) == seg);
+            if (in) lo = mid + 1; else hi = mid;
+        }
+        const int64_t len = lo - s;
+        int cur = from;
+        for (int sh = 0; sh < q.shift; sh += 8, cur ^= 1) {
+            auto digit = [&](uint2 el) {
+                return (unsigned)(((sort_bits(A.in[el.y]) - q.lo) & ((1ull << q.shift) - 1)) >> sh) & 0xFFu;
+            };
+            const uint2* src = A.e[cur] + s;
+            uint2* dst = A.e[cur ^ 1] + s;
+            if (threadIdx.x < kRadix) base[threadIdx.x] = 0;
+            __syncthreads();
+            for (int64_t i = threadIdx.x; i < len; i += blockDim.x) atomicAdd(&base[digit(src[i])], 1u);
+            __syncthreads();
+            uint32_t v = 0, x = 0;
+            if (threadIdx.x < kRadix) {
+                v = base[threadIdx.x];
+                x = v;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
+                    if (lane >= off) x += t;
+                }
+                if (lane == 31) wtot[warp] = x;
+            }
+            __syncthreads();
+            if (threadIdx.x < kRadix) {
+                uint32_t pre = 0;
+                for (int w = 0; w < warp; ++w) pre += wtot[w];
+                base[threadIdx.x] = pre + x - v;
+            }
+            for (int64_t t0 = 0; t0 < len; t0 += blockDim.x) {
+                for (int i = threadIdx.x; i < 32 * kRadix; i += blockDim.x) (&cnt[0][0])[i] = 0;
+                __syncthreads();
+                const int64_t i = t0 + threadIdx.x;
+                const bool valid = i < len;
+                const uint2 el = valid ? src[i] : make_uint2(0u, 0u);
+                const unsigned d = valid ? digit(el) : 0x100u;
+                const unsigned peers = __match_any_sync(0xffffffffu, d);
+                if (valid && (peers & lt) == 0) cnt[warp][d] = __popc(peers);
+                __syncthreads();
+                if (threadIdx.x < kRadix) {
+                    uint32_t run = base[threadIdx.x];
+                    for (int w = 0; w < 32; ++w) {
+                        const uint32_t c = cnt[w][threadIdx.x];
+                        cnt[w][threadIdx.x] = run;
+                        run += c;
+                    }
+                    base[threadIdx.x] = run;
+                }
+                __syncthreads();
+                if (valid) dst[cnt[warp][d] + __popc(peers & lt)] = el;
+                __syncthreads();
+            }
+        }
+        for (int64_t i = threadIdx.x; i < len; i += blockDim.x) {
+            const uint2 el = A.e[cur][s + i];
+            sort_put(A, s + i, sort_bits(A.in[el.y]), el.y);
+        }
+        __syncthreads();
+    }
+}
+
+// Small arrays: one CTA each (blockIdx.x), everything in one launch.  Thread t
+// of warp w holds the pairs w 32 ITEMS + 32 it + lane, so that (warp, it,
+// lane) is the current order; each pass ranks them as k_sort_scatter does and
+// writes them back to shared memory in their new order.
+constexpr int kSmallThreads = 1024;
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kSmallThreads) k_sort_small(SortPair S)
+{
+    extern __shared__ uint2 pairs[];                     // [1024 ITEMS]
+    uint32_t* wcnt = (uint32_t*)(pairs + kSmallThreads * ITEMS);   // [32][kRadix]
+    __shared__ uint32_t wsum[32];
+    __shared__ unsigned long long st[2];
+    const SortArray& A = S.a[blockIdx.x];
+    const int n = (int)A.n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int wbase = warp * 32 * ITEMS + lane;
+    if (threadIdx.x < 2) st[threadIdx.x] = 0;
+    __syncthreads();
+    uint64_t bits[ITEMS];
+    {
+        uint64_t mn = 0, mx = 0;
+        int bad = 0;
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const int i = wbase + 32 * it;
+            const double v = i < n ? A.in[i] : 0.0;
+            if (!in_domain(v)) bad = 1;
+            const uint64_t b = sort_bits(v);
+            bits[it] = b;
+            if (b && ~b > mn) mn = ~b;
+            if (b > mx) mx = b;
+        }
+        warp_range(mn, mx);
+        if (lane == 0) {
+            if (mn) atomicMax(&st[0], (unsigned long long)mn);
+            if (mx) atomicMax(&st[1], (unsigned long long)mx);
+        }
+        if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(A.flag, 1);
+    }
+    const SortQuant q = sort_quant(st);
+    uint2 el[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) el[it] = make_uint2(q.key(bits[it]), (uint32_t)(wbase + 32 * it));
+    for (int shift = 0; shift < 32; shift += 8) {
+        for (int i = threadIdx.x; i < 32 * kRadix; i += kSmallThreads) wcnt[i] = 0;
+        __syncthreads();
+        uint32_t rk[ITEMS];
+        unsigned dig[ITEMS];
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const bool valid = wbase + 32 * it < n;
+            const unsigned d = valid ? (el[it].x >> shift) & 0xFFu : 0x100u;
+            dig[it] = d;
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t prior = valid ? wcnt[warp * kRadix + d] : 0u;
+            __syncwarp();
+            if (valid && (peers & lt) == 0) wcnt[warp * kRadix + d] = prior + __popc(peers);
+            __syncwarp();
+            rk[it] = prior + __popc(peers & lt);
+        }
+        __syncthreads();
+        uint32_t tot = 0, x = 0;
+        if (threadIdx.x < kRadix) {
+            for (int w = 0; w < 32; ++w) {
+                const uint32_t t = wcnt[w * kRadix + threadIdx.x];
+                wcnt[w * kRadix + threadIdx.x] = tot;
+                tot += t;
+            }
+            x = tot;
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
+                if (lane >= off) x += t;
+            }
+            if (lane == 31) wsum[warp] = x;
+        }
+        __syncthreads();
+        if (threadIdx.x < kRadix) {
+            uint32_t pre = x - tot;
+            for (int w = 0; w < warp; ++w) pre += wsum[w];
+            for (int w = 0; w < 32; ++w) wcnt[w * kRadix + threadIdx.x] += pre;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it)
+            if (dig[it] < 0x100u) pairs[wcnt[warp * kRadix + dig[it]] + rk[it]] = el[it];
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it)
+            if (wbase + 32 * it < n) el[it] = pairs[wbase + 32 * it];
+        // (the next pass writes pairs only after a barrier)
+    }
+    // runs of equal keys: each element to its rank by full pattern
+    bool fix = false;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const int i = wbase + 32 * it;
+        if (i < n) {
+            bits[it] = sort_bits(A.in[el[it].y]);
+            if (i > 0 && pairs[i - 1].x == el[it].x && sort_bits(A.in[pairs[i - 1].y]) > bits[it]) fix = true;
+        }
+    }
+    const bool any = __syncthreads_or(fix);
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const int i = wbase + 32 * it;
+        if (i >= n) continue;
+        int pos = i;
+        if (any && el[it].x != 0) {
+            int left = 0, rank = 0;
+            for (int k = i - 1; k >= 0 && pairs[k].x == el[it].x; --k, ++left)
+                rank += sort_bits(A.in[pairs[k].y]) <= bits[it];
+            for (int k = i + 1; k < n && pairs[k].x == el[it].x; ++k) rank += sort_bits(A.in[pairs[k].y]) < bits[it];
+            pos = i - left + rank;
+        }
+        sort_put(A, pos, bits[it], el[it].y);
+    }
+}
+
+// nrep copies of a plan's sorted arrays, one after the other (derivative plans).
+__global__ void k_replicate(SortedView src, SortedView dst, int64_t n, int64_t m, int nrep)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nrep * (n > m ? n : m);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        if (i < nrep * n) {
+            const int64_t k = i % n;
+            dst.r[i] = src.r[k];
+            dst.r2[i] = src.r2[k];
+            dst.pr[i] = src.pr[k];
+        }
+        if (i < nrep * m) {
+            const int64_t k = i % m;
+            dst.w[i] = src.w[k];
+            dst.w2[i] = src.w2[k];
+            dst.pw[i] = src.pw[k];
+        }
+    }
 }
 
 __global__ void k_gather(const double* __restrict__ c, const int32_t* __restrict__ perm, int64_t n,
@@ -203,17 +558,6 @@ __global__ void k_gather(const double* __restrict__ c, const int32_t* __restrict
             const float h = (float)v;
             out2[i] = make_float2(h, (float)(v - (double)h));
         }
-    }
-}
-
-// x as double-float pairs (hi = nearest float, lo = nearest float to the rest)
-__global__ void k_split_f64(const double* __restrict__ x, int64_t n, float2* __restrict__ out)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = x[i];
-        const float h = (float)v;
-        out[i] = make_float2(h, (float)(v - (double)h));
     }
 }
 
@@ -323,24 +667,6 @@ __global__ void __launch_bounds__(kStairThreads) k_staircase(const double* __res
     }
 }
 
-// Tile i of a list: segment b with prefix[b] <= i < prefix[b + 1] (binary
-// search), then its start and count inside the segment's index range.
-__global__ void k_expand_tiles(const Seg* __restrict__ segs, const int32_t* __restrict__ prefix, int nseg,
-                               int total, Tile* __restrict__ out)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        int lo = 0, hi = nseg;   // last b with prefix[b] <= i
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (prefix[mid] <= i) lo = mid; else hi = mid;
-        }
-        const Seg sg = segs[lo];
-        const int64_t start = sg.first + (int64_t)(i - prefix[lo]) * sg.len;
-        const int64_t rem = sg.last - start + 1;
-        out[i] = Tile{sg.blk, (int32_t)(rem < sg.len ? rem : sg.len), start};
-    }
-}
-
 inline int grid_for(int64_t n, int threads)
 {
     int64_t b = (n + threads - 1) / threads;
@@ -353,94 +679,90 @@ inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
 
-cudaError_t launch_check_domain(const double* x, int64_t n, int* flag, cudaStream_t s)
+size_t sort_scratch_bytes(int64_t n)
 {
-    if (n <= 0) return cudaSuccess;
-    k_check_domain<<<grid_for(n, 256), 256, 0, s>>>(x, n, flag);
+    const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
+    return 2 * align256(sizeof(uint2) * (size_t)n) +
+           align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)(ntiles > 0 ? ntiles : 1)) +
+           align256(sizeof(uint32_t) * (size_t)kRadix) + align256(sizeof(uint32_t) * (size_t)(n / kRunMax + 2));
+}
+
+namespace {
+
+template <int ITEMS>
+cudaError_t sort_small(const SortPair& S, cudaStream_t s)
+{
+    const size_t smem = sizeof(uint2) * kSmallThreads * ITEMS + sizeof(uint32_t) * 32 * kRadix;
+    cudaError_t e = cudaFuncSetAttribute(k_sort_small<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_sort_small<ITEMS><<<2, kSmallThreads, smem, s>>>(S);
     count_launches(1);
     return cudaGetLastError();
 }
 
-size_t radix_sort_scratch_bytes(int64_t n)
+template <int KIND>
+void sort_pass(const SortPair& S, int from, int shift, bool direct, cudaStream_t s)
 {
-    int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    return 2 * align256(sizeof(uint64_t) * (size_t)n) + align256(sizeof(int32_t) * (size_t)n) +
-           align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)(ntiles > 0 ? ntiles : 1)) +
-           align256(sizeof(uint32_t) * (size_t)kRadix);
+    const int nt = S.a[0].ntiles + S.a[1].ntiles;
+    k_sort_hist<KIND><<<nt, kSortThreads, 0, s>>>(S, from, shift);
+    if (direct) {
+        k_sort_scatter<KIND, true><<<nt, kSortThreads, 0, s>>>(S, from, shift);
+    } else {
+        k_sort_colscan<<<dim3(kRadix / 32, 2), 1024, 0, s>>>(S);
+        k_sort_scatter<KIND, false><<<nt, kSortThreads, 0, s>>>(S, from, shift);
+    }
+    count_launches(direct ? 2 : 3);
 }
 
-// seg[i] = segment of the element at input index perm[i] (offsets off[0..nseg]),
-// as a radix key.
-__global__ void k_seg_keys(const int32_t* __restrict__ perm, int64_t n, const int64_t* __restrict__ off,
-                           int nseg, uint64_t* __restrict__ keys)
+}  // namespace
+
+// Checks and sorts both arrays (out, perm, split); scratch as
+// sort_scratch_bytes each, flag, stats[2] and runh[2] of each array zeroed.
+// With nseg > 1 segments (device offsets off[0..nseg], nseg <= 65536) each
+// segment is sorted on its own: the key passes are followed by stable passes
+// on the segment number, so the output keeps the segments in order.
+cudaError_t launch_sort_pair(SortPair S, char* const scratch[2], cudaStream_t s)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = perm[i];
-        int lo = 0, hi = nseg;   // last segment with off[seg] <= x
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (off[mid] <= x) lo = mid; else hi = mid;
-        }
-        keys[i] = (uint64_t)lo;
+    if (S.a[0].n <= 0 && S.a[1].n <= 0) return cudaSuccess;
+    const int64_t most = S.a[0].n > S.a[1].n ? S.a[0].n : S.a[1].n;
+    if (S.nseg <= 1 && most <= kSmallSort) {
+        if (most <= 1 * kSmallThreads) return sort_small<1>(S, s);
+        if (most <= 4 * kSmallThreads) return sort_small<4>(S, s);
+        return sort_small<kSmallSort / kSmallThreads>(S, s);
     }
+    bool direct = true;
+    for (int k = 0; k < 2; ++k) {
+        SortArray& A = S.a[k];
+        char* p = scratch[k];
+        A.ntiles = (int)((A.n + kSortTile - 1) / kSortTile);
+        A.e[0] = (uint2*)p; p += align256(sizeof(uint2) * (size_t)A.n);
+        A.e[1] = (uint2*)p; p += align256(sizeof(uint2) * (size_t)A.n);
+        A.hist = (uint32_t*)p; p += align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)(A.ntiles > 0 ? A.ntiles : 1));
+        A.tot = (uint32_t*)p; p += align256(sizeof(uint32_t) * (size_t)kRadix);
+        A.runs = (uint32_t*)p;
+        direct = direct && A.ntiles <= kSortDirectTiles;
+    }
+    const dim3 all(grid_for(most, kSortThreads), 2);
+    const int64_t few = (most + 8 * kSortThreads - 1) / (8 * kSortThreads), cap = 2 * (int64_t)device_sm_count();
+    k_sort_range<<<dim3((unsigned)(few < cap ? few : cap), 2), kSortThreads, 0, s>>>(S);
+    sort_pass<SORT_FIRST>(S, 1, 0, direct, s);
+    int cur = 0;
+    for (int shift = 8; shift < 32; shift += 8, cur ^= 1) sort_pass<SORT_KEY>(S, cur, shift, direct, s);
+    for (int shift = 0; S.nseg > 1 && (shift == 0 || (S.nseg - 1) >> shift); shift += 8, cur ^= 1)
+        sort_pass<SORT_SEG>(S, cur, shift, direct, s);
+    k_sort_finish<<<all, kSortThreads, 0, s>>>(S, cur);
+    k_sort_runs<<<dim3(device_sm_count(), 2), 1024, 0, s>>>(S, cur);
+    count_launches(3);
+    return cudaGetLastError();
 }
 
-__global__ void k_gather_keys(const double* __restrict__ in, const int32_t* __restrict__ perm, int64_t n,
-                              double* __restrict__ out)
+cudaError_t launch_replicate(const SortedView& src, const SortedView& dst, int64_t n, int64_t m, int nrep,
+                             cudaStream_t s)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double v = in[perm[i]];
-        out[i] = (v == 0.0) ? 0.0 : v;
-    }
-}
-
-// Sorts in[0..n) ascending into out, perm[i] = input index of out[i].  With
-// nseg > 1 segments (device offsets off[0..nseg], nseg <= 65536) each segment
-// is sorted on its own: the value passes are followed by two stable passes on
-// the segment number, so the output keeps the segments in order.
-cudaError_t radix_sort_f64(const double* in, int64_t n, double* out, int32_t* perm, void* scratch,
-                           size_t scratch_bytes, cudaStream_t s, const int64_t* off, int nseg)
-{
-    if (n <= 0) return cudaSuccess;
-    if (scratch_bytes < radix_sort_scratch_bytes(n)) return cudaErrorInvalidValue;
-    int ntiles = (int)((n + kSortTile - 1) / kSortTile);
-    char* p = (char*)scratch;
-    uint64_t* k0 = (uint64_t*)p; p += align256(sizeof(uint64_t) * (size_t)n);
-    uint64_t* k1 = (uint64_t*)p; p += align256(sizeof(uint64_t) * (size_t)n);
-    int32_t* v1 = (int32_t*)p; p += align256(sizeof(int32_t) * (size_t)n);
-    uint32_t* hist = (uint32_t*)p; p += align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)ntiles);
-    uint32_t* tot = (uint32_t*)p;
-    int32_t* v0 = perm;   // ping-pong between perm and v1; 8 passes end in perm
-    k_sort_init<<<grid_for(n, 256), 256, 0, s>>>(in, n, k0, v0);
-    uint64_t* ka = k0; uint64_t* kb = k1;
-    int32_t* va = v0; int32_t* vb = v1;
-    for (int pass = 0; pass < 8; ++pass) {
-        int shift = 8 * pass;
-        k_sort_hist<<<ntiles, kSortThreads, 0, s>>>(ka, n, shift, ntiles, hist);
-        k_sort_rowscan<<<kRadix, 1024, 0, s>>>(hist, ntiles, tot);
-        k_sort_scatter<<<ntiles, kSortThreads, 0, s>>>(ka, va, n, shift, ntiles, hist, tot, kb, vb);
-        uint64_t* tk = ka; ka = kb; kb = tk;
-        int32_t* tv = va; va = vb; vb = tv;
-    }
-    // after an even number of passes the data is back in (k0, perm)
-    if (nseg <= 1) {
-        k_sort_finish<<<grid_for(n, 256), 256, 0, s>>>(ka, n, out);
-        count_launches(2 + 8 * 3);
-        return cudaGetLastError();
-    }
-    k_seg_keys<<<grid_for(n, 256), 256, 0, s>>>(perm, n, off, nseg, ka);
-    for (int pass = 0; pass < 2; ++pass) {
-        const int shift = 8 * pass;
-        k_sort_hist<<<ntiles, kSortThreads, 0, s>>>(ka, n, shift, ntiles, hist);
-        k_sort_rowscan<<<kRadix, 1024, 0, s>>>(hist, ntiles, tot);
-        k_sort_scatter<<<ntiles, kSortThreads, 0, s>>>(ka, va, n, shift, ntiles, hist, tot, kb, vb);
-        uint64_t* tk = ka; ka = kb; kb = tk;
-        int32_t* tv = va; va = vb; vb = tv;
-    }
-    k_gather_keys<<<grid_for(n, 256), 256, 0, s>>>(in, perm, n, out);
-    count_launches(1 + 10 * 3 + 2);
+    const int64_t most = nrep * (n > m ? n : m);
+    if (most <= 0) return cudaSuccess;
+    k_replicate<<<grid_for(most, 256), 256, 0, s>>>(src, dst, n, m, nrep);
+    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -480,15 +802,6 @@ cudaError_t launch_staircase_many(const double* r, const double* w, int64_t m, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_expand_tiles(const Seg* segs, const int32_t* prefix, int nseg, int total, Tile* out,
-                                cudaStream_t s)
-{
-    if (total <= 0 || nseg <= 0) return cudaSuccess;
-    k_expand_tiles<<<grid_for(total, 256), 256, 0, s>>>(segs, prefix, nseg, total, out);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int stride, int comp,
                           const unsigned long long* mx, double* out, float2* out2, cudaStream_t s)
 {
@@ -522,14 +835,6 @@ cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t 
 {
     if (mb <= 0) return cudaSuccess;
     k_scatter_deriv<<<grid_for(mb, 256), 256, 0, s>>>(gs, perm, mb, stride, comp, mx, y, out);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_split_f64(const double* x, int64_t n, float2* out, cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    k_split_f64<<<grid_for(n, 256), 256, 0, s>>>(x, n, out);
     count_launches(1);
     return cudaGetLastError();
 }

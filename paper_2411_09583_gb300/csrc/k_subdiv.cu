@@ -21,9 +21,6 @@
 
 namespace nuht {
 
-// streaming multiprocessors of the current device, cached per device (k_det.cu)
-int device_sm_count();
-
 namespace {
 
 constexpr int kSubThreads = 1024;
@@ -444,28 +441,6 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide_grid(
     }
 }
 
-// Sorted values at the block edges: local blocks R = r_{j1}; asymptotic
-// blocks (r_{j0}, r_{j1}, omega_{k0}, omega_{k1}).  Counts from res (device).
-__global__ void k_block_bounds(const SubBlk* __restrict__ loc, const SubBlk* __restrict__ asy,
-                               const int64_t* __restrict__ res, const ProbParams* __restrict__ probs,
-                               const double* __restrict__ r_s, const double* __restrict__ w_s,
-                               double* __restrict__ bl, double4* __restrict__ ba)
-{
-    const int64_t nl = res[0], na = res[1];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nl + na;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < nl) {
-            const SubBlk b = loc[i];
-            bl[i] = r_s[probs[b.prob].r_off + b.j1];
-        } else {
-            const SubBlk b = asy[i - nl];
-            const ProbParams& P = probs[b.prob];
-            ba[i - nl] = make_double4(r_s[P.r_off + b.j0], r_s[P.r_off + b.j1], w_s[P.w_off + b.k0],
-                                      w_s[P.w_off + b.k1]);
-        }
-    }
-}
-
 }  // namespace
 
 int subdivide_grid_ctas()
@@ -499,14 +474,6 @@ cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const doub
     }
     k_subdivide<<<1, kSubThreads, 0, s>>>(stair, r_s, w_s, probs, nprob, min_size, n_cand, qa, qb, qcap, out, ocap,
                                           res);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_block_bounds(const SubBlk* loc, const SubBlk* asy, const int64_t* res, const ProbParams* probs,
-                                const double* r_s, const double* w_s, double* bl, double4* ba, cudaStream_t s)
-{
-    k_block_bounds<<<device_sm_count() * 8, 256, 0, s>>>(loc, asy, res, probs, r_s, w_s, bl, ba);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -155,7 +155,7 @@ struct Tile {
 };
 
 // A run of tiles: indices first..last of block blk cut into tiles of len.
-// Tile lists are expanded from these on the device (k_expand_tiles).  FFT work
+// Tile lists are expanded from these on the device (k_expand_lists).  FFT work
 // items are tiles of length one whose start is the item's ordinal in its
 // block (q for single-pass FFTs, q * lines + line for the two-pass passes).
 struct Seg {
@@ -181,12 +181,22 @@ enum { MX_DIR_ROWS, MX_DIR_COLS, MX_DIR_AREA, MX_NF2_SMALL, MX_LOG2, MX_ERR, MX_
 enum { LIST_MOM, LIST_EVAL, LIST_SPREAD, LIST_INTERP, LIST_FSMALL, LIST_FA, LIST_FB, LIST_FBLOCK,
        LIST_P0, LIST_P1, LIST_P2, kLists };
 
+// What a plan build reads back from the device in one copy (zeroed first).
+struct PlanCounts {
+    int flag[2];                    // a point / frequency is outside the domain
+    uint32_t runh[2][2];            // SortArray::runh
+    unsigned long long stats[2][2]; // SortArray::stats
+    int64_t res[4];                 // blocks of each class, lists overflowed
+    int64_t totals[kTotals];
+    int64_t maxv[kMaxv];
+    unsigned ticket;
+};
+
 struct BlockBuild {
     const int64_t* res;       // counts of local, asymptotic, direct blocks (device)
     const SubBlk* sub;        // [3][ocap] the subdivision's lists, problem-local indices
     int64_t ocap;
-    const double* bl;         // [nl] r at the last column of each local block
-    const double4* ba;        // [na] (r_j0, r_j1, omega_k0, omega_k1) of each asymptotic block
+    const double *r_s, *w_s;  // sorted points and frequencies
     const ProbParams* probs;
     int w, mom_tile, eval_tile, spread_tile, interp_tile;
     int lowp;                 // mixed precision: the FP32 FFT's lists are built too
@@ -199,7 +209,11 @@ struct BlockBuild {
     int64_t* dcnt;            // [nd][kDirCols]
     int64_t* totals;          // [kTotals] column sums
     int64_t* maxv;            // [kMaxv]
+    unsigned* ticket;         // CTAs of k_block_sizes done (zeroed, as totals and maxv)
+    int64_t* part;            // [3][ptiles][kAsyCols] column sums of every kBlockTile rows, then their prefix
+    int64_t ptiles;
 };
+constexpr int kBlockTile = 256;
 
 struct BuildLists {
     LocalBlock* loc;
@@ -208,16 +222,16 @@ struct BuildLists {
     Seg* seg[kLists];
     int32_t* pre[kLists];     // [nseg + 1] tiles before each segment
     SubBlk* blk;              // [nl + na + nd] every block in global sorted indices
+    int* status;              // the plan's device status word, cleared
 };
 
-int64_t block_scan_scratch(int64_t cap);   // int64 elements of scratch for launch_block_build
-cudaError_t launch_block_build(const BlockBuild& bb, int64_t* scratch, cudaStream_t s);
-cudaError_t launch_block_fill(const BlockBuild& bb, const BuildLists& L, cudaStream_t s);
+cudaError_t launch_block_build(const BlockBuild& bb, cudaStream_t s);
+// max_rows: the largest of the class counts
+cudaError_t launch_block_fill(const BlockBuild& bb, const BuildLists& L, int64_t max_rows, cudaStream_t s);
 
 // Kernel tables shared by every asymptotic block of a plan.
 struct Tables {
-    const double* es;      // [w][deg + 1] monomial coefficients in v = 2 z0 - 1
-    const float2* es2;     // the same as double-float (hi, lo)
+    const float2* es2;     // [w][deg + 1] monomial coefficients in v = 2 z0 - 1, double-float (hi, lo)
     int w, deg;
     int deg_comp;          // degrees above this one are evaluated in plain FP32
     const float2* ch2;     // [w][deg + 1] pieces in the Chebyshev basis T_d(v), double-float
@@ -227,8 +241,7 @@ struct Tables {
     float fold_tol;        // truncation of the spreading weights' Chebyshev form within a bin
     float fold_df_tol;     // weights' Chebyshev terms above this need double-float moments
     double half_w;         // w / 2
-    const double* ph;      // psi-hat pieces [ph_pieces][ph_deg + 1] in v in [-1, 1]
-    const float2* ph2;     // the same as double-float
+    const float2* ph2;     // psi-hat pieces [ph_pieces][ph_deg + 1] in v in [-1, 1], double-float
     double interp_const;   // sqrt(2/pi) * 4 / w^2
     float2 ic2;            // the same as double-float
     float2 ph_scale2;      // ph_scale as double-float
@@ -236,8 +249,7 @@ struct Tables {
     int ph_comp;           // psi-hat degrees above this one are evaluated in plain FP32
     double ph_scale;       // pieces per unit of xi
     double ph_xmax;        // table covers xi in [0, ph_xmax]
-    const double2* tw;     // e^{2 pi i k / 2^tw_log2}, k < 2^(tw_log2 - 1)
-    const float4* tw2;     // the same as double-float (cos.h, cos.l, sin.h, sin.l)
+    const float4* tw2;     // e^{2 pi i k / 2^tw_log2}, k < 2^(tw_log2 - 1), double-float (cos.h, cos.l, sin.h, sin.l)
     int tw_log2;
 };
 
@@ -245,11 +257,37 @@ struct Tables {
 // (each returns cudaGetLastError() of its launch and adds the number of
 // kernels it launched to the library's launch counter)
 void count_launches(int k);
-cudaError_t launch_check_domain(const double* x, int64_t n, int* flag, cudaStream_t s);
-cudaError_t radix_sort_f64(const double* in, int64_t n, double* out, int32_t* perm,
-                           void* scratch, size_t scratch_bytes, cudaStream_t s,
-                           const int64_t* seg_off = nullptr, int nseg = 1);
-size_t radix_sort_scratch_bytes(int64_t n);
+// Sorting a plan's points (a[0]) and frequencies (a[1]) (k_sort.cu).
+constexpr int kSmallSort = 8192;   // up to this many of each: one CTA per array, one launch
+struct SortArray {
+    const double* in;            // unsorted values
+    int64_t n;
+    const int64_t* off;          // segment offsets (batches)
+    double* out;                 // sorted values,
+    int32_t* perm;               // their input indices
+    float2* split;               // and double-float parts
+    int* flag;                   // set when a value is outside the domain
+    unsigned long long* stats;   // [2] value range (zeroed)
+    uint32_t* runh;              // [2] number of long runs of equal keys, whether one is unsorted (zeroed)
+    // set by launch_sort_pair
+    int ntiles;
+    uint2* e[2];
+    uint32_t *hist, *tot, *runs;
+};
+struct SortPair {
+    SortArray a[2];
+    int nseg;
+};
+size_t sort_scratch_bytes(int64_t n);
+cudaError_t launch_sort_pair(SortPair S, char* const scratch[2], cudaStream_t s);
+// The sorted arrays of a plan.
+struct SortedView {
+    double *r, *w;
+    int32_t *pr, *pw;
+    float2 *r2, *w2;
+};
+cudaError_t launch_replicate(const SortedView& src, const SortedView& dst, int64_t n, int64_t m, int nrep,
+                             cudaStream_t s);
 
 cudaError_t launch_staircase(const double* r, int64_t n, const double* w, int64_t m, double z,
                              int32_t* s_out, cudaStream_t s);
@@ -265,8 +303,6 @@ cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const doub
                              int nprob, int64_t min_size,
                              int n_cand, SubBlk* qa, SubBlk* qb, int64_t qcap, SubBlk* out, int64_t ocap,
                              int64_t* res, int4* ctot, int64_t* gst, int grid_ctas, cudaStream_t s);
-cudaError_t launch_block_bounds(const SubBlk* loc, const SubBlk* asy, const int64_t* res, const ProbParams* probs,
-                                const double* r_s, const double* w_s, double* bl, double4* ba, cudaStream_t s);
 cudaError_t launch_staircase_many(const double* r, const double* w, int64_t m, const ProbParams* probs,
                                   int nprob, int32_t* s_out, cudaStream_t s);
 // per-call input scaling (k_det.cu): *mx = the bits of the largest |x_i|
@@ -284,8 +320,16 @@ cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t 
                                  const unsigned long long* mx, const double* y, double* out, cudaStream_t s);
 cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int stride, int comp,
                           const unsigned long long* mx, double* out, float2* out2, cudaStream_t s);
-cudaError_t launch_expand_tiles(const Seg* segs, const int32_t* prefix, int nseg, int total, Tile* out,
-                                cudaStream_t s);
+// Every tile list of a plan from its segments (list i at tiles[i], ntile[i]
+// tiles), and the path of each spreading tile (modes).
+struct ExpandLists {
+    const Seg* seg[kLists];
+    const int32_t* pre[kLists];
+    Tile* tiles[kLists];
+    int nseg[kLists], ntile[kLists];
+};
+cudaError_t launch_expand_lists(const ExpandLists& E, const ProbParams* probs, const AsyBlock* blks, Tables tab,
+                                const double* r_s, int32_t* modes, cudaStream_t s);
 cudaError_t launch_scatter(const double* gs, const int32_t* perm, int64_t m, int stride, int comp,
                            const unsigned long long* mx, double* g, cudaStream_t s);
 
@@ -358,11 +402,6 @@ cudaError_t launch_local_adj_eval(const ProbParams* probs, const LocalBlock* blk
 cudaError_t launch_direct_adj(const ProbParams* probs, const DirectBlock* blks, int nblk, int max_cols,
                               int max_area, int lowp, const double* r_s, const double* w_s, const float2* r2,
                               const float2* w2, const double* g_s, double* c_s, int det, cudaStream_t s);
-// x[i] as double-float (hi, lo)
-cudaError_t launch_split_f64(const double* x, int64_t n, float2* out, cudaStream_t s);
-// Per spreading tile, the path of k_asy_spread (plan time; modes[ntiles]).
-cudaError_t launch_spread_modes(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles, int ntiles,
-                                Tables tab, const double* r_s, int32_t* modes, cudaStream_t s);
 // members: real components spread by one launch (coefficients c2 + v c_stride,
 // grids grid_b + v gb_stride); 1 in the deterministic mode.
 cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,

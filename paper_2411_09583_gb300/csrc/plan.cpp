@@ -66,6 +66,7 @@ struct nuht_plan_s {
 
     // device memory
     char* dmem = nullptr;
+    char* dsort = nullptr;   // the sorted arrays (their sizes are known before the blocks are)
     size_t dbytes = 0;
     ProbParams* d_prob = nullptr;
     double *d_r = nullptr, *d_w = nullptr;
@@ -91,8 +92,6 @@ struct nuht_plan_s {
     // moments and sums
     double *d_csb = nullptr, *d_gsb = nullptr, *d_momb = nullptr;
     float2* d_cs2b = nullptr;
-    double *d_es = nullptr, *d_ph = nullptr;
-    double2* d_tw = nullptr;
     // per-call input scaling: the bits of the largest input magnitude
     unsigned long long* d_mx = nullptr;
     // persistent local stage: queue head, per-block moment-tile counts and the
@@ -229,32 +228,20 @@ struct Staging {
 std::mutex g_stage_mu;
 Staging g_stage_in, g_stage_out;
 
-// Per-device auxiliary stream (and fork / join events) for the independent
-// halves of a plan build, used under g_stage_mu.
-struct Aux {
-    cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-    cudaEvent_t stage_done = nullptr;   // the last upload from g_stage_out on this device
-};
+// Per device, the event of the last upload from g_stage_out (under g_stage_mu).
+cudaEvent_t g_stage_done[64];
 cudaEvent_t g_stage_out_event = nullptr;   // set with the last upload; waited on before reuse
-Aux g_aux[64];
 
-cudaError_t aux_stream(Aux** out)
+cudaError_t record_stage_done(cudaStream_t s)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    Aux& a = g_aux[dev];
-    if (!a.s) {
-        e = cudaStreamCreateWithFlags(&a.s, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.join, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.stage_done, cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
-    }
-    *out = &a;
-    return cudaSuccess;
+    if (!g_stage_done[dev]) e = cudaEventCreateWithFlags(&g_stage_done[dev], cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(g_stage_done[dev], s);
+    if (e == cudaSuccess) g_stage_out_event = g_stage_done[dev];
+    return e;
 }
 
 // Per host thread and device: the stream on which the host-buffer entry point
@@ -440,8 +427,9 @@ int nuht_check_blocks(int nu, double eps, int m_terms, const double* r_sorted, i
 void nuht_destroy(nuht_plan_t p)
 {
     if (!p) return;
-    if (p->dmem) {
+    if (p->dmem || p->dsort) {
         pool_free(p->dmem, p->stream);
+        pool_free(p->dsort, p->stream);
         cudaStreamSynchronize(p->stream);
     }
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
@@ -491,7 +479,7 @@ static double ms_since(std::chrono::steady_clock::time_point& t)
 
 // Temporaries of the device work-list build (offsets into an arena).
 struct BuildTemps {
-    size_t loc, asy, dir, fcls, lcnt, acnt, dcnt, tot, maxv, scan;
+    size_t loc, asy, dir, fcls, lcnt, acnt, dcnt, part;
 };
 
 static BuildTemps reserve_build_temps(Arena& a, int64_t cap)
@@ -504,14 +492,15 @@ static BuildTemps reserve_build_temps(Arena& a, int64_t cap)
     t.lcnt = a.reserve<int64_t>(cap * kLocalCols);
     t.acnt = a.reserve<int64_t>(cap * kAsyCols);
     t.dcnt = a.reserve<int64_t>(cap * kDirCols);
-    t.tot = a.reserve<int64_t>(kTotals);
-    t.maxv = a.reserve<int64_t>(kMaxv);
-    t.scan = a.reserve<int64_t>(block_scan_scratch(cap));
+    t.part = a.reserve<int64_t>(3 * ((cap + kBlockTile - 1) / kBlockTile) * kAsyCols);
     return t;
 }
 
-static void bind_build_temps(BlockBuild& bb, char* base, const BuildTemps& t)
+static void bind_build_temps(BlockBuild& bb, char* base, const BuildTemps& t, int64_t cap)
 {
+    bb.ocap = cap;
+    bb.ptiles = (cap + kBlockTile - 1) / kBlockTile;
+    bb.part = (int64_t*)(base + t.part);
     bb.loc = (LocalBlock*)(base + t.loc);
     bb.asy = (AsyBlock*)(base + t.asy);
     bb.dir = (DirectBlock*)(base + t.dir);
@@ -519,8 +508,6 @@ static void bind_build_temps(BlockBuild& bb, char* base, const BuildTemps& t)
     bb.lcnt = (int64_t*)(base + t.lcnt);
     bb.acnt = (int64_t*)(base + t.acnt);
     bb.dcnt = (int64_t*)(base + t.dcnt);
-    bb.totals = (int64_t*)(base + t.tot);
-    bb.maxv = (int64_t*)(base + t.maxv);
 }
 
 // Checked mode (NUHT_CHECKED set and not "0"): the device-built block lists
@@ -585,15 +572,26 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
 
     // ---- sort (device) -------------------------------------------------
+    // The sorted arrays stay with the plan; the rest is scratch of the build.
+    Arena ka;
+    const size_t o_r = ka.reserve<double>(n), o_w = ka.reserve<double>(m);
+    const size_t o_pr = ka.reserve<int32_t>(n), o_pw = ka.reserve<int32_t>(m);
+    const size_t o_r2 = ka.reserve<float2>(n), o_w2 = ka.reserve<float2>(m);
+    NUHT_CK(pool_alloc((void**)&P->dsort, ka.size, s));
+    SortedView sv{(double*)(P->dsort + o_r), (double*)(P->dsort + o_w), (int32_t*)(P->dsort + o_pr),
+                  (int32_t*)(P->dsort + o_pw), (float2*)(P->dsort + o_r2), (float2*)(P->dsort + o_w2)};
+    P->d_r = sv.r; P->d_w = sv.w;
+    P->d_pr = sv.pr; P->d_pw = sv.pw;
+    P->d_r2 = sv.r2; P->d_w2 = sv.w2;
     Arena sa;
-    size_t o_r = sa.reserve<double>(n), o_w = sa.reserve<double>(m);
-    size_t o_pr = sa.reserve<int32_t>(n), o_pw = sa.reserve<int32_t>(m);
-    size_t o_st = sa.reserve<int32_t>(m);
-    size_t o_flag = sa.reserve<int>(2);
-    size_t o_prb = sa.reserve<ProbParams>(probs.size());
-    size_t o_roff = sa.reserve<int64_t>(probs.size() + 1), o_woff = sa.reserve<int64_t>(probs.size() + 1);
-    // device subdivision: two level queues, the three block lists, edge values;
-    // work-list build: descriptors, FFT classes, per-block counters, totals
+    // uploaded in one copy: problems, segment offsets, zeroed counts
+    const size_t o_prb = sa.reserve<ProbParams>(probs.size());
+    const size_t o_roff = sa.reserve<int64_t>(probs.size() + 1), o_woff = sa.reserve<int64_t>(probs.size() + 1);
+    const size_t o_cnt = sa.reserve<PlanCounts>(1);
+    const size_t up_bytes = sa.size;
+    const size_t o_st = sa.reserve<int32_t>(m);
+    // device subdivision: two level queues and the three block lists;
+    // work-list build: descriptors, FFT classes, per-block counters
     int64_t qcap = (n + m) / 4 + 4096 + nprob, ocap = (n + m) / 16 + 16384 + nprob;
     if (const char* cap = std::getenv("NUHT_SUBDIVIDE_CAPACITY")) {
         // test knob: smaller device lists exercise the host fallback
@@ -605,102 +603,81 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     size_t o_qa = sa.reserve<SubBlk>(qcap), o_qb = sa.reserve<SubBlk>(qcap);
     size_t o_out = sa.reserve<SubBlk>(3 * ocap);
-    size_t o_bl = sa.reserve<double>(ocap), o_ba = sa.reserve<double4>(ocap);
-    size_t o_res = sa.reserve<int64_t>(4);
     const int sub_ctas = subdivide_grid_ctas();
     size_t o_ctot = sa.reserve<int4>(sub_ctas > 0 ? (size_t)sub_ctas : 1), o_gst = sa.reserve<int64_t>(8);
     BuildTemps bt = reserve_build_temps(sa, ocap);
-    size_t o_scr = sa.size;
-    const size_t scr = radix_sort_scratch_bytes(n), scr_w = radix_sort_scratch_bytes(m);
-    sa.size += align256(scr);
+    const size_t o_scr = sa.size;
+    sa.size += src ? 0 : align256(sort_scratch_bytes(n));
     const size_t o_scr_w = sa.size;
-    sa.size += align256(scr_w);
+    sa.size += src ? 0 : align256(sort_scratch_bytes(m));
     char* sort_mem = nullptr;
     NUHT_CK(pool_alloc((void**)&sort_mem, sa.size, s));
     struct Free {
         char* p; cudaStream_t s;
         ~Free() { pool_free(p, s); }
     } free_sort{sort_mem, s};
-    int* d_flag = (int*)(sort_mem + o_flag);
-    NUHT_CK(cudaMemsetAsync(d_flag, 0, sizeof(int) * 2, s));
     std::lock_guard<std::mutex> stage_lock(g_stage_mu);
     // a previous build's upload from the shared staging buffer may still be in flight
     if (g_stage_out_event) NUHT_CK(cudaEventSynchronize(g_stage_out_event));
-    // problems and segment offsets (needed by the segmented sort and the staircase)
     ProbParams* d_prb = (ProbParams*)(sort_mem + o_prb);
     int64_t* d_roff = (int64_t*)(sort_mem + o_roff);
     int64_t* d_woff = (int64_t*)(sort_mem + o_woff);
+    PlanCounts* d_cnt = (PlanCounts*)(sort_mem + o_cnt);
     {
-        const size_t pb = sizeof(ProbParams) * probs.size(), ob = sizeof(int64_t) * (probs.size() + 1);
-        NUHT_CK(g_stage_out.reserve(pb + 2 * ob));
-        std::memcpy(g_stage_out.p, probs.data(), pb);
-        int64_t* ro = (int64_t*)(g_stage_out.p + pb);
-        int64_t* wo = ro + probs.size() + 1;
+        NUHT_CK(g_stage_out.reserve(up_bytes));
+        std::memcpy(g_stage_out.p + o_prb, probs.data(), sizeof(ProbParams) * probs.size());
+        int64_t* ro = (int64_t*)(g_stage_out.p + o_roff);
+        int64_t* wo = (int64_t*)(g_stage_out.p + o_woff);
         for (int i = 0; i < nprob; ++i) { ro[i] = probs[i].r_off; wo[i] = probs[i].w_off; }
         ro[nprob] = n;
         wo[nprob] = m;
-        NUHT_CK(cudaMemcpyAsync(d_prb, g_stage_out.p, pb, cudaMemcpyHostToDevice, s));
-        NUHT_CK(cudaMemcpyAsync(d_roff, ro, ob, cudaMemcpyHostToDevice, s));
-        NUHT_CK(cudaMemcpyAsync(d_woff, wo, ob, cudaMemcpyHostToDevice, s));
+        std::memset(g_stage_out.p + o_cnt, 0, sizeof(PlanCounts));
+        NUHT_CK(cudaMemcpyAsync(sort_mem, g_stage_out.p, up_bytes, cudaMemcpyHostToDevice, s));
     }
-    double* r_s = (double*)(sort_mem + o_r);
-    double* w_s = (double*)(sort_mem + o_w);
-    int32_t* pr = (int32_t*)(sort_mem + o_pr);
-    int32_t* pw = (int32_t*)(sort_mem + o_pw);
+    double* r_s = sv.r;
+    double* w_s = sv.w;
     int32_t* stair = (int32_t*)(sort_mem + o_st);
     if (src) {
         // already checked and sorted: one copy of the source's arrays per problem
-        for (int ip = 0; ip < nprob; ++ip) {
-            const ProbParams& q = probs[ip];
-            if (q.n) {
-                NUHT_CK(cudaMemcpyAsync(r_s + q.r_off, src->d_r, sizeof(double) * q.n, cudaMemcpyDeviceToDevice, s));
-                NUHT_CK(cudaMemcpyAsync(pr + q.r_off, src->d_pr, sizeof(int32_t) * q.n, cudaMemcpyDeviceToDevice, s));
-            }
-            if (q.m) {
-                NUHT_CK(cudaMemcpyAsync(w_s + q.w_off, src->d_w, sizeof(double) * q.m, cudaMemcpyDeviceToDevice, s));
-                NUHT_CK(cudaMemcpyAsync(pw + q.w_off, src->d_pw, sizeof(int32_t) * q.m, cudaMemcpyDeviceToDevice, s));
-            }
-        }
+        const SortedView from{src->d_r, src->d_w, src->d_pr, src->d_pw, src->d_r2, src->d_w2};
+        NUHT_CK(launch_replicate(from, sv, src->n, src->m, nprob, s));
     } else {
-    NUHT_CK(launch_check_domain(r, n, d_flag, s));
-    NUHT_CK(launch_check_domain(omega, m, d_flag + 1, s));
-    // the two sorts are independent: omega on the auxiliary stream
-    {
-        Aux* ax = nullptr;
-        NUHT_CK(aux_stream(&ax));
-        NUHT_CK(cudaEventRecord(ax->fork, s));
-        NUHT_CK(cudaStreamWaitEvent(ax->s, ax->fork, 0));
-        const cudaError_t ew = radix_sort_f64(omega, m, w_s, pw, sort_mem + o_scr_w, scr_w, ax->s, d_woff, nprob);
-        const cudaError_t ej = cudaEventRecord(ax->join, ax->s);
-        const cudaError_t er = radix_sort_f64(r, n, r_s, pr, sort_mem + o_scr, scr, s, d_roff, nprob);
-        // join before anything can free the sort memory
-        const cudaError_t ek = ej == cudaSuccess ? cudaStreamWaitEvent(s, ax->join, 0) : cudaStreamSynchronize(ax->s);
-        NUHT_CK(ew);
-        NUHT_CK(ej);
-        NUHT_CK(er);
-        NUHT_CK(ek);
-    }
+        SortPair sp{};
+        sp.nseg = nprob;
+        const double* in[2] = {r, omega};
+        const int64_t cnt[2] = {n, m};
+        const int64_t* off[2] = {d_roff, d_woff};
+        double* out[2] = {sv.r, sv.w};
+        int32_t* perm[2] = {sv.pr, sv.pw};
+        float2* split[2] = {sv.r2, sv.w2};
+        for (int k = 0; k < 2; ++k) {
+            SortArray& A = sp.a[k];
+            A.in = in[k]; A.n = cnt[k]; A.off = off[k];
+            A.out = out[k]; A.perm = perm[k]; A.split = split[k];
+            A.flag = &d_cnt->flag[k]; A.stats = d_cnt->stats[k]; A.runh = d_cnt->runh[k];
+        }
+        char* const scr[2] = {sort_mem + o_scr, sort_mem + o_scr_w};
+        NUHT_CK(launch_sort_pair(sp, scr, s));
     }
     if (nprob == 1) NUHT_CK(launch_staircase(r_s, n, w_s, m, probs[0].z, stair, s));
     else NUHT_CK(launch_staircase_many(r_s, w_s, m, d_prb, nprob, stair, s));
     // ---- subdivision (Algorithm 1) and work lists, on the device ------------
     SubBlk* d_out = (SubBlk*)(sort_mem + o_out);
-    int64_t* d_res = (int64_t*)(sort_mem + o_res);
-    double* d_bl = (double*)(sort_mem + o_bl);
-    double4* d_ba = (double4*)(sort_mem + o_ba);
+    int64_t* d_res = d_cnt->res;
     NUHT_CK(launch_subdivide(stair, r_s, w_s, d_prb, nprob, P->opt.min_size, P->opt.n_split_cand,
                              (SubBlk*)(sort_mem + o_qa), (SubBlk*)(sort_mem + o_qb), qcap, d_out, ocap, d_res,
                              (int4*)(sort_mem + o_ctot), (int64_t*)(sort_mem + o_gst), sub_ctas, s));
-    NUHT_CK(launch_block_bounds(d_out, d_out + ocap, d_res, d_prb, r_s, w_s, d_bl, d_ba, s));
     P->eval_threads = local_eval_threads(P->ntop_max);
     const int sp_tile = P->opt.spread_tile ? P->opt.spread_tile : spread_tile_points(P->qmax);
     P->spread_threads = sp_tile;
     BlockBuild bb{};
     bb.res = d_res;
     bb.sub = d_out;
-    bb.ocap = ocap;
-    bb.bl = d_bl;
-    bb.ba = d_ba;
+    bb.r_s = r_s;
+    bb.w_s = w_s;
+    bb.totals = d_cnt->totals;
+    bb.maxv = d_cnt->maxv;
+    bb.ticket = &d_cnt->ticket;
     bb.probs = d_prb;
     bb.w = P->w;
     bb.lowp = P->opt.precision == NUHT_PREC_MIXED;
@@ -709,33 +686,25 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     bb.spread_tile = sp_tile;
     P->interp_threads = P->opt.interp_tile ? P->opt.interp_tile : kInterpTileMax;
     bb.interp_tile = P->interp_threads;
-    bind_build_temps(bb, sort_mem, bt);
-    int64_t* bb_scan = (int64_t*)(sort_mem + bt.scan);
+    bind_build_temps(bb, sort_mem, bt, ocap);
     char* tmp_mem = nullptr;   // temporaries of the host fallback
     struct FreeTmp {
         char** p; cudaStream_t s;
         ~FreeTmp() { pool_free(*p, s); }
     } free_tmp{&tmp_mem, s};
-    NUHT_CK(cudaMemsetAsync(bb.totals, 0, sizeof(int64_t) * (kTotals + 0), s));
-    NUHT_CK(cudaMemsetAsync(bb.maxv, 0, sizeof(int64_t) * kMaxv, s));
-    NUHT_CK(launch_block_build(bb, bb_scan, s));
+    NUHT_CK(launch_block_build(bb, s));
     // the one wait of the build: flags, counts, totals and maxima to the host
-    const size_t o_hf = 0, o_hr = 64, o_ht = o_hr + 64, o_hm = o_ht + align256(sizeof(int64_t) * kTotals);
-    NUHT_CK(g_stage_in.reserve(o_hm + 256));
-    int* hflag = (int*)(g_stage_in.p + o_hf);
-    int64_t* hres = (int64_t*)(g_stage_in.p + o_hr);
-    int64_t* htot = (int64_t*)(g_stage_in.p + o_ht);
-    int64_t* hmax = (int64_t*)(g_stage_in.p + o_hm);
+    NUHT_CK(g_stage_in.reserve(sizeof(PlanCounts)));
+    PlanCounts* hc = (PlanCounts*)g_stage_in.p;
     auto fetch_results = [&]() -> cudaError_t {
-        cudaError_t e = cudaMemcpyAsync(hflag, d_flag, sizeof(int) * 2, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hres, bb.res, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(htot, bb.totals, sizeof(int64_t) * kTotals, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hmax, bb.maxv, sizeof(int64_t) * kMaxv, cudaMemcpyDeviceToHost, s);
+        cudaError_t e = cudaMemcpyAsync(hc, d_cnt, sizeof(PlanCounts), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         return e;
     };
     NUHT_CK(fetch_results());
-    if (hflag[0] || hflag[1]) return NUHT_ERR_DOMAIN;
+    if (hc->flag[0] || hc->flag[1]) return NUHT_ERR_DOMAIN;
+    int64_t* hres = hc->res;
+    const int64_t *htot = hc->totals, *hmax = hc->maxv;
     P->plan_ms[0] = ms_since(clk);
     if (hres[3]) {
         // list capacity exceeded: sorted values and staircase to the host,
@@ -751,8 +720,6 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         if (m) NUHT_CK(cudaMemcpyAsync(hst, stair, sizeof(int32_t) * m, cudaMemcpyDeviceToHost, s));
         NUHT_CK(cudaStreamSynchronize(s));
         std::vector<SubBlk> hl[3];
-        std::vector<double> hbl;
-        std::vector<double4> hba;
         std::vector<HBlock> lb, ab, db;
         for (int ip = 0; ip < nprob; ++ip) {
             const ProbParams& q = probs[ip];
@@ -773,40 +740,27 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
                     return NUHT_ERR_BAD_BLOCKS;
             }
             for (int c = 0; c < 3; ++c)
-                for (const HBlock& h : *src[c]) {
+                for (const HBlock& h : *src[c])
                     hl[c].push_back(SubBlk{(int32_t)h.k0, (int32_t)h.k1, (int32_t)h.j0, (int32_t)h.j1, ip});
-                    if (c == 0) hbl.push_back(hr[q.r_off + h.j1]);
-                    if (c == 1)
-                        hba.push_back(make_double4(hr[q.r_off + h.j0], hr[q.r_off + h.j1], hw[q.w_off + h.k0],
-                                                   hw[q.w_off + h.k1]));
-                }
         }
         int64_t cap = 1;
         for (int c = 0; c < 3; ++c) cap = (int64_t)hl[c].size() > cap ? (int64_t)hl[c].size() : cap;
         Arena ta;
-        const size_t t_sub = ta.reserve<SubBlk>(3 * cap), t_bl = ta.reserve<double>(cap);
-        const size_t t_ba = ta.reserve<double4>(cap), t_res = ta.reserve<int64_t>(4);
+        const size_t t_sub = ta.reserve<SubBlk>(3 * cap);
+        const size_t up_sub = ta.size;
         BuildTemps tt = reserve_build_temps(ta, cap);
         NUHT_CK(pool_alloc((void**)&tmp_mem, ta.size, s));
-        std::vector<char> up(t_res + 64, 0);
+        std::vector<char> up(up_sub, 0);
         for (int c = 0; c < 3; ++c)
             if (!hl[c].empty()) std::memcpy(up.data() + t_sub + sizeof(SubBlk) * c * cap, hl[c].data(),
                                             sizeof(SubBlk) * hl[c].size());
-        if (!hbl.empty()) std::memcpy(up.data() + t_bl, hbl.data(), sizeof(double) * hbl.size());
-        if (!hba.empty()) std::memcpy(up.data() + t_ba, hba.data(), sizeof(double4) * hba.size());
-        int64_t* ures = (int64_t*)(up.data() + t_res);
-        ures[0] = (int64_t)hl[0].size(); ures[1] = (int64_t)hl[1].size(); ures[2] = (int64_t)hl[2].size(); ures[3] = 0;
-        NUHT_CK(cudaMemcpyAsync(tmp_mem, up.data(), t_res + sizeof(int64_t) * 4, cudaMemcpyHostToDevice, s));
-        bb.res = (const int64_t*)(tmp_mem + t_res);
+        PlanCounts zero{};   // counts of the host's lists, everything else cleared
+        for (int c = 0; c < 3; ++c) zero.res[c] = (int64_t)hl[c].size();
+        NUHT_CK(cudaMemcpyAsync(tmp_mem, up.data(), up_sub, cudaMemcpyHostToDevice, s));
+        NUHT_CK(cudaMemcpyAsync(d_cnt, &zero, sizeof(PlanCounts), cudaMemcpyHostToDevice, s));
         bb.sub = (const SubBlk*)(tmp_mem + t_sub);
-        bb.ocap = cap;
-        bb.bl = (const double*)(tmp_mem + t_bl);
-        bb.ba = (const double4*)(tmp_mem + t_ba);
-        bind_build_temps(bb, tmp_mem, tt);
-        bb_scan = (int64_t*)(tmp_mem + tt.scan);
-        NUHT_CK(cudaMemsetAsync(bb.totals, 0, sizeof(int64_t) * kTotals, s));
-        NUHT_CK(cudaMemsetAsync(bb.maxv, 0, sizeof(int64_t) * kMaxv, s));
-        NUHT_CK(launch_block_build(bb, bb_scan, s));
+        bind_build_temps(bb, tmp_mem, tt, cap);
+        NUHT_CK(launch_block_build(bb, s));
         NUHT_CK(fetch_results());   // (the upload buffer lives until here)
     }
     if (hmax[MX_ERR]) return NUHT_ERR_UNSUPPORTED;
@@ -847,10 +801,9 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     const HostTables& T = kernel_tables(P->w);
     Arena A;
     size_t a_prob = A.reserve<ProbParams>(probs.size());
-    size_t a_es = A.reserve<double>(T.es.size()), a_ph = A.reserve<double>(T.ph.size());
     size_t a_es2 = A.reserve<float2>(T.es2.size()), a_ph2 = A.reserve<float2>(T.ph2.size());
     size_t a_ch2 = A.reserve<float2>(T.ch2.size());
-    size_t a_tw = A.reserve<double2>(T.tw.size()), a_tw2 = A.reserve<float4>(T.tw2.size());
+    size_t a_tw2 = A.reserve<float4>(T.tw2.size());
     size_t host_part = A.size;   // everything above is uploaded from one staging buffer
     size_t a_loc = A.reserve<LocalBlock>(nl);
     size_t a_asy = A.reserve<AsyBlock>(na);
@@ -862,8 +815,6 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         a_pre[i] = A.reserve<int32_t>(nseg[i] + 1);
         a_tile[i] = A.reserve<Tile>(ntile[i]);
     }
-    size_t a_r = A.reserve<double>(n), a_w = A.reserve<double>(m);
-    size_t a_pr = A.reserve<int32_t>(n), a_pw = A.reserve<int32_t>(m);
     // G >= 2 copies (a pair, or a vector group) of the per-component arrays:
     // sorted coefficients, moments and sorted outputs
     const size_t gcopies = (size_t)group_copies(P);
@@ -881,7 +832,6 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     size_t a_gb = A.reserve<double2>((size_t)P->asy_members * (size_t)P->gb_len);
     size_t a_gq = A.reserve<float4>((size_t)P->asy_members * (size_t)P->gq_len);
     size_t a_cs = A.reserve<double>(gcopies * (size_t)n), a_gs = A.reserve<double>(gcopies * (size_t)m);
-    size_t a_r2 = A.reserve<float2>(n), a_w2 = A.reserve<float2>(m);
     size_t a_cs2 = A.reserve<float2>(gcopies * (size_t)n);
     size_t a_tg = A.reserve<double2>((size_t)P->asy_members * (size_t)P->gq_len);
     size_t a_bq = A.reserve<float4>((size_t)P->asy_members * (size_t)P->gb_len);
@@ -897,7 +847,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     size_t a_mx = A.reserve<unsigned long long>(1);
     size_t a_q = A.reserve<int>((size_t)nl + 2), a_status = A.reserve<int>(1);
     NUHT_CK(pool_alloc((void**)&P->dmem, A.size, s));
-    P->dbytes = A.size;
+    P->dbytes = A.size + ka.size;
     char* D = P->dmem;
     NUHT_CK(g_stage_out.reserve(host_part));
     char* stage = g_stage_out.p;
@@ -939,21 +889,13 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     for (ProbParams& q : probs) q.tw2 = (const float4*)(D + a_tw2);
     put(a_prob, probs.data(), sizeof(ProbParams) * probs.size());
-    put(a_es, T.es.data(), sizeof(double) * T.es.size());
     put(a_es2, T.es2.data(), sizeof(float2) * T.es2.size());
     put(a_ch2, T.ch2.data(), sizeof(float2) * T.ch2.size());
-    put(a_ph, T.ph.data(), sizeof(double) * T.ph.size());
     put(a_ph2, T.ph2.data(), sizeof(float2) * T.ph2.size());
-    put(a_tw, T.tw.data(), sizeof(double2) * T.tw.size());
     put(a_tw2, T.tw2.data(), sizeof(float4) * T.tw2.size());
     P->plan_ms[2] = ms_since(clk);
     NUHT_CK(cudaMemcpyAsync(D, stage, host_part, cudaMemcpyHostToDevice, s));
-    {
-        Aux* ax = nullptr;
-        NUHT_CK(aux_stream(&ax));
-        NUHT_CK(cudaEventRecord(ax->stage_done, s));   // the next build waits on it before reusing the buffer
-        g_stage_out_event = ax->stage_done;
-    }
+    NUHT_CK(record_stage_done(s));   // the next build waits on it before reusing the buffer
     BuildLists bl{};
     bl.loc = (LocalBlock*)(D + a_loc);
     bl.asy = (AsyBlock*)(D + a_asy);
@@ -963,11 +905,15 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         bl.seg[i] = (Seg*)(D + a_seg[i]);
         bl.pre[i] = (int32_t*)(D + a_pre[i]);
     }
-    NUHT_CK(launch_block_fill(bb, bl, s));
+    P->d_status = (int*)(D + a_status);
+    bl.status = P->d_status;
+    NUHT_CK(launch_block_fill(bb, bl, std::max(nl, std::max(na, nd)), s));
     Tile* tiles[kLists];
+    ExpandLists el{};
     for (int i = 0; i < kLists; ++i) {
         tiles[i] = (Tile*)(D + a_tile[i]);
-        NUHT_CK(launch_expand_tiles(bl.seg[i], bl.pre[i], (int)nseg[i], (int)ntile[i], tiles[i], s));
+        el.seg[i] = bl.seg[i]; el.pre[i] = bl.pre[i]; el.tiles[i] = tiles[i];
+        el.nseg[i] = (int)nseg[i]; el.ntile[i] = (int)ntile[i];
     }
     P->d_tmom = tiles[LIST_MOM]; P->d_teval = tiles[LIST_EVAL];
     P->d_tspread = tiles[LIST_SPREAD]; P->d_tinterp = tiles[LIST_INTERP];
@@ -976,26 +922,14 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     for (int ps = 0; ps < 3; ++ps) P->d_fpass[ps] = tiles[LIST_P0 + ps];
     P->d_pre_mom = bl.pre[LIST_MOM];
     P->d_blk = bl.blk;
-    // sorted arrays and permutations stay on the device
-    P->d_r = (double*)(D + a_r); P->d_w = (double*)(D + a_w);
-    P->d_pr = (int32_t*)(D + a_pr); P->d_pw = (int32_t*)(D + a_pw);
-    if (n) {
-        NUHT_CK(cudaMemcpyAsync(P->d_r, r_s, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-        NUHT_CK(cudaMemcpyAsync(P->d_pr, pr, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-    }
-    if (m) {
-        NUHT_CK(cudaMemcpyAsync(P->d_w, w_s, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-        NUHT_CK(cudaMemcpyAsync(P->d_pw, pw, sizeof(int32_t) * m, cudaMemcpyDeviceToDevice, s));
-    }
     P->d_prob = (ProbParams*)(D + a_prob);
     P->d_loc = bl.loc;
     P->d_asy = bl.asy;
     P->d_dir = bl.dir;
-    P->d_es = (double*)(D + a_es); P->d_ph = (double*)(D + a_ph); P->d_tw = (double2*)(D + a_tw);
     P->d_mom = (double*)(D + a_mom); P->d_momb = P->d_mom + P->mom_len;
     P->d_gb = (double2*)(D + a_gb); P->d_gq = (float4*)(D + a_gq);
     P->d_cs = (double*)(D + a_cs); P->d_gs = (double*)(D + a_gs);
-    P->d_r2 = (float2*)(D + a_r2); P->d_w2 = (float2*)(D + a_w2); P->d_cs2 = (float2*)(D + a_cs2);
+    P->d_cs2 = (float2*)(D + a_cs2);
     P->d_csb = P->d_cs + n; P->d_gsb = P->d_gs + m; P->d_cs2b = P->d_cs2 + n;
     P->det = det;
     if (det) {
@@ -1006,13 +940,9 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     P->d_mx = (unsigned long long*)(D + a_mx);
     P->d_q = (int*)(D + a_q);
-    P->d_status = (int*)(D + a_status);
-    NUHT_CK(cudaMemsetAsync(P->d_status, 0, sizeof(int), s));
-    NUHT_CK(launch_split_f64(P->d_r, n, P->d_r2, s));
-    NUHT_CK(launch_split_f64(P->d_w, m, P->d_w2, s));
     P->d_tg = (double2*)(D + a_tg); P->d_bq = (float4*)(D + a_bq);
     Tables& tb = P->tab;
-    tb.es = P->d_es; tb.es2 = (const float2*)(D + a_es2);
+    tb.es2 = (const float2*)(D + a_es2);
     tb.w = T.w; tb.deg = T.deg; tb.half_w = 0.5 * T.w;
     // plain FP32 for the degrees whose coefficient tail T_k = max_taps sum_{k' > k} |c_k'|
     // keeps the FP32 rounding (2^-23 T_k) below kRoundBudget eps
@@ -1064,16 +994,16 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         tb.fold_tol = (float)(1e-3 * P->eps);
         tb.fold_df_tol = (float)(kRoundBudget * P->eps / ((kMomFold + 2) * 1.1920928955078125e-07));
     }
-    tb.ph = P->d_ph; tb.ph2 = (const float2*)(D + a_ph2);
+    tb.ph2 = (const float2*)(D + a_ph2);
     tb.ph_pieces = T.ph_pieces; tb.ph_deg = T.ph_deg; tb.ph_comp = T.ph_comp;
     tb.interp_const = std::sqrt(2.0 / M_PI) * 4.0 / ((double)T.w * (double)T.w);
     tb.ic2 = make_float2((float)tb.interp_const, (float)(tb.interp_const - (double)(float)tb.interp_const));
     tb.ph_scale = T.ph_scale; tb.ph_xmax = T.ph_xmax;
     tb.ph_scale2 = make_float2((float)T.ph_scale, (float)(T.ph_scale - (double)(float)T.ph_scale));
-    tb.tw = P->d_tw; tb.tw_log2 = T.tw_log2;
+    tb.tw_log2 = T.tw_log2;
     tb.tw2 = (const float4*)(D + a_tw2);
     P->d_smode = (int32_t*)(D + a_sm);
-    NUHT_CK(launch_spread_modes(P->d_prob, P->d_asy, P->d_tspread, P->n_tspread, tb, P->d_r, P->d_smode, s));
+    NUHT_CK(launch_expand_lists(el, P->d_prob, P->d_asy, tb, P->d_r, P->d_smode, s));
     P->plan_ms[3] = ms_since(clk);
     if (const char* ck = std::getenv("NUHT_CHECKED"))
         if (*ck && *ck != '0') NUHT_TRY_BUILD(verify_lists(P));
