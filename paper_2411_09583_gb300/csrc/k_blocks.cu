@@ -219,8 +219,12 @@ __device__ __forceinline__ void block_size_one(const BlockBuild& bb, int y, int6
 // Sizes, descriptors and counters of every block (CTA = kBlockTile rows of
 // class blockIdx.y), the CTAs' column sums, and by the CTA that finishes last
 // their exclusive prefix and the totals (four launches before: sizes and three
-// of scans).
-__global__ void __launch_bounds__(kBlockTile) k_block_sizes(BlockBuild bb)
+// of scans).  Bound by the latency of each asymptotic row's FP64 geometry, whose
+// instructions a warp issues 16 cycles apart: 64 rows per CTA spread it over
+// more SMs than 256 did (23 -> 16 us at 700 asymptotic blocks), and the other
+// warps help with the prefix.
+constexpr int kSizeThreads = 256;
+__global__ void __launch_bounds__(kSizeThreads) k_block_sizes(BlockBuild bb)
 {
     __shared__ unsigned long long smax[kMaxv], ssum[kAsyCols];
     __shared__ bool is_last;
@@ -230,12 +234,12 @@ __global__ void __launch_bounds__(kBlockTile) k_block_sizes(BlockBuild bb)
     if (threadIdx.x < kMaxv) smax[threadIdx.x] = 0;
     if (threadIdx.x < kAsyCols) ssum[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t i = (int64_t)blockIdx.x * kBlockTile + threadIdx.x;
+    const int64_t i = threadIdx.x < kBlockTile ? (int64_t)blockIdx.x * kBlockTile + threadIdx.x : rows;
     if (i < rows) block_size_one(bb, y, i, smax);
     __syncthreads();
     const int ncol = class_cols(y);
     const int64_t* mat = y == 0 ? bb.lcnt : (y == 1 ? bb.acnt : bb.dcnt);
-    for (int c = 0; c < ncol; ++c) {
+    for (int c = 0; threadIdx.x < kBlockTile && c < ncol; ++c) {
         int64_t v = i < rows ? mat[i * ncol + c] : 0;   // this thread's own stores
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
         if (lane == 0 && v) atomicAdd(&ssum[c], (unsigned long long)v);
@@ -254,21 +258,30 @@ __global__ void __launch_bounds__(kBlockTile) k_block_sizes(BlockBuild bb)
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    // one warp per column
-    for (int col = warp; col < kTotals; col += kBlockTile / 32) {
+    // one warp per column, four tiles per lane and step
+    for (int col = warp; col < kTotals; col += kSizeThreads / 32) {
         const int k = col >= TOT_DIR ? 2 : (col >= TOT_ASY ? 1 : 0), c = col - class_total(k);
         const int64_t nt = ceil_div(class_rows(bb, k), kBlockTile);
+        int64_t* pc = bb.part + (int64_t)k * bb.ptiles * kAsyCols + c;
         int64_t carry = 0;
-        for (int64_t t0 = 0; t0 < nt; t0 += 32) {
-            const int64_t t = t0 + lane;
-            int64_t* pp = bb.part + ((int64_t)k * bb.ptiles + t) * kAsyCols + c;
-            const int64_t v = t < nt ? __ldcg((const long long*)pp) : 0;
-            int64_t x = v;
+        for (int64_t t0 = 0; t0 < nt; t0 += 128) {
+            const int64_t t = t0 + 4 * lane;
+            int64_t v[4], sum = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = t + u < nt ? __ldcg((const long long*)(pc + (t + u) * kAsyCols)) : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) sum += v[u];
+            int64_t x = sum;
             for (int off = 1; off < 32; off <<= 1) {
                 const int64_t o = __shfl_up_sync(0xffffffffu, x, off);
                 if (lane >= off) x += o;
             }
-            if (t < nt) *pp = carry + x - v;   // exclusive offset of the tile
+            int64_t run = carry + x - sum;   // exclusive offset of the lane's first tile
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (t + u < nt) pc[(t + u) * kAsyCols] = run;
+                run += v[u];
+            }
             carry += __shfl_sync(0xffffffffu, x, 31);
         }
         if (lane == 0) bb.totals[col] = carry;
@@ -406,7 +419,7 @@ cudaError_t launch_block_build(const BlockBuild& bb, cudaStream_t s)
     dim3 grid;
     const cudaError_t e = block_grid(bb.ptiles, &grid);   // the counts are still on the device
     if (e != cudaSuccess) return e;
-    k_block_sizes<<<grid, kBlockTile, 0, s>>>(bb);
+    k_block_sizes<<<grid, kSizeThreads, 0, s>>>(bb);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -639,31 +639,78 @@ __device__ __forceinline__ int64_t first_above(const double* __restrict__ r, int
     return lo;
 }
 
-constexpr int kStairThreads = 256;
-constexpr int kStairRows = 4;   // rows per thread
+// The same by all lanes of a warp: 32 probes a step instead of one.
+__device__ __forceinline__ int64_t first_above_warp(const double* __restrict__ r, int64_t lo, int64_t hi, double wk,
+                                                    double z)
+{
+    const int lane = threadIdx.x & 31;
+    while (hi - lo > 32) {
+        const int64_t step = (hi - lo + 32) / 33, at = lo + (lane + 1) * step;   // lo < at, ascending
+        const int in = __popc(__ballot_sync(0xffffffffu, at < hi && wk * r[at < hi ? at : lo] <= z));
+        // the first `in` probes are inside: the answer lies after the last of them, up to the next
+        const int64_t nlo = in ? lo + in * step + 1 : lo, nhi = lo + (in + 1) * step;
+        lo = nlo;
+        hi = nhi < hi ? nhi : hi;
+    }
+    const int64_t at = lo + lane;
+    return lo + __popc(__ballot_sync(0xffffffffu, at < hi && wk * r[at < hi ? at : 0] <= z));
+}
+
+constexpr int kStairThreads = 256;   // rows per CTA: one each (four, one after the other, took 19 us at m = 1e5)
 
 // s[k] = max{j : omega_k * r_j <= z} (or -1): the boundary of the local region
-// in row k of the sorted matrix.  f(k) = s[k] + 1 is non-increasing in k (the
-// FP64 product is monotone in both factors), so each CTA searches its first
-// and last rows over all of r and its other rows only between those two
-// bounds: one full search of latency per CTA instead of one per row.
-__global__ void __launch_bounds__(kStairThreads) k_staircase(const double* __restrict__ r, int64_t n,
-                                                             const double* __restrict__ w, int64_t m, double z,
+// in row k of the sorted matrix, a column local to the row's problem (the one
+// with w_off <= k < w_off + m).  f(k) = s[k] + 1 is non-increasing in k within
+// a problem (the FP64 product is monotone in both factors), so a CTA whose
+// rows lie in one problem searches its first and last rows over all of r, a
+// warp each, and its other rows only between those two bounds: four steps of
+// latency per CTA instead of twenty per row (m = 1e6: 36 -> 14 us; two problems
+// of 1e6 each, every row in full: 156 -> 44).  A CTA that spans problems
+// searches every row in full.
+__global__ void __launch_bounds__(kStairThreads) k_staircase(const double* __restrict__ r,
+                                                             const double* __restrict__ w, int64_t m,
+                                                             const ProbParams* __restrict__ probs, int nprob,
                                                              int32_t* __restrict__ s)
 {
     __shared__ int64_t fb[2];
-    const int64_t span = (int64_t)kStairThreads * kStairRows;
+    __shared__ int pb[2];
+    const int64_t span = kStairThreads;
+    auto problem_of = [&](int64_t k) {
+        int lo = 0, hi = nprob;   // last problem with w_off <= k
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (probs[mid].w_off <= k) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
     for (int64_t base = (int64_t)blockIdx.x * span; base < m; base += (int64_t)gridDim.x * span) {
         const int64_t last = (base + span < m ? base + span : m) - 1;
-        if (threadIdx.x < 2) fb[threadIdx.x] = first_above(r, 0, n, w[threadIdx.x == 0 ? base : last], z);
-        __syncthreads();
-        const int64_t hi = fb[0], lo = fb[1];   // f(last) <= f(k) <= f(base)
-#pragma unroll
-        for (int i = 0; i < kStairRows; ++i) {
-            const int64_t k = base + threadIdx.x + (int64_t)i * kStairThreads;
-            if (k <= last) s[k] = (int32_t)(first_above(r, lo, hi, w[k], z) - 1);
+        const int warp = threadIdx.x >> 5;
+        if (warp < 2) {
+            const int64_t k = warp == 0 ? base : last;
+            const int p = problem_of(k);
+            const ProbParams& P = probs[p];
+            const int64_t f = first_above_warp(r + P.r_off, 0, P.n, w[k], P.z);
+            if ((threadIdx.x & 31) == 0) {
+                pb[warp] = p;
+                fb[warp] = f;
+            }
         }
-        __syncthreads();   // fb is rewritten by the next range
+        __syncthreads();
+        if (pb[0] == pb[1]) {
+            const double* rp = r + probs[pb[0]].r_off;
+            const double z = probs[pb[0]].z;
+            const int64_t hi = fb[0], lo = fb[1];   // f(last) <= f(k) <= f(base)
+            const int64_t k = base + threadIdx.x;
+            if (k <= last) s[k] = (int32_t)(first_above(rp, lo, hi, w[k], z) - 1);
+        } else {
+            const int64_t k = base + threadIdx.x;
+            if (k <= last) {
+                const ProbParams& P = probs[problem_of(k)];
+                s[k] = (int32_t)(first_above(r + P.r_off, 0, P.n, w[k], P.z) - 1);
+            }
+        }
+        __syncthreads();   // fb and pb are rewritten by the next range
     }
 }
 
@@ -766,38 +813,11 @@ cudaError_t launch_replicate(const SortedView& src, const SortedView& dst, int64
     return cudaGetLastError();
 }
 
-// Staircase of every row of a batch: row k belongs to the problem p with
-// w_off <= k < w_off + m (binary search); the search runs over that problem's
-// points and the result is a column index local to the problem.
-__global__ void k_staircase_many(const double* __restrict__ r, const double* __restrict__ w, int64_t m,
-                                 const ProbParams* __restrict__ probs, int nprob, int32_t* __restrict__ s)
-{
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nprob;   // last problem with w_off <= k
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (probs[mid].w_off <= k) lo = mid; else hi = mid;
-        }
-        const ProbParams& P = probs[lo];
-        s[k] = (int32_t)(first_above(r + P.r_off, 0, P.n, w[k], P.z) - 1);
-    }
-}
-
-cudaError_t launch_staircase(const double* r, int64_t n, const double* w, int64_t m, double z,
+cudaError_t launch_staircase(const double* r, const double* w, int64_t m, const ProbParams* probs, int nprob,
                              int32_t* s_out, cudaStream_t s)
 {
     if (m <= 0) return cudaSuccess;
-    k_staircase<<<grid_for(m, kStairThreads * kStairRows), kStairThreads, 0, s>>>(r, n, w, m, z, s_out);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_staircase_many(const double* r, const double* w, int64_t m, const ProbParams* probs,
-                                  int nprob, int32_t* s_out, cudaStream_t s)
-{
-    if (m <= 0) return cudaSuccess;
-    k_staircase_many<<<grid_for(m, 256), 256, 0, s>>>(r, w, m, probs, nprob, s_out);
+    k_staircase<<<grid_for(m, kStairThreads), kStairThreads, 0, s>>>(r, w, m, probs, nprob, s_out);
     count_launches(1);
     return cudaGetLastError();
 }

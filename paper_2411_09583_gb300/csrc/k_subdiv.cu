@@ -2,9 +2,12 @@
 //
 // The host version (subdivide.cpp) walks a first-in first-out work list.
 // Here one CTA processes that list level by level: every mixed block of a
-// level is split at once (16 candidate rows read from the staircase), its
-// four children are classified, and block-wide prefix sums give each child
-// its place in the local / asymptotic / direct lists or in the next level.
+// level is split at once by a group of 16 or 4 lanes (16 candidate rows read
+// from the staircase, then a child each), and block-wide prefix sums give each
+// child its place in the local / asymptotic / direct lists or in the next
+// level.  Bound by the latency of a level (10 at n = m = 1e5, 13 at 1e6): with
+// one thread per block its 16 candidates, one after the other, took 16,000
+// cycles a level.  n = m = 1e5 84 -> 36 us, 1e6 146 -> 79.
 // Children are placed in the order the sequential walk would append them
 // (parents in list order, children upper-left, lower-right, upper-right,
 // lower-left), so for one problem the lists equal the host's, entry for
@@ -24,7 +27,6 @@ namespace nuht {
 namespace {
 
 constexpr int kSubThreads = 1024;
-constexpr int kSubCandUnroll = 16;   // candidate rows loaded together (the default n_cand)
 constexpr int kSubWarps = kSubThreads / 32;
 
 // An asymptotic block too large for one FFT (X S > kAsyMaxXS) is queued like
@@ -60,7 +62,7 @@ __device__ __forceinline__ int classify_v(const SubBlk& b, int s0, int s1, int64
 }
 
 // Exclusive block-wide prefix sum of a 64-bit value (four 16-bit counters
-// packed; no carries since a chunk adds at most 4 x kSubThreads per field).
+// packed; no carries since a chunk adds at most kSubThreads per field).
 __device__ __forceinline__ uint64_t block_scan(uint64_t v, uint64_t* wsum, uint64_t* total)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -92,40 +94,50 @@ struct SubState {
     int64_t nout[3];   // local, asymptotic, direct blocks written so far
     int64_t nnext;     // blocks of the next level written so far
     int ovf;
+    int shared;        // the next level lies in shared memory
 };
+constexpr int kSubShared = 512;   // levels of up to this many blocks stay in shared memory (at most kSubSolo:
+                                  // a level left to the other CTAs lies in a global queue)
 
-// Places up to four children per thread (classes cls[i], 0 = none) in
-// order: class lists out[c * ocap ...] and the next level's queue.
-__device__ __forceinline__ void emit(const SubBlk* ch, const int* cls, int nch, SubState& S, uint64_t* wsum,
-                                     SubBlk* __restrict__ out, int64_t ocap, SubBlk* __restrict__ next,
-                                     int64_t qcap)
+__device__ __forceinline__ uint64_t class_count(int cls)
 {
-    uint64_t cnt = 0;
-    for (int i = 0; i < nch; ++i)
-        if (cls[i] > 0) cnt += (uint64_t)1 << (16 * ((cls[i] < 4 ? cls[i] : 4) - 1));
-    uint64_t total;
-    const uint64_t off = block_scan(cnt, wsum, &total);
-    int64_t pos[4];
-    for (int c = 0; c < 3; ++c) pos[c] = S.nout[c] + (int64_t)((off >> (16 * c)) & 0xffff);
-    pos[3] = S.nnext + (int64_t)(off >> 48);
-    bool fits = S.ovf == 0;
-    for (int c = 0; c < 3; ++c) fits = fits && S.nout[c] + (int64_t)((total >> (16 * c)) & 0xffff) <= ocap;
-    fits = fits && S.nnext + (int64_t)(total >> 48) <= qcap;
-    if (fits) {
-        for (int i = 0; i < nch; ++i) {
-            const int c = cls[i];
-            if (c == 0) continue;
-            if (c >= 4) {
-                SubBlk q = ch[i];
-                if (c == 5) q.prob |= kQuadFlag;
-                next[pos[3]++] = q;
-            } else {
-                out[(c - 1) * ocap + pos[c - 1]++] = ch[i];
-            }
-        }
+    return cls > 0 ? (uint64_t)1 << (16 * ((cls < 4 ? cls : 4) - 1)) : 0ull;
+}
+
+// This thread's child (class cls, 0 = none) at its place: pos of its class
+// list (out[c * ocap ...]) or of the next level's queue.
+__device__ __forceinline__ void place(SubBlk ch, int cls, uint64_t off, const int64_t* base, SubBlk* __restrict__ out,
+                                      int64_t ocap, SubBlk* next)
+{
+    if (cls == 0) return;
+    const int f = (cls < 4 ? cls : 4) - 1;
+    const int64_t pos = base[f] + (int64_t)((off >> (16 * f)) & 0xffff);
+    if (cls >= 4) {
+        if (cls == 5) ch.prob |= kQuadFlag;
+        next[pos] = ch;
+    } else {
+        out[f * ocap + pos] = ch;
     }
+}
+
+// Places every thread's child in thread order: class lists and the next
+// level's queue (next, or, when this is the level's only chunk and its
+// children fit, nexts in shared memory).
+__device__ __forceinline__ void emit(const SubBlk& ch, int cls, SubState& S, uint64_t* wsum,
+                                     SubBlk* __restrict__ out, int64_t ocap, SubBlk* next, int64_t qcap,
+                                     SubBlk* nexts, bool only)
+{
+    uint64_t total;
+    const uint64_t off = block_scan(class_count(cls), wsum, &total);
+    const int64_t base[4] = {S.nout[0], S.nout[1], S.nout[2], S.nnext};
+    bool fits = S.ovf == 0;
+    for (int c = 0; c < 3; ++c) fits = fits && base[c] + (int64_t)((total >> (16 * c)) & 0xffff) <= ocap;
+    fits = fits && base[3] + (int64_t)(total >> 48) <= qcap;
+    const bool sh = only && (int64_t)(total >> 48) <= kSubShared;
+    if (fits) place(ch, cls, off, base, out, ocap, sh ? nexts : next);
     __syncthreads();
     if (threadIdx.x == 0) {
+        S.shared = sh;
         if (fits) {
             for (int c = 0; c < 3; ++c) S.nout[c] += (int64_t)((total >> (16 * c)) & 0xffff);
             S.nnext += (int64_t)(total >> 48);
@@ -136,95 +148,117 @@ __device__ __forceinline__ void emit(const SubBlk* ch, const int* cls, int nch, 
     __syncthreads();
 }
 
-// The four children of mixed block qa[i] (SplitIndices at up to n_cand
-// candidate rows), or the quadrants of a flagged asymptotic block, and their
-// classes (0 none / empty, 1..3 a list, 4 the next level, 5 quadrants next);
-// nothing for i >= na.
-__device__ __forceinline__ void make_children(int64_t i, int64_t na, const SubBlk* qa,
-                                              const int32_t* __restrict__ stair, const double* __restrict__ r_s,
-                                              const double* __restrict__ w_s, const ProbParams* __restrict__ probs,
-                                              int64_t min_size, int n_cand, SubBlk* ch, int* cls)
+// W lanes (16 or 4) share mixed block qa[i]: SplitIndices over up to n_cand
+// candidate rows, one lane each at a time (the candidate row minimising the
+// mixed area, its column the last local one; ties keep the first), or the
+// quadrants of a flagged asymptotic block; then lane c < 4 of the group takes
+// child c and its class (0 none / empty, 1..3 a list, 4 the next level, 5
+// quadrants next).  Nothing for i >= na.
+template <int W>
+__device__ __forceinline__ void make_child(int64_t i, int64_t na, const SubBlk* qa, const int32_t* __restrict__ stair,
+                                           const double* __restrict__ r_s, const double* __restrict__ w_s,
+                                           const ProbParams* __restrict__ probs, int64_t min_size, int n_cand,
+                                           bool may_exceed, SubBlk* ch, int* cls)
 {
-    if (i < na && (qa[i].prob & kQuadFlag)) {
-        // an asymptotic block too large for one FFT: its quadrants
-        SubBlk b = qa[i];
-        b.prob &= ~kQuadFlag;
-        const ProbParams& P = probs[b.prob];
-        const int km = (b.k0 + b.k1) >> 1, jm = (b.j0 + b.j1) >> 1;
-        ch[0] = SubBlk{b.k0, km, b.j0, jm, b.prob};
-        ch[1] = SubBlk{km + 1, b.k1, jm + 1, b.j1, b.prob};
-        ch[2] = SubBlk{b.k0, km, jm + 1, b.j1, b.prob};
-        ch[3] = SubBlk{km + 1, b.k1, b.j0, jm, b.prob};
+    const int sub = threadIdx.x & (W - 1);
+    const bool live = i < na;
+    SubBlk b = live ? qa[i] : SubBlk{0, -1, 0, -1, 0};
+    const bool quad = (b.prob & kQuadFlag) != 0;
+    b.prob &= ~kQuadFlag;
+    const ProbParams& P = probs[b.prob];
+    const int32_t* st = stair + P.w_off;
+    const int rows = b.k1 - b.k0 + 1;
+    const int nc = !live || quad ? 0 : (rows <= n_cand ? rows : n_cand);
+    // the product fits 32 bits for up to 2^32 / n_cand rows
+    const bool narrow = (int64_t)n_cand * rows <= 0xffffffffLL;
+    int64_t best = INT64_MAX;
+    int bc = 0x7fffffff, bk = b.k0, bj = b.j0 - 1;
+    for (int c0 = sub; c0 < nc; c0 += 4 * W) {
+        int kv[4], jv[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const bool ne = ch[c].k1 >= ch[c].k0 && ch[c].j1 >= ch[c].j0;
-            cls[c] = ne ? (asy_too_big(r_s + P.r_off, w_s + P.w_off, ch[c]) ? 5 : 2) : 0;
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + u * W;
+            kv[u] = b.k0;
+            if (c < nc) {
+                if (rows <= n_cand) kv[u] += c;
+                else if (narrow) kv[u] += (int)((unsigned)c * (unsigned)(rows - 1) / (unsigned)(n_cand - 1));
+                else kv[u] += (int)((int64_t)c * (rows - 1) / (n_cand - 1));
+            }
         }
-    } else if (i < na) {
-        const SubBlk b = qa[i];
-        const int32_t* st = stair + probs[b.prob].w_off;
-        // SplitIndices: the candidate row minimising the mixed area,
-        // its column the last local one (ties keep the first)
-        const int rows = b.k1 - b.k0 + 1;
-        const int nc = rows <= n_cand ? rows : n_cand;
-        int64_t best = -1;
-        int bk = b.k0, bj = b.j0 - 1;
-        auto cand_row = [&](int c) {
-            return rows <= n_cand ? b.k0 + c : b.k0 + (int)(((int64_t)c * (b.k1 - b.k0)) / (n_cand - 1));
-        };
-        auto consider = [&](int k, int j) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) jv[u] = c0 + u * W < nc ? st[kv[u]] : 0;   // all in flight
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + u * W, k = kv[u];
+            int j = jv[u];
             if (j > b.j1) j = b.j1;
             if (j < b.j0) j = b.j0 - 1;
             const int64_t area = (int64_t)(k - b.k0 + 1) * (b.j1 - j) + (int64_t)(b.k1 - k) * (j - b.j0 + 1);
-            if (best < 0 || area < best) {
+            if (c < nc && area < best) {
                 best = area;
+                bc = c;
                 bk = k;
                 bj = j;
             }
-        };
-        if (nc <= kSubCandUnroll) {
-            // all candidate loads in flight at once
-            int jv[kSubCandUnroll];
-#pragma unroll
-            for (int c = 0; c < kSubCandUnroll; ++c) jv[c] = c < nc ? st[cand_row(c)] : 0;
-#pragma unroll
-            for (int c = 0; c < kSubCandUnroll; ++c)
-                if (c < nc) consider(cand_row(c), jv[c]);
-        } else {
-            for (int c = 0; c < nc; ++c) {
-                const int k = cand_row(c);
-                consider(k, st[k]);
-            }
-        }
-        ch[0] = SubBlk{b.k0, bk, b.j0, bj, b.prob};           // upper left: local
-        ch[1] = SubBlk{bk + 1, b.k1, bj + 1, b.j1, b.prob};   // lower right: asymptotic
-        ch[2] = SubBlk{b.k0, bk, bj + 1, b.j1, b.prob};       // upper right: mixed
-        ch[3] = SubBlk{bk + 1, b.k1, b.j0, bj, b.prob};       // lower left: mixed
-        // the children's end rows, loaded together
-        int sk1[4], sk0[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const bool ne = ch[c].k1 >= ch[c].k0 && ch[c].j1 >= ch[c].j0;
-            sk1[c] = ne ? st[ch[c].k1] : 0;
-            sk0[c] = ne ? st[ch[c].k0] : 0;
-        }
-        const ProbParams& P = probs[b.prob];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            cls[c] = classify_v(ch[c], sk0[c], sk1[c], min_size);
-            if (cls[c] == 2 && asy_too_big(r_s + P.r_off, w_s + P.w_off, ch[c])) cls[c] = 5;
         }
     }
+#pragma unroll
+    for (int off = W / 2; off > 0; off >>= 1) {
+        const int64_t oa = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oc = __shfl_xor_sync(0xffffffffu, bc, off);
+        const int ok = __shfl_xor_sync(0xffffffffu, bk, off), oj = __shfl_xor_sync(0xffffffffu, bj, off);
+        if (oa < best || (oa == best && oc < bc)) {
+            best = oa;
+            bc = oc;
+            bk = ok;
+            bj = oj;
+        }
+    }
+    if (quad) {
+        bk = (b.k0 + b.k1) >> 1;
+        bj = (b.j0 + b.j1) >> 1;
+    }
+    // 0 upper left (local), 1 lower right (asymptotic), 2 upper right, 3 lower left
+    const bool low = sub & 1, right = sub == 1 || sub == 2;
+    *ch = SubBlk{low ? bk + 1 : b.k0, low ? b.k1 : bk, right ? bj + 1 : b.j0, right ? b.j1 : bj, b.prob};
+    *cls = 0;
+    if (!live || sub >= 4 || ch->k1 < ch->k0 || ch->j1 < ch->j0) return;
+    if (quad) {
+        *cls = 2;
+    } else {
+        const int s0 = st[ch->k0], s1 = st[ch->k1];
+        *cls = classify_v(*ch, s0, s1, min_size);
+    }
+    if (may_exceed && *cls == 2 && asy_too_big(r_s + P.r_off, w_s + P.w_off, *ch)) *cls = 5;
 }
 
-__global__ void __launch_bounds__(kSubThreads) k_subdivide(
-    const int32_t* __restrict__ stair, const double* __restrict__ r_s, const double* __restrict__ w_s,
-    const ProbParams* __restrict__ probs, int nprob, int64_t min_size,
-    int n_cand, SubBlk* qa, SubBlk* qb, int64_t qcap, SubBlk* __restrict__ out, int64_t ocap,
-    int64_t* __restrict__ res)
+// Whether some problem's whole range exceeds one FFT: only then can a block
+// (the test loads its corner values otherwise, one more step of latency for
+// every level).
+__device__ __forceinline__ bool any_may_exceed(const double* __restrict__ r_s, const double* __restrict__ w_s,
+                                               const ProbParams* __restrict__ probs, int nprob)
 {
-    __shared__ uint64_t wsum[kSubWarps];
-    __shared__ SubState S;
+    bool big = false;
+    for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
+        const ProbParams& P = probs[p];
+        if (P.m > 0 && P.n > 0)
+            big = big || !(0.5 * (r_s[P.r_off + P.n - 1] - r_s[P.r_off]) * 0.5 *
+                               (w_s[P.w_off + P.m - 1] - w_s[P.w_off]) <= kAsyMaxXS);
+    }
+    return __syncthreads_or(big);
+}
+
+// The roots and the levels of up to max_level blocks, by one CTA: levels of up
+// to kSubShared blocks stay in shared memory (sq), larger ones in the global
+// queues.  Returns the size of the level left over (in qa) and whether the
+// global queues were swapped an odd number of times.
+__device__ __forceinline__ int64_t solo_walk(const int32_t* __restrict__ stair, const double* __restrict__ r_s,
+                                             const double* __restrict__ w_s, const ProbParams* __restrict__ probs,
+                                             int nprob, int64_t min_size, int n_cand, bool may_exceed, SubBlk*& qa,
+                                             SubBlk*& qb, int64_t qcap, SubBlk* __restrict__ out, int64_t ocap,
+                                             int64_t max_level, SubState& S, uint64_t* wsum,
+                                             SubBlk (*sq)[kSubShared], int* swapped)
+{
     if (threadIdx.x == 0) {
         S.nout[0] = S.nout[1] = S.nout[2] = 0;
         S.nnext = 0;
@@ -242,25 +276,54 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide(
             cls = classify(stair + P.w_off, ch, min_size);
             if (cls == 2 && asy_too_big(r_s + P.r_off, w_s + P.w_off, ch)) cls = 5;
         }
-        emit(&ch, &cls, 1, S, wsum, out, ocap, qa, qcap);
+        emit(ch, cls, S, wsum, out, ocap, qa, qcap, sq[0], nprob <= kSubThreads);
     }
     int64_t na = S.nnext;
-    while (na > 0 && S.ovf == 0) {
-        __syncthreads();   // every thread has read S.nnext and S.ovf
+    bool sh = S.shared;
+    int cur = 0, sw = 0;
+    while (na > 0 && na <= max_level && S.ovf == 0) {
+        __syncthreads();   // every thread has read S.nnext, S.shared and S.ovf
         if (threadIdx.x == 0) S.nnext = 0;
         __syncthreads();
-        for (int64_t base = 0; base < na; base += kSubThreads) {
-            const int64_t i = base + threadIdx.x;
-            SubBlk ch[4];
-            int cls[4] = {0, 0, 0, 0};
-            make_children(i, na, qa, stair, r_s, w_s, probs, min_size, n_cand, ch, cls);
-            emit(ch, cls, 4, S, wsum, out, ocap, qb, qcap);
+        const bool wide = na <= kSubThreads / 16;
+        const int per = wide ? kSubThreads / 16 : kSubThreads / 4;   // blocks per chunk
+        const SubBlk* lv = sh ? sq[cur] : qa;
+        for (int64_t base = 0; base < na; base += per) {
+            SubBlk ch;
+            int cls;
+            if (wide)
+                make_child<16>(base + threadIdx.x / 16, na, lv, stair, r_s, w_s, probs, min_size, n_cand, may_exceed,
+                               &ch, &cls);
+            else
+                make_child<4>(base + threadIdx.x / 4, na, lv, stair, r_s, w_s, probs, min_size, n_cand, may_exceed,
+                              &ch, &cls);
+            emit(ch, cls, S, wsum, out, ocap, qb, qcap, sq[cur ^ 1], na <= per);
         }
         na = S.nnext;
+        sh = S.shared;
+        cur ^= 1;
         SubBlk* tmp = qa;
         qa = qb;
         qb = tmp;
+        sw ^= 1;
     }
+    *swapped = sw;
+    return na;
+}
+
+__global__ void __launch_bounds__(kSubThreads) k_subdivide(
+    const int32_t* __restrict__ stair, const double* __restrict__ r_s, const double* __restrict__ w_s,
+    const ProbParams* __restrict__ probs, int nprob, int64_t min_size,
+    int n_cand, SubBlk* qa, SubBlk* qb, int64_t qcap, SubBlk* __restrict__ out, int64_t ocap,
+    int64_t* __restrict__ res)
+{
+    __shared__ uint64_t wsum[kSubWarps];
+    __shared__ SubState S;
+    __shared__ SubBlk sq[2][kSubShared];
+    int swapped;
+    const bool big = any_may_exceed(r_s, w_s, probs, nprob);
+    solo_walk(stair, r_s, w_s, probs, nprob, min_size, n_cand, big, qa, qb, qcap, out, ocap, (int64_t)1 << 62, S,
+              wsum, sq, &swapped);
     if (threadIdx.x == 0) {
         res[0] = S.nout[0];
         res[1] = S.nout[1];
@@ -272,13 +335,13 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide(
 // Multi-CTA form of k_subdivide (cooperative launch).  CTA 0 walks the first
 // levels alone, as k_subdivide, while a level holds at most kSubSolo blocks;
 // from the first larger level on, every CTA takes consecutive chunks of
-// kSubThreads blocks of a level.  After its block-wide scan a CTA publishes
+// kSubThreads / 4 blocks of a level.  After its block-wide scan a CTA publishes
 // its four counts (ctot), and after a grid-wide barrier each CTA forms its
 // chunk's offsets from the counts of the chunks before it: the offsets of the
 // one-CTA walk, so the lists are the same entry for entry.  Every CTA keeps
 // the same copy of the list counts (SubState), so all take the same number of
 // barriers.  gst carries CTA 0's state to the others.
-constexpr int64_t kSubSolo = 2 * kSubThreads;
+constexpr int64_t kSubSolo = 512;   // two chunks of 4-lane groups
 
 __global__ void __launch_bounds__(kSubThreads) k_subdivide_grid(
     const int32_t* __restrict__ stair, const double* __restrict__ r_s, const double* __restrict__ w_s,
@@ -292,44 +355,12 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide_grid(
     __shared__ SubState S;
     __shared__ int64_t cpre[4], ctall[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ SubBlk sq[2][kSubShared];
+    const bool big = any_may_exceed(r_s, w_s, probs, nprob);
     if (blockIdx.x == 0) {
-        if (threadIdx.x == 0) {
-            S.nout[0] = S.nout[1] = S.nout[2] = 0;
-            S.nnext = 0;
-            S.ovf = 0;
-        }
-        __syncthreads();
-        for (int base = 0; base < nprob; base += kSubThreads) {
-            const int p = base + threadIdx.x;
-            SubBlk ch{0, -1, 0, -1, 0};
-            int cls = 0;
-            if (p < nprob) {
-                const ProbParams& P = probs[p];
-                ch = SubBlk{0, (int32_t)P.m - 1, 0, (int32_t)P.n - 1, p};
-                cls = classify(stair + P.w_off, ch, min_size);
-                if (cls == 2 && asy_too_big(r_s + P.r_off, w_s + P.w_off, ch)) cls = 5;
-            }
-            emit(&ch, &cls, 1, S, wsum, out, ocap, qa, qcap);
-        }
-        int64_t na = S.nnext;
-        int swapped = 0;
-        while (na > 0 && na <= kSubSolo && S.ovf == 0) {
-            __syncthreads();   // every thread has read S.nnext and S.ovf
-            if (threadIdx.x == 0) S.nnext = 0;
-            __syncthreads();
-            for (int64_t base = 0; base < na; base += kSubThreads) {
-                const int64_t i = base + threadIdx.x;
-                SubBlk ch[4];
-                int cls[4] = {0, 0, 0, 0};
-                make_children(i, na, qa, stair, r_s, w_s, probs, min_size, n_cand, ch, cls);
-                emit(ch, cls, 4, S, wsum, out, ocap, qb, qcap);
-            }
-            na = S.nnext;
-            SubBlk* tmp = qa;
-            qa = qb;
-            qb = tmp;
-            swapped ^= 1;
-        }
+        int swapped;
+        const int64_t na = solo_walk(stair, r_s, w_s, probs, nprob, min_size, n_cand, big, qa, qb, qcap, out, ocap,
+                                     kSubSolo, S, wsum, sq, &swapped);
         if (threadIdx.x == 0) {
             gst[0] = S.nout[0];
             gst[1] = S.nout[1];
@@ -356,21 +387,18 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide_grid(
         qb = tmp;
     }
     int64_t na = S.nnext;
-    const int64_t per_round = (int64_t)gridDim.x * kSubThreads;
+    const int64_t per_round = (int64_t)gridDim.x * (kSubThreads / 4);
     while (na > 0 && S.ovf == 0) {
         __syncthreads();   // every thread has read S.nnext and S.ovf
         if (threadIdx.x == 0) S.nnext = 0;
         __syncthreads();
         for (int64_t r0 = 0; r0 < na; r0 += per_round) {
-            const int64_t i = r0 + (int64_t)blockIdx.x * kSubThreads + threadIdx.x;
-            SubBlk ch[4];
-            int cls[4] = {0, 0, 0, 0};
-            make_children(i, na, qa, stair, r_s, w_s, probs, min_size, n_cand, ch, cls);
-            uint64_t cnt = 0;
-            for (int c = 0; c < 4; ++c)
-                if (cls[c] > 0) cnt += (uint64_t)1 << (16 * ((cls[c] < 4 ? cls[c] : 4) - 1));
+            SubBlk ch;
+            int cls;
+            make_child<4>(r0 + (int64_t)blockIdx.x * (kSubThreads / 4) + threadIdx.x / 4, na, qa, stair, r_s, w_s,
+                          probs, min_size, n_cand, big, &ch, &cls);
             uint64_t total;
-            const uint64_t off = block_scan(cnt, wsum, &total);
+            const uint64_t off = block_scan(class_count(cls), wsum, &total);
             if (threadIdx.x == 0)
                 ctot[blockIdx.x] = make_int4((int)(total & 0xffff), (int)((total >> 16) & 0xffff),
                                              (int)((total >> 32) & 0xffff), (int)(total >> 48));
@@ -402,20 +430,9 @@ __global__ void __launch_bounds__(kSubThreads) k_subdivide_grid(
             for (int c = 0; c < 3; ++c) fits = fits && S.nout[c] + ctall[c] <= ocap;
             fits = fits && S.nnext + ctall[3] <= qcap;
             if (fits) {
-                int64_t pos[4];
-                for (int c = 0; c < 3; ++c) pos[c] = S.nout[c] + cpre[c] + (int64_t)((off >> (16 * c)) & 0xffff);
-                pos[3] = S.nnext + cpre[3] + (int64_t)(off >> 48);
-                for (int c = 0; c < 4; ++c) {
-                    const int k = cls[c];
-                    if (k == 0) continue;
-                    if (k >= 4) {
-                        SubBlk q = ch[c];
-                        if (k == 5) q.prob |= kQuadFlag;
-                        qb[pos[3]++] = q;
-                    } else {
-                        out[(k - 1) * ocap + pos[k - 1]++] = ch[c];
-                    }
-                }
+                const int64_t base[4] = {S.nout[0] + cpre[0], S.nout[1] + cpre[1], S.nout[2] + cpre[2],
+                                         S.nnext + cpre[3]};
+                place(ch, cls, off, base, out, ocap, qb);
             }
             __syncthreads();
             if (threadIdx.x == 0) {

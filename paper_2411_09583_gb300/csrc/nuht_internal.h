@@ -213,7 +213,7 @@ struct BlockBuild {
     int64_t* part;            // [3][ptiles][kAsyCols] column sums of every kBlockTile rows, then their prefix
     int64_t ptiles;
 };
-constexpr int kBlockTile = 256;
+constexpr int kBlockTile = 64;   // rows (blocks) per CTA of the list build
 
 struct BuildLists {
     LocalBlock* loc;
@@ -289,7 +289,7 @@ struct SortedView {
 cudaError_t launch_replicate(const SortedView& src, const SortedView& dst, int64_t n, int64_t m, int nrep,
                              cudaStream_t s);
 
-cudaError_t launch_staircase(const double* r, int64_t n, const double* w, int64_t m, double z,
+cudaError_t launch_staircase(const double* r, const double* w, int64_t m, const ProbParams* probs, int nprob,
                              int32_t* s_out, cudaStream_t s);
 // Algorithm 1 on the device: lists out[0..ocap) local, out[ocap..2 ocap)
 // asymptotic, out[2 ocap..3 ocap) direct; res = {counts, overflow}.  With
@@ -298,13 +298,14 @@ cudaError_t launch_staircase(const double* r, int64_t n, const double* w, int64_
 // gst[8]); otherwise, or if that launch is refused, one CTA.  The lists are the
 // same either way.
 constexpr int kSubGridMax = 1024;
+// up to this many points + frequencies: one CTA, no cooperative launch (levels of
+// up to ~120 blocks there: 52 -> 22 us at 4000 in all, the grid's barriers included)
+constexpr int64_t kSubOneCta = 32768;
 int subdivide_grid_ctas();
 cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const double* w_s, const ProbParams* probs,
                              int nprob, int64_t min_size,
                              int n_cand, SubBlk* qa, SubBlk* qb, int64_t qcap, SubBlk* out, int64_t ocap,
                              int64_t* res, int4* ctot, int64_t* gst, int grid_ctas, cudaStream_t s);
-cudaError_t launch_staircase_many(const double* r, const double* w, int64_t m, const ProbParams* probs,
-                                  int nprob, int32_t* s_out, cudaStream_t s);
 // per-call input scaling (k_det.cu): *mx = the bits of the largest |x_i|
 // (gather scales the inputs by 2^-E of it, scatter the outputs back,
 // input_exponent); Fx128 sums to FP64

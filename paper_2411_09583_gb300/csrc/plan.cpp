@@ -603,7 +603,8 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     size_t o_qa = sa.reserve<SubBlk>(qcap), o_qb = sa.reserve<SubBlk>(qcap);
     size_t o_out = sa.reserve<SubBlk>(3 * ocap);
-    const int sub_ctas = subdivide_grid_ctas();
+    // up to kSubOneCta points and frequencies no level outgrows one CTA's walk
+    const int sub_ctas = n + m <= kSubOneCta ? 0 : subdivide_grid_ctas();
     size_t o_ctot = sa.reserve<int4>(sub_ctas > 0 ? (size_t)sub_ctas : 1), o_gst = sa.reserve<int64_t>(8);
     BuildTemps bt = reserve_build_temps(sa, ocap);
     const size_t o_scr = sa.size;
@@ -659,8 +660,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         char* const scr[2] = {sort_mem + o_scr, sort_mem + o_scr_w};
         NUHT_CK(launch_sort_pair(sp, scr, s));
     }
-    if (nprob == 1) NUHT_CK(launch_staircase(r_s, n, w_s, m, probs[0].z, stair, s));
-    else NUHT_CK(launch_staircase_many(r_s, w_s, m, d_prb, nprob, stair, s));
+    NUHT_CK(launch_staircase(r_s, w_s, m, d_prb, nprob, stair, s));
     // ---- subdivision (Algorithm 1) and work lists, on the device ------------
     SubBlk* d_out = (SubBlk*)(sort_mem + o_out);
     int64_t* d_res = d_cnt->res;
