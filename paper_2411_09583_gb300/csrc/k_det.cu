@@ -18,22 +18,48 @@ namespace {
 
 constexpr int kDetThreads = 256;
 
-// *mx = max |x_i| as the bit pattern of a non-negative double (whose integer
-// order is the order of the values): a maximum does not depend on the order
-// of the updates, so the scale is the same on every run.
-__global__ void __launch_bounds__(kDetThreads) k_absmax_bits(const double* __restrict__ x, int64_t count,
-                                                             unsigned long long* __restrict__ mx)
+// Clears the accumulators of a call (Z) and writes every CTA's maximum |x_i|
+// to part[blockIdx.x], as the bit pattern of a non-negative double (whose
+// integer order is the order of the values); the gather kernel reduces the
+// CTAs' maxima.  A maximum does not depend on the order, so the scale is the
+// same on every run.  x may be absent, or weighted: |x[perm[i]] ws[i]| (i < nb,
+// every vector of comps).
+__global__ void __launch_bounds__(kDetThreads) k_prepare(ZeroList Z, const double* __restrict__ x, int64_t count,
+                                                         const int32_t* __restrict__ perm,
+                                                         const double* __restrict__ ws, int comps,
+                                                         unsigned long long* __restrict__ part)
 {
+    __shared__ unsigned long long wmax[kDetThreads / 32];
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int z = 0; z < Z.n; ++z) {
+        double2* p = (double2*)Z.p[z];
+        const int64_t n2 = Z.bytes[z] / 16;
+        for (int64_t i = t0; i < n2; i += step) p[i] = make_double2(0.0, 0.0);
+        if (t0 == 0 && (Z.bytes[z] & 8)) ((double*)Z.p[z])[2 * n2] = 0.0;
+    }
+    if (!x) return;
     unsigned long long m = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(x[i]) & 0x7fffffffffffffffull;
+    for (int64_t i = t0; i < count; i += step) {
+        double v;
+        if (perm) {
+            const int64_t i0 = i / comps;
+            v = x[(int64_t)perm[i0] * comps + (i - i0 * comps)] * ws[i0];
+        } else {
+            v = x[i];
+        }
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
         m = b > m ? b : m;
     }
     for (int off = 16; off > 0; off >>= 1) {
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
         m = o > m ? o : m;
     }
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(mx, m);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kDetThreads / 32; ++w) m = wmax[w] > m ? wmax[w] : m;
+        part[blockIdx.x] = m;
+    }
 }
 
 __global__ void __launch_bounds__(kDetThreads) k_fx_decode(const Fx128* __restrict__ src, double* __restrict__ dst,
@@ -42,6 +68,13 @@ __global__ void __launch_bounds__(kDetThreads) k_fx_decode(const Fx128* __restri
     const int fxs = probs[0].fxs;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
         dst[i] = fx_decode(src[i], fxs);
+}
+
+// CTAs of k_prepare: four elements a thread, at most kMaxParts
+int prepare_parts(int64_t work)
+{
+    const int64_t need = (work + 4 * kDetThreads - 1) / (4 * kDetThreads);
+    return (int)(need < 1 ? 1 : (need < kMaxParts ? need : kMaxParts));
 }
 
 int grid_for(int64_t count)
@@ -65,14 +98,16 @@ int device_sm_count()
     return sms;
 }
 
-cudaError_t launch_input_scale(const double* x, int64_t count, unsigned long long* mx, cudaStream_t s)
+cudaError_t launch_prepare(const ZeroList& Z, const double* x, int64_t count, const int32_t* perm, const double* ws,
+                           int comps, unsigned long long* part, int* parts, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(mx, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    if (count > 0) {
-        k_absmax_bits<<<grid_for(count), kDetThreads, 0, s>>>(x, count, mx);
-        count_launches(1);
-    }
+    if (!x && Z.n == 0) return cudaSuccess;
+    int64_t work = x ? count : 0;
+    for (int z = 0; z < Z.n; ++z) work = (int64_t)(Z.bytes[z] / 16) > work ? (int64_t)(Z.bytes[z] / 16) : work;
+    const int grid = prepare_parts(work);
+    if (parts) *parts = grid;
+    k_prepare<<<grid, kDetThreads, 0, s>>>(Z, x, count, perm, ws, comps, part);
+    count_launches(1);
     return cudaGetLastError();
 }
 

@@ -306,21 +306,37 @@ cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const doub
                              int nprob, int64_t min_size,
                              int n_cand, SubBlk* qa, SubBlk* qb, int64_t qcap, SubBlk* out, int64_t ocap,
                              int64_t* res, int4* ctot, int64_t* gst, int grid_ctas, cudaStream_t s);
-// per-call input scaling (k_det.cu): *mx = the bits of the largest |x_i|
-// (gather scales the inputs by 2^-E of it, scatter the outputs back,
-// input_exponent); Fx128 sums to FP64
-cudaError_t launch_input_scale(const double* x, int64_t count, unsigned long long* mx, cudaStream_t s);
+// Start of a call (k_det.cu): clears the accumulators of Z (16-byte aligned)
+// and, with x, writes *parts CTA maxima of |x| (bits) to part[kMaxParts], which
+// launch_gather reduces to *mx: it scales the inputs by 2^-E of the largest
+// magnitude, the scatter the outputs back (input_exponent).  perm and ws:
+// |x[perm[i]] ws[i]| (derivative plans).
+constexpr int kMaxParts = 512;
+struct ZeroList {
+    void* p[6];
+    size_t bytes[6];   // multiples of 8
+    int n;
+    void add(void* q, size_t b)
+    {
+        if (b) {
+            p[n] = q;
+            bytes[n++] = b;
+        }
+    }
+};
+cudaError_t launch_prepare(const ZeroList& Z, const double* x, int64_t count, const int32_t* perm, const double* ws,
+                           int comps, unsigned long long* part, int* parts, cudaStream_t s);
 cudaError_t launch_fx_decode(const void* src, double* dst, int64_t count, const ProbParams* probs, cudaStream_t s);
-// derivative plans (k_sort.cu): weighted gather into both problems' copies,
-// the weighted input maximum, and the half difference scattered times y
-cudaError_t launch_gather_deriv(const double* x, const int32_t* perm, const double* ws, int64_t nb, int stride,
-                                int comp, const unsigned long long* mx, double* out, float2* out2, cudaStream_t s);
-cudaError_t launch_absmax_weighted(const double* x, const int32_t* perm, const double* ws, int64_t nb, int comps,
-                                   unsigned long long* mx, cudaStream_t s);
-cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int stride, int comp,
+// Components comp .. comp + G - 1 between user and sorted order (k_sort.cu).
+// ws (derivative plans, else null): the weighted input, n = 2 nb, into both
+// problems' copies; launch_scatter_deriv the half difference times y.
+cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int64_t nb, const double* ws, int stride,
+                          int comp, int G, const unsigned long long* part, int parts, unsigned long long* mx,
+                          double* out, float2* out2, cudaStream_t s);
+cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int stride, int comp, int G,
                                  const unsigned long long* mx, const double* y, double* out, cudaStream_t s);
-cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int stride, int comp,
-                          const unsigned long long* mx, double* out, float2* out2, cudaStream_t s);
+cudaError_t launch_scatter(const double* gs, const int32_t* perm, int64_t m, int stride, int comp, int G,
+                           const unsigned long long* mx, double* g, cudaStream_t s);
 // Every tile list of a plan from its segments (list i at tiles[i], ntile[i]
 // tiles), and the path of each spreading tile (modes).
 struct ExpandLists {
@@ -331,8 +347,7 @@ struct ExpandLists {
 };
 cudaError_t launch_expand_lists(const ExpandLists& E, const ProbParams* probs, const AsyBlock* blks, Tables tab,
                                 const double* r_s, int32_t* modes, cudaStream_t s);
-cudaError_t launch_scatter(const double* gs, const int32_t* perm, int64_t m, int stride, int comp,
-                           const unsigned long long* mx, double* g, cudaStream_t s);
+
 
 cudaError_t launch_local_moments(const ProbParams* probs, const LocalBlock* blks, const Tile* tiles,
                                  int ntiles, int lmax, const float2* r2, const float2* c2,

@@ -92,8 +92,9 @@ struct nuht_plan_s {
     // moments and sums
     double *d_csb = nullptr, *d_gsb = nullptr, *d_momb = nullptr;
     float2* d_cs2b = nullptr;
-    // per-call input scaling: the bits of the largest input magnitude
-    unsigned long long* d_mx = nullptr;
+    // per-call input scaling: the bits of the largest input magnitude, and the
+    // CTAs' maxima it comes from
+    unsigned long long *d_mx = nullptr, *d_part = nullptr;
     // persistent local stage: queue head, per-block moment-tile counts and the
     // moment tiles' prefix per block; status word of bounded device waits
     int* d_q = nullptr;
@@ -844,7 +845,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     size_t a_fmomb = A.reserve<Fx128>(det ? (size_t)P->mom_len : f1);
     size_t a_fgb = A.reserve<Fx128>(det ? 2 * (size_t)P->gb_len : f1);
     size_t a_ftg = A.reserve<Fx128>(det ? 2 * (size_t)P->gq_len : f1);
-    size_t a_mx = A.reserve<unsigned long long>(1);
+    size_t a_mx = A.reserve<unsigned long long>(1), a_part = A.reserve<unsigned long long>(kMaxParts);
     size_t a_q = A.reserve<int>((size_t)nl + 2), a_status = A.reserve<int>(1);
     NUHT_CK(pool_alloc((void**)&P->dmem, A.size, s));
     P->dbytes = A.size + ka.size;
@@ -939,6 +940,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         P->f_gb = (Fx128*)(D + a_fgb); P->f_tg = (Fx128*)(D + a_ftg);
     }
     P->d_mx = (unsigned long long*)(D + a_mx);
+    P->d_part = (unsigned long long*)(D + a_part);
     P->d_q = (int*)(D + a_q);
     P->d_tg = (double2*)(D + a_tg); P->d_bq = (float4*)(D + a_bq);
     Tables& tb = P->tab;
@@ -1204,7 +1206,6 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
     const cudaStream_t ls = fk.local(s), as = fk.asy(s);
     if (loc && group) {
         NUHT_TRY(T.begin(NUHT_STAGE_LOCAL_MOMENTS, ls));
-        NUHT_CK(cudaMemsetAsync(P->d_mom, 0, sizeof(double) * P->mom_len * ng, ls));
         NUHT_CK(launch_local_moments_group(P->d_prob, P->d_loc, P->d_tmom, P->n_tmom, P->lmax, P->d_r2,
                                            P->d_cs2, P->n, ng, P->d_mom, P->mom_len, ls));
         NUHT_TRY(T.end(NUHT_STAGE_LOCAL_MOMENTS, ls));
@@ -1216,8 +1217,6 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         // moments and evaluation in one persistent launch (per-block waits)
         NUHT_TRY(T.begin(NUHT_STAGE_LOCAL_MOMENTS, ls));
         double* momb = ng == 2 ? P->d_momb : nullptr;
-        NUHT_CK(cudaMemsetAsync(P->d_mom, 0, sizeof(double) * P->mom_len, ls));
-        if (momb) NUHT_CK(cudaMemsetAsync(momb, 0, sizeof(double) * P->mom_len, ls));
         const char* st = std::getenv("NUHT_QUEUE_STALL");
         const bool stall = st && *st && *st != '0';
         NUHT_CK(launch_local_persistent(P->d_prob, P->d_loc, P->d_tmom, P->n_tmom, P->d_teval, P->n_teval,
@@ -1227,13 +1226,11 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         NUHT_TRY(T.end(NUHT_STAGE_LOCAL_MOMENTS, ls));
     } else if (loc) {
         NUHT_TRY(T.begin(NUHT_STAGE_LOCAL_MOMENTS, ls));
-        NUHT_CK(cudaMemsetAsync(mom_acc, 0, acc_bytes(P, P->mom_len), ls));
         // a pair's moments in one pass (one Chebyshev recurrence per point for
         // both components) when its accumulators fit, else a second launch (the
         // group kernel at G = 2 was measured slower on the complex n = m = 4e6
         // workload: 5.68 against 5.38 ms per execute)
         double* momb = ng == 2 ? P->d_momb : nullptr;
-        if (momb) NUHT_CK(cudaMemsetAsync(momb_acc, 0, acc_bytes(P, P->mom_len), ls));
         if (momb && local_moments2_fits(P->lmax)) {
             NUHT_CK(launch_local_moments2(P->d_prob, P->d_loc, P->d_tmom, P->n_tmom, P->lmax, P->d_r2,
                                           P->d_cs2, P->d_cs2b, mom_acc, momb_acc, ls));
@@ -1278,7 +1275,7 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         const float2* c2 = member_c2(P, v0);
         double* gv = member_g_acc(P, v0);
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_SPREAD, as));
-        NUHT_CK(cudaMemsetAsync(gb_acc, 0, acc_bytes(P, 2 * P->gb_len * nv), as));
+        if (v0 > 0) NUHT_CK(cudaMemsetAsync(gb_acc, 0, acc_bytes(P, 2 * P->gb_len * nv), as));
         if (lowp)
             NUHT_CK(launch_asy_spread_f32(P->d_prob, P->d_asy, P->d_tspread, P->d_smode, P->n_tspread, P->qmax,
                                           P->spread_threads, P->tab, P->d_r, P->d_r2, c2, P->n, nv, gb_acc,
@@ -1322,14 +1319,40 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
     return NUHT_OK;
 }
 
+// Accumulators that a group of ng components starts from zero: the sums
+// (rows elements each), the moments, and the grid of the first asymptotic
+// launch (grid_len complex values per member; fx twins in the deterministic
+// mode, where groups are pairs).
+static ZeroList group_zeros(nuht_plan_t P, int ng, double* sum, Fx128* fsum, Fx128* fsumb, int64_t rows,
+                            double2* grid, Fx128* fgrid, int64_t grid_len)
+{
+    const int mask = P->opt.class_mask;
+    const bool loc = (mask & 1) && P->n_loc, asy = (mask & 2) && P->n_asy;
+    ZeroList Z{};
+    if (P->det) {
+        Z.add(fsum, sizeof(Fx128) * (size_t)rows);
+        if (ng > 1) Z.add(fsumb, sizeof(Fx128) * (size_t)rows);
+        if (loc) Z.add(P->f_mom, sizeof(Fx128) * (size_t)P->mom_len);
+        if (loc && ng > 1) Z.add(P->f_momb, sizeof(Fx128) * (size_t)P->mom_len);
+        if (asy) Z.add(fgrid, 2 * sizeof(Fx128) * (size_t)grid_len);   // one member per launch
+        return Z;
+    }
+    Z.add(sum, sizeof(double) * (size_t)rows * ng);
+    if (loc) Z.add(P->d_mom, sizeof(double) * (size_t)P->mom_len * ng);
+    if (asy) Z.add(grid, sizeof(double2) * (size_t)grid_len * std::min(ng, P->asy_members));
+    return Z;
+}
+
 // The component loop of a forward transform, in groups of G real components
 // (opts.vec_group; 1 when the plan has no local or direct blocks to share):
-// gather(comp, c, c2) writes a component's sorted, scaled input into its
-// member's arrays, apply_forward adds every block class into the members'
-// sums, scatter(comp, g) writes a member's sums out.
+// prepare(Z, first) clears a group's accumulators (and with the first finds
+// the input's largest magnitude), gather(comp, ng) writes the group's sorted,
+// scaled inputs into its members' arrays, apply_forward adds every block class
+// into the members' sums, scatter(comp, ng) writes them out.
 extern "C++" {
-template <class Gather, class Scatter>
-static int drive_forward(nuht_plan_t P, int comps, cudaStream_t s, Gather&& gather, Scatter&& scatter)
+template <class Prepare, class Gather, class Scatter>
+static int drive_forward(nuht_plan_t P, int comps, cudaStream_t s, Prepare&& prepare, Gather&& gather,
+                         Scatter&& scatter)
 {
     NUHT_TRY(ensure_events(P, comps));
     const bool share = ((P->opt.class_mask & 4) && P->n_dir > 0) || ((P->opt.class_mask & 1) && P->n_loc > 0);
@@ -1340,19 +1363,15 @@ static int drive_forward(nuht_plan_t P, int comps, cudaStream_t s, Gather&& gath
         const int ng = comps - c0 < G ? comps - c0 : G;
         StageTimer T{P, c0};
         NUHT_TRY(T.begin(NUHT_STAGE_GATHER, s));
-        for (int v = 0; v < ng; ++v) {
-            NUHT_CK(cudaMemsetAsync(member_g_acc(P, v), 0, acc_bytes(P, P->m), s));
-            NUHT_CK(gather(c0 + v, member_c(P, v), member_c2(P, v)));
-        }
+        NUHT_CK(prepare(group_zeros(P, ng, P->d_gs, P->f_gs, P->f_gsb, P->m, P->d_gb, P->f_gb, P->gb_len), c0 == 0));
+        NUHT_CK(gather(c0, ng));
         NUHT_TRY(T.end(NUHT_STAGE_GATHER, s));
         NUHT_TRY(apply_forward(P, c0, ng, s));
-        for (int v = 0; v < ng; ++v) {
-            StageTimer Tv{P, c0 + v};
-            NUHT_TRY(Tv.begin(NUHT_STAGE_SCATTER, s));
-            if (P->det) NUHT_CK(launch_fx_decode(member_g_acc(P, v), member_g(P, v), P->m, P->d_prob, s));
-            NUHT_CK(scatter(c0 + v, member_g(P, v)));
-            NUHT_TRY(Tv.end(NUHT_STAGE_SCATTER, s));
-        }
+        NUHT_TRY(T.begin(NUHT_STAGE_SCATTER, s));
+        for (int v = 0; P->det && v < ng; ++v)
+            NUHT_CK(launch_fx_decode(member_g_acc(P, v), member_g(P, v), P->m, P->d_prob, s));
+        NUHT_CK(scatter(c0, ng));
+        NUHT_TRY(T.end(NUHT_STAGE_SCATTER, s));
     }
     return NUHT_OK;
 }
@@ -1370,11 +1389,18 @@ int nuht_execute(nuht_plan_t P, const double* c, double* g, int nvec, int is_com
         return NUHT_OK;
     }
     // c is scaled by a power of two from its largest magnitude
-    NUHT_CK(launch_input_scale(c, P->n * comps, P->d_mx, s));
+    int parts = 0;
     return drive_forward(
         P, comps, s,
-        [&](int cp, double* o, float2* o2) { return launch_gather(c, P->d_pr, P->n, comps, cp, P->d_mx, o, o2, s); },
-        [&](int cp, const double* src) { return launch_scatter(src, P->d_pw, P->m, comps, cp, P->d_mx, g, s); });
+        [&](const ZeroList& Z, bool first) {
+            return launch_prepare(Z, first ? c : nullptr, P->n * comps, nullptr, nullptr, 1, P->d_part,
+                                  first ? &parts : nullptr, s);
+        },
+        [&](int cp, int ng) {
+            return launch_gather(c, P->d_pr, P->n, P->n, nullptr, comps, cp, ng, P->d_part, parts, P->d_mx, P->d_cs,
+                                 P->d_cs2, s);
+        },
+        [&](int cp, int ng) { return launch_scatter(P->d_gs, P->d_pw, P->m, comps, cp, ng, P->d_mx, g, s); });
 }
 
 // The accumulation target of member v's adjoint sums (d_cs + v n, or f_cs /
@@ -1412,7 +1438,6 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
         NUHT_TRY(T.begin(NUHT_STAGE_LOCAL_MOMENTS, ls));
         if (ng > 2) {
             // a group: one Miller sweep per row and one basis per point for all members
-            NUHT_CK(cudaMemsetAsync(P->d_mom, 0, sizeof(double) * P->mom_len * ng, ls));
             NUHT_CK(launch_local_adj_group(P->d_prob, P->d_loc, P->d_teval, P->n_teval, P->d_tmom, P->n_tmom,
                                            P->lmax, P->ntop_max, local_adj_group_threads(P->ntop_max), P->d_w2,
                                            P->d_r2, P->d_gs, P->m, ng, P->d_mom, P->mom_len, P->d_cs, P->n, true,
@@ -1426,8 +1451,6 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
         }
         for (int v = 0; ng <= 2 && v < ng; v += pairs ? 2 : 1) {
             const bool two = pairs && v + 1 < ng;
-            NUHT_CK(cudaMemsetAsync(mom_acc(v), 0, acc_bytes(P, P->mom_len * (two && !P->det ? 2 : 1)), ls));
-            if (two && P->det) NUHT_CK(cudaMemsetAsync(mom_acc(v + 1), 0, acc_bytes(P, P->mom_len), ls));
             NUHT_CK(launch_local_adj_moments(P->d_prob, P->d_loc, P->d_teval, P->n_teval, P->ntop_max, thr,
                                              P->d_w2, member_g(P, v), mom_acc(v),
                                              two ? member_g(P, v + 1) : nullptr, two ? mom_acc(v + 1) : nullptr,
@@ -1460,7 +1483,7 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
         const int nv = ng - v0 < am ? ng - v0 : am;
         StageTimer Tv{P, c0 + v0};
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_SPREAD, as));
-        NUHT_CK(cudaMemsetAsync(tg_acc, 0, acc_bytes(P, 2 * P->gq_len * nv), as));
+        if (v0 > 0) NUHT_CK(cudaMemsetAsync(tg_acc, 0, acc_bytes(P, 2 * P->gq_len * nv), as));
         NUHT_CK(launch_asy_adj_spread(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->qmax, P->interp_threads,
                                       P->tab, P->d_w, member_g(P, v0), P->m, nv, tg_acc, P->gq_len, as));
         if (P->det) NUHT_CK(launch_fx_decode(P->f_tg, (double*)P->d_tg, 2 * P->gq_len, P->d_prob, as));
@@ -1479,13 +1502,14 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
     return NUHT_OK;
 }
 
-// The component loop of an adjoint transform (drive_forward transposed), in
-// groups as in drive_forward: gather(comp, g) writes a component's sorted,
-// scaled input into its member's array, apply_adjoint adds every block class
-// into the members' sums, scatter(comp, c) writes a member's sums out.
+// The component loop of an adjoint transform (drive_forward transposed):
+// gather(comp, ng) writes the group's sorted, scaled inputs into its members'
+// arrays, apply_adjoint adds every block class into the members' sums,
+// scatter(comp, ng) writes them out.
 extern "C++" {
-template <class Gather, class Scatter>
-static int drive_adjoint(nuht_plan_t P, int comps, cudaStream_t s, Gather&& gather, Scatter&& scatter)
+template <class Prepare, class Gather, class Scatter>
+static int drive_adjoint(nuht_plan_t P, int comps, cudaStream_t s, Prepare&& prepare, Gather&& gather,
+                         Scatter&& scatter)
 {
     NUHT_TRY(ensure_events(P, comps));
     const bool share = (P->opt.class_mask & 1) && P->n_loc > 0;
@@ -1499,19 +1523,15 @@ static int drive_adjoint(nuht_plan_t P, int comps, cudaStream_t s, Gather&& gath
         const int ng = comps - c0 < G ? comps - c0 : G;
         StageTimer T{P, c0};
         NUHT_TRY(T.begin(NUHT_STAGE_GATHER, s));
-        for (int v = 0; v < ng; ++v) {
-            NUHT_CK(cudaMemsetAsync(member_c_acc(P, v), 0, acc_bytes(P, P->n), s));
-            NUHT_CK(gather(c0 + v, member_g(P, v)));
-        }
+        NUHT_CK(prepare(group_zeros(P, ng, P->d_cs, P->f_cs, P->f_csb, P->n, P->d_tg, P->f_tg, P->gq_len), c0 == 0));
+        NUHT_CK(gather(c0, ng));
         NUHT_TRY(T.end(NUHT_STAGE_GATHER, s));
         NUHT_TRY(apply_adjoint(P, c0, ng, pairs, s));
-        for (int v = 0; v < ng; ++v) {
-            StageTimer Tv{P, c0 + v};
-            NUHT_TRY(Tv.begin(NUHT_STAGE_SCATTER, s));
-            if (P->det) NUHT_CK(launch_fx_decode(member_c_acc(P, v), member_c(P, v), P->n, P->d_prob, s));
-            NUHT_CK(scatter(c0 + v, member_c(P, v)));
-            NUHT_TRY(Tv.end(NUHT_STAGE_SCATTER, s));
-        }
+        NUHT_TRY(T.begin(NUHT_STAGE_SCATTER, s));
+        for (int v = 0; P->det && v < ng; ++v)
+            NUHT_CK(launch_fx_decode(member_c_acc(P, v), member_c(P, v), P->n, P->d_prob, s));
+        NUHT_CK(scatter(c0, ng));
+        NUHT_TRY(T.end(NUHT_STAGE_SCATTER, s));
     }
     return NUHT_OK;
 }
@@ -1529,11 +1549,18 @@ int nuht_adjoint(nuht_plan_t P, const double* g, double* c, int nvec, int is_com
         return NUHT_OK;
     }
     // g is scaled by a power of two from its largest magnitude
-    NUHT_CK(launch_input_scale(g, P->m * comps, P->d_mx, s));
+    int parts = 0;
     return drive_adjoint(
         P, comps, s,
-        [&](int cp, double* o) { return launch_gather(g, P->d_pw, P->m, comps, cp, P->d_mx, o, nullptr, s); },
-        [&](int cp, const double* src) { return launch_scatter(src, P->d_pr, P->n, comps, cp, P->d_mx, c, s); });
+        [&](const ZeroList& Z, bool first) {
+            return launch_prepare(Z, first ? g : nullptr, P->m * comps, nullptr, nullptr, 1, P->d_part,
+                                  first ? &parts : nullptr, s);
+        },
+        [&](int cp, int ng) {
+            return launch_gather(g, P->d_pw, P->m, P->m, nullptr, comps, cp, ng, P->d_part, parts, P->d_mx, P->d_gs,
+                                 nullptr, s);
+        },
+        [&](int cp, int ng) { return launch_scatter(P->d_cs, P->d_pr, P->n, comps, cp, ng, P->d_mx, c, s); });
 }
 
 int nuht_plan_deriv(nuht_plan_t* out, nuht_plan_t base, void* stream)
@@ -1579,14 +1606,19 @@ int nuht_grad_omega(nuht_plan_t D, const double* c, const double* e, double* gra
         return NUHT_OK;
     }
     // the forward transform of r c, scaled by a power of two from its largest magnitude
-    NUHT_CK(launch_absmax_weighted(c, D->d_pr, D->d_r, nb, nvec, D->d_mx, s));
+    int parts = 0;
     return drive_forward(
         D, nvec, s,
-        [&](int cp, double* o, float2* o2) {
-            return launch_gather_deriv(c, D->d_pr, D->d_r, nb, nvec, cp, D->d_mx, o, o2, s);
+        [&](const ZeroList& Z, bool first) {
+            return launch_prepare(Z, first ? c : nullptr, nb * nvec, D->d_pr, D->d_r, nvec, D->d_part,
+                                  first ? &parts : nullptr, s);
         },
-        [&](int cp, const double* src) {
-            return launch_scatter_deriv(src, D->d_pw, mb, nvec, cp, D->d_mx, e, grad_omega, s);
+        [&](int cp, int ng) {
+            return launch_gather(c, D->d_pr, 2 * nb, nb, D->d_r, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_cs,
+                                 D->d_cs2, s);
+        },
+        [&](int cp, int ng) {
+            return launch_scatter_deriv(D->d_gs, D->d_pw, mb, nvec, cp, ng, D->d_mx, e, grad_omega, s);
         });
 }
 
@@ -1602,12 +1634,19 @@ int nuht_grad_r(nuht_plan_t D, const double* c, const double* e, double* grad_r,
         return NUHT_OK;
     }
     // the adjoint transform of omega e, scaled by a power of two from its largest magnitude
-    NUHT_CK(launch_absmax_weighted(e, D->d_pw, D->d_w, mb, nvec, D->d_mx, s));
+    int parts = 0;
     return drive_adjoint(
         D, nvec, s,
-        [&](int cp, double* o) { return launch_gather_deriv(e, D->d_pw, D->d_w, mb, nvec, cp, D->d_mx, o, nullptr, s); },
-        [&](int cp, const double* src) {
-            return launch_scatter_deriv(src, D->d_pr, nb, nvec, cp, D->d_mx, c, grad_r, s);
+        [&](const ZeroList& Z, bool first) {
+            return launch_prepare(Z, first ? e : nullptr, mb * nvec, D->d_pw, D->d_w, nvec, D->d_part,
+                                  first ? &parts : nullptr, s);
+        },
+        [&](int cp, int ng) {
+            return launch_gather(e, D->d_pw, 2 * mb, mb, D->d_w, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_gs,
+                                 nullptr, s);
+        },
+        [&](int cp, int ng) {
+            return launch_scatter_deriv(D->d_cs, D->d_pr, nb, nvec, cp, ng, D->d_mx, c, grad_r, s);
         });
 }
 
