@@ -136,40 +136,62 @@ __device__ __forceinline__ df psihat_fx(const Tables& T, const AsyBlock& B, long
     return psihat_of(T, df_mul(df{B.alpha_h, B.alpha_l}, df{s.h * sc, s.l * sc}));
 }
 
-constexpr int kSpreadSub = 8;       // point sub-ranges per moment, combined by shuffles
-constexpr int kMomMinPerBin = 16;   // tiles with at least this many points per bin use moments
 constexpr int kMaxTileBins = 32;
+constexpr int kSpreadSub = 8;       // point sub-ranges per moment, combined by shuffles
 
-// Row strides of the moment path's shared arrays: = 2 mod 4 elements, so
-// that the eight point rows a quarter-warp reads (16-byte loads of float2
-// pairs, or 8-byte loads of float pairs) fall in distinct banks.
-__host__ __device__ __forceinline__ int mom_stride(int n) { return ((n + 1) & ~1) + (((n + 1) & 2) ? 0 : 2); }
-
-struct MomLayout {
-    int ndf, nf;     // degree pairs accumulated in double-float / in FP32
-    int sud, suf;    // row strides of the basis: double-float part (float2), FP32 part (float)
-    int sx;          // row stride of the weighted values (float2)
-    int dpad;        // rows of the moment matrix (2 ndf + 2 nf)
-};
-
-__host__ __device__ __forceinline__ MomLayout mom_layout(int nb, int dcs, int Q2)
+// The tile's largest magnitude bound: every warp leaves its own (warp_mag, all
+// threads), and after a barrier every thread reads the tile's (up to 8 warps).
+__device__ __forceinline__ void warp_mag(unsigned* wmag, float mag)
 {
-    MomLayout L;
-    L.ndf = (dcs + 1) >> 1;
-    L.nf = (nb - dcs + 1) >> 1;
-    L.sud = mom_stride(2 * L.ndf);
-    L.suf = L.nf > 0 ? mom_stride(2 * L.nf) : 0;
-    L.sx = mom_stride(Q2);
-    L.dpad = 2 * (L.ndf + L.nf);
-    return L;
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mag));
+    if ((threadIdx.x & 31) == 0) wmag[threadIdx.x >> 5] = m;
+}
+__device__ __forceinline__ float tile_mag(const unsigned* wmag)
+{
+    unsigned m = wmag[0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = wmag[w] > m ? wmag[w] : m;
+    return __uint_as_float(m);
 }
 
-// Degree of row e of the moment matrix (pairs of double-float degrees
-// 0..2 ndf - 1, then pairs of FP32 degrees from dcs); -1 for padding.
-__device__ __forceinline__ int mom_degree(int e, int ndf, int dcs, int nb)
+// Small shared arrays of the dense paths (one set for all their instances).
+struct MomShared {
+    int bstart[kMaxTileBins + 3];      // first point of each bin
+    unsigned wmag[8];                  // per warp, the largest magnitude bound (float bits)
+    uint16_t items[kMaxMomItems];      // (degree pair, Hankel pair) of every moment item, by cost
+};
+
+// A bound of |re| and |im| of c (double-float high parts; 1.001 covers the low
+// parts and the rounding of what is derived from them).
+__device__ __forceinline__ float mag_of(float re, float im) { return 1.001f * fmaxf(fabsf(re), fabsf(im)); }
+constexpr int kMomBins = 2;         // bins whose moments are formed and added to the grid together
+constexpr int kMomMinPerBin = 16;   // tiles with at least this many points per bin use moments
+
+// Row strides of the dense paths' shared arrays, whose points (rows) eight or
+// sixteen consecutive lanes read side by side: loads of two elements want half
+// the stride odd, loads of four a quarter of it.
+__host__ __device__ __forceinline__ int mom_stride2(int n) { return ((n + 1) & ~1) + (((n + 1) & 2) ? 0 : 2); }
+__host__ __device__ __forceinline__ int mom_stride4(int n) { return ((n + 3) & ~3) + (((n + 3) & 4) ? 0 : 4); }
+
+// Double-float arrays are kept as two planes of floats: the FP32 items, more
+// than half of the work, read the high parts alone.
+struct MomLayout {
+    int ndf, nf;     // degree pairs with low parts / without
+    int suh, sul;    // row strides of the basis: high parts (all degrees), low parts (degrees < dcs)
+    int sxh, sxl;    // row strides of the weighted values: high parts, low parts (the first nlow pairs)
+    int dpad;        // rows of the moment matrix (2 ndf + 2 nf): degree = row, zero from nb on
+};
+
+__host__ __device__ __forceinline__ MomLayout mom_layout(int nb, int dcs, int Q2, int nlow)
 {
-    const int d = e < 2 * ndf ? e : dcs + (e - 2 * ndf);
-    return (e < 2 * ndf ? d < dcs : d < nb) ? d : -1;
+    MomLayout L;
+    L.ndf = dcs >> 1;
+    L.nf = nb > dcs ? (nb - dcs + 1) >> 1 : 0;
+    L.dpad = 2 * (L.ndf + L.nf);
+    L.suh = mom_stride2(L.dpad);
+    L.sul = mom_stride2(2 * L.ndf);
+    L.sxh = mom_stride4(Q2);
+    L.sxl = mom_stride4(4 * nlow);
+    return L;
 }
 
 // Dense tile: all points of one bin (same l0) share the cells, so
@@ -182,63 +204,91 @@ __device__ __forceinline__ int mom_degree(int e, int ndf, int dcs, int nb)
 // in double-float.
 //
 // Shared by the spreading of points (forward) and of frequencies (adjoint):
-// target(j, &v, xq) gives target j's cell and kernel coordinate v and writes
-// its 2M weighted values as double-float (re, im) pairs xq[2q], xq[2q + 1];
+// target(j, &v, xh, xl, &mag) gives target j's cell and kernel coordinate v and
+// writes its 2M weighted values as (re, im) pairs [2q], [2q + 1], high parts to
+// xh and the low parts of the first nlow Hankel pairs to xl, and a bound of
+// their magnitudes;
 // cell(c) is the grid index of cell c, or -1 for a cell outside the grid.
 // Members (forward spreading of V real components): target writes member 0's
-// values; values(vm, xq) rewrites this thread's point's values for member vm,
+// values; values(vm, xh, xl) rewrites this thread's point's values for member vm
+// (returning their bound),
 // whose grid sits moff accumulator elements after member 0's.  The basis,
 // the cells and the bins are formed once for all members.
-template <class Target, class Values, class Cell, class Acc>
-__device__ __forceinline__ void spread_moments(int Q, int qs, const Tile& t, const Tables& tab, Target&& target,
-                                               Values&& values, int V, int64_t moff, Cell&& cell, Acc gb,
-                                               float2* sm)
+//
+// Bound: issue slots, and the longest lane's chain between two barriers.  So
+//  - double-float items take 16 lanes, FP32 ones 8, on different warps, and two
+//    bins share the barriers and one grid update (a cell of both gets one sum);
+//  - the lanes' partial sums are exchanged and halved (8 exchanges for 8 outputs)
+//    instead of each summed by all lanes (24);
+//  - with ANCHORED sums (tab.anchored, eps >= kAnchorMinEps) a product takes 6
+//    instructions instead of 12, from an anchor above the tile's largest value
+//    times the points of a lane.
+// n = m = 1e6, eps 1e-12 (forward, with the folded tiles): 1.02 -> 0.92 ms;
+// eps 1e-10 0.98 -> 0.81 (forward), 1.33 -> 1.00 per transform (adjoint);
+// one vector of 16 at 1.5e5 points 0.128 -> 0.108.  Outputs differ by 9e-15 of
+// their norm at eps 1e-12 and by 5e-13 at 1e-10.  Skipping a phase in a
+// timing-only build at eps 1e-12 (0.96 ms then): double-float items 0.11, FP32
+// items 0.11 (before the high parts had a plane of their own), grid update
+// 0.09; of the folded tiles N 0.04, beta 0.02, M 0.06, grid update 0.11.
+// Per Hankel pair (a quad of values) only the degrees that need it are summed in
+// double-float (ProbParams::items).
+template <bool ANCHORED, class Target, class Values, class Cell, class Acc>
+__device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& t, const Tables& tab,
+                                               Target&& target, Values&& values, int V, int64_t moff, Cell&& cell,
+                                               Acc gb, float* sm, MomShared& sh)
 {
     const int nt = blockDim.x, tid = threadIdx.x, cnt = t.count;
     const int w = tab.w, nb = tab.nb, dcs = tab.dcs;
-    const int Q2 = 2 * Q;
-    const MomLayout L = mom_layout(nb, dcs, Q2);
-    const int nq = Q2 >> 2;
-    float2* Ud = sm;                                  // [nt][sud]  T_d(v_p), d < dcs
-    float2* X = Ud + nt * L.sud;                      // [nt][sx]   x_q'(p)
-    float2* Mb = X + nt * L.sx;                       // [dpad][Q2] moments of the current bin
-    float2* Ach = Mb + L.dpad * Q2;                   // [w][dpad]  Chebyshev coefficients, row order of Mb
-    float* Uf = (float*)(Ach + w * L.dpad);           // [nt][suf]  T_d(v_p), d >= dcs
-    int* l0s = (int*)(Uf + nt * L.suf);               // [nt]
-    __shared__ int bstart[kMaxTileBins + 3];
+    const int Q = P.Q, qs = P.qs, Q2 = 2 * Q;
+    const MomLayout L = mom_layout(nb, dcs, Q2, P.nlow);
+    float2* Mb = (float2*)sm;                         // [kMomBins][dpad][Q2] moments of a group of bins
+    float2* Ach = Mb + kMomBins * L.dpad * Q2;        // [w][dpad]  Chebyshev coefficients
+    float* Xh = (float*)(Ach + w * L.dpad);           // [nt][sxh]  x_q'(p), high parts
+    float* Xl = Xh + nt * L.sxh;                      // [nt][sxl]  low parts
+    float* Uh = Xl + nt * L.sxl;                      // [nt][suh]  T_d(v_p), high parts
+    float* Ul = Uh + nt * L.suh;                      // [nt][sul]  low parts, d < dcs
+    int* l0s = (int*)(Ul + nt * L.sul);               // [nt]
+    int* bstart = sh.bstart;
+    unsigned* wmag = sh.wmag;
+    uint16_t* items = sh.items;
+    const int ntask = P.nitems, nA = P.nwide;
+    for (int i = tid; i < ntask; i += nt) items[i] = P.items[i];
     for (int i = tid; i < w * L.dpad; i += nt) {
-        const int r = i / L.dpad, e = i - r * L.dpad;
-        const int d = mom_degree(e, L.ndf, dcs, nb);
-        Ach[i] = d >= 0 ? tab.ch2[r * (tab.deg + 1) + d] : make_float2(0.f, 0.f);
+        const int r = i / L.dpad, d = i - r * L.dpad;
+        Ach[i] = d < nb ? tab.ch2[r * (tab.deg + 1) + d] : make_float2(0.f, 0.f);
     }
+    float mag = 0.f;
     if (tid < cnt) {
         df vd;
-        l0s[tid] = target(t.start + tid, &vd, X + tid * L.sx);
+        l0s[tid] = target(t.start + tid, &vd, Xh + tid * L.sxh, Xl + tid * L.sxl, &mag);
         // Chebyshev basis by T_{d+1} = 2 v T_d - T_{d-1}
-        float2* ud = Ud + tid * L.sud;
-        float* uf = Uf + tid * L.suf;
+        float* uh = Uh + tid * L.suh;
+        float* ul = Ul + tid * L.sul;
         const float vh = vd.h, vl = vd.l;
         df tm{1.f, 0.f}, tc{vh, vl};
-        ud[0] = make_float2(1.f, 0.f);
-        ud[1] = make_float2(vh, vl);                 // dcs >= 2
+        uh[0] = 1.f;
+        ul[0] = 0.f;
+        uh[1] = vh;                                  // dcs >= 2
+        ul[1] = vl;
         const df v2{2.f * vh, 2.f * vl};
         int d = 2;
         for (; d < dcs; ++d) {
             const df tn = cheb_step(v2, tc, tm);
-            ud[d] = make_float2(tn.h, tn.l);
+            uh[d] = tn.h;
+            ul[d] = tn.l;
             tm = tc;
             tc = tn;
         }
-        for (int e = dcs; e < L.sud; ++e) ud[e] = make_float2(0.f, 0.f);
         float fm = tm.h, fc = tc.h;
         for (; d < nb; ++d) {
             const float fn = fmaf(2.f * vh, fc, -fm);
-            uf[d - dcs] = fn;
+            uh[d] = fn;
             fm = fc;
             fc = fn;
         }
-        for (int e = nb - dcs; e < L.suf; ++e) uf[e] = 0.f;
+        for (; d < L.dpad; ++d) uh[d] = 0.f;
     }
+    if (ANCHORED) warp_mag(wmag, mag);
     __syncthreads();
     const int lfirst = l0s[0];
     const int nbins = l0s[cnt - 1] - lfirst + 1;
@@ -250,144 +300,140 @@ __device__ __forceinline__ void spread_moments(int Q, int qs, const Tile& t, con
         bstart[b] = lo;
     }
     __syncthreads();
-    const int npairs = L.ndf + L.nf;
-    const int nitems = npairs * nq * kSpreadSub;
-    const int nqA = min(nq, (qs + 1) >> 1);        // quads holding a term q < qs
-    const int nA = L.ndf * nqA, nB = L.ndf * (nq - nqA);
-    const int nitems_pad = (nitems + 31) & ~31;
     for (int vm = 0; vm < V; ++vm) {
     if (vm > 0) {
-        if (tid < cnt) values(vm, X + tid * L.sx);
+        if (tid < cnt) mag = values(vm, Xh + tid * L.sxh, Xl + tid * L.sxl);
+        if (ANCHORED) warp_mag(wmag, mag);
         __syncthreads();
     }
+    const float tmag = ANCHORED ? tile_mag(wmag) : 0.f;
     const Acc gv = gb.at(vm * moff);
-    for (int b = 0; b < nbins; ++b) {
-        const int p0 = bstart[b], p1 = bstart[b + 1];
-        if (p0 == p1) continue;
-        for (int it = tid; it < nitems_pad; it += nt) {
-            const bool live = it < nitems;
-            const int sub = it & (kSpreadSub - 1);
-            const int o = live ? it / kSpreadSub : 0;
-            // outputs (degree pair dp, value quad qq) ordered by cost so that warps
-            // are uniform: double-float degrees with a quad holding a term q < qs,
-            // then double-float degrees with quads of small terms, then FP32 degrees
-            int dp, qq;
-            if (o < nA) {
-                dp = o / nqA;
-                qq = o - dp * nqA;
-            } else if (o < nA + nB) {
-                const int ob = o - nA;
-                dp = ob / (nq - nqA);
-                qq = nqA + (ob - dp * (nq - nqA));
-            } else {
-                const int ob = o - nA - nB;
-                dp = L.ndf + ob / nq;
-                qq = ob - (dp - L.ndf) * nq;
-            }
-            const bool lowd = dp >= L.ndf;       // FP32-tier degrees
-            const bool lowq = o >= nA && !lowd;  // double-float degrees, small Hankel terms only
+    for (int g0 = 0; g0 < nbins; g0 += kMomBins) {
+        const int gn = nbins - g0 < kMomBins ? nbins - g0 : kMomBins;
+        if (bstart[g0] == bstart[g0 + gn]) continue;
+        // double-float items, 16 lanes each (whole warps)
+        const int nwide = (gn * nA * 2 * kSpreadSub + 31) & ~31;
+        for (int it = tid; it < nwide; it += nt) {
+            const int sub = it & (2 * kSpreadSub - 1), u = it / (2 * kSpreadSub);
+            const bool live = u < gn * nA;
+            const int b = live && u >= nA ? u / nA : 0, o = live ? u - b * nA : 0;
+            const int dp = items[o] >> 8, qq = items[o] & 255;
+            const int p0 = bstart[g0 + b], p1 = live ? bstart[g0 + b + 1] : p0;
+            const float anc =
+                ANCHORED ? acc_anchor(tmag * (float)((p1 - p0 + 2 * kSpreadSub - 1) / (2 * kSpreadSub))) : 0.f;
             acc2 A[2][4];
 #pragma unroll
             for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int f = 0; f < 4; ++f) A[e][f] = acc2{0.f, 0.f};
-            if (live && !lowd && lowq) {
-                const float2* up = Ud + 2 * dp;
+                for (int f = 0; f < 4; ++f) A[e][f] = acc2{anc, 0.f};
+            const float *uph = Uh + 2 * dp, *upl = Ul + 2 * dp, *xph = Xh + 4 * qq, *xpl = Xl + 4 * qq;
 #pragma unroll 2
-                for (int p = p0 + sub; p < p1; p += kSpreadSub) {
-                    const float4 uu = *(const float4*)(up + p * L.sud);
-                    const float4 xa = *(const float4*)(X + p * L.sx + 4 * qq);
-                    const float4 xb = *(const float4*)(X + p * L.sx + 4 * qq + 2);
-                    const float xs[4] = {xa.x, xa.z, xb.x, xb.z};
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        A[0][f].s = fmaf(uu.x, xs[f], A[0][f].s);
-                        A[1][f].s = fmaf(uu.z, xs[f], A[1][f].s);
-                    }
-                }
-            } else if (live && !lowd) {
-                const float2* up = Ud + 2 * dp;
-#pragma unroll 2
-                for (int p = p0 + sub; p < p1; p += kSpreadSub) {
-                    const float4 uu = *(const float4*)(up + p * L.sud);
-                    const float4 xa = *(const float4*)(X + p * L.sx + 4 * qq);
-                    const float4 xb = *(const float4*)(X + p * L.sx + 4 * qq + 2);
-                    const df xs[4] = {{xa.x, xa.y}, {xa.z, xa.w}, {xb.x, xb.y}, {xb.z, xb.w}};
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        acc_fma(A[0][f], df{uu.x, uu.y}, xs[f]);
-                        acc_fma(A[1][f], df{uu.z, uu.w}, xs[f]);
-                    }
-                }
-            } else if (live) {
-                const float* up = Uf + 2 * (dp - L.ndf);
-#pragma unroll 2
-                for (int p = p0 + sub; p < p1; p += kSpreadSub) {
-                    const float2 uu = *(const float2*)(up + p * L.suf);
-                    const float4 xa = *(const float4*)(X + p * L.sx + 4 * qq);
-                    const float4 xb = *(const float4*)(X + p * L.sx + 4 * qq + 2);
-                    const float xs[4] = {xa.x, xa.z, xb.x, xb.z};
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        A[0][f].s = fmaf(uu.x, xs[f], A[0][f].s);
-                        A[1][f].s = fmaf(uu.y, xs[f], A[1][f].s);
-                    }
-                }
-            }
-            // combine the kSpreadSub partial sums (adjacent lanes)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
+            for (int p = p0 + sub; p < p1; p += 2 * kSpreadSub) {
+                const float2 uh = *(const float2*)(uph + p * L.suh), ul = *(const float2*)(upl + p * L.sul);
+                const float4 xh = *(const float4*)(xph + p * L.sxh), xl = *(const float4*)(xpl + p * L.sxl);
+                const df xs[4] = {{xh.x, xl.x}, {xh.y, xl.y}, {xh.z, xl.z}, {xh.w, xl.w}};
 #pragma unroll
                 for (int f = 0; f < 4; ++f) {
-                    acc2 a = A[e][f];
-#pragma unroll
-                    for (int off = kSpreadSub >> 1; off > 0; off >>= 1) {
-                        const float os = __shfl_xor_sync(0xffffffffu, a.s, off);
-                        const float oc = __shfl_xor_sync(0xffffffffu, a.c, off);
-                        float s2, q2;
-                        two_sum(a.s, os, s2, q2);
-                        a.s = s2;
-                        a.c += oc + q2;
-                    }
-                    if (live && sub == 0) {
-                        const df m = fast_two_sum(a.s, a.c);
-                        Mb[(2 * dp + e) * Q2 + 4 * qq + f] = make_float2(m.h, m.l);
-                    }
-                }
-        }
-        __syncthreads();
-        // grid[l0 + i][q'] += sum_d A[i][d] M[d][q']
-        const int l0 = lfirst + b;
-        for (int o = tid; o < w * Q2; o += nt) {
-            const int i = o / Q2, qv = o - i * Q2;
-            const int64_t idx = cell(l0 + i);
-            if (idx < 0) continue;
-            acc2 s{0.f, 0.f};
-            const float2* ar = Ach + i * L.dpad;
-            float sf = 0.f;
-            int e = 0;
-            if ((qv >> 1) < qs) {
-                for (; e < 2 * L.ndf; ++e) {
-                    const float2 a2 = ar[e], m2 = Mb[e * Q2 + qv];
-                    acc_fma(s, df{a2.x, a2.y}, df{m2.x, m2.y});
+                    acc_mul<ANCHORED>(A[0][f], df{uh.x, ul.x}, xs[f]);
+                    acc_mul<ANCHORED>(A[1][f], df{uh.y, ul.y}, xs[f]);
                 }
             }
-            for (; e < L.dpad; ++e) sf = fmaf(ar[e].x, Mb[e * Q2 + qv].x, sf);
-            const double val = acc_value(s) + (double)sf;
-            if (val != 0.0) gv.add(2 * ((int64_t)idx * Q + (qv >> 1)) + (qv & 1), val);
+            if (ANCHORED) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int f = 0; f < 4; ++f) A[e][f].s -= anc;
+            }
+            // each exchange halves the outputs a lane carries: lane sub ends
+            // with degree e = bit 3, value f = bits 2 and 1, summed over bit 0
+            acc2 h4[4], h2[2];
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                h4[f] = acc_exchange((sub & 8) ? A[1][f] : A[0][f], (sub & 8) ? A[0][f] : A[1][f], 8);
+#pragma unroll
+            for (int f = 0; f < 2; ++f)
+                h2[f] = acc_exchange((sub & 4) ? h4[2 + f] : h4[f], (sub & 4) ? h4[f] : h4[2 + f], 4);
+            acc2 h = acc_exchange((sub & 2) ? h2[1] : h2[0], (sub & 2) ? h2[0] : h2[1], 2);
+            h = acc_exchange(h, h, 1);
+            if (live && (sub & 1) == 0) {
+                const df m = fast_two_sum(h.s, h.c);
+                Mb[(b * L.dpad + 2 * dp + (sub >> 3)) * Q2 + 4 * qq + ((sub >> 1) & 3)] = make_float2(m.h, m.l);
+            }
+        }
+        // FP32 items, 8 lanes each, on the threads after the ones above
+        const int nF = ntask - nA;
+        const int nnarrow = (gn * nF * kSpreadSub + 31) & ~31;
+        const int shift = nwide % nt;
+        for (int it = tid >= shift ? tid - shift : tid - shift + nt; it < nnarrow; it += nt) {
+            const int sub = it & (kSpreadSub - 1), u = it / kSpreadSub;
+            const bool live = u < gn * nF;
+            const int b = live && u >= nF ? u / nF : 0, o = live ? nA + u - b * nF : 0;
+            const int dp = items[o] >> 8, qq = items[o] & 255;
+            const int p0 = bstart[g0 + b], p1 = live ? bstart[g0 + b + 1] : p0;
+            const float *uph = Uh + 2 * dp, *xph = Xh + 4 * qq;
+            float A[2][4] = {};
+#pragma unroll 2
+            for (int p = p0 + sub; p < p1; p += kSpreadSub) {
+                const float2 uh = *(const float2*)(uph + p * L.suh);
+                const float4 xh = *(const float4*)(xph + p * L.sxh);
+                const float a0 = uh.x, a1 = uh.y, xs[4] = {xh.x, xh.y, xh.z, xh.w};
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    A[0][f] = fmaf(a0, xs[f], A[0][f]);
+                    A[1][f] = fmaf(a1, xs[f], A[1][f]);
+                }
+            }
+            float h4[4], h2[2];
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                h4[f] = ((sub & 4) ? A[1][f] : A[0][f]) +
+                        __shfl_xor_sync(0xffffffffu, (sub & 4) ? A[0][f] : A[1][f], 4);
+#pragma unroll
+            for (int f = 0; f < 2; ++f)
+                h2[f] = ((sub & 2) ? h4[2 + f] : h4[f]) +
+                        __shfl_xor_sync(0xffffffffu, (sub & 2) ? h4[f] : h4[2 + f], 2);
+            const float h = ((sub & 1) ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? h2[0] : h2[1], 1);
+            if (live) Mb[(b * L.dpad + 2 * dp + (sub >> 2)) * Q2 + 4 * qq + (sub & 3)] = make_float2(h, 0.f);
+        }
+        __syncthreads();
+        // grid[l0 + c][q'] += sum_b sum_d A[c - b][d] M_b[d][q'] over the group's bins b with 0 <= c - b < w
+        const int l0 = lfirst + g0, ncell = gn + w - 1;
+        for (int o = tid; o < ncell * Q2; o += nt) {
+            const int c = o / Q2, qv = o - c * Q2;
+            const int64_t idx = cell(l0 + c);
+            if (idx < 0) continue;
+            const int ed = (qv >> 1) < qs ? 2 * L.ndf : 0;
+            const int b_lo = c - w + 1 > 0 ? c - w + 1 : 0, b_hi = c < gn - 1 ? c : gn - 1;
+            acc2 s{0.f, 0.f};
+            float sf = 0.f;
+            for (int b = b_lo; b <= b_hi; ++b) {
+                const float2* ar = Ach + (c - b) * L.dpad;
+                const float2* mb = Mb + b * L.dpad * Q2 + qv;
+                int e = 0;
+                for (; e < ed; ++e) {
+                    const float2 a2 = ar[e], m2 = mb[e * Q2];
+                    acc_fma(s, df{a2.x, a2.y}, df{m2.x, m2.y});
+                }
+                for (; e < L.dpad; ++e) sf = fmaf(ar[e].x, mb[e * Q2].x, sf);
+            }
+            // (one FP64 sum per value: FP64 issues 64 times slower)
+            float h, l;
+            two_sum(s.s, sf, h, l);
+            l += s.c;
+            if (h != 0.f || l != 0.f)
+                gv.add(2 * ((int64_t)idx * Q + (qv >> 1)) + (qv & 1), (double)h + (double)l);
         }
         __syncthreads();
     }
     }
 }
 
-// Shared memory (bytes) of the moment path for nt points and Q = 2M.
-__host__ __device__ __forceinline__ size_t spread_moments_smem(int nt, int Q, int w, int nb, int dcs)
+// Shared memory (bytes) of the moment path for nt points, Q = 2M and nlow.
+__host__ __device__ __forceinline__ size_t spread_moments_smem(int nt, int Q, int nlow, int w, int nb, int dcs)
 {
-    const MomLayout L = mom_layout(nb, dcs, 2 * Q);
-    return sizeof(float2) * ((size_t)nt * L.sud + (size_t)nt * L.sx + (size_t)L.dpad * 2 * Q +
-                             (size_t)w * L.dpad) +
-           sizeof(float) * (size_t)nt * L.suf + sizeof(int) * (size_t)nt;
+    const MomLayout L = mom_layout(nb, dcs, 2 * Q, nlow);
+    return sizeof(float2) * ((size_t)kMomBins * L.dpad * 2 * Q + (size_t)w * L.dpad) +
+           sizeof(float) * (size_t)nt * (L.sxh + L.sxl + L.suh + L.sul) + sizeof(int) * (size_t)nt;
 }
 
 // q-folded dense tile.  Within the bin of cell L, r_p = R_L - (h/2) v_p with
@@ -503,10 +549,10 @@ __host__ __device__ __forceinline__ int fold_edf_max(int nb, int dcs)
 // Shared memory (bytes) of the folded path for nt points and Q = 2M (its largest layout).
 __host__ __device__ __forceinline__ size_t spread_fold_smem(int nt, int Q, int w, int nb, int dcs)
 {
-    const MomLayout L = mom_layout(nb, dcs, 2 * Q);
+    const MomLayout L = mom_layout(nb, dcs, 2 * Q, 0);
     const int G = fold_group_bins(L.dpad, 2 * Q);
     const int em = fold_emax(nb), edm = fold_edf_max(nb, dcs);
-    const int sud = mom_stride(edm), suf = mom_stride(em - 2);
+    const int sud = mom_stride2(edm), suf = mom_stride2(em - 2);
     return sizeof(float4) * ((size_t)nt + (size_t)G * em) +
            sizeof(float2) * ((size_t)nt * sud + (size_t)G * L.dpad * (2 * Q + 1) + (size_t)G * Q * kBetaStride +
                              (size_t)w * L.dpad) +
@@ -516,18 +562,18 @@ __host__ __device__ __forceinline__ size_t spread_fold_smem(int nt, int Q, int w
 // Members (MULTI): V real components with coefficients c2 + vm c_stride,
 // grids moff accumulator elements apart; the points' cells, bases and phase
 // factors and the bins are formed once for all members.
-template <bool MULTI, class Acc>
-__device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, const Tables& tab, FoldPlan F,
+template <bool ANCHORED, bool MULTI, class Acc>
+__device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& t, const Tables& tab, FoldPlan F,
                             const double* __restrict__ r_s, const float2* __restrict__ r2,
                             const float2* __restrict__ c2, int64_t c_stride, int V, int64_t moff, Acc gb,
-                            float4* sm4)
+                            float4* sm4, MomShared& sh)
 {
     const int nt = blockDim.x, tid = threadIdx.x, cnt = t.count;
     const int w = tab.w, nb = tab.nb, dcs = tab.dcs;
-    const int Q2 = 2 * Q, K = F.K, E = F.E, Edf = F.Edf;
-    const MomLayout L = mom_layout(nb, dcs, Q2);
+    const int Q = P.Q, qs = P.qs, Q2 = 2 * Q, K = F.K, E = F.E, Edf = F.Edf;
+    const MomLayout L = mom_layout(nb, dcs, Q2, 0);
     const int G = fold_group_bins(L.dpad, Q2);
-    const int sud = mom_stride(Edf), suf = mom_stride(E - Edf);
+    const int sud = mom_stride2(Edf), suf = mom_stride2(E - Edf);
     float4* Y = sm4;                                  // [nt] y_p as (re.h, re.l, im.h, im.l)
     float4* N = Y + nt;                               // [G][E] N[e] of a group of bins
     float2* Ud = (float2*)(N + G * E);                // [nt][sud] T_e(v_p), e < Edf
@@ -539,11 +585,14 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
     float2* Ach = beta + G * Q * kBetaStride;         // [w][dpad] Chebyshev coefficients of the taps
     float* Uf = (float*)(Ach + w * L.dpad);           // [nt][suf] T_e(v_p), Edf <= e < E
     int* l0s = (int*)(Uf + nt * suf);                 // [nt]
-    __shared__ int bstart[kMaxTileBins + 3];
+    int* bstart = sh.bstart;
+    unsigned* wmag = sh.wmag;
+    uint16_t* items = sh.items;
+    const int nA = P.nwide;
+    for (int i = tid; i < P.nitems; i += nt) items[i] = P.items[i];
     for (int i = tid; i < w * L.dpad; i += nt) {
-        const int r = i / L.dpad, e = i - r * L.dpad;
-        const int d = mom_degree(e, L.ndf, dcs, nb);
-        Ach[i] = d >= 0 ? tab.ch2[r * (tab.deg + 1) + d] : make_float2(0.f, 0.f);
+        const int r = i / L.dpad, d = i - r * L.dpad;
+        Ach[i] = d < nb ? tab.ch2[r * (tab.deg + 1) + d] : make_float2(0.f, 0.f);
     }
     // this thread's point: (r_j/rho)^(-1/2) e^{i w_c x_j} (the weight without c_j)
     df yr{0.f, 0.f}, yi{0.f, 0.f};
@@ -577,6 +626,7 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
         spread_weight_fx(B, tab.tw2, X, r2[j], MULTI ? make_float2(1.f, 0.f) : c2[j], &yr, &yi, &rat);
         if (!MULTI) Y[tid] = make_float4(yr.h, yr.l, yi.h, yi.l);
     }
+    if (ANCHORED && !MULTI) warp_mag(wmag, tid < cnt ? mag_of(yr.h, yi.h) : 0.f);
     __syncthreads();
     const int lfirst = l0s[0];
     const int nbins = l0s[cnt - 1] - lfirst + 1;
@@ -592,13 +642,17 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
     const df rho{B.rho_h, B.rho_l};
     for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
     if (MULTI) {
+        float mag = 0.f;
         if (tid < cnt) {
             const float2 cv = c2[vm * c_stride + j];
             const df wr = df_mul(df{cv.x, cv.y}, yr), wi = df_mul(df{cv.x, cv.y}, yi);
             Y[tid] = make_float4(wr.h, wr.l, wi.h, wi.l);
+            mag = mag_of(wr.h, wi.h);
         }
+        if (ANCHORED) warp_mag(wmag, mag);
         __syncthreads();
     }
+    const float tmag = ANCHORED ? tile_mag(wmag) : 0.f;
     const Acc gv = gb.at(vm * moff);
     for (int g0 = 0; g0 < nbins; g0 += G) {
         const int gn = nbins - g0 < G ? nbins - g0 : G;
@@ -623,7 +677,9 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
                 dfi = false;
             }
             const int p0 = bstart[g0 + b], p1 = bstart[g0 + b + 1];
-            acc2 a00{0.f, 0.f}, a01{0.f, 0.f}, a10{0.f, 0.f}, a11{0.f, 0.f};
+            const float anc = ANCHORED && live && dfi
+                                  ? acc_anchor(tmag * (float)((p1 - p0 + kSpreadSub - 1) / kSpreadSub)) : 0.f;
+            acc2 a00{anc, 0.f}, a01{anc, 0.f}, a10{anc, 0.f}, a11{anc, 0.f};
             if (live && dfi) {
                 const float2* up = Ud + 2 * pr;
 #pragma unroll 2
@@ -631,10 +687,10 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
                     const float4 uu = *(const float4*)(up + p * sud);
                     const float4 yv = Y[p];
                     const df u0{uu.x, uu.y}, u1{uu.z, uu.w}, yr{yv.x, yv.y}, yi{yv.z, yv.w};
-                    acc_fma(a00, u0, yr);
-                    acc_fma(a01, u0, yi);
-                    acc_fma(a10, u1, yr);
-                    acc_fma(a11, u1, yi);
+                    acc_mul<ANCHORED>(a00, u0, yr);
+                    acc_mul<ANCHORED>(a01, u0, yi);
+                    acc_mul<ANCHORED>(a10, u1, yr);
+                    acc_mul<ANCHORED>(a11, u1, yi);
                 }
             } else if (live) {
                 const float* up = Uf + 2 * pr;
@@ -648,27 +704,23 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
                     a11.s = fmaf(uu.y, yv.z, a11.s);
                 }
             }
-            acc2* accs[4] = {&a00, &a01, &a10, &a11};
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                acc2 a = *accs[f];
-#pragma unroll
-                for (int off = kSpreadSub >> 1; off > 0; off >>= 1) {
-                    const float os = __shfl_xor_sync(0xffffffffu, a.s, off);
-                    const float oc = __shfl_xor_sync(0xffffffffu, a.c, off);
-                    float s2, q2;
-                    two_sum(a.s, os, s2, q2);
-                    a.s = s2;
-                    a.c += oc + q2;
-                }
-                *accs[f] = a;
+            if (ANCHORED) {
+                a00.s -= anc;
+                a01.s -= anc;
+                a10.s -= anc;
+                a11.s -= anc;
             }
-            if (live && sub == 0) {
-                const int e0 = dfi ? 2 * pr : Edf + 2 * pr;
-                const df n00 = fast_two_sum(a00.s, a00.c), n01 = fast_two_sum(a01.s, a01.c);
-                const df n10 = fast_two_sum(a10.s, a10.c), n11 = fast_two_sum(a11.s, a11.c);
-                N[b * E + e0] = make_float4(n00.h, n00.l, n01.h, n01.l);
-                N[b * E + e0 + 1] = make_float4(n10.h, n10.l, n11.h, n11.l);
+            // lanes exchange halves: lane sub ends with degree e0 + (sub >> 2),
+            // part (re, im) = (sub >> 1) & 1, then the last pair is summed
+            const bool hi4 = sub & 4, hi2 = sub & 2;
+            const acc2 hr = acc_exchange(hi4 ? a10 : a00, hi4 ? a00 : a10, 4);
+            const acc2 hm = acc_exchange(hi4 ? a11 : a01, hi4 ? a01 : a11, 4);
+            acc2 h = acc_exchange(hi2 ? hm : hr, hi2 ? hr : hm, 2);
+            h = acc_exchange(h, h, 1);
+            if (live && (sub & 1) == 0) {
+                const int e = (dfi ? 2 * pr : Edf + 2 * pr) + (sub >> 2);
+                const df v = fast_two_sum(h.s, h.c);
+                *((float2*)(N + b * E + e) + ((sub >> 1) & 1)) = make_float2(v.h, v.l);
             }
         }
         // beta_qk = s^q sum_{j >= k, j = k mod 2} t_j MC(j, k), t_j = C(q+j-1, j) eta^j,
@@ -705,18 +757,19 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
         // (b) M[d][q] = sum_k beta_qk (N[d+k] + N[|d-k|]) / 2 into the row order of Mb;
         // each item forms two consecutive q, so one sum N[d+k] + N[|d-k|]
         // (an unevaluated (hi, lo) pair) serves both
+        // (items of a group of bins in the order of list_items, two rows each,
+        // so that the double-float ones fill warps)
         for (int o = tid; o < gn * L.dpad * (Q >> 1); o += nt) {
-            const int b = o / (L.dpad * (Q >> 1)), rem = o - b * (L.dpad * (Q >> 1));
-            const int e = rem / (Q >> 1), q0 = 2 * (rem - e * (Q >> 1));
-            const int d = mom_degree(e, L.ndf, dcs, nb);
+            const int row = o / gn, b = o - row * gn;
+            const int it = items[row >> 1], q0 = 2 * (it & 255), e = 2 * (it >> 8) + (row & 1);
+            const int d = e < nb ? e : -1;
             float2 mr0 = make_float2(0.f, 0.f), mi0 = mr0, mr1 = mr0, mi1 = mr0;
             if (d >= 0) {
                 const float2* bt0 = beta + (b * Q + q0) * kBetaStride;
                 const float2* bt1 = bt0 + kBetaStride;
                 const float4* Nb = N + b * E;
                 const float4 n0 = Nb[d];
-                const bool dfe = e < 2 * L.ndf;
-                if (dfe && q0 < qs) {
+                if ((row >> 1) < nA) {
                     const bool df1 = q0 + 1 < qs;
                     acc2 ar0{0.f, 0.f}, ai0{0.f, 0.f}, ar1{0.f, 0.f}, ai1{0.f, 0.f};
                     const float2 b00 = bt0[0], b10 = bt1[0];
@@ -793,18 +846,16 @@ __device__ void spread_fold(const AsyBlock& B, int Q, int qs, const Tile& t, con
             if (idx < 0 || idx >= nf1) continue;
             const int b_lo = c - w + 1 > 0 ? c - w + 1 : 0;
             const int b_hi = c < gn - 1 ? c : gn - 1;
-            const bool dq = (qv >> 1) < qs;
+            const int ed = (qv >> 1) < qs ? 2 * L.ndf : 0;
             acc2 sacc{0.f, 0.f};
             for (int b = b_lo; b <= b_hi; ++b) {
                 const float2* ar = Ach + (c - b) * L.dpad;
                 const float2* mb = Mb + b * L.dpad * Q2s + qv;
                 float sf = 0.f;
                 int e = 0;
-                if (dq) {
-                    for (; e < 2 * L.ndf; ++e) {
-                        const float2 a2 = ar[e], m2 = mb[e * Q2s];
-                        acc_fma(sacc, df{a2.x, a2.y}, df{m2.x, m2.y});
-                    }
+                for (; e < ed; ++e) {
+                    const float2 a2 = ar[e], m2 = mb[e * Q2s];
+                    acc_fma(sacc, df{a2.x, a2.y}, df{m2.x, m2.y});
                 }
                 for (; e < L.dpad; ++e) sf = fmaf(ar[e].x, mb[e * Q2s].x, sf);
                 float s2, e2;
@@ -998,13 +1049,14 @@ __global__ void k_expand_lists(ExpandLists E, int total, const ProbParams* __res
 // or taps and phase factor once.  MULTI: the instance for V > 1 (V = 1 runs
 // the instance without the member loop's registers and barriers).
 template <bool DET, bool MULTI>
-__global__ void k_asy_spread(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
+__global__ void __launch_bounds__(256, 3) k_asy_spread(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
                              const Tile* __restrict__ tiles, const int32_t* __restrict__ modes, Tables tab,
                              const double* __restrict__ r_s, const float2* __restrict__ r2,
                              const float2* __restrict__ c2, int64_t c_stride, int V,
                              double2* __restrict__ grid_b, int64_t gb_stride)
 {
     extern __shared__ float4 smem4[];
+    __shared__ MomShared sh;
     const Tile t = tiles[blockIdx.x];
     if (t.count <= 0) return;
     const int mode = modes[blockIdx.x];
@@ -1013,35 +1065,52 @@ __global__ void k_asy_spread(const ProbParams* __restrict__ probs, const AsyBloc
     using Acc = typename AccumOf<DET>::type;
     const Acc gb = Acc{(double*)grid_b, probs[B.prob].fxs}.at(2 * B.b_off);
     const int64_t moff = 2 * gb_stride;
-    if ((mode & 3) == 2)
-        spread_fold<MULTI>(B, Q, probs[B.prob].qs, t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V, moff, gb,
-                           smem4);
-    else if (mode & 3) {
+    if ((mode & 3) == 2) {
+        if (tab.anchored)
+            spread_fold<true, MULTI>(B, probs[B.prob], t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V, moff,
+                                     gb, smem4, sh);
+        else
+            spread_fold<false, MULTI>(B, probs[B.prob], t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V,
+                                      moff, gb, smem4, sh);
+    } else if (mode & 3) {
         // c_j (r_j/rho)^(-q-1/2) e^{i w_c x_j} onto the 2 N1 + 1 modes
         const int nf1 = 2 * B.N1 + 1;
         df yr{0.f, 0.f}, yi{0.f, 0.f}, rat{0.f, 0.f};   // this thread's point's weight without c_j
         int64_t jt = 0;
-        auto put = [&](float2* xq, float2 cv) {
+        const int nlow = 2 * probs[B.prob].nlow;   // terms kept in double-float
+        auto put = [&](float* xh, float* xl, float2 cv) {
             df wr = df_mul(df{cv.x, cv.y}, yr), wi = df_mul(df{cv.x, cv.y}, yi);
-            for (int q = 0; q < Q; ++q) {
-                xq[2 * q] = make_float2(wr.h, wr.l);
-                xq[2 * q + 1] = make_float2(wi.h, wi.l);
+            int q = 0;
+            for (; q < nlow; ++q) {
+                *(float2*)(xh + 2 * q) = make_float2(wr.h, wi.h);
+                *(float2*)(xl + 2 * q) = make_float2(wr.l, wi.l);
                 wr = df_mul(wr, rat);
                 wi = df_mul(wi, rat);
             }
+            float fr = wr.h, fi = wi.h;
+            for (; q < Q; ++q) {
+                *(float2*)(xh + 2 * q) = make_float2(fr, fi);
+                fr *= rat.h;
+                fi *= rat.h;
+            }
+            return mag_of(xh[0], xh[1]);   // the ratio is at most one
         };
-        spread_moments(Q, probs[B.prob].qs, t, tab,
-            [&](int64_t j, df* v, float2* xq) {
-                long long Xp;
-                const int l0 = spread_cell_fx(B, tab.w, r_s[j], &Xp, v);
-                spread_weight_fx(B, tab.tw2, Xp, r2[j], make_float2(1.f, 0.f), &yr, &yi, &rat);
-                jt = j;
-                put(xq, c2[j]);
-                return l0;
-            },
-            [&](int vm, float2* xq) { put(xq, c2[vm * c_stride + jt]); }, MULTI ? V : 1, moff,
-            [&](int c) -> int64_t { const int x = c + B.N1; return (x >= 0 && x < nf1) ? x : -1; },
-            gb, (float2*)smem4);
+        auto target = [&](int64_t j, df* v, float* xh, float* xl, float* mag) {
+            long long Xp;
+            const int l0 = spread_cell_fx(B, tab.w, r_s[j], &Xp, v);
+            spread_weight_fx(B, tab.tw2, Xp, r2[j], make_float2(1.f, 0.f), &yr, &yi, &rat);
+            jt = j;
+            *mag = put(xh, xl, c2[j]);
+            return l0;
+        };
+        auto values = [&](int vm, float* xh, float* xl) { return put(xh, xl, c2[vm * c_stride + jt]); };
+        auto cell = [&](int c) -> int64_t { const int x = c + B.N1; return (x >= 0 && x < nf1) ? x : -1; };
+        if (tab.anchored)
+            spread_moments<true>(probs[B.prob], t, tab, target, values, MULTI ? V : 1, moff, cell, gb,
+                                 (float*)smem4, sh);
+        else
+            spread_moments<false>(probs[B.prob], t, tab, target, values, MULTI ? V : 1, moff, cell, gb,
+                                  (float*)smem4, sh);
     }
     else
         spread_taps<MULTI>(B, Q, t, tab, r_s, r2, c2, c_stride, V, moff, gb, smem4);
@@ -1434,12 +1503,15 @@ __device__ __forceinline__ int adj_spread_factor(const AsyBlock& B, const ProbPa
     return t0;
 }
 
-// The 2M values x_q for g_k from the frequency's factor.
-__device__ __forceinline__ void adj_values(const ProbParams& P, const AdjFactor& F, double gk, float2* xq)
+// The 2M values x_q for g_k from the frequency's factor, handed to put(q, re,
+// im); returns a bound of their magnitudes.
+template <class Put>
+__device__ __forceinline__ float adj_values(const ProbParams& P, const AdjFactor& F, double gk, Put&& put)
 {
     const df g = df_from(gk);
     const df fr = df_mul(F.fr, g), fi = df_mul(F.fi, g), mz = F.mz;
     df mq{1.f, 0.f};
+    float mag = 0.f;
     for (int q = 0; q < P.Q; ++q) {
         const df cq = df_mul(df{P.a2[q].x, P.a2[q].y}, mq);
         // (fr + i fi) i^q cq
@@ -1452,10 +1524,11 @@ __device__ __forceinline__ void adj_values(const ProbParams& P, const AdjFactor&
         }
         ur = df_mul(ur, cq);
         ui = df_mul(ui, cq);
-        xq[2 * q] = make_float2(ur.h, ur.l);
-        xq[2 * q + 1] = make_float2(ui.h, ui.l);
+        put(q, ur, ui);
+        mag = fmaxf(mag, mag_of(ur.h, ui.h));
         mq = df_mul(mq, mz);
     }
+    return mag;
 }
 
 // Frequencies of a tile -> FFT grid (periodic, atomics into tgrid).  Dense
@@ -1465,12 +1538,13 @@ __device__ __forceinline__ void adj_values(const ProbParams& P, const AdjFactor&
 // (g_s + vm g_stride into tgrid + vm tg_stride) share each frequency's cell,
 // basis or taps and factor (MULTI: the instance for V > 1).
 template <bool MULTI>
-__global__ void k_asy_adj_spread(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
+__global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
                                  const Tile* __restrict__ tiles, Tables tab,
                                  const double* __restrict__ w_s, const double* __restrict__ g_s,
                                  int64_t g_stride, int V, double2* __restrict__ tgrid, int64_t tg_stride)
 {
     extern __shared__ float4 sma[];
+    __shared__ MomShared sh;
     __shared__ int use_mom;
     const Tile t = tiles[blockIdx.x];
     const AsyBlock B = blks[t.blk];
@@ -1491,16 +1565,27 @@ __global__ void k_asy_adj_spread(const ProbParams* __restrict__ probs, const Asy
     if (use_mom) {
         AdjFactor F{};
         int64_t kt = 0;
-        spread_moments(Q, P.qs, t, tab,
-            [&](int64_t k, df* v, float2* xq) {
-                const int t0 = adj_spread_factor(B, P, tab, w_s[k], v, &F);
-                kt = k;
-                adj_values(P, F, g_s[k], xq);
-                return t0;
-            },
-            [&](int vm, float2* xq) { adj_values(P, F, g_s[vm * g_stride + kt], xq); }, MULTI ? V : 1,
-            2 * tg_stride,
-            [&](int c) -> int64_t { return c & mask; }, tg, (float2*)sma);
+        const int nlow = 2 * P.nlow;   // terms kept in double-float
+        auto put = [&](float* xh, float* xl, double gk) {
+            return adj_values(P, F, gk, [&](int q, df re, df im) {
+                *(float2*)(xh + 2 * q) = make_float2(re.h, im.h);
+                if (q < nlow) *(float2*)(xl + 2 * q) = make_float2(re.l, im.l);
+            });
+        };
+        auto target = [&](int64_t k, df* v, float* xh, float* xl, float* mag) {
+            const int t0 = adj_spread_factor(B, P, tab, w_s[k], v, &F);
+            kt = k;
+            *mag = put(xh, xl, g_s[k]);
+            return t0;
+        };
+        auto values = [&](int vm, float* xh, float* xl) { return put(xh, xl, g_s[vm * g_stride + kt]); };
+        auto cell = [&](int c) -> int64_t { return c & mask; };
+        if (tab.anchored)
+            spread_moments<true>(P, t, tab, target, values, MULTI ? V : 1, 2 * tg_stride, cell, tg,
+                                 (float*)sma, sh);
+        else
+            spread_moments<false>(P, t, tab, target, values, MULTI ? V : 1, 2 * tg_stride, cell, tg,
+                                  (float*)sma, sh);
         return;
     }
     const int ncoef = w * (deg + 1);
@@ -1515,7 +1600,9 @@ __global__ void k_asy_adj_spread(const ProbParams* __restrict__ probs, const Asy
     if (tid < cnt) {
         df vdf;
         const int t0 = adj_spread_factor(B, P, tab, w_s[k], &vdf, &F);
-        adj_values(P, F, g_s[k], (float2*)(uval + tid * Q));
+        adj_values(P, F, g_s[k], [&](int q, df re, df im) {
+            uval[tid * Q + q] = make_float4(re.h, re.l, im.h, im.l);
+        });
         for (int i = 0; i < w; ++i) {
             const df tp = horner_comp(coef + i * (deg + 1), deg, vdf.h, vdf.l, tab.deg_comp);
             taps[tid * w + i] = make_float2(tp.h, tp.l);
@@ -1529,7 +1616,10 @@ __global__ void k_asy_adj_spread(const ProbParams* __restrict__ probs, const Asy
     for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
     if (MULTI && vm > 0) {
         __syncthreads();   // the previous member's reads of uval are done
-        if (tid < cnt) adj_values(P, F, g_s[vm * g_stride + k], (float2*)(uval + tid * Q));
+        if (tid < cnt)
+            adj_values(P, F, g_s[vm * g_stride + k], [&](int q, df re, df im) {
+                uval[tid * Q + q] = make_float4(re.h, re.l, im.h, im.l);
+            });
         __syncthreads();
     }
     const Accum tgv = tg.at(2 * vm * tg_stride);
@@ -1723,7 +1813,7 @@ __device__ void spread_moments_f32(const AsyBlock& B, int Q, const Tile& t, cons
     const int w = tab.w, nb = tab.nb;
     const int Q2 = 2 * Q;
     const int ndp = (nb + 1) >> 1, dpad = 2 * ndp, nq = Q2 >> 2;
-    const int su = mom_stride(nb), sx = f32_stride4(Q2);
+    const int su = mom_stride2(nb), sx = f32_stride4(Q2);
     const int GB = f32_group_bins(dpad, Q2);
     float* U = sm;                               // [nt][su]
     float* X = U + nt * su;                      // [nt][sx]
@@ -1857,7 +1947,7 @@ __device__ void spread_moments_f32(const AsyBlock& B, int Q, const Tile& t, cons
 __host__ __device__ __forceinline__ size_t spread_moments_f32_smem(int nt, int Q, int w, int nb)
 {
     const int dpad = 2 * ((nb + 1) >> 1);
-    return sizeof(float) * ((size_t)nt * mom_stride(nb) + (size_t)nt * f32_stride4(2 * Q) +
+    return sizeof(float) * ((size_t)nt * mom_stride2(nb) + (size_t)nt * f32_stride4(2 * Q) +
                             (size_t)f32_group_bins(dpad, 2 * Q) * dpad * 2 * Q + (size_t)w * dpad) +
            sizeof(int) * (size_t)nt;
 }
@@ -2119,7 +2209,7 @@ cudaError_t launch_asy_adj_spread(const ProbParams* probs, const AsyBlock* blks,
     if (nt < 32 || nt > kInterpTileThreads || (nt & 31)) return cudaErrorInvalidValue;
     size_t smem = sizeof(float4) * (size_t)nt * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
                   sizeof(float2) * (size_t)nt * tab.w + sizeof(int) * (size_t)nt;
-    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.w, tab.nb, tab.dcs);
+    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
     if (smem_mom > smem) smem = smem_mom;
     if (members < 1) return cudaErrorInvalidValue;
     auto kern = members > 1 ? k_asy_adj_spread<true> : k_asy_adj_spread<false>;
@@ -2204,7 +2294,7 @@ cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, con
     if (ntiles <= 0) return cudaSuccess;
     size_t smem = sizeof(float4) * (size_t)nt * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
                   sizeof(float2) * (size_t)nt * tab.w + sizeof(int) * (size_t)nt;
-    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.w, tab.nb, tab.dcs);
+    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
     if (smem_mom > smem) smem = smem_mom;
     const size_t smem_fold = spread_fold_smem(nt, qmax, tab.w, tab.nb, tab.dcs);
     if (smem_fold > smem) smem = smem_fold;

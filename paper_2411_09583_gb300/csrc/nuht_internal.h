@@ -22,6 +22,10 @@ constexpr int kMaxDeg = 20;         // degree of the kernel piece polynomials
 // spreading grid then has N1 ~ 2 X S / pi + w/2 <= ~2.04e6 cells and its FFT
 // at most 2^23 points (the single-FFT limit is 2^kFftMaxLog2).
 constexpr double kAsyMaxXS = 3.2e6;
+// Tolerance from which the spreading sums are anchored: their rounding
+// (measured ~3e-13 of the result, against ~1e-14 for the compensated sums)
+// stays far below it.
+constexpr double kAnchorMinEps = 1e-11;
 constexpr int kMomFold = 32;        // FP32 partial sums of the spreading moments span at most this many points
 constexpr int kMaxNtop = 400;       // largest Bessel index kept by the local evaluation
                                     // (the transposed moments then stay within 205 KB of shared memory)
@@ -75,6 +79,10 @@ __host__ __device__ inline FftTile fft_tile(int LN, int pass, int Q)
     return T;
 }
 
+// Items of the moment contraction: pairs of the up to kMaxDeg + 1 degrees
+// (double-float ones rounded up to even) times Hankel pairs.
+constexpr int kMaxMomItems = ((kMaxDeg + 2) / 2) * (kMaxQ / 2);
+
 // Per-problem constants.
 struct ProbParams {
     int nu;        // |nu|
@@ -85,6 +93,12 @@ struct ProbParams {
     int fxs;       // accumulation: kFxOff = FP64 atomics; else the deterministic mode's
                    // fixed-point scale kFxScale (contributions add round(v 2^fxs) exactly)
     int8_t dcp[kMaxQ / 2];   // per Hankel pair (2p, 2p+1): double-float degrees of the interpolation sums
+    // Items of a spreading tile's moment contraction, (degree pair << 8 | Hankel
+    // pair): the nwide double-float ones first (pairs of degrees below a Hankel
+    // pair's need), then the FP32 ones; the first nlow Hankel pairs have some
+    // double-float item (their values keep low parts)
+    int16_t nitems, nwide, nlow;
+    uint16_t items[kMaxMomItems];
     double z;      // crossover
     double cphi, sphi;           // cos, sin of phi = -(2 nu + 1) pi / 4
     float2 cphi2, sphi2;         // the same as double-float
@@ -236,11 +250,13 @@ struct Tables {
     int deg_comp;          // degrees above this one are evaluated in plain FP32
     const float2* ch2;     // [w][deg + 1] pieces in the Chebyshev basis T_d(v), double-float
     int nb;                // Chebyshev terms kept (tail below 1e-3 eps)
-    int dcs;               // spreading moments of degree >= dcs accumulate in plain FP32
+    int dcs;               // spreading moments of degree >= dcs (even) accumulate in plain FP32
+    int nlow;              // largest ProbParams::nlow (sizes the spreading tiles)
     int dci;               // interpolation terms of degree >= dci are summed in plain FP32
     float fold_tol;        // truncation of the spreading weights' Chebyshev form within a bin
     float fold_df_tol;     // weights' Chebyshev terms above this need double-float moments
     double half_w;         // w / 2
+    int anchored;          // anchored accumulation (acc_fma_anchored): eps >= kAnchorMinEps
     const float2* ph2;     // psi-hat pieces [ph_pieces][ph_deg + 1] in v in [-1, 1], double-float
     double interp_const;   // sqrt(2/pi) * 4 / w^2
     float2 ic2;            // the same as double-float

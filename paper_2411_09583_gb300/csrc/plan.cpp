@@ -550,6 +550,26 @@ static int verify_lists(nuht_plan_t P)
         if (rc_ != NUHT_OK) return rc_; \
     } while (0)
 
+// The moment items of a problem whose Hankel pair p needs double-float for the
+// degrees below dsp[p] (none from term qs on).
+static void list_moment_items(ProbParams& pp, const int* dsp, int nb, int dcs)
+{
+    const int ndf = dcs / 2, npairs = ndf + (nb - dcs + 1) / 2, nq = pp.Q / 2;
+    auto wide_rows = [&](int q) { return 2 * q >= pp.qs ? 0 : std::min((dsp[q] + 1) / 2, ndf); };
+    int k = 0;
+    pp.nlow = 0;
+    for (int q = 0; q < nq; ++q)
+        for (int d = 0; d < wide_rows(q); ++d) {
+            pp.items[k++] = (uint16_t)(d << 8 | q);
+            pp.nlow = (int16_t)(q + 1);
+        }
+    pp.nwide = (int16_t)k;
+    for (int d = 0; d < npairs; ++d)
+        for (int q = 0; q < nq; ++q)
+            if (d >= wide_rows(q)) pp.items[k++] = (uint16_t)(d << 8 | q);
+    pp.nitems = (int16_t)k;
+}
+
 // src: build from the sorted arrays and permutations of that plan, repeated
 // once per problem (derivative plans), instead of checking and sorting r and omega.
 static int build_plan(nuht_plan_t P, const double* r, const double* omega, const nuht_plan_s* src = nullptr)
@@ -864,17 +884,36 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     // the expansions' truncation of at most eps per entry (Lemma 3.1, Sec. 3.2
     // eq. asy-error) and inside the 10 eps ||c||_1 contract.
     constexpr double kRoundBudget = 0.1;
-    // Per Hankel pair, the degrees of the interpolation's per-bin and
-    // per-frequency sums that need double-float: term q enters g with weight
+    // Per Hankel pair, the degrees of the spreading moments and of the
+    // interpolation's per-bin and per-frequency sums that need double-float: term q enters g with weight
     // at most |a_q| z^-q, so degree d may round in FP32 once the rounding bound
     // of the degrees from d on (as for tab.dci, whose weight is one) times the
     // pair's larger weight stays below kRoundBudget eps.
+    int nb = 0, dcs = 0, nlow_max = 0;
     {
         const int nc = T.deg + 1;
-        std::vector<double> colsum(nc, 0.0);
-        for (int i = 0; i < T.w; ++i)
-            for (int d = 0; d < nc; ++d) colsum[d] += std::fabs(T.ch[(size_t)i * nc + d]);
-        for (ProbParams& pp : probs)
+        std::vector<double> colsum(nc, 0.0), tailmax(nc + 1, 0.0);
+        for (int i = 0; i < T.w; ++i) {
+            double sum = 0.0;
+            for (int d = nc - 1; d >= 0; --d) {
+                sum += std::fabs(T.ch[(size_t)i * nc + d]);
+                colsum[d] += std::fabs(T.ch[(size_t)i * nc + d]);
+                tailmax[d] = std::max(tailmax[d], sum);
+            }
+        }
+        // partial sums of a moment: at most ceil(tile / 8) points and the degrees' sum
+        const int chain = (std::max(P->spread_threads, P->interp_threads) + 7) / 8 + 3 + nc;
+        // Chebyshev terms kept (tail below 1e-3 eps), and those of the spreading
+        // moments in double-float: FP32 ones accumulate over at most ceil(tile / 8)
+        // points each, with rounding below kRoundBudget eps
+        nb = nc;
+        while (nb > 2 && tailmax[nb - 1] <= 1e-3 * P->eps) --nb;
+        dcs = nb;
+        const int terms = (P->spread_threads + 7) / 8 + 3 + nb;
+        while (dcs > 2 && tailmax[dcs - 1] * terms * 1.1920928955078125e-07 <= kRoundBudget * P->eps) --dcs;
+        dcs = std::min((dcs + 1) & ~1, (nb + 1) & ~1);
+        for (ProbParams& pp : probs) {
+            int dsp[kMaxQ / 2];
             for (int pr = 0; pr < kMaxQ / 2; ++pr) {
                 double wmax = 0.0;
                 for (int q = 2 * pr; q < 2 * pr + 2 && q < pp.Q; ++q)
@@ -886,7 +925,15 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
                     if (acc * wmax <= kRoundBudget * P->eps) --d; else break;
                 }
                 pp.dcp[pr] = (int8_t)d;
+                // the spreading moments of degrees >= dsp in FP32 (as tab.dcs,
+                // whose weight is one)
+                int ds = nc;
+                while (ds > 0 && tailmax[ds - 1] * wmax * chain * 1.1920928955078125e-07 <= kRoundBudget * P->eps) --ds;
+                dsp[pr] = ds;
             }
+            list_moment_items(pp, dsp, nb, dcs);
+            nlow_max = std::max(nlow_max, (int)pp.nlow);
+        }
     }
     for (ProbParams& q : probs) q.tw2 = (const float4*)(D + a_tw2);
     put(a_prob, probs.data(), sizeof(ProbParams) * probs.size());
@@ -958,30 +1005,17 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
         }
         if (tail * 1.1920928955078125e-07 <= kRoundBudget * P->eps) tb.deg_comp = k; else break;
     }
-    // Chebyshev form of the taps (moment paths): nb terms, dropping a tail
-    // below 1e-3 eps; degrees >= dcs of the spreading moments accumulate in
-    // FP32 over at most ceil(tile / 8) points each, degrees >= dci of the
-    // interpolation sum in FP32, both with rounding below kRoundBudget eps.
+    // Chebyshev form of the taps (moment paths): degrees >= dci of the
+    // interpolation sum in FP32 with rounding below kRoundBudget eps.
     tb.ch2 = (const float2*)(D + a_ch2);
     {
         const int nc = T.deg + 1;
-        std::vector<double> tailmax(nc + 1, 0.0), colsum(nc, 0.0);
-        for (int i = 0; i < T.w; ++i) {
-            double sum = 0.0;
-            for (int d = nc - 1; d >= 0; --d) {
-                const double a = std::fabs(T.ch[(size_t)i * nc + d]);
-                sum += a;
-                colsum[d] += a;
-                tailmax[d] = sum > tailmax[d] ? sum : tailmax[d];
-            }
-        }
-        int nb = nc;
-        while (nb > 2 && tailmax[nb - 1] <= 1e-3 * P->eps) --nb;
+        std::vector<double> colsum(nc, 0.0);
+        for (int i = 0; i < T.w; ++i)
+            for (int d = 0; d < nc; ++d) colsum[d] += std::fabs(T.ch[(size_t)i * nc + d]);
         tb.nb = nb;
-        const int nsub = (P->spread_threads + 7) / 8;
-        int dcs = nb;
-        while (dcs > 2 && tailmax[dcs - 1] * (nsub + nb) * 1.1920928955078125e-07 <= kRoundBudget * P->eps) --dcs;
         tb.dcs = dcs;
+        tb.nlow = nlow_max;
         int dci = nb;
         double acc = 0.0;
         while (dci > 2) {
@@ -989,6 +1023,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
             if (acc <= kRoundBudget * P->eps) --dci; else break;
         }
         tb.dci = dci;
+        tb.anchored = P->eps >= kAnchorMinEps;
         // q-folded spreading: the weights' Chebyshev terms are kept down to
         // 1e-3 eps; a term above kRoundBudget eps / ((kMomFold + 2) 2^-23) multiplies
         // moments whose FP32 partial sums (kMomFold points) would show, so
