@@ -611,21 +611,22 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const double* __restri
 // out[u] (+)= sum_v y_u (gs[k] + gs[mb + k]) / 2 back at the input's scale, u = perm[k]:
 // the two problems' sums (orders nu - 1 and nu + 1, the second negated) give
 // J_nu' = (J_{nu-1} - J_{nu+1}) / 2 (DLMF 10.6.1); vectors after the first add on.
+// With one problem (nrep = 1) its sums are the derivative.
 __global__ void __launch_bounds__(kSortThreads) k_scatter_deriv(const double* __restrict__ gs,
                                                                 const int32_t* __restrict__ perm, int64_t mb,
-                                                                int stride, int comp, int G,
+                                                                int nrep, int stride, int comp, int G,
                                                                 const unsigned long long* __restrict__ mx,
                                                                 const double* __restrict__ y,
                                                                 double* __restrict__ out)
 {
-    const int e = input_exponent(*mx) - 1;
+    const int e = input_exponent(*mx) - (nrep == 2 ? 1 : 0);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < mb;
          k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t u = perm[k];
         double sum = comp == 0 ? 0.0 : out[u];
         for (int v = 0; v < G; ++v) {
-            const double* gv = gs + v * 2 * mb;
-            const double x = scalbn(gv[k] + gv[mb + k], e) * y[u * stride + comp + v];
+            const double* gv = gs + v * nrep * mb;
+            const double x = scalbn(nrep == 2 ? gv[k] + gv[mb + k] : gv[k], e) * y[u * stride + comp + v];
             sum = comp + v == 0 ? x : sum + x;
         }
         out[u] = sum;
@@ -837,11 +838,12 @@ cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int64
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int stride, int comp, int G,
+cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int nrep, int stride, int comp, int G,
                                  const unsigned long long* mx, const double* y, double* out, cudaStream_t s)
 {
     if (mb <= 0) return cudaSuccess;
-    k_scatter_deriv<<<grid_for(mb, kSortThreads), kSortThreads, 0, s>>>(gs, perm, mb, stride, comp, G, mx, y, out);
+    k_scatter_deriv<<<grid_for(mb, kSortThreads), kSortThreads, 0, s>>>(gs, perm, mb, nrep, stride, comp, G, mx, y,
+                                                                        out);
     count_launches(1);
     return cudaGetLastError();
 }

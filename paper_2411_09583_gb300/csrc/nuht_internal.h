@@ -344,12 +344,12 @@ cudaError_t launch_prepare(const ZeroList& Z, const double* x, int64_t count, co
                            int comps, unsigned long long* part, int* parts, cudaStream_t s);
 cudaError_t launch_fx_decode(const void* src, double* dst, int64_t count, const ProbParams* probs, cudaStream_t s);
 // Components comp .. comp + G - 1 between user and sorted order (k_sort.cu).
-// ws (derivative plans, else null): the weighted input, n = 2 nb, into both
-// problems' copies; launch_scatter_deriv the half difference times y.
+// ws (derivative plans, else null): the weighted input, n = nb or 2 nb, into the
+// problems' copies; launch_scatter_deriv the (half) difference times y.
 cudaError_t launch_gather(const double* c, const int32_t* perm, int64_t n, int64_t nb, const double* ws, int stride,
                           int comp, int G, const unsigned long long* part, int parts, unsigned long long* mx,
                           double* out, float2* out2, cudaStream_t s);
-cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int stride, int comp, int G,
+cudaError_t launch_scatter_deriv(const double* gs, const int32_t* perm, int64_t mb, int nrep, int stride, int comp, int G,
                                  const unsigned long long* mx, const double* y, double* out, cudaStream_t s);
 cudaError_t launch_scatter(const double* gs, const int32_t* perm, int64_t m, int stride, int comp, int G,
                            const unsigned long long* mx, double* g, cudaStream_t s);

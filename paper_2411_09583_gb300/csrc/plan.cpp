@@ -53,7 +53,8 @@ struct nuht_plan_s {
     int nu_user = 0;
     // derivative plan (nuht_plan_deriv): problems nu - 1 and nu + 1 (the
     // second with its sign flipped) over two copies of the base plan's sorted
-    // points and frequencies; n_base, m_base are the base plan's sizes
+    // points and frequencies, or for nu = 0, where J_0' = -J_1, one problem of
+    // order 1 (its sign flipped); n_base, m_base are the base plan's sizes
     bool deriv = false;
     int64_t n_base = 0, m_base = 0;
     double eps = 0.0;
@@ -1613,15 +1614,21 @@ int nuht_plan_deriv(nuht_plan_t* out, nuht_plan_t base, void* stream)
     P->nu_user = nu;
     P->eps = base->eps;
     P->opt = base->opt;
-    P->n = 2 * base->n;
-    P->m = 2 * base->m;
+    // J_nu' = (J_{nu-1} - J_{nu+1}) / 2, and J_{-1} = -J_1: at nu = 0 both terms
+    // are the same transform, run once (half the work: n = m = 1e6, eps 1e-10,
+    // one gradient 6.4 -> 3.3 ms)
+    const size_t nprob = nu == 0 ? 1 : 2;
+    P->n = (int64_t)nprob * base->n;
+    P->m = (int64_t)nprob * base->m;
     P->stream = (cudaStream_t)stream;
-    P->probs.resize(2);
-    int rc = init_problem(P->probs[0], nu - 1, P->eps, P->opt.m_terms, base->n, base->m, 0, 0);
+    P->probs.resize(nprob);
+    int rc = NUHT_OK;
+    if (nprob == 2) rc = init_problem(P->probs[0], nu - 1, P->eps, P->opt.m_terms, base->n, base->m, 0, 0);
     if (rc == NUHT_OK)
-        rc = init_problem(P->probs[1], nu + 1, P->eps, P->opt.m_terms, base->n, base->m, base->n, base->m);
+        rc = init_problem(P->probs[nprob - 1], nu + 1, P->eps, P->opt.m_terms, base->n, base->m,
+                          P->n - base->n, P->m - base->m);
     if (rc != NUHT_OK) { delete P; return rc; }
-    P->probs[1].sgn = -P->probs[1].sgn;   // its sums enter with -J_{nu+1}
+    P->probs[nprob - 1].sgn = -P->probs[nprob - 1].sgn;   // its sums enter with -J_{nu+1}
     P->w = nufft_width(P->eps);
     rc = build_plan(P, nullptr, nullptr, base);
     if (rc != NUHT_OK) { nuht_destroy(P); return rc; }
@@ -1649,11 +1656,11 @@ int nuht_grad_omega(nuht_plan_t D, const double* c, const double* e, double* gra
                                   first ? &parts : nullptr, s);
         },
         [&](int cp, int ng) {
-            return launch_gather(c, D->d_pr, 2 * nb, nb, D->d_r, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_cs,
+            return launch_gather(c, D->d_pr, D->n, nb, D->d_r, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_cs,
                                  D->d_cs2, s);
         },
         [&](int cp, int ng) {
-            return launch_scatter_deriv(D->d_gs, D->d_pw, mb, nvec, cp, ng, D->d_mx, e, grad_omega, s);
+            return launch_scatter_deriv(D->d_gs, D->d_pw, mb, (int)D->probs.size(), nvec, cp, ng, D->d_mx, e, grad_omega, s);
         });
 }
 
@@ -1677,11 +1684,11 @@ int nuht_grad_r(nuht_plan_t D, const double* c, const double* e, double* grad_r,
                                   first ? &parts : nullptr, s);
         },
         [&](int cp, int ng) {
-            return launch_gather(e, D->d_pw, 2 * mb, mb, D->d_w, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_gs,
+            return launch_gather(e, D->d_pw, D->m, mb, D->d_w, nvec, cp, ng, D->d_part, parts, D->d_mx, D->d_gs,
                                  nullptr, s);
         },
         [&](int cp, int ng) {
-            return launch_scatter_deriv(D->d_cs, D->d_pr, nb, nvec, cp, ng, D->d_mx, c, grad_r, s);
+            return launch_scatter_deriv(D->d_cs, D->d_pr, nb, (int)D->probs.size(), nvec, cp, ng, D->d_mx, c, grad_r, s);
         });
 }
 
