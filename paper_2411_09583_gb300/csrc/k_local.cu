@@ -418,9 +418,105 @@ __device__ __forceinline__ void series_sum_nu0(df y, int L, const float2* mu, co
     *sumb = Ab;
 }
 
-// One thread per row of a local block.  J_0..J_ntop(x/2) by Miller's backward
-// recurrence, kept (unnormalised) in this thread's column of shared memory,
-// then sum_l C_l mu_l divided by the square of the normalisation.  With momb
+// nu > 0: sum_l C_l mu_l while Miller's backward recurrence produces the J_n.
+// The two orders of C_l = J_{hp+l} J_{|hm-l|}, hp + hm = nu, add up to nu
+// (l <= hm) or differ by nu (l > hm), so J_n meets its partners J_{n+nu} and
+// J_{nu-n} among the last nu + 1 values: those are kept in a ring of
+// min(nu, ntop) + 1 slots (J_n in slot n modulo the ring's size) of this
+// thread's column instead of all ntop + 1 -- at nu = 18, L = 65 that is 19
+// columns instead of 75, and ten CTAs of an SM instead of two (256 problems of
+// orders 0..20: evaluation 3.44 -> 1.97 ms).  Steps, start
+// and rescaling as in miller_store_df; a rescale by 2^-20 scales the sums by
+// 2^-40.  Returns S.
+__device__ __forceinline__ int ring_slots(int nu, int ntop) { return (nu < ntop ? nu : ntop) + 1; }
+
+__device__ __forceinline__ void ring_term(acc2* sum, acc2* sumb, bool two, df a, float2 b, float2 mu, const float2* mub)
+{
+    // the product stays an unevaluated (hi, lo) pair
+    const float p = a.h * b.x;
+    const float e = fmaf(a.l, b.x, fmaf(a.h, b.y, fmaf(a.h, b.x, -p)));
+    acc_fma(*sum, df{p, e}, df{mu.x, mu.y});
+    if (two) acc_fma(*sumb, df{p, e}, df{mub->x, mub->y});
+}
+
+__device__ __forceinline__ df miller_sum_ring(df y, int nu, int hp, int hm, int L, int ns, const float2* mu,
+                                              const float2* mub, bool two, float2* jb, int nt, int tid, acc2* sum,
+                                              acc2* sumb)
+{
+    const int ntop = hp + L, R = ring_slots(nu, ntop);
+    const df iy = df_recip(y);
+    const float ih = 2.f * iy.h, il = 2.f * iy.l;   // 2 / y
+    float f1, f0, fS;
+    const int i0 = miller_fp32_head(ns, miller_fp32_floor(ntop, y.h), ih, &f1, &f0, &fS);
+    const float s0 = ldexpf(1.f, -ilogbf(f0));
+    float jh = f0 * s0, jl = 0.f, ph = f1 * s0, pl = 0.f;
+    acc2 S{fS * s0, 0.f};
+    acc2 A{0.f, 0.f}, Ab{0.f, 0.f};
+    int slot = -1;   // of the last stored value (i0 > ntop, so every order up to ntop is stored)
+    auto take = [&](int n) {
+        if (n > ntop) return;
+        slot = slot < 0 ? n % R : (slot == 0 ? R - 1 : slot - 1);
+        jb[slot * nt + tid] = make_float2(jh, jl);
+        const int l1 = hm + n, l0 = hm - n;
+        if (n >= 1 && l1 <= L)   // J_{n+nu}, in the slot the next value takes
+            ring_term(&A, &Ab, two, df{jh, jl}, jb[(slot == 0 ? R - 1 : slot - 1) * nt + tid], mu[l1], mub + l1);
+        if (l0 >= 0 && l0 <= L)
+            ring_term(&A, &Ab, two, df{jh, jl}, jb[(nu - n) * nt + tid], mu[l0], mub + l0);
+    };
+    for (int i = i0; i >= 2; i -= 2) {
+        miller_step(i, ih, il, jh, jl, ph, pl);
+        take(i - 1);
+        miller_step(i - 1, ih, il, jh, jl, ph, pl);
+        take(i - 2);
+        float s2, e2;
+        two_sum(S.s, 2.f * jh, s2, e2);
+        S.s = s2;
+        S.c += e2 + 2.f * jl;
+        if (fabsf(jh) > 1048576.f) {
+            const float sc = 9.5367431640625e-07f;    // 2^-20
+            const float sc2 = 9.094947017729282e-13f; // 2^-40
+            jh *= sc; jl *= sc; ph *= sc; pl *= sc; S.s *= sc; S.c *= sc;
+            A.s *= sc2; A.c *= sc2; Ab.s *= sc2; Ab.c *= sc2;
+            // (slots not written yet hold anything; they are written before they are read)
+            for (int q = 0; slot >= 0 && q < R; ++q) {
+                const float2 v = jb[q * nt + tid];
+                jb[q * nt + tid] = make_float2(v.x * sc, v.y * sc);
+            }
+        }
+    }
+    *sum = A;
+    *sumb = Ab;
+    // J_0 was added with weight 2; it counts once
+    float s2, e2;
+    two_sum(S.s, -jh, s2, e2);
+    return fast_two_sum(s2, S.c + e2 - jl);
+}
+
+// nu > 0, y < 1: the same sums from the power series values (normalised),
+// orders ascending: J_n meets J_{|nu-n|}, one of the last nu + 1 values.
+__device__ __forceinline__ void series_sum_ring(df y, int nu, int hp, int L, const float2* mu, const float2* mub,
+                                                bool two, float2* jb, int nt, int tid, acc2* sum, acc2* sumb)
+{
+    const int ntop = hp + L, R = ring_slots(nu, ntop);
+    const df h{0.5f * y.h, 0.5f * y.l};
+    const df q = df_neg(df_mul(h, h));
+    df lead{1.f, 0.f};   // (y/2)^n / n!
+    acc2 A{0.f, 0.f}, Ab{0.f, 0.f};
+    for (int n = 0; n <= ntop; ++n) {
+        if (n > 0) lead = df_mul(df_mul(lead, h), df_inv_int(n));
+        if (lead.h == 0.f) break;   // every later term has a vanishing factor
+        const df v = jn_series_sum(n, lead, q);
+        jb[(n % R) * nt + tid] = make_float2(v.h, v.l);
+        const int l = n - hp, b = nu > n ? nu - n : n - nu;
+        if (l >= 0) ring_term(&A, &Ab, two, v, jb[(b % R) * nt + tid], mu[l], mub + l);
+    }
+    *sum = A;
+    *sumb = Ab;
+}
+
+// One thread per row of a local block: sum_l C_l mu_l, formed while Miller's
+// backward recurrence produces J_0..J_ntop(x/2) (unnormalised), divided by the
+// square of the normalisation.  With momb
 // (the moments of a second real component) the same C_l also give
 // sum_l C_l mub_l into g_sb.
 // coherent: read the moments past L1 (they were just written by other CTAs
@@ -438,7 +534,7 @@ __device__ __forceinline__ void local_eval_tile(const ProbParams* __restrict__ p
     const bool two = momb != nullptr;
     float2* mu = sm2;                 // [L + 1] moments of this block, double-float
     float2* mub = sm2 + (P.ntop + 1); // [L + 1] the second component's (two)
-    float2* jb = sm2 + (two ? 2 : 1) * (P.ntop + 1);  // [ntop + 1][nt]
+    float2* jb = sm2 + (two ? 2 : 1) * (P.ntop + 1);  // [ring_slots][nt] (nu > 0)
     const int hp = (nu & 1) ? (nu + 1) / 2 : nu / 2;   // index paired with +l
     const int hm = (nu & 1) ? (nu - 1) / 2 : nu / 2;   // index paired with -l
     // the moments times the sign and weight of their term: C_l = sgn_l J_{hp+l} J_{|hm-l|},
@@ -479,25 +575,13 @@ __device__ __forceinline__ void local_eval_tile(const ProbParams* __restrict__ p
             else
                 series_sum_nu0(ydf, L, mu, mub, two, &sum, &sumb);
         } else if (ydf.h >= 1.f) {
-            S = miller_store_df(ydf, ntop, ns, jb, nt, tid);
+            S = miller_sum_ring(ydf, nu, hp, hm, L, ns, mu, mub, two, jb, nt, tid, &sum, &sumb);
         } else {
-            S = series_store_df(ydf, ntop, jb, nt, tid);
+            series_sum_ring(ydf, nu, hp, L, mu, mub, two, jb, nt, tid, &sum, &sumb);
         }
-        // The stored values stay below 2^36 and the signed moments below 2^33
-        // (inputs scaled below 2, at most 2^31 points), so the products
-        // J_a J_b mu_l (each an unevaluated (hi, lo) pair) and their sums stay
-        // inside the FP32 range; S^2 is divided out at the end.
-        if (nu != 0) {
-            for (int l = 0; l <= L; ++l) {
-                const int b = hm - l;
-                const float2 va = jb[(hp + l) * nt + tid];
-                const float2 vb = jb[(b >= 0 ? b : -b) * nt + tid];
-                const float p = va.x * vb.x;
-                const float e = fmaf(va.y, vb.x, fmaf(va.x, vb.y, fmaf(va.x, vb.x, -p)));
-                acc_fma(sum, df{p, e}, df{mu[l].x, mu[l].y});
-                if (two) acc_fma(sumb, df{p, e}, df{mub[l].x, mub[l].y});
-            }
-        }
+        // The values stay below 2^36 and the signed moments below 2^33 (inputs
+        // scaled below 2, at most 2^31 points), so the products J_a J_b mu_l and
+        // their sums stay inside the FP32 range; S^2 is divided out at the end.
         const df iS = df_recip(S);
         val = df_to(df_mul(df_mul(fast_two_sum(sum.s, sum.c), iS), iS));
         if (two) valb = df_to(df_mul(df_mul(fast_two_sum(sumb.s, sumb.c), iS), iS));
@@ -1798,14 +1882,14 @@ int local_eval_threads(int ntop_max)
 }
 
 cudaError_t launch_local_eval(const ProbParams* probs, const LocalBlock* blks, const Tile* tiles,
-                                   int ntiles, int ntop_max, bool column, int threads, const float2* w2,
+                                   int ntiles, int ntop_max, int nu_max, int threads, const float2* w2,
                                    const double* mom, double* g_s, const double* momb, double* g_sb,
                                    cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
     const size_t nmu = momb ? 2 : 1;
     // rows of order 0 keep no Bessel column (their sums are formed during the sweep)
-    const size_t col = column ? (size_t)(ntop_max + 1) * threads : 0;
+    const size_t col = nu_max > 0 ? (size_t)(std::min(nu_max, ntop_max) + 1) * threads : 0;
     size_t smem = sizeof(float2) * (col + nmu * (size_t)(ntop_max + 1));
     cudaError_t e = cudaFuncSetAttribute(k_local_eval, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);

@@ -1286,7 +1286,7 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
                                           P->eval_threads, P->d_w2, P->d_mom, gs, momb, gsb, ls));
         else
             NUHT_CK(launch_local_eval(P->d_prob, P->d_loc, P->d_teval, P->n_teval, P->ntop_max,
-                                      P->nu_max > 0, P->eval_threads, P->d_w2, P->d_mom, gs, momb, gsb, ls));
+                                      P->nu_max, P->eval_threads, P->d_w2, P->d_mom, gs, momb, gsb, ls));
         NUHT_TRY(T.end(NUHT_STAGE_LOCAL_EVAL, ls));
     }
     if (dir) {
