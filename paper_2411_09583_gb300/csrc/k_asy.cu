@@ -1122,6 +1122,19 @@ __global__ void __launch_bounds__(256, 3) k_asy_spread(const ProbParams* __restr
 constexpr int kInterpHBytesPerThread = 128;
 constexpr int kAdjInterpHBytes = kInterpHBytesPerThread * kAdjInterpThreads;
 
+// Cells of a sparse tile's window, rows of ws float4: it may run over the
+// taps' coefficients and the room of the per-bin sums (hbytes) behind a dense
+// tile's window, since the taps are formed before it is filled.
+// Reading a cell's 2M terms from L2 once per output and tap bounds a tile that
+// cannot stage its window; with 64 cells most tiles of a far field (about one
+// output per two cells) could not: interpolation of 4e6 outputs, eps 1e-8,
+// 1.71 -> 1.16 ms, 16 members of 1.2e5 outputs 1.48 -> 1.38 ms.
+__device__ __forceinline__ int sparse_win_cells(int Q, int ws, int w, int deg, int hbytes)
+{
+    const int bytes = (int)(sizeof(float4) * kWinCells * Q + sizeof(float2) * ((w * (deg + 1) + 1) & ~1)) + hbytes;
+    return bytes / (int)(sizeof(float4) * ws);
+}
+
 // Shared memory (bytes) of k_asy_interp for 2M = qmax.
 __host__ __device__ __forceinline__ size_t interp_smem(int qmax, int w, int deg, int threads,
                                                       int hbytes)
@@ -1339,7 +1352,7 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
     Tables tab, const double* __restrict__ w_s, const float2* __restrict__ w2, const float4* __restrict__ grid_q,
     int64_t gq_stride, int V, double* __restrict__ g_s, int64_t g_stride)
 {
-    extern __shared__ float4 win[];          // [kWinCells][Q] grid cells of this tile
+    extern __shared__ float4 win[];          // [kWinCells][ws] grid cells of this tile
     const Tile t = tiles[blockIdx.x];
     const AsyBlock B = blks[t.blk];
     const ProbParams& P = probs[B.prob];
@@ -1365,9 +1378,12 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
     const int nbins = t0s[t.count - 1] - wstart + 1;
     const int wlen = nbins - 1 + w;
     const int mask = B.nf2 - 1;
-    const bool staged = wlen <= kWinCells;
     const int maxbins = hbytes / (int)(sizeof(float2) * hs);
-    const bool mom = staged && nbins <= maxbins && t.count >= kMomMinPerBin * nbins;
+    const bool mom = wlen <= kWinCells && nbins <= maxbins && t.count >= kMomMinPerBin * nbins;
+    // the rows of a dense tile's window are read by lanes of one bin, those of a
+    // sparse tile's by lanes in different cells: an odd stride keeps these apart
+    const int ws = mom ? Q : Q | 1;
+    const bool staged = mom || wlen <= sparse_win_cells(Q, ws, w, deg, hbytes);
     if (mom) {
         for (int i = threadIdx.x; i < w * nb; i += blockDim.x) {
             const int r = i / nb, d = i - r * nb;
@@ -1403,11 +1419,14 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
     const df cph{P.cphi2.x, P.cphi2.y}, sph{P.sphi2.x, P.sphi2.y};
     for (int vm = 0; vm < V; ++vm) {
         const float4* gq = grid_q + vm * gq_stride + B.q_off;
-        if (vm > 0) __syncthreads();   // the previous member's reads of the window and H are done
+        // the previous member's reads of the window and H are done, and the taps are
+        // formed before a sparse tile's window takes their coefficients' place
+        if (vm > 0 || !mom) __syncthreads();
         if (staged) {
             for (int idx = threadIdx.x; idx < wlen * Q; idx += blockDim.x) {
                 const int cc = idx / Q;
-                win[idx] = gq[(int64_t)((wstart + cc) & mask) * Q + (idx - cc * Q)];
+                const int q = idx - cc * Q;
+                win[cc * ws + q] = gq[(int64_t)((wstart + cc) & mask) * Q + q];
             }
         }
         __syncthreads();
@@ -1447,7 +1466,7 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
             bin_sums_eval(Hb, u, nb, dci, Q, qs, P.dcp, combine);
         else
             tap_sums_eval(u, w, Q, qs, [&](int i, int q) {
-                return staged ? win[(t0 + i - wstart) * Q + q] : gq[(int64_t)((t0 + i) & mask) * Q + q];
+                return staged ? win[(t0 + i - wstart) * ws + q] : gq[(int64_t)((t0 + i) & mask) * Q + q];
             }, combine);
         // Re(e^{i (omega r_c + phi)} T) = Re(e^{i omega r_c} (e^{i phi} T))
         const df tre = fast_two_sum(tr.s, tr.c), tim = fast_two_sum(ti.s, ti.c);
@@ -1674,7 +1693,7 @@ __global__ void __launch_bounds__(kAdjInterpThreads) k_asy_adj_interp(
     Tables tab, const double* __restrict__ r_s, const float4* __restrict__ bgrid, int64_t bg_stride, int V,
     double* __restrict__ c_s, int64_t c_stride)
 {
-    extern __shared__ float4 win[];          // [kWinCells][Q] modes of this pass
+    extern __shared__ float4 win[];          // [kWinCells][ws] modes of this pass
     const Tile t = tiles[blockIdx.x];
     const AsyBlock B = blks[t.blk];
     const ProbParams& P = probs[B.prob];
@@ -1702,8 +1721,9 @@ __global__ void __launch_bounds__(kAdjInterpThreads) k_asy_adj_interp(
         const int wstart = l0s[0];
         const int nbins = l0s[cnt - 1] - wstart + 1;
         const int wlen = nbins - 1 + w;
-        const bool staged = wlen <= kWinCells;
-        const bool mom = staged && nbins <= maxbins && cnt >= kMomMinPerBin * nbins;
+        const bool mom = wlen <= kWinCells && nbins <= maxbins && cnt >= kMomMinPerBin * nbins;
+        const int ws = mom ? Q : Q | 1;   // as in k_asy_interp
+        const bool staged = mom || wlen <= sparse_win_cells(Q, ws, w, deg, kAdjInterpHBytes);
         if (mom) {
             for (int i = threadIdx.x; i < w * nb; i += blockDim.x) {
                 const int r = i / nb, d = i - r * nb;
@@ -1731,13 +1751,15 @@ __global__ void __launch_bounds__(kAdjInterpThreads) k_asy_adj_interp(
         }
         for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
             const float4* gb = bgrid + vm * bg_stride + B.b_off;
-            if (vm > 0) __syncthreads();   // the previous member's reads of the window and H are done
+            // as in k_asy_interp
+            if (vm > 0 || !mom) __syncthreads();
             if (staged)
                 for (int idx = threadIdx.x; idx < wlen * Q; idx += blockDim.x) {
                     const int cc = idx / Q;
                     const int li = wstart + cc + B.N1;
-                    win[idx] = (li >= 0 && li < nf1) ? gb[(int64_t)li * Q + (idx - cc * Q)]
-                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int q = idx - cc * Q;
+                    win[cc * ws + q] = (li >= 0 && li < nf1) ? gb[(int64_t)li * Q + q]
+                                                             : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             __syncthreads();
             if (mom) {
@@ -1758,7 +1780,7 @@ __global__ void __launch_bounds__(kAdjInterpThreads) k_asy_adj_interp(
             else
                 tap_sums_eval(u, w, Q, qs, [&](int i, int q) {
                     const int li = l0 + i + B.N1;
-                    if (staged) return win[(l0 + i - wstart) * Q + q];
+                    if (staged) return win[(l0 + i - wstart) * ws + q];
                     return (li >= 0 && li < nf1) ? gb[(int64_t)li * Q + q] : make_float4(0.f, 0.f, 0.f, 0.f);
                 }, combine);
             // c_j += Re( e^{i w_c x} (r/rho)^(-1/2) T )
