@@ -872,12 +872,79 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
     }
 }
 
+// Sums of a sparse tile: output (cell first + c, q), c < span, is the sum over
+// the rows p whose taps cover the cell (l0[p] <= cell < l0[p] + w, ascending
+// l0) of taps[p][cell - l0[p]] vals[p][q], handed to put(cell, q, re, im).
+// One lane per output, or two (halves of its rows) where a pass has fewer
+// outputs than half the threads.  start[x], the first row with l0 >= first
+// cell of the pass - (w - 1) + x, gives a cell's rows as [start[c], start[c +
+// w]); it has room for cap cells and w more.  With build it is formed (cells
+// ready at a barrier), else it stands from the previous member.
+// FP32 issue and shared reads of the products bound it.  Two binary searches per
+// lane and output and the FP64 (1/64 rate) halves of every output cost more than
+// the products before: 4e6 far-field points (eps 1e-12, half a point a cell) 1.80 ->
+// 1.05 ms, 256 problems of 3e2 to 1e5 points 5.3 -> 4.7 ms.
+template <class Put>
+__device__ __forceinline__ void tap_cell_sums(const int* l0s, int cnt, int first, int span, int w, int Q,
+                                              const float2* taps, const float4* vals, uint16_t* start, int cap,
+                                              bool build, Put&& put)
+{
+    const int nt = blockDim.x, tid = threadIdx.x;
+    const unsigned qinv = 0xffffffffu / (unsigned)Q + 1;   // item / Q, exact while nout Q < 2^32 (Q >= 2)
+    for (int c0 = 0; c0 < span; c0 += cap) {
+        const int nc = min(cap, span - c0);
+        if (build || span > cap) {
+            if (c0 > 0 || !build) __syncthreads();   // the last pass's reads of start are done
+            for (int x = tid; x < nc + w; x += nt) {
+                const int key = first + c0 - (w - 1) + x;
+                int lo = 0, hi = cnt;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (l0s[mid] < key) lo = mid + 1; else hi = mid;
+                }
+                start[x] = (uint16_t)lo;
+            }
+            __syncthreads();
+        }
+        const int nout = nc * Q;
+        const int sh = 2 * nout <= nt ? 1 : 0;
+        const int sub = tid & sh;
+        for (int item = tid >> sh; item < nout; item += nt >> sh) {
+            const int c = (int)__umulhi((unsigned)item, qinv), q = item - c * Q;
+            int p = start[c], hi = start[c + w];
+            const bool any = p < hi;
+            if (sh) {
+                const int mid = (p + hi + 1) >> 1;
+                if (sub) p = mid; else hi = mid;
+            }
+            const int cell = first + c0 + c;
+            acc2 ar{0.f, 0.f}, ai{0.f, 0.f};
+            for (; p < hi; ++p) {
+                const float2 k2 = taps[p * w + (cell - l0s[p])];
+                const float4 av = vals[p * Q + q];
+                acc_fma(ar, df{k2.x, k2.y}, df{av.x, av.y});
+                acc_fma(ai, df{k2.x, k2.y}, df{av.z, av.w});
+            }
+            if (sh) {
+                const unsigned pair = 0x3u << (tid & 30);
+                const acc2 br{__shfl_xor_sync(pair, ar.s, 1), __shfl_xor_sync(pair, ar.c, 1)};
+                const acc2 bi{__shfl_xor_sync(pair, ai.s, 1), __shfl_xor_sync(pair, ai.c, 1)};
+                float e;
+                two_sum(ar.s, br.s, ar.s, e);
+                ar.c += br.c + e;
+                two_sum(ai.s, bi.s, ai.s, e);
+                ai.c += bi.c + e;
+            }
+            if (any && !sub) put(cell, q, acc_value(ar), acc_value(ai));
+        }
+    }
+}
+
 // Sparse tile (points spread over many cells): each thread prepares one point
-// (cell l0, w kernel taps, the 2M weighted, pre-phased values), then each
-// (cell, q) output of the tile's window is owned by one thread, which sums
-// over the points whose taps cover that cell and adds the sum to the block's
-// global grid.  Members as in spread_fold: the taps and phase factors are
-// formed once, the weighted values and the sums per member.
+// (cell l0, w kernel taps, the 2M weighted, pre-phased values), then
+// tap_cell_sums adds each (cell, q) of the tile's window to the block's global
+// grid.  Members as in spread_fold: the taps and phase factors are formed
+// once, the weighted values and the sums per member.
 template <bool MULTI, class Acc>
 __device__ void spread_taps(const AsyBlock& B, int Q, const Tile& t, const Tables& tab,
                             const double* __restrict__ r_s, const float2* __restrict__ r2,
@@ -917,20 +984,6 @@ __device__ void spread_taps(const AsyBlock& B, int Q, const Tile& t, const Table
     const int lfirst = l0s[0];
     const int span = l0s[cnt - 1] - lfirst + w;
     const int nf1 = 2 * B.N1 + 1;
-    // Outputs (cell, q), q fastest.  For a tile whose span of cells is close
-    // to the kernel width every thread walks all the tile's points in
-    // lockstep (one row of taps / values per step: broadcast or contiguous
-    // reads) and skips points whose taps miss its cell; otherwise it
-    // binary-searches the few points that reach its cell.  Each output is
-    // split between kSub lanes (halves of the point range) combined by a
-    // shuffle, so that more threads than outputs can work.
-    constexpr int kSub = 2;
-    const bool dense = span <= 2 * w;
-    const int nout = span * Q;
-    const int lane = tid & 31;
-    const int sub = lane & (kSub - 1);
-    const unsigned gmask = 0x3u << (lane & ~(kSub - 1));
-    const int half = (cnt + 1) >> 1;
     for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
     if (MULTI) {
         if (tid < cnt) {
@@ -945,47 +998,15 @@ __device__ void spread_taps(const AsyBlock& B, int Q, const Tile& t, const Table
         __syncthreads();
     }
     const Acc gv = gb.at(vm * moff);
-    for (int base = tid - sub; base < nout * kSub; base += nt) {
-        const int item = (base + sub) / kSub;   // same item for both lanes of a pair
-        const bool live = item < nout;
-        const int c = live ? item / Q : 0, q = live ? item - c * Q : 0;
-        const int cell = lfirst + c;
-        int p_lo, p_hi;
-        if (dense) {
-            p_lo = sub * half;
-            p_hi = sub ? cnt : half;
-        } else {
-            int lo = 0, hi = cnt;
-            const int key = cell - w + 1;
-            while (lo < hi) { int mid = (lo + hi) >> 1; if (l0s[mid] < key) lo = mid + 1; else hi = mid; }
-            const int plo = lo;
-            hi = cnt;
-            while (lo < hi) { int mid = (lo + hi) >> 1; if (l0s[mid] <= cell) lo = mid + 1; else hi = mid; }
-            const int mid2 = (plo + lo + 1) >> 1;
-            p_lo = sub ? mid2 : plo;
-            p_hi = sub ? lo : mid2;
-        }
-        if (!live) p_hi = p_lo;
-        acc2 ar{0.f, 0.f}, ai{0.f, 0.f};
-        for (int p = p_lo; p < p_hi; ++p) {
-            const int i = cell - l0s[p];
-            if (i >= 0 && i < w) {
-                const float2 k2 = taps[p * w + i];
-                const float4 av = aval[p * Q + q];
-                const df k{k2.x, k2.y};
-                acc_fma(ar, k, df{av.x, av.y});
-                acc_fma(ai, k, df{av.z, av.w});
-            }
-        }
-        double vr = acc_value(ar), vi = acc_value(ai);
-        vr += __shfl_down_sync(gmask, vr, 1, kSub);
-        vi += __shfl_down_sync(gmask, vi, 1, kSub);
+    // the taps are formed: their coefficients' room (4 w (deg + 1) 16-bit words) holds the cells' first rows
+    tap_cell_sums(l0s, cnt, lfirst, span, w, Q, taps, aval, (uint16_t*)coef, w * (4 * deg + 3), vm == 0,
+                  [&](int cell, int q, double vr, double vi) {
         const int idx = cell + B.N1;
-        if (live && sub == 0 && idx >= 0 && idx < nf1 && (vr != 0.0 || vi != 0.0)) {
+        if (idx >= 0 && idx < nf1) {
             gv.add(2 * ((int64_t)idx * Q + q), vr);
             gv.add(2 * ((int64_t)idx * Q + q) + 1, vi);
         }
-    }
+    });
     if (MULTI) __syncthreads();   // aval is rewritten for the next member
     }
 }
@@ -1127,7 +1148,7 @@ constexpr int kAdjInterpHBytes = kInterpHBytesPerThread * kAdjInterpThreads;
 // tile's window, since the taps are formed before it is filled.
 // Reading a cell's 2M terms from L2 once per output and tap bounds a tile that
 // cannot stage its window; with 64 cells most tiles of a far field (about one
-// output per two cells) could not: interpolation of 4e6 outputs, eps 1e-8,
+// output per two cells) could not: interpolation of 4e6 outputs, eps 1e-12,
 // 1.71 -> 1.16 ms, 16 members of 1.2e5 outputs 1.48 -> 1.38 ms.
 __device__ __forceinline__ int sparse_win_cells(int Q, int ws, int w, int deg, int hbytes)
 {
@@ -1631,7 +1652,6 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const 
     __syncthreads();
     const int tfirst = t0s[0];
     const int span = t0s[cnt - 1] - tfirst + w;
-    const bool dense = span <= 2 * w;
     for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
     if (MULTI && vm > 0) {
         __syncthreads();   // the previous member's reads of uval are done
@@ -1642,38 +1662,13 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const 
         __syncthreads();
     }
     const Accum tgv = tg.at(2 * vm * tg_stride);
-    for (int item = tid; item < span * Q; item += nt) {
-        const int c = item / Q, q = item - c * Q;
-        const int cell = tfirst + c;
-        int p_lo = 0, p_hi = cnt;
-        if (!dense) {
-            int lo = 0, hi = cnt;
-            const int key = cell - w + 1;
-            while (lo < hi) { int mid = (lo + hi) >> 1; if (t0s[mid] < key) lo = mid + 1; else hi = mid; }
-            p_lo = lo;
-            hi = cnt;
-            while (lo < hi) { int mid = (lo + hi) >> 1; if (t0s[mid] <= cell) lo = mid + 1; else hi = mid; }
-            p_hi = lo;
-        }
-        acc2 ar{0.f, 0.f}, ai{0.f, 0.f};
-        bool any = false;
-        for (int p = p_lo; p < p_hi; ++p) {
-            const int i = cell - t0s[p];
-            if (i >= 0 && i < w) {
-                const float2 k2 = taps[p * w + i];
-                const float4 uv = uval[p * Q + q];
-                const df kk{k2.x, k2.y};
-                acc_fma(ar, kk, df{uv.x, uv.y});
-                acc_fma(ai, kk, df{uv.z, uv.w});
-                any = true;
-            }
-        }
-        if (any) {
-            const int64_t o = (int64_t)(cell & mask) * Q + q;
-            tgv.add(2 * o, acc_value(ar));
-            tgv.add(2 * o + 1, acc_value(ai));
-        }
-    }
+    // as in spread_taps
+    tap_cell_sums(t0s, cnt, tfirst, span, w, Q, taps, uval, (uint16_t*)coef, w * (4 * deg + 3), vm == 0,
+                  [&](int cell, int q, double vr, double vi) {
+        const int64_t o = (int64_t)(cell & mask) * Q + q;
+        tgv.add(2 * o, vr);
+        tgv.add(2 * o + 1, vi);
+    });
     }
 }
 
