@@ -30,10 +30,35 @@ __device__ __forceinline__ df fast_two_sum(float a, float b)
     return df{s, b - (s - a)};
 }
 
+// x = h + l, h = x rounded to FP32 and l the rest rounded, from the bits of x:
+// the top 24 bits of the significand rounded to nearest even, and the signed
+// remainder of 29 bits.  The three conversions and the subtraction in FP64
+// (below; values whose parts are not both normal FP32 numbers) hold a warp's
+// FP64 pipe, 1/64 of the FP32 rate, for 256 cycles.
 __device__ __forceinline__ df df_from(double x)
 {
-    const float h = (float)x;
-    return df{h, (float)(x - (double)h)};
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7ff) - 1023;
+    if (e < -74 || e > 126) {
+        if (e == -1023) return df{__uint_as_float(hi & 0x80000000u), 0.f};   // zero and subnormals
+        const float h = (float)x;
+        return df{h, (float)(x - (double)h)};
+    }
+    const unsigned top = ((hi & 0xfffffu) << 3) | (lo >> 29);   // without the leading one
+    int rem = (int)(lo & 0x1fffffffu);
+    const unsigned up = rem + (int)(top & 1u) > 0x10000000 ? 1u : 0u;
+    rem -= (int)(up << 29);
+    const float h = __uint_as_float((hi & 0x80000000u) | (((unsigned)(e + 127) << 23) + top + up));
+    const float ulp = __uint_as_float((unsigned)(e + 75) << 23);   // 2^(e - 52)
+    return df{h, (float)((int)hi < 0 ? -rem : rem) * ulp};
+}
+
+// x 2^e, exactly scalbn(x, e): on the exponent bits while both are normal.
+__device__ __forceinline__ double scale_pow2(double x, int e)
+{
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    if (ex == 0 || ex == 0x7ff || ex + e <= 0 || ex + e >= 0x7ff) return scalbn(x, e);
+    return __hiloint2double(hi + e * (1 << 20), __double2loint(x));
 }
 
 __device__ __forceinline__ double df_to(df a) { return (double)a.h + (double)a.l; }

@@ -1536,8 +1536,8 @@ __device__ __forceinline__ int adj_spread_factor(const AsyBlock& B, const ProbPa
     const df cph{P.cphi2.x, P.cphi2.y}, sph{P.sphi2.x, P.sphi2.y};
     const df er = df_add(df_mul(cs, cph), df_negate(df_mul(sn, sph)));
     const df ei = df_add(df_mul(sn, cph), df_mul(cs, sph));
-    const df amp = df_mul(df_mul(df_from((double)P.sgn * tab.interp_const), df_sqrt(m1d)),
-                          df_recip(psihat_fx(tab, B, Sw)));
+    df amp = df_mul(df_mul(df{tab.ic2.x, tab.ic2.y}, df_sqrt(m1d)), df_recip(psihat_fx(tab, B, Sw)));
+    if (P.sgn < 0) amp = df_negate(amp);
     F->fr = df_mul(amp, er);
     F->fi = df_mul(amp, ei);
     return t0;

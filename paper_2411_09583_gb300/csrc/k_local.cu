@@ -65,13 +65,41 @@ __device__ __forceinline__ acc2 warp_sum_acc(acc2 a)
     return a;
 }
 
+// Sums that lane 0 of a warp gets one after another (slot = 0, 1, ..., the same
+// in all lanes), kept one per lane, so that one conversion to FP64 (1/64 of the
+// FP32 rate, as slow for one lane as for 32) and one add serve up to 32 of them.
+struct LaneSums {
+    acc2 v{0.f, 0.f};
+    int at = -1;   // where this lane's sum belongs, -1: none
+    __device__ __forceinline__ void take(int slot, acc2 a, int index)
+    {
+        a.s = __shfl_sync(0xffffffffu, a.s, 0);
+        a.c = __shfl_sync(0xffffffffu, a.c, 0);
+        if ((int)(threadIdx.x & 31) == (slot & 31)) {
+            v = a;
+            at = index;
+        }
+    }
+    // add(index, sum) for the sums held, once 32 are (or all are: last)
+    template <class Add>
+    __device__ __forceinline__ void flush(int slot, bool last, Add&& add)
+    {
+        if (!last && (slot & 31) != 31) return;
+        if (at >= 0) add(at, acc_value(v));
+        at = -1;
+    }
+};
+
 // dst[l] += sum over the CTA's threads of acc[l * nt + thread], l <= L: one
-// warp per l, compensated FP32 sums, one conversion and one FP64 atomic per l
-// (FP64 runs at 1/64 of the FP32 rate).
+// warp per l, compensated FP32 sums, one conversion and one FP64 atomic for
+// up to 32 l.
 __device__ __forceinline__ void reduce_columns_add(const acc2* acc, int nt, int L, Accum dst)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int l = warp; l <= L; l += nw) {
+    LaneSums sums;
+    const auto add = [&](int l, double v) { dst.add(l, v); };
+    int slot = 0;
+    for (int l = warp; l <= L; l += nw, ++slot) {
         acc2 a{0.f, 0.f};
         for (int k = lane; k < nt; k += 32) {
             const acc2 v = acc[l * nt + k];
@@ -80,9 +108,10 @@ __device__ __forceinline__ void reduce_columns_add(const acc2* acc, int nt, int 
             a.s = s;
             a.c += v.c + e;
         }
-        a = warp_sum_acc(a);
-        if (lane == 0) dst.add(l, acc_value(a));
+        sums.take(slot, warp_sum_acc(a), l);
+        sums.flush(slot, false, add);
     }
+    sums.flush(slot, true, add);
 }
 
 // One CTA per tile of columns of one local block.  Each thread keeps its own
@@ -544,12 +573,12 @@ __device__ __forceinline__ void local_eval_tile(const ProbParams* __restrict__ p
         float sgn = (b < 0 && ((-b) & 1)) ? -1.f : 1.f;
         if (l > 0 || (nu & 1)) sgn *= 2.f;
         const double v = coherent ? __ldcg(&mom[B.mom_off + l]) : mom[B.mom_off + l];
-        const float h = (float)v;
-        mu[l] = make_float2(sgn * h, sgn * (float)(v - (double)h));
+        const df m = df_from(v);
+        mu[l] = make_float2(sgn * m.h, sgn * m.l);
         if (two) {
             const double vb = coherent ? __ldcg(&momb[B.mom_off + l]) : momb[B.mom_off + l];
-            const float hb = (float)vb;
-            mub[l] = make_float2(sgn * hb, sgn * (float)(vb - (double)hb));
+            const df mb = df_from(vb);
+            mub[l] = make_float2(sgn * mb.h, sgn * mb.l);
         }
     }
     __syncthreads();
@@ -586,8 +615,8 @@ __device__ __forceinline__ void local_eval_tile(const ProbParams* __restrict__ p
         val = df_to(df_mul(df_mul(fast_two_sum(sum.s, sum.c), iS), iS));
         if (two) valb = df_to(df_mul(df_mul(fast_two_sum(sumb.s, sumb.c), iS), iS));
     }
-    Accum{g_s, P.fxs}.add(k, (double)P.sgn * val);
-    if (two) Accum{g_sb, P.fxs}.add(k, (double)P.sgn * valb);
+    Accum{g_s, P.fxs}.add(k, P.sgn < 0 ? -val : val);
+    if (two) Accum{g_sb, P.fxs}.add(k, P.sgn < 0 ? -valb : valb);
 }
 
 __global__ void k_local_eval(const ProbParams* __restrict__ probs, const LocalBlock* __restrict__ blks,
@@ -987,8 +1016,8 @@ __device__ __forceinline__ DirFx direct_frame(const double* __restrict__ r_s, co
 // multiply: m = ceil(2^32 / d) gives floor(e m / 2^32) = floor(e / d) exactly
 // whenever e d < 2^32 (direct blocks hold at most a few thousand entries).
 struct ColDiv {
-    unsigned long long m;
-    __device__ __forceinline__ explicit ColDiv(int d) : m(((1ull << 32) + (unsigned)d - 1) / (unsigned)d) {}
+    unsigned long long m;   // floor((2^32 - 1) / d) + 1 (a 32-bit division)
+    __device__ __forceinline__ explicit ColDiv(int d) : m((unsigned long long)(0xffffffffu / (unsigned)d) + 1) {}
     __device__ __forceinline__ int operator()(int e) const { return (int)(((unsigned long long)(unsigned)e * m) >> 32); }
 };
 
@@ -1007,7 +1036,7 @@ __device__ __forceinline__ int direct_partition(const ProbParams& P, const Direc
     const int rows = area / cols;
     if (threadIdx.x == 0) { cnt[0] = 0; cnt[1] = 0; }
     __syncthreads();
-    const float zf = (float)P.z;
+    const float zf = P.z2.x;   // z rounded to FP32
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int area_pad = (area + 31) & ~31;
@@ -1108,14 +1137,20 @@ __global__ void k_direct(const ProbParams* __restrict__ probs, const DirectBlock
         // a row's S <= 32 slots summed by one warp, compensated FP32 sums
         // through the shuffles (no FP64 adds: FP64 runs at 1/64 of the rate)
         const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int i = threadIdx.x >> 5; i < rows; i += nw) {
-            const acc2 a = warp_sum_acc(acc2{lane < S ? rowf[i * S + lane] : 0.f, 0.f});
-            if (lane == 0) atomicAdd(&g_s[B.k0 + i], (double)P.sgn * acc_value(a));
+        LaneSums sums, sumsb;
+        const auto add = [&](int i, double v) { atomicAdd(&g_s[B.k0 + i], P.sgn < 0 ? -v : v); };
+        const auto addb = [&](int i, double v) { atomicAdd(&g_sb[B.k0 + i], P.sgn < 0 ? -v : v); };
+        int slot = 0;
+        for (int i = threadIdx.x >> 5; i < rows; i += nw, ++slot) {
+            sums.take(slot, warp_sum_acc(acc2{lane < S ? rowf[i * S + lane] : 0.f, 0.f}), i);
+            sums.flush(slot, false, add);
             if (two) {
-                const acc2 ab = warp_sum_acc(acc2{lane < S ? rowfb[i * S + lane] : 0.f, 0.f});
-                if (lane == 0) atomicAdd(&g_sb[B.k0 + i], (double)P.sgn * acc_value(ab));
+                sumsb.take(slot, warp_sum_acc(acc2{lane < S ? rowfb[i * S + lane] : 0.f, 0.f}), i);
+                sumsb.flush(slot, false, addb);
             }
         }
+        sums.flush(slot, true, add);
+        if (two) sumsb.flush(slot, true, addb);
         return;
     }
     if (det) {
@@ -1173,8 +1208,8 @@ __global__ void k_direct(const ProbParams* __restrict__ probs, const DirectBlock
     }
     __syncthreads();
     for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-        atomicAdd(&g_s[B.k0 + i], (double)P.sgn * rowacc[i]);
-        if (two) atomicAdd(&g_sb[B.k0 + i], (double)P.sgn * rowaccb[i]);
+        atomicAdd(&g_s[B.k0 + i], P.sgn < 0 ? -rowacc[i] : rowacc[i]);
+        if (two) atomicAdd(&g_sb[B.k0 + i], P.sgn < 0 ? -rowaccb[i] : rowaccb[i]);
     }
 }
 
@@ -1218,8 +1253,8 @@ k_local_adj_moments(const ProbParams* __restrict__ probs, const LocalBlock* __re
         const int cnt = t.count - base < nt ? t.count - base : nt;
         if (tid < cnt) {
             const int64_t k = t.start + base + tid;
-            const double gk = (double)P.sgn * g_s[k];
-            const double gkb = TWO ? (double)P.sgn * g_sb[k] : 0.0;
+            const double gk = P.sgn < 0 ? -g_s[k] : g_s[k];
+            const double gkb = !TWO ? 0.0 : P.sgn < 0 ? -g_sb[k] : g_sb[k];
             const float2 wk = w2[k];
             const df ydf = df_mul(df{wk.x, wk.y}, df{0.5f * B.R_h, 0.5f * B.R_l});   // y = omega R / 2
             if (!(ydf.h > 0.f)) {
@@ -1263,7 +1298,11 @@ k_local_adj_moments(const ProbParams* __restrict__ probs, const LocalBlock* __re
                 grb[TWO ? i : 0] = df{gb.x, gb.y};
             }
         }
-        for (int l = warp; l <= L; l += nw) {
+        LaneSums sums, sumsb;
+        const auto add = [&](int l, double v) { Accum{mom, P.fxs}.add(B.mom_off + l, v); };
+        const auto addb = [&](int l, double v) { Accum{momb, P.fxs}.add(B.mom_off + l, v); };
+        int slot = 0;
+        for (int l = warp; l <= L; l += nw, ++slot) {
             const int b = hm - l, bi = b >= 0 ? b : -b;
             float sgn = (b < 0 && (bi & 1)) ? -1.f : 1.f;
             if (l > 0 || (nu & 1)) sgn *= 2.f;
@@ -1280,13 +1319,15 @@ k_local_adj_moments(const ProbParams* __restrict__ probs, const LocalBlock* __re
                     if (TWO) acc_fma(ab, cl, grb[TWO ? i : 0]);
                 }
             }
-            a = warp_sum_acc(a);
-            if (lane == 0) Accum{mom, P.fxs}.add(B.mom_off + l, acc_value(a));
+            sums.take(slot, warp_sum_acc(a), l);
+            sums.flush(slot, false, add);
             if (TWO) {
-                ab = warp_sum_acc(ab);
-                if (lane == 0) Accum{momb, P.fxs}.add(B.mom_off + l, acc_value(ab));
+                sumsb.take(slot, warp_sum_acc(ab), l);
+                sumsb.flush(slot, false, addb);
             }
         }
+        sums.flush(slot, true, add);
+        if (TWO) sumsb.flush(slot, true, addb);
         __syncthreads();   // jb and gsm are rewritten by the next pass
     }
 }
@@ -1304,8 +1345,8 @@ k_local_adj_eval(const ProbParams* __restrict__ probs, const LocalBlock* __restr
     const int nt = blockDim.x, tid = threadIdx.x;
     for (int l = tid; l <= L; l += nt) {
         const double v = mom[B.mom_off + l];
-        const float h = (float)v;
-        mu2[l] = make_float2(h, (float)(v - (double)h));
+        const df m = df_from(v);
+        mu2[l] = make_float2(m.h, m.l);
     }
     __syncthreads();
     const df invR{B.iR_h, B.iR_l};
@@ -1388,7 +1429,7 @@ __global__ void k_direct_adj(const ProbParams* __restrict__ probs, const DirectB
     }
     __syncthreads();
     for (int i = threadIdx.x; i < cols; i += blockDim.x)
-        atomicAdd(&c_s[B.j0 + i], (double)P.sgn * colacc[i]);
+        atomicAdd(&c_s[B.j0 + i], P.sgn < 0 ? -colacc[i] : colacc[i]);
 }
 
 // ------------------------------------------------------------ vector groups
@@ -1520,8 +1561,8 @@ __global__ void k_local_eval_group(const ProbParams* __restrict__ probs, const L
     for (int i = tid; i < (L + 1) * GM; i += nt) {
         const int l = i / GM, v = i - l * GM;
         const double x = v < G ? mom[v * mom_stride + B.mom_off + l] : 0.0;
-        const float h = (float)x;
-        mu[i] = make_float2(h, (float)(x - (double)h));
+        const df m = df_from(x);
+        mu[i] = make_float2(m.h, m.l);
     }
     __syncthreads();
     if (tid >= t.count) return;
@@ -1577,8 +1618,10 @@ __global__ void k_local_eval_group(const ProbParams* __restrict__ probs, const L
         const df iS2 = df_mul(iS, iS);
 #pragma unroll
         for (int v = 0; v < GM; ++v)
-            if (v < G)
-                dst.add(v * g_stride + k, (double)P.sgn * df_to(df_mul(fast_two_sum(sum[v].s, sum[v].c), iS2)));
+            if (v < G) {
+                const df val = df_mul(fast_two_sum(sum[v].s, sum[v].c), iS2);
+                dst.add(v * g_stride + k, df_to(P.sgn < 0 ? df_negate(val) : val));
+            }
     }
 }
 
@@ -1609,9 +1652,8 @@ __global__ void k_direct_group(const ProbParams* __restrict__ probs, const Direc
     for (int t = threadIdx.x; t < area; t += blockDim.x) {
         const int e = list[t];
         const int rr = cdiv(e), cc = e - rr * cols;
-        const double v = direct_entry_fx(P, F, w_s[B.k0 + rr], r_s[B.j0 + cc], t >= nloc, lowp != 0);
-        const float h = (float)v;
-        E[cc * rows + rr] = make_float2(h, (float)(v - (double)h));
+        const df v = direct_entry_df(P, F, w_s[B.k0 + rr], r_s[B.j0 + cc], t >= nloc, lowp != 0);
+        E[cc * rows + rr] = make_float2(v.h, v.l);
     }
     __syncthreads();
     const Accum dst{g_s, P.fxs};
@@ -1623,7 +1665,7 @@ __global__ void k_direct_group(const ProbParams* __restrict__ probs, const Direc
             const float2 ev = E[cc * rows + rr], cf = cv[cc];
             acc_fma(s, df{ev.x, ev.y}, df{cf.x, cf.y});
         }
-        dst.add(v * g_stride + B.k0 + rr, (double)P.sgn * acc_value(s));
+        dst.add(v * g_stride + B.k0 + rr, acc_value(P.sgn < 0 ? acc2{-s.s, -s.c} : s));
     }
 }
 
@@ -1673,7 +1715,11 @@ k_local_adj_moments_group(const ProbParams* __restrict__ probs, const LocalBlock
             }
             p2m[tid] = p2;
             for (int v = 0; v < GM; ++v) {
-                const df gs = v < G ? df_mul(df_from((double)P.sgn * g_s[v * g_stride + k]), iS2) : df{0.f, 0.f};
+                df gs{0.f, 0.f};
+                if (v < G) {
+                    const double gk = g_s[v * g_stride + k];
+                    gs = df_mul(df_from(P.sgn < 0 ? -gk : gk), iS2);
+                }
                 gsm[v * nt + tid] = make_float2(gs.h, gs.l);
             }
         }
@@ -1698,14 +1744,13 @@ k_local_adj_moments_group(const ProbParams* __restrict__ probs, const LocalBlock
                     }
                 }
             }
-            const Accum dst{mom, P.fxs};
+            LaneSums sums;   // of this l, one member per lane
 #pragma unroll
-            for (int v = 0; v < GM; ++v) {
-                if (v < G) {
-                    const acc2 sv = warp_sum_acc(a[v]);
-                    if (lane == 0) dst.add(v * mom_stride + B.mom_off + l, acc_value(sv));
-                }
-            }
+            for (int v = 0; v < GM; ++v)
+                if (v < G) sums.take(v, warp_sum_acc(a[v]), v);
+            sums.flush(0, true, [&](int v, double x) {
+                Accum{mom, P.fxs}.add(v * mom_stride + B.mom_off + l, x);
+            });
         }
         __syncthreads();   // jb and gsm are rewritten by the next pass
     }
@@ -1730,8 +1775,8 @@ k_local_adj_eval_group(const ProbParams* __restrict__ probs, const LocalBlock* _
     for (int i = tid; i < (L + 1) * GM; i += nt) {
         const int l = i / GM, v = i - l * GM;
         const double x = v < G ? mom[v * mom_stride + B.mom_off + l] : 0.0;
-        const float h = (float)x;
-        mu2[i] = make_float2(h, (float)(x - (double)h));
+        const df m = df_from(x);
+        mu2[i] = make_float2(m.h, m.l);
     }
     __syncthreads();
     const df invR{B.iR_h, B.iR_l};

@@ -20,6 +20,7 @@
 // 1e6 and by launch latency below 1e5.
 #include <cstdint>
 
+#include "df64.cuh"
 #include "nuht_internal.h"
 
 namespace nuht {
@@ -272,8 +273,8 @@ __device__ __forceinline__ void sort_put(const SortArray& A, int64_t pos, uint64
     const double v = __longlong_as_double((long long)bits);
     A.out[pos] = v;
     A.perm[pos] = (int32_t)idx;
-    const float h = (float)v;
-    A.split[pos] = make_float2(h, (float)(v - (double)h));
+    const df s = df_from(v);
+    A.split[pos] = make_float2(s.h, s.l);
 }
 
 // Writes the sorted values, their indices and their double-float parts.  An
@@ -583,11 +584,11 @@ __global__ void __launch_bounds__(kSortThreads) k_gather(const double* __restric
         const double* row = c + (int64_t)perm[i0] * stride + comp;
         const double wt = ws ? ws[i0] : 1.0;
         for (int v = 0; v < G; ++v) {
-            const double x = scalbn(ws ? row[v] * wt : row[v], e);
+            const double x = scale_pow2(ws ? row[v] * wt : row[v], e);
             out[v * n + i] = x;
             if (out2) {
-                const float h = (float)x;
-                out2[v * n + i] = make_float2(h, (float)(x - (double)h));
+                const df s = df_from(x);
+                out2[v * n + i] = make_float2(s.h, s.l);
             }
         }
     }
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const double* __restri
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
          i += (int64_t)gridDim.x * blockDim.x) {
         double* row = g + (int64_t)perm[i] * stride + comp;
-        for (int v = 0; v < G; ++v) row[v] = scalbn(gs[v * m + i], e);
+        for (int v = 0; v < G; ++v) row[v] = scale_pow2(gs[v * m + i], e);
     }
 }
 
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter_deriv(const double* __
         double sum = comp == 0 ? 0.0 : out[u];
         for (int v = 0; v < G; ++v) {
             const double* gv = gs + v * nrep * mb;
-            const double x = scalbn(nrep == 2 ? gv[k] + gv[mb + k] : gv[k], e) * y[u * stride + comp + v];
+            const double x = scale_pow2(nrep == 2 ? gv[k] + gv[mb + k] : gv[k], e) * y[u * stride + comp + v];
             sum = comp + v == 0 ? x : sum + x;
         }
         out[u] = sum;
