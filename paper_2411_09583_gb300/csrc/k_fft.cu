@@ -8,6 +8,7 @@
 // points; every CTA takes a tile of up to kFftTileVals values -- some lines,
 // each with a run of the block's Hankel terms q, which are adjacent in memory.
 // Mixed-precision forward transforms: FP32 butterflies (the _f32 kernels).
+#include <algorithm>
 #include <cstdint>
 
 #include "asy_dev.cuh"
@@ -489,24 +490,12 @@ __global__ void k_asy_fft_small_f32(const ProbParams* __restrict__ probs, const 
     for (int tt = threadIdx.x; tt < N; tt += blockDim.x) dst[B.q_off + (int64_t)tt * Q + q] = cf4_of(Xf[tt]);
 }
 
-// All Q grids of one small block (nf2 * Q <= kFftSmemMax) in one CTA: the
+// All Q grids of one small block (nf2 * Q <= kFftSmemMax) by one CTA: the
 // deconvolution factor of each mode is computed once and used for every q;
-// the Q transforms share every butterfly stage.  A launch takes the blocks
-// with pts_lo < nf2 * Q <= pts_hi (the others return at once), so that small
-// blocks run in CTAs sized for them.
-__global__ void k_asy_fft_block_f32(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
-                                    const Tile* __restrict__ items, Tables tab,
-                                    const double2* __restrict__ src, float4* __restrict__ dst, int pts_lo,
-                                    int pts_hi, int64_t src_stride, int64_t dst_stride)
+// the Q transforms share every butterfly stage.
+__device__ __forceinline__ void fft_whole_f32(const AsyBlock& B, int Q, const Tables& tab,
+                                              const double2* __restrict__ src, float4* __restrict__ dst, float2* Xf)
 {
-    extern __shared__ float2 Xf[];   // [Q][N], each grid bit-reversed
-    src += blockIdx.y * src_stride;   // member blockIdx.y of a batch of real components
-    dst += blockIdx.y * dst_stride;
-    const Tile it = items[blockIdx.x];
-    const AsyBlock B = blks[it.blk];
-    const int Q = probs[B.prob].Q;
-    const int pts = B.nf2 * Q;
-    if (pts <= pts_lo || pts > pts_hi) return;
     const int N = B.nf2, logN = B.log2nf2, half = N >> 1;
     for (int tt = threadIdx.x; tt < N; tt += blockDim.x) {
         const int l = (tt < half) ? tt : tt - N;
@@ -525,6 +514,47 @@ __global__ void k_asy_fft_block_f32(const ProbParams* __restrict__ probs, const 
     for (int idx = threadIdx.x; idx < N * Q; idx += blockDim.x) {
         const int tt = idx / Q, q = idx - tt * Q;
         gq[idx] = cf4_of(Xf[q * N + tt]);
+    }
+}
+
+// The blocks with pts_lo < nf2 * Q <= pts_hi.  SCAN = false (the small class,
+// nearly all blocks): one CTA per item, the others return at once.  SCAN (the
+// few large ones): every thread of a CTA looks at one item, the items a grid
+// apart, and the CTA transforms those of the class that it found.  With a CTA
+// per item here too, 1.26e5 CTAs of which almost none had work took 0.11 of
+// the 0.64 ms of a complex mixed-precision transform's FFTs (n = m = 4e6).
+template <bool SCAN>
+__global__ void k_asy_fft_block_f32(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
+                                    const Tile* __restrict__ items, int nitems, Tables tab,
+                                    const double2* __restrict__ src, float4* __restrict__ dst, int pts_lo,
+                                    int pts_hi, int64_t src_stride, int64_t dst_stride)
+{
+    extern __shared__ float2 Xf[];   // [Q][N], each grid bit-reversed
+    src += blockIdx.y * src_stride;   // member blockIdx.y of a batch of real components
+    dst += blockIdx.y * dst_stride;
+    if constexpr (!SCAN) {
+        const AsyBlock B = blks[items[blockIdx.x].blk];
+        const int Q = probs[B.prob].Q, pts = B.nf2 * Q;
+        if (pts > pts_lo && pts <= pts_hi) fft_whole_f32(B, Q, tab, src, dst, Xf);
+    } else {
+        __shared__ int found[256], nfound;
+        for (int64_t base = 0; base < nitems; base += (int64_t)blockDim.x * gridDim.x) {
+            if (threadIdx.x == 0) nfound = 0;
+            __syncthreads();
+            const int64_t i = base + (int64_t)threadIdx.x * gridDim.x + blockIdx.x;
+            if (i < nitems) {
+                const int b = items[i].blk;
+                const int pts = blks[b].nf2 * probs[blks[b].prob].Q;
+                if (pts > pts_lo && pts <= pts_hi) found[atomicAdd(&nfound, 1)] = b;
+            }
+            __syncthreads();
+            const int nf = nfound;
+            for (int f = 0; f < nf; ++f) {
+                const AsyBlock B = blks[found[f]];
+                fft_whole_f32(B, probs[B.prob].Q, tab, src, dst, Xf);
+                __syncthreads();   // Xf is rewritten by the next block, found by the next round
+            }
+        }
     }
 }
 
@@ -653,9 +683,9 @@ cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* bl
     if (members < 1 || members > 65535) return cudaErrorInvalidValue;
     if (max_pts < 1 || max_pts > kFftSmemMax) max_pts = kFftSmemMax;
     // blocks of up to kFftSmallPts points in small CTAs (8 KiB, many per SM),
-    // the larger ones in CTAs sized for the largest; each launch skips the
-    // other size class at once
+    // the larger ones in CTAs sized for the largest
     constexpr int kFftSmallPts = 1024;
+    constexpr int kFftScanCtas = 8 * 152;   // at least eight CTAs per SM look for the larger ones
     const int ranges[2][2] = {{0, max_pts < kFftSmallPts ? max_pts : kFftSmallPts}, {kFftSmallPts, max_pts}};
     int launched = 0;
     for (int r = 0; r < 2; ++r) {
@@ -666,10 +696,13 @@ cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* bl
         if (r == 0 && nt > 128) nt = 128;
         if (nt > 256) nt = 256;
         if (nt < 32) nt = 32;
-        cudaError_t e = cudaFuncSetAttribute(k_asy_fft_block_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        auto kern = r ? k_asy_fft_block_f32<true> : k_asy_fft_block_f32<false>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_asy_fft_block_f32<<<dim3(nitems, members), nt, smem, s>>>(probs, blks, items, tab, src, dst, lo, hi,
-                                                                    src_stride, dst_stride);
+        int gx = nitems;
+        if (r) gx = std::min(nitems, std::max((nitems + nt - 1) / nt, kFftScanCtas));
+        kern<<<dim3(gx, members), nt, smem, s>>>(probs, blks, items, nitems, tab, src, dst, lo, hi, src_stride,
+                                                 dst_stride);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         ++launched;

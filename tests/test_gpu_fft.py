@@ -51,3 +51,23 @@ def test_one_block_at_every_pass_count(LN, eps, m_terms, members):
     assert np.all(err <= tol(eps, c)), (err, tol(eps, c))
     err = np.max(np.abs(ca - oracle.direct(1, omega, r, e)), axis=0)
     assert np.all(err <= tol(eps, e)), (err, tol(eps, e))
+
+
+@pytest.mark.parametrize("count,n", [(1, 60), (3, 4000), (40, 500), (60, 1500)])
+def test_mixed_blocks_of_both_size_classes(count, n):
+    # mixed precision transforms a block's grids whole in one CTA, small and
+    # large ones in launches of their own: none, few or many of either kind
+    from paper_2411_09583_gb300 import Plan
+    rng = np.random.default_rng(count)
+    ns, ms = rng.integers(n // 2, n + 1, count), rng.integers(n // 2, n + 1, count)
+    r, omega = rng.uniform(0.0, 1.0, ns.sum()), rng.uniform(0.0, 1.0, ms.sum()) * n
+    c = rng.standard_normal(r.size)
+    nus = np.arange(count) % 4
+    with Plan.many(nus, to_dev(r), ns, to_dev(omega), ms, 1e-5, precision="mixed", min_size=64) as p:
+        g = p.execute(to_dev(c)).cpu().numpy()
+    jo = io = 0
+    for nu, a, b in zip(nus, ns, ms):
+        ref = oracle.direct(int(nu), r[jo:jo + a], omega[io:io + b], c[jo:jo + a])
+        assert np.max(np.abs(g[io:io + b] - ref)) <= tol(1e-5, c[jo:jo + a])
+        jo += a
+        io += b
