@@ -15,8 +15,8 @@
 // by their full patterns where they lie.  Points and frequencies share every
 // launch, and up to kSmallSort of each are sorted by one CTA in one launch.
 // Measured, both arrays on an idle GPU (sum of the launches): n = m = 1e6
-// 0.45 ms in 52 launches on two streams -> 0.17 in 15; 1e5 0.16 -> 0.05; 2000
-// 0.12 -> 0.02 in one launch.  Bound by the scatters' 8-byte stores (L2) at
+// 0.45 ms in 52 launches on two streams -> 0.17 in 15; 1e5 0.16 -> 0.06; 2000
+// 48 launches -> one of 0.02.  Bound by the scatters' 8-byte stores (L2) at
 // 1e6 and by launch latency below 1e5.
 #include <cstdint>
 

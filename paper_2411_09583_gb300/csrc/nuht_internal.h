@@ -315,7 +315,7 @@ cudaError_t launch_staircase(const double* r, const double* w, int64_t m, const 
 // same either way.
 constexpr int kSubGridMax = 1024;
 // up to this many points + frequencies: one CTA, no cooperative launch (levels of
-// up to ~120 blocks there: 52 -> 22 us at 4000 in all, the grid's barriers included)
+// up to ~120 blocks there: 52 -> 20 us at 4000 in all, the grid's barriers included)
 constexpr int64_t kSubOneCta = 32768;
 int subdivide_grid_ctas();
 cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const double* w_s, const ProbParams* probs,
