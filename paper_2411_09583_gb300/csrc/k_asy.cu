@@ -173,6 +173,18 @@ constexpr int kMomBins = 2;         // bins whose moments are formed and added t
 // interpolations up to 1.5 % at 8.
 constexpr int kMomMinPerBin = 16;
 
+// Tiles of up to kSmallTile points or frequencies run in CTAs of as many threads,
+// in a launch of their own, where a plan has at least kSplitBlocks asymptotic
+// blocks (the last tile of a block is its only partial one): a wide CTA holds its
+// SM's threads and shared memory for a few rows and waits at every barrier for warps
+// without any.  A row's sums are the same in either.  Both launches visit all
+// tiles, so fewer blocks would pay for more than they give (a launch of 1.6e4 idle
+// CTAs: some 10 us; one block: no small tile at all).  Interpolation and spreading
+// together: 62786 blocks (mixed precision, complex 4e6) 3.25 -> 2.87 ms, 50113 (256
+// problems) 9.2 -> 8.7, 3181 (1e6 points) call 2.72 -> 2.68.
+constexpr int kSmallTile = 64;
+constexpr int kSplitBlocks = 2048;
+
 // Row strides of the dense paths' shared arrays, whose points (rows) eight or
 // sixteen consecutive lanes read side by side: loads of two elements want half
 // the stride odd, loads of four a quarter of it.
@@ -1081,12 +1093,12 @@ __global__ void __launch_bounds__(256, 3) k_asy_spread(const ProbParams* __restr
                              const Tile* __restrict__ tiles, const int32_t* __restrict__ modes, Tables tab,
                              const double* __restrict__ r_s, const float2* __restrict__ r2,
                              const float2* __restrict__ c2, int64_t c_stride, int V,
-                             double2* __restrict__ grid_b, int64_t gb_stride)
+                             double2* __restrict__ grid_b, int64_t gb_stride, int over, int upto)
 {
     extern __shared__ float4 smem4[];
     __shared__ MomShared sh;
     const Tile t = tiles[blockIdx.x];
-    if (t.count <= 0) return;
+    if (t.count <= over || t.count > upto) return;   // the other launch's
     const int mode = modes[blockIdx.x];
     const AsyBlock B = blks[t.blk];
     const int Q = probs[B.prob].Q;
@@ -1378,10 +1390,12 @@ __device__ __forceinline__ void tap_sums_eval(const float2* u, int w, int Q, int
 __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
     const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks, const Tile* __restrict__ tiles,
     Tables tab, const double* __restrict__ w_s, const float2* __restrict__ w2, const float4* __restrict__ grid_q,
-    int64_t gq_stride, int V, double* __restrict__ g_s, int64_t g_stride)
+    int64_t gq_stride, int V, double* __restrict__ g_s, int64_t g_stride, int hbytes,
+    int over, int upto)
 {
     extern __shared__ float4 win[];          // [kWinCells][ws] grid cells of this tile
     const Tile t = tiles[blockIdx.x];
+    if (t.count <= over || t.count > upto) return;   // the other launch's
     const AsyBlock B = blks[t.blk];
     const ProbParams& P = probs[B.prob];
     const int w = tab.w, deg = tab.deg, nb = tab.nb, dci = tab.dci;
@@ -1390,7 +1404,6 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_interp(
     const int hs = nb * Q2 + 2;                                  // bin stride of H (float2)
     float2* coef2 = (float2*)(win + kWinCells * Q);              // [w][deg + 1] taps, or [w][nb] Chebyshev
     float2* H = coef2 + ((w * (deg + 1) + 1) & ~1);              // [bins][hs], 16-byte aligned
-    const int hbytes = kInterpHBytesPerThread * (int)blockDim.x;
     float2* U = H + hbytes / sizeof(float2);                     // [threads][us]
     int* t0s = (int*)(U + blockDim.x * us);                      // [threads]
     const bool valid = (int)threadIdx.x < t.count;
@@ -1588,12 +1601,14 @@ template <bool MULTI>
 __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const ProbParams* __restrict__ probs, const AsyBlock* __restrict__ blks,
                                  const Tile* __restrict__ tiles, Tables tab,
                                  const double* __restrict__ w_s, const double* __restrict__ g_s,
-                                 int64_t g_stride, int V, double2* __restrict__ tgrid, int64_t tg_stride)
+                                 int64_t g_stride, int V, double2* __restrict__ tgrid, int64_t tg_stride,
+                                 int over, int upto)
 {
     extern __shared__ float4 sma[];
     __shared__ MomShared sh;
     __shared__ int use_mom;
     const Tile t = tiles[blockIdx.x];
+    if (t.count <= over || t.count > upto) return;   // the other launch's
     const AsyBlock B = blks[t.blk];
     const ProbParams& P = probs[B.prob];
     const int Q = P.Q;
@@ -1601,7 +1616,6 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const 
     const int mask = B.nf2 - 1;
     const Accum tg = Accum{(double*)tgrid, P.fxs}.at(2 * B.q_off);
     const int cnt = t.count;
-    if (cnt <= 0) return;
     if (tid == 0) {
         long long Om, Sw, svw;
         const int tfirst = interp_cell_sv(B, w, w_s[t.start], &Om, &Sw, &svw);
@@ -1796,16 +1810,6 @@ __global__ void __launch_bounds__(kAdjInterpThreads) k_asy_adj_interp(
 }
 
 // ------------------------------------------------------ mixed precision (FP32)
-// Tiles of up to kSmallTile points or frequencies run in CTAs of as many threads,
-// in a launch of their own, where a plan has at least kSplitTiles tiles: a wide
-// CTA holds its SM's threads and shared memory for a few rows and waits at every
-// barrier for warps without any.  Both launches visit all tiles; below that many the
-// second launch costs what it gives.  A row's sums are the same in either.
-// Complex n = m = 4e6, half of 1.08e5 interpolation and a fifth of 1.9e5 spreading
-// tiles small: interpolation 1.44 -> 1.10 ms, spreading 1.81 -> 1.77.
-constexpr int kSmallTile = 64;
-constexpr int kSplitTiles = 8192;
-
 __device__ __forceinline__ float horner_f32(const float2* __restrict__ c, int deg, float v)
 {
     float acc = c[deg].x;
@@ -2236,23 +2240,30 @@ __global__ void __launch_bounds__(kInterpTileThreads, 4) k_asy_interp_f32(
 }  // namespace
 
 cudaError_t launch_asy_adj_spread(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  int ntiles, int qmax, int nt, Tables tab, const double* w_s, const double* g_s,
+                                  int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const double* g_s,
                                   int64_t g_stride, int members, double2* tgrid, int64_t tg_stride,
                                   cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
     if (nt < 32 || nt > kInterpTileThreads || (nt & 31)) return cudaErrorInvalidValue;
-    size_t smem = sizeof(float4) * (size_t)nt * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
-                  sizeof(float2) * (size_t)nt * tab.w + sizeof(int) * (size_t)nt;
-    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
-    if (smem_mom > smem) smem = smem_mom;
     if (members < 1) return cudaErrorInvalidValue;
     auto kern = members > 1 ? k_asy_adj_spread<true> : k_asy_adj_spread<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<ntiles, nt, smem, s>>>(probs, blks, tiles, tab, w_s, g_s, g_stride, members, tgrid, tg_stride);
-    count_launches(1);
-    return cudaGetLastError();
+    int over = 0;
+    for (int n : {nblk >= kSplitBlocks && nt > kSmallTile ? kSmallTile : 0, nt}) {
+        if (n <= 0) continue;
+        size_t smem = sizeof(float4) * (size_t)n * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
+                      sizeof(float2) * (size_t)n * tab.w + sizeof(int) * (size_t)n;
+        const size_t smem_mom = spread_moments_smem(n, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
+        if (smem_mom > smem) smem = smem_mom;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<ntiles, n, smem, s>>>(probs, blks, tiles, tab, w_s, g_s, g_stride, members, tgrid, tg_stride, over, n);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        count_launches(1);
+        over = n;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_asy_adj_interp(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
@@ -2272,7 +2283,7 @@ cudaError_t launch_asy_adj_interp(const ProbParams* probs, const AsyBlock* blks,
 }
 
 cudaError_t launch_asy_spread_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  const int32_t* modes, int ntiles, int qmax, int nt, Tables tab,
+                                  const int32_t* modes, int ntiles, int nblk, int qmax, int nt, Tables tab,
                                   const double* r_s, const float2* r2, const float2* c2, int64_t c_stride,
                                   int members, double2* grid_b, int64_t gb_stride, cudaStream_t s)
 {
@@ -2280,7 +2291,7 @@ cudaError_t launch_asy_spread_f32(const ProbParams* probs, const AsyBlock* blks,
     if (members < 1) return cudaErrorInvalidValue;
     auto kern = members > 1 ? k_asy_spread_f32<true> : k_asy_spread_f32<false>;
     int over = 0;
-    for (int n : {ntiles >= kSplitTiles && nt > kSmallTile ? kSmallTile : 0, nt}) {
+    for (int n : {nblk >= kSplitBlocks && nt > kSmallTile ? kSmallTile : 0, nt}) {
         if (n <= 0) continue;
         size_t smem = sizeof(float2) * (size_t)n * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
                       sizeof(float) * (size_t)n * tab.w + sizeof(int) * (size_t)n;
@@ -2299,7 +2310,7 @@ cudaError_t launch_asy_spread_f32(const ProbParams* probs, const AsyBlock* blks,
 }
 
 cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  int ntiles, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
+                                  int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
                                   const float4* grid_q, int64_t gq_stride, int members, double* g_s,
                                   int64_t g_stride, cudaStream_t s)
 {
@@ -2307,7 +2318,7 @@ cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks,
     if (nt < 32 || nt > kInterpTileThreads || (nt & 31)) return cudaErrorInvalidValue;
     if (members < 1) return cudaErrorInvalidValue;
     int over = 0;
-    for (int n : {ntiles >= kSplitTiles && nt > kSmallTile ? kSmallTile : 0, nt}) {
+    for (int n : {nblk >= kSplitBlocks && nt > kSmallTile ? kSmallTile : 0, nt}) {
         if (n <= 0) continue;
         // room for the sums of every bin that a dense tile of n frequencies can have,
         // so that a tile takes the path that it takes at nt threads
@@ -2342,43 +2353,63 @@ cudaError_t launch_expand_lists(const ExpandLists& E, const ProbParams* probs, c
 }
 
 cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                              const int32_t* modes, int ntiles, int qmax, int nt, Tables tab, const double* r_s,
+                              const int32_t* modes, int ntiles, int nblk, int qmax, int nt, Tables tab, const double* r_s,
                               const float2* r2, const float2* c2, int64_t c_stride, int members,
                               double2* grid_b, int64_t gb_stride, int det, cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
-    size_t smem = sizeof(float4) * (size_t)nt * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
-                  sizeof(float2) * (size_t)nt * tab.w + sizeof(int) * (size_t)nt;
-    const size_t smem_mom = spread_moments_smem(nt, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
-    if (smem_mom > smem) smem = smem_mom;
-    const size_t smem_fold = spread_fold_smem(nt, qmax, tab.w, tab.nb, tab.dcs);
-    if (smem_fold > smem) smem = smem_fold;
+    if (members < 1 || (det && members != 1)) return cudaErrorInvalidValue;
     auto kern = det ? k_asy_spread<true, false>
                     : (members > 1 ? k_asy_spread<false, true> : k_asy_spread<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (members < 1 || (det && members != 1)) return cudaErrorInvalidValue;
-    kern<<<ntiles, nt, smem, s>>>(probs, blks, tiles, modes, tab, r_s, r2, c2, c_stride, members, grid_b,
-                                  gb_stride);
-    count_launches(1);
-    return cudaGetLastError();
+    int over = 0;
+    for (int n : {nblk >= kSplitBlocks && nt > kSmallTile ? kSmallTile : 0, nt}) {
+        if (n <= 0) continue;
+        size_t smem = sizeof(float4) * (size_t)n * qmax + sizeof(float2) * (size_t)tab.w * (tab.deg + 1) +
+                      sizeof(float2) * (size_t)n * tab.w + sizeof(int) * (size_t)n;
+        const size_t smem_mom = spread_moments_smem(n, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
+        if (smem_mom > smem) smem = smem_mom;
+        const size_t smem_fold = spread_fold_smem(n, qmax, tab.w, tab.nb, tab.dcs);
+        if (smem_fold > smem) smem = smem_fold;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<ntiles, n, smem, s>>>(probs, blks, tiles, modes, tab, r_s, r2, c2, c_stride, members, grid_b,
+                                     gb_stride, over, n);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        count_launches(1);
+        over = n;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_asy_interp(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                              int ntiles, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
+                              int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
                               const float4* grid_q, int64_t gq_stride, int members, double* g_s,
                               int64_t g_stride, cudaStream_t s)
 {
     if (ntiles <= 0) return cudaSuccess;
     if (nt < 32 || nt > kInterpTileThreads || (nt & 31)) return cudaErrorInvalidValue;
-    const size_t smem = interp_smem(qmax, tab.w, tab.deg, nt, kInterpHBytesPerThread * nt);
-    cudaError_t e = cudaFuncSetAttribute(k_asy_interp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     if (members < 1) return cudaErrorInvalidValue;
-    k_asy_interp<<<ntiles, nt, smem, s>>>(probs, blks, tiles, tab, w_s, w2, grid_q, gq_stride, members, g_s,
-                                          g_stride);
-    count_launches(1);
-    return cudaGetLastError();
+    int over = 0;
+    for (int n : {nblk >= kSplitBlocks && nt > kSmallTile ? kSmallTile : 0, nt}) {
+        if (n <= 0) continue;
+        // room for the sums of every bin that a dense tile of n frequencies can have,
+        // so that a tile takes the path that it takes at nt threads
+        const int bins = (int)sizeof(float2) * (tab.nb * 2 * qmax + 2) * (n / kMomMinPerBin);
+        const int hbytes = n == nt ? kInterpHBytesPerThread * n
+                                   : std::min(kInterpHBytesPerThread * nt,
+                                              std::max(kInterpHBytesPerThread * n, (bins + 15) & ~15));
+        const size_t smem = interp_smem(qmax, tab.w, tab.deg, n, hbytes);
+        cudaError_t e = cudaFuncSetAttribute(k_asy_interp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_asy_interp<<<ntiles, n, smem, s>>>(probs, blks, tiles, tab, w_s, w2, grid_q, gq_stride, members, g_s,
+                                             g_stride, hbytes, over, n);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        count_launches(1);
+        over = n;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace nuht

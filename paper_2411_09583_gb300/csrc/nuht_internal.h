@@ -437,12 +437,12 @@ cudaError_t launch_direct_adj(const ProbParams* probs, const DirectBlock* blks, 
 // members: real components spread by one launch (coefficients c2 + v c_stride,
 // grids grid_b + v gb_stride); 1 in the deterministic mode.
 cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                              const int32_t* modes, int ntiles, int qmax, int nt, Tables tab, const double* r_s,
+                              const int32_t* modes, int ntiles, int nblk, int qmax, int nt, Tables tab, const double* r_s,
                               const float2* r2, const float2* c2, int64_t c_stride, int members,
                               double2* grid_b, int64_t gb_stride, int det, cudaStream_t s);
 // members as in launch_asy_spread (inputs g_s + v g_stride, grids tgrid + v tg_stride)
 cudaError_t launch_asy_adj_spread(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  int ntiles, int qmax, int nt, Tables tab, const double* w_s, const double* g_s,
+                                  int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const double* g_s,
                                   int64_t g_stride, int members, double2* tgrid, int64_t tg_stride,
                                   cudaStream_t s);
 // members as in launch_asy_interp (modes bgrid + v bg_stride, sums into c_s + v c_stride)
@@ -450,11 +450,11 @@ cudaError_t launch_asy_adj_interp(const ProbParams* probs, const AsyBlock* blks,
                                   int ntiles, int qmax, Tables tab, const double* r_s, const float4* bgrid,
                                   int64_t bg_stride, int members, double* c_s, int64_t c_stride, cudaStream_t s);
 cudaError_t launch_asy_spread_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  const int32_t* modes, int ntiles, int qmax, int nt, Tables tab,
+                                  const int32_t* modes, int ntiles, int nblk, int qmax, int nt, Tables tab,
                                   const double* r_s, const float2* r2, const float2* c2, int64_t c_stride,
                                   int members, double2* grid_b, int64_t gb_stride, cudaStream_t s);
 cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                                  int ntiles, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
+                                  int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
                                   const float4* grid_q, int64_t gq_stride, int members, double* g_s,
                                   int64_t g_stride, cudaStream_t s);
 // One pass of the double-float FFTs (pass 0 reads src, the last one of a block
@@ -480,7 +480,7 @@ cudaError_t launch_asy_fft_large_f32(const ProbParams* probs, const AsyBlock* bl
 // members: real components interpolated by one launch (FFT outputs grid_q + v
 // gq_stride, sums into g_s + v g_stride).
 cudaError_t launch_asy_interp(const ProbParams* probs, const AsyBlock* blks, const Tile* tiles,
-                              int ntiles, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
+                              int ntiles, int nblk, int qmax, int nt, Tables tab, const double* w_s, const float2* w2,
                               const float4* grid_q, int64_t gq_stride, int members, double* g_s,
                               int64_t g_stride, cudaStream_t s);
 

@@ -1313,12 +1313,12 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_SPREAD, as));
         if (v0 > 0) NUHT_CK(cudaMemsetAsync(gb_acc, 0, acc_bytes(P, 2 * P->gb_len * nv), as));
         if (lowp)
-            NUHT_CK(launch_asy_spread_f32(P->d_prob, P->d_asy, P->d_tspread, P->d_smode, P->n_tspread, P->qmax,
-                                          P->spread_threads, P->tab, P->d_r, P->d_r2, c2, P->n, nv, gb_acc,
+            NUHT_CK(launch_asy_spread_f32(P->d_prob, P->d_asy, P->d_tspread, P->d_smode, P->n_tspread, P->n_asy,
+                                          P->qmax, P->spread_threads, P->tab, P->d_r, P->d_r2, c2, P->n, nv, gb_acc,
                                           P->gb_len, as));
         else
-            NUHT_CK(launch_asy_spread(P->d_prob, P->d_asy, P->d_tspread, P->d_smode, P->n_tspread, P->qmax,
-                                      P->spread_threads, P->tab, P->d_r, P->d_r2, c2, P->n, nv, gb_acc,
+            NUHT_CK(launch_asy_spread(P->d_prob, P->d_asy, P->d_tspread, P->d_smode, P->n_tspread, P->n_asy,
+                                      P->qmax, P->spread_threads, P->tab, P->d_r, P->d_r2, c2, P->n, nv, gb_acc,
                                       P->gb_len, P->det ? 1 : 0, as));
         if (P->det) NUHT_CK(launch_fx_decode(P->f_gb, (double*)P->d_gb, 2 * P->gb_len, P->d_prob, as));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_SPREAD, as));
@@ -1342,11 +1342,11 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_FFT, as));
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_INTERP, as));
         if (lowp)
-            NUHT_CK(launch_asy_interp_f32(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->qmax,
+            NUHT_CK(launch_asy_interp_f32(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->n_asy, P->qmax,
                                           P->interp_threads, P->tab, P->d_w, P->d_w2, P->d_gq, P->gq_len, nv,
                                           gv, P->m, as));
         else
-            NUHT_CK(launch_asy_interp(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->qmax,
+            NUHT_CK(launch_asy_interp(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->n_asy, P->qmax,
                                       P->interp_threads, P->tab, P->d_w, P->d_w2, P->d_gq, P->gq_len, nv, gv,
                                       P->m, as));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_INTERP, as));
@@ -1520,7 +1520,7 @@ static int apply_adjoint(nuht_plan_t P, int c0, int ng, bool pairs, cudaStream_t
         StageTimer Tv{P, c0 + v0};
         NUHT_TRY(Tv.begin(NUHT_STAGE_ASY_SPREAD, as));
         if (v0 > 0) NUHT_CK(cudaMemsetAsync(tg_acc, 0, acc_bytes(P, 2 * P->gq_len * nv), as));
-        NUHT_CK(launch_asy_adj_spread(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->qmax, P->interp_threads,
+        NUHT_CK(launch_asy_adj_spread(P->d_prob, P->d_asy, P->d_tinterp, P->n_tinterp, P->n_asy, P->qmax, P->interp_threads,
                                       P->tab, P->d_w, member_g(P, v0), P->m, nv, tg_acc, P->gq_len, as));
         if (P->det) NUHT_CK(launch_fx_decode(P->f_tg, (double*)P->d_tg, 2 * P->gq_len, P->d_prob, as));
         NUHT_TRY(Tv.end(NUHT_STAGE_ASY_SPREAD, as));

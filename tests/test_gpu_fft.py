@@ -73,22 +73,27 @@ def test_mixed_blocks_of_both_size_classes(count, n):
         io += b
 
 
-def test_mixed_with_many_small_tiles():
-    # enough tiles that the mixed-precision spreading and interpolation run small
-    # and large ones in launches of their own
+@pytest.mark.parametrize("precision,eps", [("mixed", 1e-5), ("fp64", 1e-8)])
+def test_many_small_tiles(precision, eps):
+    # enough blocks that the spreading and interpolation run small and large tiles
+    # in launches of their own
     from paper_2411_09583_gb300 import Plan
     rng = np.random.default_rng(9)
     count, big = 500, 3
     ns = np.r_[np.full(count, 700), np.full(big, 6000)]
     nus = np.arange(ns.size) % 3
     r, omega = rng.uniform(0.0, 1.0, ns.sum()), rng.uniform(0.0, 1.0, ns.sum()) * np.repeat(ns, ns)
-    c = rng.standard_normal(r.size)
-    with Plan.many(nus, to_dev(r), ns, to_dev(omega), ns, 1e-5, precision="mixed", min_size=32) as p:
+    c, e = rng.standard_normal(r.size), rng.standard_normal(r.size)
+    with Plan.many(nus, to_dev(r), ns, to_dev(omega), ns, eps, precision=precision, min_size=32) as p:
         assert p.info()["n_asy"] >= 8192
         g = p.execute(to_dev(c)).cpu().numpy()
+        ca = p.adjoint(to_dev(e)).cpu().numpy()
     at = 0
     for nu, n in zip(nus, ns):
+        sl = slice(at, at + n)
         rows = rng.integers(0, n, 8)
-        ref = oracle.direct(int(nu), r[at:at + n], omega[at:at + n][rows], c[at:at + n])
-        assert np.max(np.abs(g[at:at + n][rows] - ref)) <= tol(1e-5, c[at:at + n])
+        ref = oracle.direct(int(nu), r[sl], omega[sl][rows], c[sl])
+        assert np.max(np.abs(g[sl][rows] - ref)) <= tol(eps, c[sl])
+        ref = oracle.direct(int(nu), omega[sl], r[sl][rows], e[sl])
+        assert np.max(np.abs(ca[sl][rows] - ref)) <= tol(eps, e[sl])
         at += n
