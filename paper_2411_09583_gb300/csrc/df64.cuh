@@ -130,34 +130,6 @@ __device__ __forceinline__ void acc_fma(acc2& A, df a, df b)
 
 __device__ __forceinline__ double acc_value(acc2 A) { return (double)A.s + (double)A.c; }
 
-// Anchored accumulation: the running sum starts from an anchor 1.5 2^K with
-// 2^K > 2 bound, bound >= |any partial sum|, so that it stays in one binade and
-// its rounding error is exactly what A.s - s leaves of the product: six
-// instructions a product instead of the twelve of acc_fma (no two_sum).  The
-// sum is (A.s - anchor) + A.c; against acc_fma the anchor's distance from the
-// actual sum (bound / |sum|) costs that many bits of the 48.
-__device__ __forceinline__ float acc_anchor(float bound)
-{
-    const unsigned e = (__float_as_uint(bound) & 0x7f800000u) + 0x01000000u;   // 2^(floor(log2 bound) + 2)
-    return __uint_as_float((e < 0x7e000000u ? e : 0x7e000000u) | 0x00400000u);
-}
-
-__device__ __forceinline__ void acc_fma_anchored(acc2& A, df a, df b)
-{
-    const float s = fmaf(a.h, b.h, A.s);
-    const float e = fmaf(a.h, b.h, A.s - s);   // exact but for its own rounding
-    A.c = fmaf(a.l, b.h, fmaf(a.h, b.l, A.c)) + e;
-    A.s = s;
-}
-
-// One of the two (uniform choice per kernel path).
-template <bool ANCHORED>
-__device__ __forceinline__ void acc_mul(acc2& A, df a, df b)
-{
-    if (ANCHORED) acc_fma_anchored(A, a, b);
-    else acc_fma(A, a, b);
-}
-
 // a += the value of lane ^ off (two-sum through the shuffles), where this lane
 // keeps `keep` and hands over `give`.
 __device__ __forceinline__ acc2 acc_exchange(acc2 keep, acc2 give, int off)

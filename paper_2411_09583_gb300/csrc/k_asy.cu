@@ -139,30 +139,12 @@ __device__ __forceinline__ df psihat_fx(const Tables& T, const AsyBlock& B, long
 constexpr int kMaxTileBins = 32;
 constexpr int kSpreadSub = 8;       // point sub-ranges per moment, combined by shuffles
 
-// The tile's largest magnitude bound: every warp leaves its own (warp_mag, all
-// threads), and after a barrier every thread reads the tile's (up to 8 warps).
-__device__ __forceinline__ void warp_mag(unsigned* wmag, float mag)
-{
-    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mag));
-    if ((threadIdx.x & 31) == 0) wmag[threadIdx.x >> 5] = m;
-}
-__device__ __forceinline__ float tile_mag(const unsigned* wmag)
-{
-    unsigned m = wmag[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = wmag[w] > m ? wmag[w] : m;
-    return __uint_as_float(m);
-}
-
 // Small shared arrays of the dense paths (one set for all their instances).
 struct MomShared {
     int bstart[kMaxTileBins + 3];      // first point of each bin
-    unsigned wmag[8];                  // per warp, the largest magnitude bound (float bits)
     uint16_t items[kMaxMomItems];      // (degree pair, Hankel pair) of every moment item, by cost
 };
 
-// A bound of |re| and |im| of c (double-float high parts; 1.001 covers the low
-// parts and the rounding of what is derived from them).
-__device__ __forceinline__ float mag_of(float re, float im) { return 1.001f * fmaxf(fabsf(re), fabsf(im)); }
 constexpr int kMomBins = 2;         // bins whose moments are formed and added to the grid together
 // Tiles with at least this many points per bin use moments (spreading) or per-bin
 // sums (interpolation).  One line for all four stages: the dense paths cut the
@@ -223,14 +205,12 @@ __host__ __device__ __forceinline__ MomLayout mom_layout(int nb, int dcs, int Q2
 // in double-float.
 //
 // Shared by the spreading of points (forward) and of frequencies (adjoint):
-// target(j, &v, xh, xl, &mag) gives target j's cell and kernel coordinate v and
+// target(j, &v, xh, xl) gives target j's cell and kernel coordinate v and
 // writes its 2M weighted values as (re, im) pairs [2q], [2q + 1], high parts to
-// xh and the low parts of the first nlow Hankel pairs to xl, and a bound of
-// their magnitudes;
+// xh and the low parts of the first nlow Hankel pairs to xl;
 // cell(c) is the grid index of cell c, or -1 for a cell outside the grid.
 // Members (forward spreading of V real components): target writes member 0's
-// values; values(vm, xh, xl) rewrites this thread's point's values for member vm
-// (returning their bound),
+// values; values(vm, xh, xl) rewrites this thread's point's values for member vm,
 // whose grid sits moff accumulator elements after member 0's.  The basis,
 // the cells and the bins are formed once for all members.
 //
@@ -238,20 +218,18 @@ __host__ __device__ __forceinline__ MomLayout mom_layout(int nb, int dcs, int Q2
 //  - double-float items take 16 lanes, FP32 ones 8, on different warps, and two
 //    bins share the barriers and one grid update (a cell of both gets one sum);
 //  - the lanes' partial sums are exchanged and halved (8 exchanges for 8 outputs)
-//    instead of each summed by all lanes (24);
-//  - with ANCHORED sums (tab.anchored, eps >= kAnchorMinEps) a product takes 6
-//    instructions instead of 12, from an anchor above the tile's largest value
-//    times the points of a lane.
+//    instead of each summed by all lanes (24).
 // n = m = 1e6, eps 1e-12 (forward, with the folded tiles): 1.02 -> 0.92 ms;
-// eps 1e-10 0.98 -> 0.81 (forward), 1.33 -> 1.00 per transform (adjoint);
-// one vector of 16 at 1.5e5 points 0.128 -> 0.108.  Outputs differ by 9e-15 of
-// their norm at eps 1e-12 and by 5e-13 at 1e-10.  Skipping a phase in a
+// one vector of 16 at 1.5e5 points 0.128 -> 0.108.  Sums of six instructions a
+// product, from an anchor above the tile's largest value, take 2 % off a gradient
+// at eps 1e-10 (8.62 -> 8.47 ms) but round 4 to 75 times coarser there and at
+// 1e-11, up to 1.7e-12 of the result.  Skipping a phase in a
 // timing-only build at eps 1e-12 (0.96 ms then): double-float items 0.11, FP32
 // items 0.11 (before the high parts had a plane of their own), grid update
 // 0.09; of the folded tiles N 0.04, beta 0.02, M 0.06, grid update 0.11.
 // Per Hankel pair (a quad of values) only the degrees that need it are summed in
 // double-float (ProbParams::items).
-template <bool ANCHORED, class Target, class Values, class Cell, class Acc>
+template <class Target, class Values, class Cell, class Acc>
 __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& t, const Tables& tab,
                                                Target&& target, Values&& values, int V, int64_t moff, Cell&& cell,
                                                Acc gb, float* sm, MomShared& sh)
@@ -268,7 +246,6 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
     float* Ul = Uh + nt * L.suh;                      // [nt][sul]  low parts, d < dcs
     int* l0s = (int*)(Ul + nt * L.sul);               // [nt]
     int* bstart = sh.bstart;
-    unsigned* wmag = sh.wmag;
     uint16_t* items = sh.items;
     const int ntask = P.nitems, nA = P.nwide;
     for (int i = tid; i < ntask; i += nt) items[i] = P.items[i];
@@ -276,10 +253,9 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
         const int r = i / L.dpad, d = i - r * L.dpad;
         Ach[i] = d < nb ? tab.ch2[r * (tab.deg + 1) + d] : make_float2(0.f, 0.f);
     }
-    float mag = 0.f;
     if (tid < cnt) {
         df vd;
-        l0s[tid] = target(t.start + tid, &vd, Xh + tid * L.sxh, Xl + tid * L.sxl, &mag);
+        l0s[tid] = target(t.start + tid, &vd, Xh + tid * L.sxh, Xl + tid * L.sxl);
         // Chebyshev basis by T_{d+1} = 2 v T_d - T_{d-1}
         float* uh = Uh + tid * L.suh;
         float* ul = Ul + tid * L.sul;
@@ -307,7 +283,6 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
         }
         for (; d < L.dpad; ++d) uh[d] = 0.f;
     }
-    if (ANCHORED) warp_mag(wmag, mag);
     __syncthreads();
     const int lfirst = l0s[0];
     const int nbins = l0s[cnt - 1] - lfirst + 1;
@@ -321,11 +296,9 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
     __syncthreads();
     for (int vm = 0; vm < V; ++vm) {
     if (vm > 0) {
-        if (tid < cnt) mag = values(vm, Xh + tid * L.sxh, Xl + tid * L.sxl);
-        if (ANCHORED) warp_mag(wmag, mag);
+        if (tid < cnt) values(vm, Xh + tid * L.sxh, Xl + tid * L.sxl);
         __syncthreads();
     }
-    const float tmag = ANCHORED ? tile_mag(wmag) : 0.f;
     const Acc gv = gb.at(vm * moff);
     for (int g0 = 0; g0 < nbins; g0 += kMomBins) {
         const int gn = nbins - g0 < kMomBins ? nbins - g0 : kMomBins;
@@ -338,13 +311,11 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
             const int b = live && u >= nA ? u / nA : 0, o = live ? u - b * nA : 0;
             const int dp = items[o] >> 8, qq = items[o] & 255;
             const int p0 = bstart[g0 + b], p1 = live ? bstart[g0 + b + 1] : p0;
-            const float anc =
-                ANCHORED ? acc_anchor(tmag * (float)((p1 - p0 + 2 * kSpreadSub - 1) / (2 * kSpreadSub))) : 0.f;
             acc2 A[2][4];
 #pragma unroll
             for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int f = 0; f < 4; ++f) A[e][f] = acc2{anc, 0.f};
+                for (int f = 0; f < 4; ++f) A[e][f] = acc2{0.f, 0.f};
             const float *uph = Uh + 2 * dp, *upl = Ul + 2 * dp, *xph = Xh + 4 * qq, *xpl = Xl + 4 * qq;
 #pragma unroll 2
             for (int p = p0 + sub; p < p1; p += 2 * kSpreadSub) {
@@ -353,15 +324,9 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
                 const df xs[4] = {{xh.x, xl.x}, {xh.y, xl.y}, {xh.z, xl.z}, {xh.w, xl.w}};
 #pragma unroll
                 for (int f = 0; f < 4; ++f) {
-                    acc_mul<ANCHORED>(A[0][f], df{uh.x, ul.x}, xs[f]);
-                    acc_mul<ANCHORED>(A[1][f], df{uh.y, ul.y}, xs[f]);
+                    acc_fma(A[0][f], df{uh.x, ul.x}, xs[f]);
+                    acc_fma(A[1][f], df{uh.y, ul.y}, xs[f]);
                 }
-            }
-            if (ANCHORED) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) A[e][f].s -= anc;
             }
             // each exchange halves the outputs a lane carries: lane sub ends
             // with degree e = bit 3, value f = bits 2 and 1, summed over bit 0
@@ -581,7 +546,7 @@ __host__ __device__ __forceinline__ size_t spread_fold_smem(int nt, int Q, int w
 // Members (MULTI): V real components with coefficients c2 + vm c_stride,
 // grids moff accumulator elements apart; the points' cells, bases and phase
 // factors and the bins are formed once for all members.
-template <bool ANCHORED, bool MULTI, class Acc>
+template <bool MULTI, class Acc>
 __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& t, const Tables& tab, FoldPlan F,
                             const double* __restrict__ r_s, const float2* __restrict__ r2,
                             const float2* __restrict__ c2, int64_t c_stride, int V, int64_t moff, Acc gb,
@@ -605,7 +570,6 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
     float* Uf = (float*)(Ach + w * L.dpad);           // [nt][suf] T_e(v_p), Edf <= e < E
     int* l0s = (int*)(Uf + nt * suf);                 // [nt]
     int* bstart = sh.bstart;
-    unsigned* wmag = sh.wmag;
     uint16_t* items = sh.items;
     const int nA = P.nwide;
     for (int i = tid; i < P.nitems; i += nt) items[i] = P.items[i];
@@ -645,7 +609,6 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
         spread_weight_fx(B, tab.tw2, X, r2[j], MULTI ? make_float2(1.f, 0.f) : c2[j], &yr, &yi, &rat);
         if (!MULTI) Y[tid] = make_float4(yr.h, yr.l, yi.h, yi.l);
     }
-    if (ANCHORED && !MULTI) warp_mag(wmag, tid < cnt ? mag_of(yr.h, yi.h) : 0.f);
     __syncthreads();
     const int lfirst = l0s[0];
     const int nbins = l0s[cnt - 1] - lfirst + 1;
@@ -661,17 +624,13 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
     const df rho{B.rho_h, B.rho_l};
     for (int vm = 0; vm < (MULTI ? V : 1); ++vm) {
     if (MULTI) {
-        float mag = 0.f;
         if (tid < cnt) {
             const float2 cv = c2[vm * c_stride + j];
             const df wr = df_mul(df{cv.x, cv.y}, yr), wi = df_mul(df{cv.x, cv.y}, yi);
             Y[tid] = make_float4(wr.h, wr.l, wi.h, wi.l);
-            mag = mag_of(wr.h, wi.h);
         }
-        if (ANCHORED) warp_mag(wmag, mag);
         __syncthreads();
     }
-    const float tmag = ANCHORED ? tile_mag(wmag) : 0.f;
     const Acc gv = gb.at(vm * moff);
     for (int g0 = 0; g0 < nbins; g0 += G) {
         const int gn = nbins - g0 < G ? nbins - g0 : G;
@@ -696,9 +655,7 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
                 dfi = false;
             }
             const int p0 = bstart[g0 + b], p1 = bstart[g0 + b + 1];
-            const float anc = ANCHORED && live && dfi
-                                  ? acc_anchor(tmag * (float)((p1 - p0 + kSpreadSub - 1) / kSpreadSub)) : 0.f;
-            acc2 a00{anc, 0.f}, a01{anc, 0.f}, a10{anc, 0.f}, a11{anc, 0.f};
+            acc2 a00{0.f, 0.f}, a01{0.f, 0.f}, a10{0.f, 0.f}, a11{0.f, 0.f};
             if (live && dfi) {
                 const float2* up = Ud + 2 * pr;
 #pragma unroll 2
@@ -706,10 +663,10 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
                     const float4 uu = *(const float4*)(up + p * sud);
                     const float4 yv = Y[p];
                     const df u0{uu.x, uu.y}, u1{uu.z, uu.w}, yr{yv.x, yv.y}, yi{yv.z, yv.w};
-                    acc_mul<ANCHORED>(a00, u0, yr);
-                    acc_mul<ANCHORED>(a01, u0, yi);
-                    acc_mul<ANCHORED>(a10, u1, yr);
-                    acc_mul<ANCHORED>(a11, u1, yi);
+                    acc_fma(a00, u0, yr);
+                    acc_fma(a01, u0, yi);
+                    acc_fma(a10, u1, yr);
+                    acc_fma(a11, u1, yi);
                 }
             } else if (live) {
                 const float* up = Uf + 2 * pr;
@@ -722,12 +679,6 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
                     a10.s = fmaf(uu.y, yv.x, a10.s);
                     a11.s = fmaf(uu.y, yv.z, a11.s);
                 }
-            }
-            if (ANCHORED) {
-                a00.s -= anc;
-                a01.s -= anc;
-                a10.s -= anc;
-                a11.s -= anc;
             }
             // lanes exchange halves: lane sub ends with degree e0 + (sub >> 2),
             // part (re, im) = (sub >> 1) & 1, then the last pair is summed
@@ -1106,12 +1057,8 @@ __global__ void __launch_bounds__(256, 3) k_asy_spread(const ProbParams* __restr
     const Acc gb = Acc{(double*)grid_b, probs[B.prob].fxs}.at(2 * B.b_off);
     const int64_t moff = 2 * gb_stride;
     if ((mode & 3) == 2) {
-        if (tab.anchored)
-            spread_fold<true, MULTI>(B, probs[B.prob], t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V, moff,
-                                     gb, smem4, sh);
-        else
-            spread_fold<false, MULTI>(B, probs[B.prob], t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V,
-                                      moff, gb, smem4, sh);
+        spread_fold<MULTI>(B, probs[B.prob], t, tab, fold_unpack(mode), r_s, r2, c2, c_stride, V, moff, gb, smem4,
+                           sh);
     } else if (mode & 3) {
         // c_j (r_j/rho)^(-q-1/2) e^{i w_c x_j} onto the 2 N1 + 1 modes
         const int nf1 = 2 * B.N1 + 1;
@@ -1133,24 +1080,18 @@ __global__ void __launch_bounds__(256, 3) k_asy_spread(const ProbParams* __restr
                 fr *= rat.h;
                 fi *= rat.h;
             }
-            return mag_of(xh[0], xh[1]);   // the ratio is at most one
         };
-        auto target = [&](int64_t j, df* v, float* xh, float* xl, float* mag) {
+        auto target = [&](int64_t j, df* v, float* xh, float* xl) {
             long long Xp;
             const int l0 = spread_cell_fx(B, tab.w, r_s[j], &Xp, v);
             spread_weight_fx(B, tab.tw2, Xp, r2[j], make_float2(1.f, 0.f), &yr, &yi, &rat);
             jt = j;
-            *mag = put(xh, xl, c2[j]);
+            put(xh, xl, c2[j]);
             return l0;
         };
-        auto values = [&](int vm, float* xh, float* xl) { return put(xh, xl, c2[vm * c_stride + jt]); };
+        auto values = [&](int vm, float* xh, float* xl) { put(xh, xl, c2[vm * c_stride + jt]); };
         auto cell = [&](int c) -> int64_t { const int x = c + B.N1; return (x >= 0 && x < nf1) ? x : -1; };
-        if (tab.anchored)
-            spread_moments<true>(probs[B.prob], t, tab, target, values, MULTI ? V : 1, moff, cell, gb,
-                                 (float*)smem4, sh);
-        else
-            spread_moments<false>(probs[B.prob], t, tab, target, values, MULTI ? V : 1, moff, cell, gb,
-                                  (float*)smem4, sh);
+        spread_moments(probs[B.prob], t, tab, target, values, MULTI ? V : 1, moff, cell, gb, (float*)smem4, sh);
     }
     else
         spread_taps<MULTI>(B, Q, t, tab, r_s, r2, c2, c_stride, V, moff, gb, smem4);
@@ -1564,14 +1505,13 @@ __device__ __forceinline__ int adj_spread_factor(const AsyBlock& B, const ProbPa
 }
 
 // The 2M values x_q for g_k from the frequency's factor, handed to put(q, re,
-// im); returns a bound of their magnitudes.
+// im).
 template <class Put>
-__device__ __forceinline__ float adj_values(const ProbParams& P, const AdjFactor& F, double gk, Put&& put)
+__device__ __forceinline__ void adj_values(const ProbParams& P, const AdjFactor& F, double gk, Put&& put)
 {
     const df g = df_from(gk);
     const df fr = df_mul(F.fr, g), fi = df_mul(F.fi, g), mz = F.mz;
     df mq{1.f, 0.f};
-    float mag = 0.f;
     for (int q = 0; q < P.Q; ++q) {
         const df cq = df_mul(df{P.a2[q].x, P.a2[q].y}, mq);
         // (fr + i fi) i^q cq
@@ -1585,10 +1525,8 @@ __device__ __forceinline__ float adj_values(const ProbParams& P, const AdjFactor
         ur = df_mul(ur, cq);
         ui = df_mul(ui, cq);
         put(q, ur, ui);
-        mag = fmaxf(mag, mag_of(ur.h, ui.h));
         mq = df_mul(mq, mz);
     }
-    return mag;
 }
 
 // Frequencies of a tile -> FFT grid (periodic, atomics into tgrid).  Dense
@@ -1628,25 +1566,20 @@ __global__ void __launch_bounds__(kInterpTileThreads, 3) k_asy_adj_spread(const 
         int64_t kt = 0;
         const int nlow = 2 * P.nlow;   // terms kept in double-float
         auto put = [&](float* xh, float* xl, double gk) {
-            return adj_values(P, F, gk, [&](int q, df re, df im) {
+            adj_values(P, F, gk, [&](int q, df re, df im) {
                 *(float2*)(xh + 2 * q) = make_float2(re.h, im.h);
                 if (q < nlow) *(float2*)(xl + 2 * q) = make_float2(re.l, im.l);
             });
         };
-        auto target = [&](int64_t k, df* v, float* xh, float* xl, float* mag) {
+        auto target = [&](int64_t k, df* v, float* xh, float* xl) {
             const int t0 = adj_spread_factor(B, P, tab, w_s[k], v, &F);
             kt = k;
-            *mag = put(xh, xl, g_s[k]);
+            put(xh, xl, g_s[k]);
             return t0;
         };
-        auto values = [&](int vm, float* xh, float* xl) { return put(xh, xl, g_s[vm * g_stride + kt]); };
+        auto values = [&](int vm, float* xh, float* xl) { put(xh, xl, g_s[vm * g_stride + kt]); };
         auto cell = [&](int c) -> int64_t { return c & mask; };
-        if (tab.anchored)
-            spread_moments<true>(P, t, tab, target, values, MULTI ? V : 1, 2 * tg_stride, cell, tg,
-                                 (float*)sma, sh);
-        else
-            spread_moments<false>(P, t, tab, target, values, MULTI ? V : 1, 2 * tg_stride, cell, tg,
-                                  (float*)sma, sh);
+        spread_moments(P, t, tab, target, values, MULTI ? V : 1, 2 * tg_stride, cell, tg, (float*)sma, sh);
         return;
     }
     const int ncoef = w * (deg + 1);

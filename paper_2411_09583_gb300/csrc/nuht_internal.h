@@ -22,10 +22,6 @@ constexpr int kMaxDeg = 20;         // degree of the kernel piece polynomials
 // spreading grid then has N1 ~ 2 X S / pi + w/2 <= ~2.04e6 cells and its FFT
 // at most 2^23 points (the single-FFT limit is 2^kFftMaxLog2).
 constexpr double kAsyMaxXS = 3.2e6;
-// Tolerance from which the spreading sums are anchored: their rounding
-// (measured ~3e-13 of the result, against ~1e-14 for the compensated sums)
-// stays far below it.
-constexpr double kAnchorMinEps = 1e-11;
 constexpr int kMomFold = 32;        // FP32 partial sums of the spreading moments span at most this many points
 constexpr int kMaxNtop = 400;       // largest Bessel index kept by the local evaluation
                                     // (the transposed moments then stay within 205 KB of shared memory)
@@ -256,7 +252,6 @@ struct Tables {
     float fold_tol;        // truncation of the spreading weights' Chebyshev form within a bin
     float fold_df_tol;     // weights' Chebyshev terms above this need double-float moments
     double half_w;         // w / 2
-    int anchored;          // anchored accumulation (acc_fma_anchored): eps >= kAnchorMinEps
     const float2* ph2;     // psi-hat pieces [ph_pieces][ph_deg + 1] in v in [-1, 1], double-float
     double interp_const;   // sqrt(2/pi) * 4 / w^2
     float2 ic2;            // the same as double-float

@@ -1024,7 +1024,6 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
             if (acc <= kRoundBudget * P->eps) --dci; else break;
         }
         tb.dci = dci;
-        tb.anchored = P->eps >= kAnchorMinEps;
         // q-folded spreading: the weights' Chebyshev terms are kept down to
         // 1e-3 eps; a term above kRoundBudget eps / ((kMomFold + 2) 2^-23) multiplies
         // moments whose FP32 partial sums (kMomFold points) would show, so

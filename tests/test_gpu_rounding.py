@@ -1,0 +1,39 @@
+"""The rounding of the asymptotic pipeline, apart from its truncation.
+
+The transform is linear, and its truncation with it: what execute(3 c) / 3 and
+execute(c) differ by is rounding alone (3 c rounds to 2^-53 of itself).  The sums
+are compensated pairs of floats (48 bits) except where an FP32 tier keeps its bound
+below a tenth of the tolerance.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from gpu_helpers import to_dev  # noqa: E402
+
+
+def _rms(x):
+    return np.sqrt(np.mean(x * x))
+
+
+def _noise(nu, eps, n, cells, seed):
+    # one asymptotic block, r in [1, 2] over `cells` cells of the spreading grid
+    from paper_2411_09583_gb300 import Plan
+    rng = np.random.default_rng(seed)
+    s = 0.5 * np.pi * cells
+    r, omega = rng.uniform(1.0, 2.0, n), rng.uniform(600.0, 600.0 + 2 * s, n)
+    out = []
+    with Plan(nu, to_dev(r), to_dev(omega), eps) as p:
+        for apply, x in ((p.execute, rng.standard_normal(n)), (p.adjoint, rng.standard_normal(n))):
+            y, y3 = apply(to_dev(x)).cpu().numpy(), apply(to_dev(3.0 * x)).cpu().numpy()
+            out.append(_rms(y3 / 3.0 - y) / _rms(y))
+    return out
+
+
+@pytest.mark.parametrize("nu,n,cells", [(0, 4000, 3), (0, 4000, 30), (17, 4000, 30), (1, 20000, 100)])
+def test_dense_sums_keep_their_48_bits(nu, n, cells):
+    # eps = 1e-11: the budget of the four FP32 tiers is 0.1 eps each for some 40
+    # roundings of one sign; of random signs they leave 4 * 0.1 eps / 40 = 1e-13
+    noise = np.mean([_noise(nu, 1e-11, n, cells, seed) for seed in range(3)], axis=0)
+    assert np.all(noise <= 1e-13), noise
