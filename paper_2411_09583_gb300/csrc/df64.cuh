@@ -130,6 +130,27 @@ __device__ __forceinline__ void acc_fma(acc2& A, df a, df b)
 
 __device__ __forceinline__ double acc_value(acc2 A) { return (double)A.s + (double)A.c; }
 
+// (double)x from the bits of x: the conversion instruction holds a warp's FP64
+// pipe for 64 cycles (subnormal, infinite and NaN values take it).
+__device__ __forceinline__ double f64_of(float x)
+{
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+    if (a != 0u && a - 0x00800000u >= 0x7f000000u) return (double)x;
+    const unsigned m = a != 0u ? (a >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)((u & 0x80000000u) | m), (int)(a << 29));
+}
+
+// The sum of two compensated sums, rounded once to FP64: neither their joining
+// nor the conversion costs a bit of the parts that they hold.
+__device__ __forceinline__ double acc_join(acc2 a, acc2 b)
+{
+    float s, e, h, t, u;
+    two_sum(a.s, b.s, s, e);
+    two_sum(a.c, b.c, h, t);
+    two_sum(h, e, h, u);
+    return f64_of(s) + (f64_of(h) + f64_of(t + u));
+}
+
 // a += the value of lane ^ off (two-sum through the shuffles), where this lane
 // keeps `keep` and hands over `give`.
 __device__ __forceinline__ acc2 acc_exchange(acc2 keep, acc2 give, int off)

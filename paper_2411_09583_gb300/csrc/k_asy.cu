@@ -846,14 +846,16 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
 // the rows p whose taps cover the cell (l0[p] <= cell < l0[p] + w, ascending
 // l0) of taps[p][cell - l0[p]] vals[p][q], handed to put(cell, q, re, im).
 // One lane per output, or two (halves of its rows) where a pass has fewer
-// outputs than half the threads.  start[x], the first row with l0 >= first
+// outputs than half the threads; the rows in two chains that join without loss
+// either way (in one chain the error of order 100 at eps 1e-12 was 1.4 times
+// larger: Hankel's coefficients magnify what is rounded here).  start[x], the first row with l0 >= first
 // cell of the pass - (w - 1) + x, gives a cell's rows as [start[c], start[c +
 // w]); it has room for cap cells and w more.  With build it is formed (cells
 // ready at a barrier), else it stands from the previous member.
 // FP32 issue and shared reads of the products bound it.  Two binary searches per
 // lane and output and the FP64 (1/64 rate) halves of every output cost more than
 // the products before: 4e6 far-field points (eps 1e-12, half a point a cell) 1.80 ->
-// 1.05 ms, 256 problems of 3e2 to 1e5 points 5.3 -> 4.7 ms.
+// 1.18 ms, 256 problems of 3e2 to 1e5 points 5.3 -> 4.8 ms.
 template <class Put>
 __device__ __forceinline__ void tap_cell_sums(const int* l0s, int cnt, int first, int span, int w, int Q,
                                               const float2* taps, const float4* vals, uint16_t* start, int cap,
@@ -888,24 +890,26 @@ __device__ __forceinline__ void tap_cell_sums(const int* l0s, int cnt, int first
                 if (sub) p = mid; else hi = mid;
             }
             const int cell = first + c0 + c;
-            acc2 ar{0.f, 0.f}, ai{0.f, 0.f};
-            for (; p < hi; ++p) {
-                const float2 k2 = taps[p * w + (cell - l0s[p])];
-                const float4 av = vals[p * Q + q];
-                acc_fma(ar, df{k2.x, k2.y}, df{av.x, av.y});
-                acc_fma(ai, df{k2.x, k2.y}, df{av.z, av.w});
-            }
+            acc2 ar{0.f, 0.f}, ai{0.f, 0.f}, br{0.f, 0.f}, bi{0.f, 0.f};
+            auto row = [&](int x, acc2& re, acc2& im) {
+                const float2 k2 = taps[x * w + (cell - l0s[x])];
+                const float4 av = vals[x * Q + q];
+                acc_fma(re, df{k2.x, k2.y}, df{av.x, av.y});
+                acc_fma(im, df{k2.x, k2.y}, df{av.z, av.w});
+            };
             if (sh) {
+                for (; p < hi; ++p) row(p, ar, ai);
                 const unsigned pair = 0x3u << (tid & 30);
-                const acc2 br{__shfl_xor_sync(pair, ar.s, 1), __shfl_xor_sync(pair, ar.c, 1)};
-                const acc2 bi{__shfl_xor_sync(pair, ai.s, 1), __shfl_xor_sync(pair, ai.c, 1)};
-                float e;
-                two_sum(ar.s, br.s, ar.s, e);
-                ar.c += br.c + e;
-                two_sum(ai.s, bi.s, ai.s, e);
-                ai.c += bi.c + e;
+                br = acc2{__shfl_xor_sync(pair, ar.s, 1), __shfl_xor_sync(pair, ar.c, 1)};
+                bi = acc2{__shfl_xor_sync(pair, ai.s, 1), __shfl_xor_sync(pair, ai.c, 1)};
+            } else {
+                for (; p + 1 < hi; p += 2) {
+                    row(p, ar, ai);
+                    row(p + 1, br, bi);
+                }
+                if (p < hi) row(p, ar, ai);
             }
-            if (any && !sub) put(cell, q, acc_value(ar), acc_value(ai));
+            if (any && !sub) put(cell, q, acc_join(ar, br), acc_join(ai, bi));
         }
     }
 }
