@@ -146,6 +146,7 @@ struct MomShared {
 };
 
 constexpr int kMomBins = 2;         // bins whose moments are formed and added to the grid together
+static_assert(kMomBins <= 2, "the grid update joins the sums of two bins");
 // Tiles with at least this many points per bin use moments (spreading) or per-bin
 // sums (interpolation).  One line for all four stages: the dense paths cut the
 // taps' Chebyshev tail at 1e-3 eps, and the adjoint is the forward's transpose to
@@ -388,9 +389,13 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
             if (idx < 0) continue;
             const int ed = (qv >> 1) < qs ? 2 * L.ndf : 0;
             const int b_lo = c - w + 1 > 0 ? c - w + 1 : 0, b_hi = c < gn - 1 ? c : gn - 1;
-            acc2 s{0.f, 0.f};
+            acc2 s{0.f, 0.f}, s1{0.f, 0.f};   // of either bin: joined without rounding
             float sf = 0.f;
             for (int b = b_lo; b <= b_hi; ++b) {
+                if (b > b_lo) {
+                    s1 = s;
+                    s = acc2{0.f, 0.f};
+                }
                 const float2* ar = Ach + (c - b) * L.dpad;
                 const float2* mb = Mb + b * L.dpad * Q2 + qv;
                 int e = 0;
@@ -400,12 +405,9 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
                 }
                 for (; e < L.dpad; ++e) sf = fmaf(ar[e].x, mb[e * Q2].x, sf);
             }
-            // (one FP64 sum per value: FP64 issues 64 times slower)
-            float h, l;
-            two_sum(s.s, sf, h, l);
-            l += s.c;
-            if (h != 0.f || l != 0.f)
-                gv.add(2 * ((int64_t)idx * Q + (qv >> 1)) + (qv & 1), (double)h + (double)l);
+            const double val = acc_join(s, s1) + f64_of(sf);
+            if (__double_as_longlong(val) << 1)   // (an integer test: FP64 issues 64 times slower)
+                gv.add(2 * ((int64_t)idx * Q + (qv >> 1)) + (qv & 1), val);
         }
         __syncthreads();
     }
