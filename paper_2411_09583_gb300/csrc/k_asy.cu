@@ -2194,7 +2194,7 @@ cudaError_t launch_asy_adj_spread(const ProbParams* probs, const AsyBlock* blks,
                       sizeof(float2) * (size_t)n * tab.w + sizeof(int) * (size_t)n;
         const size_t smem_mom = spread_moments_smem(n, qmax, tab.nlow, tab.w, tab.nb, tab.dcs);
         if (smem_mom > smem) smem = smem_mom;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<ntiles, n, smem, s>>>(probs, blks, tiles, tab, w_s, g_s, g_stride, members, tgrid, tg_stride, over, n);
         e = cudaGetLastError();
@@ -2213,7 +2213,7 @@ cudaError_t launch_asy_adj_interp(const ProbParams* probs, const AsyBlock* blks,
     const size_t smem = interp_smem(qmax, tab.w, tab.deg, kAdjInterpThreads, kAdjInterpHBytes);
     if (members < 1) return cudaErrorInvalidValue;
     auto kern = members > 1 ? k_asy_adj_interp<true> : k_asy_adj_interp<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<ntiles, kAdjInterpThreads, smem, s>>>(probs, blks, tiles, tab, r_s, bgrid, bg_stride, members, c_s,
                                                  c_stride);
@@ -2236,7 +2236,7 @@ cudaError_t launch_asy_spread_f32(const ProbParams* probs, const AsyBlock* blks,
                       sizeof(float) * (size_t)n * tab.w + sizeof(int) * (size_t)n;
         const size_t smem_mom = spread_moments_f32_smem(n, qmax, tab.w, tab.nb);
         if (smem_mom > smem) smem = smem_mom;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<ntiles, n, smem, s>>>(probs, blks, tiles, modes, tab, r_s, r2, c2, c_stride, members, grid_b,
                                      gb_stride, over, n);
@@ -2266,7 +2266,7 @@ cudaError_t launch_asy_interp_f32(const ProbParams* probs, const AsyBlock* blks,
                                    : std::min(kInterpHBytesPerThread * nt,
                                               std::max(kInterpHBytesPerThread * n, (bins + 15) & ~15));
         const size_t smem = interp_f32_smem(qmax, tab.w, tab.deg, n, hbytes);
-        cudaError_t e = cudaFuncSetAttribute(k_asy_interp_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_asy_interp_f32, smem);
         if (e != cudaSuccess) return e;
         k_asy_interp_f32<<<ntiles, n, smem, s>>>(probs, blks, tiles, tab, w_s, w2, grid_q, gq_stride, members, g_s,
                                                  g_stride, hbytes, over, n);
@@ -2309,7 +2309,7 @@ cudaError_t launch_asy_spread(const ProbParams* probs, const AsyBlock* blks, con
         if (smem_mom > smem) smem = smem_mom;
         const size_t smem_fold = spread_fold_smem(n, qmax, tab.w, tab.nb, tab.dcs);
         if (smem_fold > smem) smem = smem_fold;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<ntiles, n, smem, s>>>(probs, blks, tiles, modes, tab, r_s, r2, c2, c_stride, members, grid_b,
                                      gb_stride, over, n);
@@ -2339,7 +2339,7 @@ cudaError_t launch_asy_interp(const ProbParams* probs, const AsyBlock* blks, con
                                    : std::min(kInterpHBytesPerThread * nt,
                                               std::max(kInterpHBytesPerThread * n, (bins + 15) & ~15));
         const size_t smem = interp_smem(qmax, tab.w, tab.deg, n, hbytes);
-        cudaError_t e = cudaFuncSetAttribute(k_asy_interp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_asy_interp, smem);
         if (e != cudaSuccess) return e;
         k_asy_interp<<<ntiles, n, smem, s>>>(probs, blks, tiles, tab, w_s, w2, grid_q, gq_stride, members, g_s,
                                              g_stride, hbytes, over, n);

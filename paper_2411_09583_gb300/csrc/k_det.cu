@@ -7,6 +7,9 @@
 // largest magnitude lies in [1, 2), and scales the output back by 2^E: both
 // exact in FP64, and the transform is linear, so any finite input range works.
 #include <cstdint>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "nuht_internal.h"
 
@@ -96,6 +99,21 @@ int device_sm_count()
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
     if (dev >= 0 && dev < 64) cache[dev] = sms;
     return sms;
+}
+
+cudaError_t allow_smem_of(const void* kernel, size_t bytes)
+{
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, size_t> allowed;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& most = allowed[{kernel, dev}];
+    if (bytes <= most) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) most = bytes;
+    return e;
 }
 
 cudaError_t launch_prepare(const ZeroList& Z, const double* x, int64_t count, const int32_t* perm, const double* ws,

@@ -649,7 +649,7 @@ cudaError_t launch_asy_fft(const ProbParams* probs, const AsyBlock* blks, const 
     if (members < 1 || members > 65535) return cudaErrorInvalidValue;
     auto kern = pass == 0 ? (adj ? k_asy_fft<true, true> : k_asy_fft<false, true>)
                           : (adj ? k_asy_fft<true, false> : k_asy_fft<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(nitems, members), kFftThreads, smem, s>>>(probs, blks, items, tab, pass, src, tmp, dst, src_stride,
                                                           tmp_stride, dst_stride);
@@ -664,7 +664,7 @@ cudaError_t launch_asy_fft_small_f32(const ProbParams* probs, const AsyBlock* bl
     if (nitems <= 0) return cudaSuccess;
     if (members < 1 || members > 65535) return cudaErrorInvalidValue;
     size_t smem = sizeof(float2) * (size_t)max_nf2;
-    cudaError_t e = cudaFuncSetAttribute(k_asy_fft_small_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_asy_fft_small_f32, smem);
     if (e != cudaSuccess) return e;
     int nt = max_nf2 / 2;
     if (nt > 256) nt = 256;
@@ -697,7 +697,7 @@ cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* bl
         if (nt > 256) nt = 256;
         if (nt < 32) nt = 32;
         auto kern = r ? k_asy_fft_block_f32<true> : k_asy_fft_block_f32<false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         int gx = nitems;
         if (r) gx = std::min(nitems, std::max((nitems + nt - 1) / nt, kFftScanCtas));

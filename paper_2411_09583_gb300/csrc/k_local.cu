@@ -1835,7 +1835,7 @@ cudaError_t launch_local_adj_moments(const ProbParams* probs, const LocalBlock* 
     size_t smem = sizeof(float2) * (size_t)(ntop_max + 1) * threads + (sizeof(float2) + sizeof(float)) * threads +
                   (two ? sizeof(float2) * threads : 0);
     auto kern = two ? k_local_adj_moments<true> : k_local_adj_moments<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<ntiles, threads, smem, s>>>(probs, blks, tiles, w2, g_s, mom, g_sb, momb);
     count_launches(1);
@@ -1860,7 +1860,7 @@ cudaError_t launch_direct_adj(const ProbParams* probs, const DirectBlock* blks, 
     if (nblk <= 0) return cudaSuccess;
     size_t smem = sizeof(double) * (det ? 1 : (size_t)(max_cols > 0 ? max_cols : 1)) +
                   sizeof(int) * (size_t)max_area;
-    cudaError_t e = cudaFuncSetAttribute(k_direct_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_direct_adj, smem);
     if (e != cudaSuccess) return e;
     k_direct_adj<<<nblk, 256, smem, s>>>(probs, blks, r_s, w_s, r2, w2, g_s, c_s, lowp, det);
     count_launches(1);
@@ -1874,8 +1874,7 @@ cudaError_t launch_local_moments(const ProbParams* probs, const LocalBlock* blks
     if (ntiles <= 0) return cudaSuccess;
     const int threads = local_moment_threads(lmax);
     size_t smem = sizeof(acc2) * (size_t)(lmax + 1) * threads;
-    cudaError_t e = cudaFuncSetAttribute(k_local_moments, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_moments, smem);
     if (e != cudaSuccess) return e;
     k_local_moments<<<ntiles, threads, smem, s>>>(probs, blks, tiles, r2, c2, mom);
     count_launches(1);
@@ -1893,8 +1892,7 @@ cudaError_t launch_local_moments2(const ProbParams* probs, const LocalBlock* blk
     const int threads = local_moment_threads(lmax);
     const size_t smem = 2 * sizeof(acc2) * (size_t)(lmax + 1) * threads;
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_local_moments2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_moments2, smem);
     if (e != cudaSuccess) return e;
     k_local_moments2<<<ntiles, threads, smem, s>>>(probs, blks, tiles, r2, c2, c2b, mom, momb);
     count_launches(1);
@@ -1936,8 +1934,7 @@ cudaError_t launch_local_eval(const ProbParams* probs, const LocalBlock* blks, c
     // rows of order 0 keep no Bessel column (their sums are formed during the sweep)
     const size_t col = nu_max > 0 ? (size_t)(std::min(nu_max, ntop_max) + 1) * threads : 0;
     size_t smem = sizeof(float2) * (col + nmu * (size_t)(ntop_max + 1));
-    cudaError_t e = cudaFuncSetAttribute(k_local_eval, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_eval, smem);
     if (e != cudaSuccess) return e;
     k_local_eval<<<ntiles, threads, smem, s>>>(probs, blks, tiles, w2, mom, g_s, momb, g_sb);
     count_launches(1);
@@ -1956,7 +1953,7 @@ cudaError_t launch_local_persistent(const ProbParams* probs, const LocalBlock* b
     const size_t sm_mom = sizeof(acc2) * (size_t)(lmax + 1) * threads;
     const size_t sm_eval = sizeof(float2) * ((size_t)(ntop_max + 1) * threads + nmu * (size_t)(ntop_max + 1));
     const size_t smem = sm_mom > sm_eval ? sm_mom : sm_eval;
-    cudaError_t e = cudaFuncSetAttribute(k_local_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_local_persistent, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     e = cudaGetDevice(&dev);
@@ -1999,8 +1996,7 @@ cudaError_t launch_local_eval_f32(const ProbParams* probs, const LocalBlock* blk
     if (ntiles <= 0) return cudaSuccess;
     const size_t nmu = momb ? 2 : 1;
     size_t smem = sizeof(float) * ((size_t)(ntop_max + 1) * threads + nmu * (size_t)(ntop_max + 1));
-    cudaError_t e = cudaFuncSetAttribute(k_local_eval_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_eval_f32, smem);
     if (e != cudaSuccess) return e;
     k_local_eval_f32<<<ntiles, threads, smem, s>>>(probs, blks, tiles, w2, mom, g_s, momb, g_sb);
     count_launches(1);
@@ -2017,7 +2013,7 @@ cudaError_t launch_direct(const ProbParams* probs, const DirectBlock* blks, int 
     const size_t acc = det ? 1 : (g_sb ? 2 : 1) *
                        (mode == 2 ? (size_t)kDirSlotFloats / 2 : (size_t)(max_rows > 0 ? max_rows : 1));
     size_t smem = sizeof(double) * acc + sizeof(int) * (size_t)max_area;
-    cudaError_t e = cudaFuncSetAttribute(k_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_direct, smem);
     if (e != cudaSuccess) return e;
     k_direct<<<nblk, 256, smem, s>>>(probs, blks, r_s, w_s, r2, w2, c_s, c2, g_s, c_sb, c2b, g_sb, mode, det);
     count_launches(1);
@@ -2040,8 +2036,7 @@ cudaError_t launch_local_moments_group(const ProbParams* probs, const LocalBlock
     if (ntiles <= 0) return cudaSuccess;
     if (G < 1 || G > kGroupMax || (lmax + 1) * G > kMomGroupOut * kMomThreads) return cudaErrorInvalidValue;
     const size_t smem = sizeof(float2) * (size_t)(lmax + 1 + G) * (kMomThreads + 8);
-    cudaError_t e = cudaFuncSetAttribute(k_local_moments_group, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_moments_group, smem);
     if (e != cudaSuccess) return e;
     k_local_moments_group<<<ntiles, kMomThreads, smem, s>>>(probs, blks, tiles, r2, c2, c_stride, G, mom,
                                                             mom_stride);
@@ -2055,8 +2050,7 @@ static cudaError_t eval_group_as(const ProbParams* probs, const LocalBlock* blks
                                  int64_t mom_stride, int G, double* g_s, int64_t g_stride, cudaStream_t s)
 {
     const size_t smem = sizeof(float2) * (size_t)(ntop_max + 1) * (threads + GM);
-    cudaError_t e = cudaFuncSetAttribute(k_local_eval_group<GM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(k_local_eval_group<GM>, smem);
     if (e != cudaSuccess) return e;
     k_local_eval_group<GM><<<ntiles, threads, smem, s>>>(probs, blks, tiles, w2, mom, mom_stride, G, g_s,
                                                           g_stride);
@@ -2088,7 +2082,7 @@ cudaError_t launch_direct_group(const ProbParams* probs, const DirectBlock* blks
     if (nblk <= 0) return cudaSuccess;
     if (G < 1 || G > kGroupMax) return cudaErrorInvalidValue;
     const size_t smem = (sizeof(float2) + sizeof(int)) * (size_t)(max_area > 0 ? max_area : 1);
-    cudaError_t e = cudaFuncSetAttribute(k_direct_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_direct_group, smem);
     if (e != cudaSuccess) return e;
     k_direct_group<<<nblk, 128, smem, s>>>(probs, blks, r_s, w_s, r2, w2, c2, c_stride, G, g_s, g_stride, lowp);
     count_launches(1);
@@ -2104,16 +2098,14 @@ static cudaError_t adj_group_as(const ProbParams* probs, const LocalBlock* blks,
     if (moments) {
         if (n_teval <= 0) return cudaSuccess;
         const size_t smem = sizeof(float2) * (size_t)(ntop_max + 1 + GM) * threads + sizeof(float) * threads;
-        cudaError_t e = cudaFuncSetAttribute(k_local_adj_moments_group<GM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_local_adj_moments_group<GM>, smem);
         if (e != cudaSuccess) return e;
         k_local_adj_moments_group<GM><<<n_teval, threads, smem, s>>>(probs, blks, teval, w2, g_s, g_stride, G, mom,
                                                                      mom_stride);
     } else {
         if (n_tmom <= 0) return cudaSuccess;
         const size_t smem = sizeof(float2) * (size_t)(lmax + 1) * GM;
-        cudaError_t e = cudaFuncSetAttribute(k_local_adj_eval_group<GM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = allow_smem(k_local_adj_eval_group<GM>, smem);
         if (e != cudaSuccess) return e;
         k_local_adj_eval_group<GM><<<n_tmom, kMomThreads, smem, s>>>(probs, blks, tmom, r2, mom, mom_stride, G, c_s,
                                                                      c_stride);

@@ -215,7 +215,7 @@ extern "C" int nuht_local_apply_noalloc(int nu, double eps, const double* r, int
     {
         const int threads = local_moment_threads(L);   // (L + 1) doubles per thread
         const size_t smem = sizeof(double) * (size_t)(L + 1) * threads;
-        e = cudaFuncSetAttribute(k_noalloc_moments, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_noalloc_moments, smem);
         if (e != cudaSuccess) return NUHT_ERR_CUDA;
         int dev = 0, sms = 0;
         e = cudaGetDevice(&dev);
@@ -233,7 +233,7 @@ extern "C" int nuht_local_apply_noalloc(int nu, double eps, const double* r, int
     {
         const int threads = local_eval_threads(ntop);
         const size_t smem = sizeof(double) * (size_t)(ntop + 1) * threads;
-        e = cudaFuncSetAttribute(k_noalloc_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem(k_noalloc_eval, smem);
         if (e != cudaSuccess) return NUHT_ERR_CUDA;
         const int64_t blocks = (m + threads - 1) / threads;
         k_noalloc_eval<<<(unsigned)blocks, threads, smem, s>>>(anu, sgn, L, ntop, omega, m, Rm, mom, nvec, g);

@@ -746,7 +746,7 @@ template <int ITEMS>
 cudaError_t sort_small(const SortPair& S, cudaStream_t s)
 {
     const size_t smem = sizeof(uint2) * kSmallThreads * ITEMS + sizeof(uint32_t) * 32 * kRadix;
-    cudaError_t e = cudaFuncSetAttribute(k_sort_small<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_sort_small<ITEMS>, smem);
     if (e != cudaSuccess) return e;
     k_sort_small<ITEMS><<<2, kSmallThreads, smem, s>>>(S);
     count_launches(1);

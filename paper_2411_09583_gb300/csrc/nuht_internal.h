@@ -268,6 +268,15 @@ struct Tables {
 // (each returns cudaGetLastError() of its launch and adds the number of
 // kernels it launched to the library's launch counter)
 void count_launches(int k);
+// Lets a kernel be launched with `bytes` of dynamic shared memory on the current
+// device (k_det.cu).  The attribute belongs to the process: it is only ever
+// raised, so that no host thread lowers it between another's call and its launch.
+cudaError_t allow_smem_of(const void* kernel, size_t bytes);
+template <class Kernel>
+cudaError_t allow_smem(Kernel* kernel, size_t bytes)
+{
+    return allow_smem_of((const void*)kernel, bytes);
+}
 // Sorting a plan's points (a[0]) and frequencies (a[1]) (k_sort.cu).
 constexpr int kSmallSort = 8192;   // up to this many of each: one CTA per array, one launch
 struct SortArray {
