@@ -12,12 +12,14 @@
 // that the input spans (zero has a key of its own), in four 8-bit passes
 // instead of the eight a 64-bit pattern takes and over 8-byte (key, index)
 // pairs instead of 12 bytes; the few values that share a key are then ordered
-// by their full patterns where they lie.  Points and frequencies share every
+// by their full patterns where they lie, or, if they are many, by passes over the
+// bits that the key left out.  Points and frequencies share every
 // launch, and up to kSmallSort of each are sorted by one CTA in one launch.
 // Measured, both arrays on an idle GPU (sum of the launches): n = m = 1e6
 // 0.45 ms in 52 launches on two streams -> 0.17 in 15; 1e5 0.16 -> 0.06; 2000
 // 48 launches -> one of 0.02.  Bound by the scatters' 8-byte stores (L2) at
 // 1e6 and by launch latency below 1e5.
+#include <cooperative_groups.h>
 #include <cstdint>
 
 #include "df64.cuh"
@@ -53,11 +55,8 @@ struct SortQuant {
     uint64_t lo;
     int shift;
     __device__ __forceinline__ uint32_t key(uint64_t b) const { return b == 0 ? 0u : 1u + (uint32_t)((b - lo) >> shift); }
-    // digit of the bits below the key, from bit `at` on
-    __device__ __forceinline__ unsigned low(uint64_t b, int at) const
-    {
-        return (unsigned)(((b - lo) & ((1ull << shift) - 1)) >> at) & 0xFFu;
-    }
+    // the bits below the key (32 at most, for a finite range)
+    __device__ __forceinline__ uint32_t low(uint64_t b) const { return (uint32_t)((b - lo) & ((1ull << shift) - 1)); }
 };
 
 // stats[0] = the largest ~bits over non-zero values, stats[1] = the largest bits
@@ -143,6 +142,25 @@ __device__ __forceinline__ int sort_tile_of(const SortPair& S, int blk, int* til
     return w;
 }
 
+// Adds a tile's digit counts to h.  SKEWED: many elements may share a digit (a
+// warp's are then added once).
+template <int KIND, bool SKEWED>
+__device__ __forceinline__ void sort_count_tile(const SortArray& A, const SortQuant& q, int nseg, int from, int shift,
+                                                int tile, uint32_t* h)
+{
+    const int64_t base = (int64_t)tile * kSortTile;
+#pragma unroll
+    for (int it = 0; it < kSortItems; ++it) {
+        const int64_t i = base + it * kSortThreads + threadIdx.x;
+        const unsigned d = i < A.n ? sort_digit<KIND>(A, nseg, sort_load<KIND>(A, q, A.e[from], i), shift) : 0x100u;
+        if (SKEWED && __all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+            if ((threadIdx.x & 31) == 0 && d < 0x100u) atomicAdd(&h[d], 32u);
+        } else if (d < 0x100u) {
+            atomicAdd(&h[d], 1u);
+        }
+    }
+}
+
 // Digit counts of every tile: hist[tile * kRadix + d].
 template <int KIND>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortPair S, int from, int shift)
@@ -151,15 +169,9 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(SortPair S, int from
     int tile;
     const SortArray& A = S.a[sort_tile_of(S, blockIdx.x, &tile)];
     const SortQuant q = KIND == SORT_FIRST ? sort_quant(A.stats) : SortQuant{0, 0};
-    const uint2* src = A.e[from];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)tile * kSortTile;
-#pragma unroll
-    for (int it = 0; it < kSortItems; ++it) {
-        const int64_t i = base + it * kSortThreads + threadIdx.x;
-        if (i < A.n) atomicAdd(&h[sort_digit<KIND>(A, S.nseg, sort_load<KIND>(A, q, src, i), shift)], 1u);
-    }
+    sort_count_tile<KIND, false>(A, q, S.nseg, from, shift, tile, h);
     __syncthreads();
     A.hist[(int64_t)tile * kRadix + threadIdx.x] = h[threadIdx.x];
 }
@@ -186,55 +198,46 @@ __global__ void __launch_bounds__(1024) k_sort_colscan(SortPair S)
     }
 }
 
-// Stable scatter of one pass.  Warp w of a tile owns its 128 consecutive
-// elements, in rounds of 32, so (warp, round, lane) is the input order: each
-// warp ranks its elements among equal digits with a per-warp digit count in
-// shared memory (warp-synchronous, no CTA barrier per round), then one
-// exclusive prefix over the warps per digit places every warp's run after
-// the earlier warps' in the tile's part of each digit bucket.  With DIRECT
-// (few tiles) the CTA forms the counts of the tiles before it and the totals
-// itself instead of a scan launch between.
-template <int KIND, bool DIRECT>
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(SortPair S, int from, int shift)
+struct ScatterShared {
+    uint32_t wcnt[kSortThreads / 32][kRadix];   // per-warp digit counts, then the warps' starts
+    uint32_t wsum[kSortThreads / 32];
+};
+
+// Start of digit threadIdx.x's bucket from its total v: exclusive scan over the
+// digits (blockDim.x == kRadix; all threads).
+__device__ __forceinline__ uint32_t digit_start(uint32_t v, ScatterShared& sh)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += t;
+    }
+    if (lane == 31) sh.wsum[warp] = x;
+    __syncthreads();
+    uint32_t pre = 0;
+    for (int w = 0; w < warp; ++w) pre += sh.wsum[w];
+    return pre + x - v;
+}
+
+// Stable scatter of a tile in one pass, its elements of digit threadIdx.x from
+// mybase on (returned: where the next tile's go).  Warp w of a tile owns its 128
+// consecutive elements, in rounds of 32, so (warp, round, lane) is the input
+// order: each warp ranks its elements among equal digits with a per-warp digit
+// count in shared memory (warp-synchronous, no CTA barrier per round), then one
+// exclusive prefix over the warps per digit places every warp's run after the
+// earlier warps' in the tile's part of each digit bucket.
+template <int KIND>
+__device__ __forceinline__ uint32_t sort_scatter_tile(const SortArray& A, const SortQuant& q, int nseg, int from,
+                                                      int shift, int tile, uint32_t mybase, ScatterShared& sh)
 {
     constexpr int kWarps = kSortThreads / 32;
-    __shared__ uint32_t wcnt[kWarps][kRadix];   // per-warp digit counts, then the warps' starts
-    __shared__ uint32_t wsum[kWarps];
-    int tile;
-    const SortArray& A = S.a[sort_tile_of(S, blockIdx.x, &tile)];
-    const SortQuant q = KIND == SORT_FIRST ? sort_quant(A.stats) : SortQuant{0, 0};
-    const uint2* src = A.e[from];
+    uint32_t (*wcnt)[kRadix] = sh.wcnt;
     uint2* dst = A.e[from ^ 1];
     const int64_t n = A.n;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // start of digit threadIdx.x's bucket for this tile: exclusive scan of the
-    // 256 digit totals plus this tile's offset inside the bucket
-    uint32_t mybase;
-    {
-        uint32_t v = 0, mine = 0;
-        if (DIRECT) {
-#pragma unroll 8
-            for (int t = 0; t < A.ntiles; ++t) {
-                const uint32_t c = A.hist[(int64_t)t * kRadix + threadIdx.x];
-                mine += t < tile ? c : 0u;
-                v += c;
-            }
-        } else {
-            v = A.tot[threadIdx.x];     // blockDim.x == kRadix
-            mine = A.hist[(int64_t)tile * kRadix + threadIdx.x];
-        }
-        uint32_t x = v;
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += t;
-        }
-        if (lane == 31) wsum[warp] = x;
-        for (int i = threadIdx.x; i < kWarps * kRadix; i += blockDim.x) (&wcnt[0][0])[i] = 0;
-        __syncthreads();
-        uint32_t pre = 0;
-        for (int w = 0; w < warp; ++w) pre += wsum[w];
-        mybase = pre + x - v + mine;
-    }
+    for (int i = lane; i < kRadix; i += 32) wcnt[warp][i] = 0;
+    __syncwarp();
     const unsigned lt = (1u << lane) - 1u;
     const int64_t wbase = (int64_t)tile * kSortTile + (int64_t)warp * (32 * kSortItems);
     uint2 el[kSortItems];
@@ -243,12 +246,12 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(SortPair S, int f
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
         const int64_t i = wbase + it * 32 + lane;
-        el[it] = i < n ? sort_load<KIND>(A, q, src, i) : make_uint2(0u, 0u);
+        el[it] = i < n ? sort_load<KIND>(A, q, A.e[from], i) : make_uint2(0u, 0u);
     }
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it) {
         const bool valid = wbase + it * 32 + lane < n;
-        const unsigned d = valid ? sort_digit<KIND>(A, S.nseg, el[it], shift) : 0x100u;
+        const unsigned d = valid ? sort_digit<KIND>(A, nseg, el[it], shift) : 0x100u;
         dig[it] = d;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const uint32_t prior = valid ? wcnt[warp][d] : 0u;
@@ -258,19 +261,42 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(SortPair S, int f
         rk[it] = prior + __popc(peers & lt);
     }
     __syncthreads();
-    {
-        const int d = threadIdx.x;
-        uint32_t run = mybase;
-        for (int w = 0; w < kWarps; ++w) {
-            const uint32_t t = wcnt[w][d];
-            wcnt[w][d] = run;
-            run += t;
-        }
+    uint32_t run = mybase;
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t t = wcnt[w][threadIdx.x];
+        wcnt[w][threadIdx.x] = run;
+        run += t;
     }
     __syncthreads();
 #pragma unroll
     for (int it = 0; it < kSortItems; ++it)
         if (dig[it] < 0x100u) dst[wcnt[warp][dig[it]] + rk[it]] = el[it];
+    return run;
+}
+
+// With DIRECT (few tiles) the CTA forms the counts of the tiles before it and
+// the totals itself instead of a scan launch between.
+template <int KIND, bool DIRECT>
+__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(SortPair S, int from, int shift)
+{
+    __shared__ ScatterShared sh;
+    int tile;
+    const SortArray& A = S.a[sort_tile_of(S, blockIdx.x, &tile)];
+    const SortQuant q = KIND == SORT_FIRST ? sort_quant(A.stats) : SortQuant{0, 0};
+    uint32_t v = 0, mine = 0;
+    if (DIRECT) {
+#pragma unroll 8
+        for (int t = 0; t < A.ntiles; ++t) {
+            const uint32_t c = A.hist[(int64_t)t * kRadix + threadIdx.x];
+            mine += t < tile ? c : 0u;
+            v += c;
+        }
+    } else {
+        v = A.tot[threadIdx.x];
+        mine = A.hist[(int64_t)tile * kRadix + threadIdx.x];
+    }
+    const uint32_t start = digit_start(v, sh) + mine;
+    sort_scatter_tile<KIND>(A, q, S.nseg, from, shift, tile, start, sh);
 }
 
 __device__ __forceinline__ void sort_put(const SortArray& A, int64_t pos, uint64_t bits, uint32_t idx)
@@ -285,129 +311,183 @@ __device__ __forceinline__ void sort_put(const SortArray& A, int64_t pos, uint64
 // Writes the sorted values, their indices and their double-float parts.  An
 // element of a run of equal keys (and segments) goes to its rank by full
 // pattern within the run; equal patterns keep their order.  Runs of more than
-// kRunMax stay as they are, are listed, and set runh[1] when two neighbours
-// of one are out of order (k_sort_runs then sorts them).
+// kRunMax stay as they are: unsorted[0] is set when two neighbours of one are out
+// of order (k_sort_long then sorts the array), unsorted[1] collects the bits in
+// which the neighbours of any run differ.  A segment's elements lie where its input does, at
+// off[seg].. of the sorted array.
 __global__ void __launch_bounds__(kSortThreads) k_sort_finish(SortPair S, int from)
 {
     const SortArray& A = S.a[blockIdx.y];
     const uint2* e = A.e[from];
     const SortQuant q = sort_quant(A.stats);
     auto bits_of = [&](int64_t i) { return sort_bits(A.in[e[i].y]); };
+    uint32_t differ = 0;
+    bool wrong = false;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint2 el = e[i];
         const uint64_t b = sort_bits(A.in[el.y]);
-        auto same = [&](int64_t k) {
-            if (k < 0 || k >= A.n) return false;
-            const uint2 o = e[k];
-            return o.x == el.x && (S.nseg <= 1 || seg_of(A.off, S.nseg, o.y) == seg_of(A.off, S.nseg, el.y));
-        };
         int64_t pos = i;
         if (q.shift > 0 && el.x != 0) {
-            int left = 0, right = 0;
-            while (left < kRunMax && same(i - left - 1)) ++left;
-            while (right < kRunMax && same(i + right + 1)) ++right;
-            if (left + right + 1 <= kRunMax) {
-                int rank = 0;
-                for (int k = 1; k <= left; ++k) rank += bits_of(i - k) <= b;
-                for (int k = 1; k <= right; ++k) rank += bits_of(i + k) < b;
-                pos = i - left + rank;
-            } else {
-                if (left == 0) {
-                    const uint32_t slot = atomicAdd(A.runh, 1u);
-                    A.runs[slot] = (uint32_t)i;   // at most n / kRunMax long runs
+            int64_t first = 0, end = A.n;
+            if (S.nseg > 1) {
+                const uint32_t seg = seg_of(A.off, S.nseg, i);
+                first = A.off[seg];
+                end = A.off[seg + 1];
+            }
+            auto same = [&](int64_t k) { return k >= first && k < end && e[k].x == el.x; };
+            const bool before = same(i - 1);
+            if (before || same(i + 1)) {
+                int left = 0, right = 0;
+                bool over = same(i - kRunMax) || same(i + kRunMax);
+                while (!over && same(i - left - 1)) ++left;
+                while (!over && same(i + right + 1)) ++right;
+                over = over || left + right + 1 > kRunMax;
+                if (before) {
+                    const uint64_t o = bits_of(i - 1);
+                    wrong = wrong || (over && o > b);
+                    differ |= q.low(o) ^ q.low(b);
                 }
-                if (left > 0 && bits_of(i - 1) > b) A.runh[1] = 1u;
+                if (!over) {
+                    int rank = 0;
+                    for (int k = 1; k <= left; ++k) rank += bits_of(i - k) <= b;
+                    for (int k = 1; k <= right; ++k) rank += bits_of(i + k) < b;
+                    pos = i - left + rank;
+                }
             }
         }
         sort_put(A, pos, b, el.y);
     }
+    // one pair of global updates per CTA, and only where it adds something (a store
+    // per element took 0.6 ms for 1e6 elements of one run)
+    __shared__ uint32_t cta;
+    if (threadIdx.x == 0) cta = 0;
+    const bool any = __syncthreads_or(wrong || differ != 0);
+    if (!any) return;
+    differ = __reduce_or_sync(0xffffffffu, differ);
+    if ((threadIdx.x & 31) == 0) atomicOr(&cta, differ);
+    wrong = __syncthreads_or(wrong);
+    if (threadIdx.x == 0) {
+        volatile uint32_t* u = A.unsorted;
+        if (wrong && u[0] == 0) u[0] = 1u;
+        if ((cta & ~u[1]) != 0) atomicOr(A.unsorted + 1, cta);
+    }
 }
 
-// Runs of more than kRunMax equal keys that are out of order: one CTA per run,
-// a stable radix sort of the remaining low bits of the patterns, ping-pong
-// between the two pair arrays' parts of the run (which other runs' searches
-// may read: every pair there has this run's key and segment).  Inputs need values packed
-// more densely than 1 / kRunMax of a 2^-31 step of their range for it; it
-// returns at once otherwise.
-__global__ void __launch_bounds__(1024) k_sort_runs(SortPair S, int from)
+// The arrays with a run of more than kRunMax equal keys out of order (values
+// packed more densely than 1 / kRunMax of a 2^-31 step of their range), sorted
+// once more by all CTAs together: stable passes over the bits below the keys in
+// which a run's values differ, the keys and the segments.  A CTA takes consecutive
+// tiles and counts their digits together; grid barriers lie between the counts of
+// a pass, their prefix over the CTAs and the scatter.  Returns at once otherwise.
+// One CTA per run took 12 ms for 1e6 values of one run; 0.11 here where they differ
+// in their last bits, 0.40 for 4e6 that differ in 22.
+constexpr int kLongRuns = 32, kLongLen = 20;              // the CTAs' counts: runs of up to kLongLen of them
+constexpr int kLongMaxCtas = kLongRuns * kLongLen;
+
+__global__ void __launch_bounds__(kSortThreads, 4) k_sort_long(SortPair S)
 {
-    __shared__ uint32_t cnt[32][kRadix];
-    __shared__ uint32_t base[kRadix], wtot[kRadix / 32];
-    const SortArray& A = S.a[blockIdx.y];
-    if (A.runh[1] == 0) return;
-    const uint32_t nruns = A.runh[0];
-    const SortQuant q = sort_quant(A.stats);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    for (uint32_t rr = blockIdx.x; rr < nruns; rr += gridDim.x) {
-        const int64_t s = A.runs[rr];
-        const uint2 first = A.e[from][s];
-        const uint32_t seg = S.nseg > 1 ? seg_of(A.off, S.nseg, first.y) : 0u;
-        // end of the run: first later pair with another segment or key
-        int64_t lo = s + 1, hi = A.n;
-        while (lo < hi) {
-            const int64_t mid = lo + ((hi - lo) >> 1);
-            const uint2 o = A.e[from][mid];
-            const bool in = o.x == first.x && (S.nseg <= 1 || seg_of(A.off, S.nseg, o.y) == seg);
-            if (in) lo = mid + 1; else hi = mid;
+    if (S.a[0].unsorted[0] == 0 && S.a[1].unsorted[0] == 0) return;
+    __shared__ ScatterShared sh;
+    __shared__ uint32_t part[kLongRuns][9];
+    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    auto sync = [&]() {
+        if (gridDim.x > 1) grid.sync();
+        else __syncthreads();
+    };
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    SortQuant q[2];
+    int low_at[2][4], nlow[2], npass[2], per[2], most = 0;   // the low digits, passes over them and in all, tiles per CTA
+    for (int w = 0; w < 2; ++w) {
+        const SortArray& A = S.a[w];
+        q[w] = sort_quant(A.stats);
+        nlow[w] = 0;
+        for (uint32_t m = A.unsorted[1]; m != 0; ++nlow[w]) {
+            const int at = __ffs(m) - 1;
+            low_at[w][nlow[w]] = at;
+            m &= ~(0xFFu << at);
         }
-        const int64_t len = lo - s;
-        int cur = from;
-        for (int sh = 0; sh < q.shift; sh += 8, cur ^= 1) {
-            auto digit = [&](uint2 el) {
-                return (unsigned)(((sort_bits(A.in[el.y]) - q.lo) & ((1ull << q.shift) - 1)) >> sh) & 0xFFu;
-            };
-            const uint2* src = A.e[cur] + s;
-            uint2* dst = A.e[cur ^ 1] + s;
-            if (threadIdx.x < kRadix) base[threadIdx.x] = 0;
+        npass[w] = A.unsorted[0] ? nlow[w] + 4 + (S.nseg <= 1 ? 0 : (S.nseg - 1) >> 8 ? 2 : 1) : 0;
+        per[w] = (A.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
+        most = npass[w] > most ? npass[w] : most;
+        for (int64_t i = t0; npass[w] && i < A.n; i += step)
+            A.e[0][i] = make_uint2(q[w].low(sort_bits(A.in[i])), (uint32_t)i);
+    }
+    for (int pass = 0; pass < most; ++pass) {
+        const int from = pass & 1;
+        sync();
+        bool keys = false;
+        for (int w = 0; w < 2; ++w) {
+            if (npass[w] == 0 || pass != nlow[w]) continue;
+            const SortArray& A = S.a[w];
+            keys = true;
+            for (int64_t i = t0; i < A.n; i += step) A.e[from][i].x = q[w].key(sort_bits(A.in[A.e[from][i].y]));
+        }
+        if (keys) sync();
+        for (int w = 0; w < 2; ++w) {
+            const SortArray& A = S.a[w];
+            const int first = blockIdx.x * per[w], end = first + per[w] < A.ntiles ? first + per[w] : A.ntiles;
+            if (pass >= npass[w] || first >= end) continue;
+            const int p = pass - nlow[w], at = p < 0 ? low_at[w][pass] : 8 * (p & 3);
+            uint32_t* h = sh.wcnt[0];
+            h[threadIdx.x] = 0;
             __syncthreads();
-            for (int64_t i = threadIdx.x; i < len; i += blockDim.x) atomicAdd(&base[digit(src[i])], 1u);
-            __syncthreads();
-            uint32_t v = 0, x = 0;
-            if (threadIdx.x < kRadix) {
-                v = base[threadIdx.x];
-                x = v;
-                for (int off = 1; off < 32; off <<= 1) {
-                    const uint32_t t = __shfl_up_sync(0xffffffffu, x, off);
-                    if (lane >= off) x += t;
-                }
-                if (lane == 31) wtot[warp] = x;
+            for (int t = first; t < end; ++t) {
+                if (p < 4) sort_count_tile<SORT_KEY, true>(A, q[w], S.nseg, from, at, t, h);
+                else sort_count_tile<SORT_SEG, true>(A, q[w], S.nseg, from, at, t, h);
             }
             __syncthreads();
-            if (threadIdx.x < kRadix) {
-                uint32_t pre = 0;
-                for (int w = 0; w < warp; ++w) pre += wtot[w];
-                base[threadIdx.x] = pre + x - v;
+            A.hist[(int64_t)blockIdx.x * kRadix + threadIdx.x] = h[threadIdx.x];
+        }
+        sync();
+        // prefix of 8 digits' counts over the CTAs
+        for (int u = blockIdx.x; u < 2 * kRadix / 8; u += gridDim.x) {
+            const int w = u >= kRadix / 8;
+            if (pass >= npass[w]) continue;
+            const SortArray& A = S.a[w];
+            const int nb = (A.ntiles + per[w] - 1) / per[w];   // CTAs with tiles, at most kLongMaxCtas
+            const int c = threadIdx.x & 7, d = 8 * (u & (kRadix / 8 - 1)) + c, run = threadIdx.x >> 3;
+            uint32_t v[kLongLen], sum = 0;
+#pragma unroll
+            for (int k = 0; k < kLongLen; ++k) {   // all in flight
+                const int b = run * kLongLen + k;
+                v[k] = b < nb ? A.hist[(int64_t)b * kRadix + d] : 0u;
             }
-            for (int64_t t0 = 0; t0 < len; t0 += blockDim.x) {
-                for (int i = threadIdx.x; i < 32 * kRadix; i += blockDim.x) (&cnt[0][0])[i] = 0;
-                __syncthreads();
-                const int64_t i = t0 + threadIdx.x;
-                const bool valid = i < len;
-                const uint2 el = valid ? src[i] : make_uint2(0u, 0u);
-                const unsigned d = valid ? digit(el) : 0x100u;
-                const unsigned peers = __match_any_sync(0xffffffffu, d);
-                if (valid && (peers & lt) == 0) cnt[warp][d] = __popc(peers);
-                __syncthreads();
-                if (threadIdx.x < kRadix) {
-                    uint32_t run = base[threadIdx.x];
-                    for (int w = 0; w < 32; ++w) {
-                        const uint32_t c = cnt[w][threadIdx.x];
-                        cnt[w][threadIdx.x] = run;
-                        run += c;
-                    }
-                    base[threadIdx.x] = run;
-                }
-                __syncthreads();
-                if (valid) dst[cnt[warp][d] + __popc(peers & lt)] = el;
-                __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kLongLen; ++k) sum += v[k];
+            part[run][c] = sum;
+            __syncthreads();
+            uint32_t acc = 0;
+            for (int r = 0; r < run; ++r) acc += part[r][c];
+            if (run == kLongRuns - 1) A.tot[d] = acc + sum;
+#pragma unroll
+            for (int k = 0; k < kLongLen; ++k) {
+                const int b = run * kLongLen + k;
+                if (b < nb) A.hist[(int64_t)b * kRadix + d] = acc;
+                acc += v[k];
+            }
+            __syncthreads();   // part is rewritten by the next digits
+        }
+        sync();
+        for (int w = 0; w < 2; ++w) {
+            const SortArray& A = S.a[w];
+            const int first = blockIdx.x * per[w], end = first + per[w] < A.ntiles ? first + per[w] : A.ntiles;
+            if (pass >= npass[w] || first >= end) continue;
+            const int p = pass - nlow[w], at = p < 0 ? low_at[w][pass] : 8 * (p & 3);
+            uint32_t base = digit_start(A.tot[threadIdx.x], sh) + A.hist[(int64_t)blockIdx.x * kRadix + threadIdx.x];
+            for (int t = first; t < end; ++t) {
+                if (p < 4) base = sort_scatter_tile<SORT_KEY>(A, q[w], S.nseg, from, at, t, base, sh);
+                else base = sort_scatter_tile<SORT_SEG>(A, q[w], S.nseg, from, at, t, base, sh);
+                __syncthreads();   // sh is rewritten by the next tile
             }
         }
-        for (int64_t i = threadIdx.x; i < len; i += blockDim.x) {
-            const uint2 el = A.e[cur][s + i];
-            sort_put(A, s + i, sort_bits(A.in[el.y]), el.y);
+    }
+    sync();
+    for (int w = 0; w < 2; ++w) {
+        const SortArray& A = S.a[w];
+        for (int64_t i = t0; npass[w] && i < A.n; i += step) {
+            const uint2 el = A.e[npass[w] & 1][i];
+            sort_put(A, i, sort_bits(A.in[el.y]), el.y);
         }
-        __syncthreads();
     }
 }
 
@@ -473,7 +553,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_sort_small(SortPair S)
             for (int it = 0; it < ITEMS; ++it) {
                 const bool valid = wbase + 32 * it < n;
                 unsigned d = 0x100u;
-                if (valid) d = pass < nlow ? q.low(sort_bits(A.in[el[it].y]), 8 * pass) : (el[it].x >> (8 * (pass - nlow))) & 0xFFu;
+                if (valid) d = pass < nlow ? (q.low(sort_bits(A.in[el[it].y])) >> (8 * pass)) & 0xFFu : (el[it].x >> (8 * (pass - nlow))) & 0xFFu;
                 dig[it] = d;
                 const unsigned peers = __match_any_sync(0xffffffffu, d);
                 const uint32_t prior = valid ? wcnt[warp * kRadix + d] : 0u;
@@ -757,7 +837,7 @@ size_t sort_scratch_bytes(int64_t n)
     const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
     return 2 * align256(sizeof(uint2) * (size_t)n) +
            align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)(ntiles > 0 ? ntiles : 1)) +
-           align256(sizeof(uint32_t) * (size_t)kRadix) + align256(sizeof(uint32_t) * (size_t)(n / kRunMax + 2));
+           align256(sizeof(uint32_t) * (size_t)kRadix);
 }
 
 namespace {
@@ -787,10 +867,30 @@ void sort_pass(const SortPair& S, int from, int shift, bool direct, cudaStream_t
     count_launches(direct ? 2 : 3);
 }
 
+// k_sort_long by the CTAs that are resident together (up to four per SM, and
+// kLongMaxCtas), or by one where a cooperative launch is refused.
+cudaError_t sort_long(const SortPair& S, cudaStream_t s)
+{
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_long, kSortThreads, 0) == cudaSuccess && per_sm > 0) {
+        void* args[] = {(void*)&S};
+        const int all = (per_sm < 4 ? per_sm : 4) * device_sm_count();
+        if (cudaLaunchCooperativeKernel((const void*)k_sort_long, dim3(all < kLongMaxCtas ? all : kLongMaxCtas),
+                                        dim3(kSortThreads), args, 0, s) == cudaSuccess) {
+            count_launches(1);
+            return cudaSuccess;
+        }
+    }
+    (void)cudaGetLastError();
+    k_sort_long<<<1, kSortThreads, 0, s>>>(S);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 // Checks and sorts both arrays (out, perm, split); scratch as
-// sort_scratch_bytes each, flag, stats[2] and runh[2] of each array zeroed.
+// sort_scratch_bytes each, flag, stats[2] and unsorted[2] of each array zeroed.
 // With nseg > 1 segments (device offsets off[0..nseg], nseg <= 65536) each
 // segment is sorted on its own: the key passes are followed by stable passes
 // on the segment number, so the output keeps the segments in order.
@@ -811,8 +911,7 @@ cudaError_t launch_sort_pair(SortPair S, char* const scratch[2], cudaStream_t s)
         A.e[0] = (uint2*)p; p += align256(sizeof(uint2) * (size_t)A.n);
         A.e[1] = (uint2*)p; p += align256(sizeof(uint2) * (size_t)A.n);
         A.hist = (uint32_t*)p; p += align256(sizeof(uint32_t) * (size_t)kRadix * (size_t)(A.ntiles > 0 ? A.ntiles : 1));
-        A.tot = (uint32_t*)p; p += align256(sizeof(uint32_t) * (size_t)kRadix);
-        A.runs = (uint32_t*)p;
+        A.tot = (uint32_t*)p;
         direct = direct && A.ntiles <= kSortDirectTiles;
     }
     const dim3 all(grid_for(most, kSortThreads), 2);
@@ -824,9 +923,9 @@ cudaError_t launch_sort_pair(SortPair S, char* const scratch[2], cudaStream_t s)
     for (int shift = 0; S.nseg > 1 && (shift == 0 || (S.nseg - 1) >> shift); shift += 8, cur ^= 1)
         sort_pass<SORT_SEG>(S, cur, shift, direct, s);
     k_sort_finish<<<all, kSortThreads, 0, s>>>(S, cur);
-    k_sort_runs<<<dim3(device_sm_count(), 2), 1024, 0, s>>>(S, cur);
-    count_launches(3);
-    return cudaGetLastError();
+    count_launches(2);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? sort_long(S, s) : e;
 }
 
 cudaError_t launch_replicate(const SortedView& src, const SortedView& dst, int64_t n, int64_t m, int nrep,

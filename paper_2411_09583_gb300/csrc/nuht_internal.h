@@ -194,7 +194,7 @@ enum { LIST_MOM, LIST_EVAL, LIST_SPREAD, LIST_INTERP, LIST_FSMALL, LIST_FA, LIST
 // What a plan build reads back from the device in one copy (zeroed first).
 struct PlanCounts {
     int flag[2];                    // a point / frequency is outside the domain
-    uint32_t runh[2][2];            // SortArray::runh
+    uint32_t unsorted[2][2];        // SortArray::unsorted
     unsigned long long stats[2][2]; // SortArray::stats
     int64_t res[4];                 // blocks of each class, lists overflowed
     int64_t totals[kTotals];
@@ -288,11 +288,11 @@ struct SortArray {
     float2* split;               // and double-float parts
     int* flag;                   // set when a value is outside the domain
     unsigned long long* stats;   // [2] value range (zeroed)
-    uint32_t* runh;              // [2] number of long runs of equal keys, whether one is unsorted (zeroed)
+    uint32_t* unsorted;          // [2] whether a long run of equal keys is out of order, the bits it differs in (zeroed)
     // set by launch_sort_pair
     int ntiles;
     uint2* e[2];
-    uint32_t *hist, *tot, *runs;
+    uint32_t *hist, *tot;
 };
 struct SortPair {
     SortArray a[2];

@@ -677,7 +677,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
             SortArray& A = sp.a[k];
             A.in = in[k]; A.n = cnt[k]; A.off = off[k];
             A.out = out[k]; A.perm = perm[k]; A.split = split[k];
-            A.flag = &d_cnt->flag[k]; A.stats = d_cnt->stats[k]; A.runh = d_cnt->runh[k];
+            A.flag = &d_cnt->flag[k]; A.stats = d_cnt->stats[k]; A.unsorted = d_cnt->unsorted[k];
         }
         char* const scr[2] = {sort_mem + o_scr, sort_mem + o_scr_w};
         NUHT_CK(launch_sort_pair(sp, scr, s));

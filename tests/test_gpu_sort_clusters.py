@@ -53,3 +53,38 @@ def _check(n, k, outlier):
 @pytest.mark.parametrize("k,outlier", [(1, 1e-3), (4, 0.0), (2, 1e-300)])
 def test_clusters_in_one_cta(n, k, outlier):
     _check(n, k, outlier)
+
+
+@pytest.mark.parametrize("n", [8193, 100003, 1000003])
+@pytest.mark.parametrize("k,outlier", [(1, 1e-3), (4, 0.0), (2, 1e-300)])
+def test_clusters_over_many_ctas(n, k, outlier):
+    _check(n, k, outlier)
+
+
+@pytest.mark.parametrize("nprob,top", [(2, 9000), (300, 3000), (700, 400)])
+def test_clusters_in_segments(nprob, top):
+    from paper_2411_09583_gb300 import Plan
+    rng = np.random.default_rng(nprob)
+    n, m = rng.integers(0, top, nprob), rng.integers(0, 90, nprob)
+    n[0] = top
+    r, omega = _circles(rng, int(n.sum()), 2, 1e-3), _circles(rng, int(m.sum()), 1, 1e-5)
+    with Plan.many(rng.integers(0, 4, nprob), to_dev(r), n, to_dev(omega), m, 1e-6) as p:
+        pr, pw = p.permutations()
+
+    def want(x, cnt):
+        off = np.concatenate([[0], np.cumsum(cnt)])
+        return np.concatenate([off[i] + np.argsort(x[off[i]:off[i + 1]], kind="stable") for i in range(len(cnt))])
+    assert np.array_equal(pr, want(r, n))
+    assert np.array_equal(pw, want(omega, m))
+
+
+@pytest.mark.parametrize("n", [5000, 60000])
+def test_short_runs_beside_a_long_one(n):
+    # pairs and triples of equal keys that differ in other bits than the long run's
+    from paper_2411_09583_gb300 import Plan
+    rng = np.random.default_rng(n)
+    v = np.concatenate([rng.uniform(0.5, 0.6, n), 1.0 + 2.0 ** -52 * rng.integers(0, 5, n), [1e-300]])
+    r, omega = rng.permutation(v), rng.uniform(0.0, 1.0, 9000)
+    with Plan(0, to_dev(r), to_dev(omega), 1e-8) as p:
+        pr, _ = p.permutations()
+    assert np.array_equal(pr, np.argsort(r, kind="stable"))
