@@ -215,7 +215,9 @@ int nuht_adjoint(nuht_plan_t p, const double *g, double *c, int nvec, int is_com
  *   d/domega_k sum_k e_k g_k = e_k sum_j c_j r_j J_nu'(omega_k r_j)
  *
  * The two orders run as two problems of one plan whose sums are added with
- * opposite signs, so each gradient is one pass of the pipeline.  The plan
+ * opposite signs, so each gradient is one pass of the pipeline.  For nu = 0,
+ * where both are -J_1, one transform of order 1 serves both; the plan reports
+ * two all the same (nuht_info, nuht_get_blocks, nuht_get_permutations).  The plan
  * reuses the base plan's sorted values and permutations (no second sort or
  * domain check); it needs |nu| + 1 <= 100 (else NUHT_ERR_UNSUPPORTED) and uses
  * the base plan's eps and options.  The base plan may be destroyed afterwards.

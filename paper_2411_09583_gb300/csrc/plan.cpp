@@ -1757,6 +1757,10 @@ int nuht_transform_host(int nu, const double* r, int64_t n, const double* omega,
     return rc;
 }
 
+// Copies of its problems that a plan reports: a derivative plan at order 0 runs
+// one transform (of order 1) for its two problems.
+static int reported_copies(const nuht_plan_s* P) { return P->deriv && P->probs.size() == 1 ? 2 : 1; }
+
 int nuht_info(nuht_plan_t P, nuht_plan_info* out)
 {
     if (!P || !out) return NUHT_ERR_INVALID_ARG;
@@ -1769,15 +1773,16 @@ int nuht_info(nuht_plan_t P, nuht_plan_info* out)
     out->asy_members = P->asy_members;
     out->z = P->probs[0].z;
     out->eps = P->eps;
-    out->n = P->n;
-    out->m = P->m;
-    out->n_local = P->n_loc;
-    out->n_asy = P->n_asy;
-    out->n_direct = P->n_dir;
-    out->direct_entries = P->direct_entries;
-    out->local_rows_cols = P->local_rc;
-    out->asy_rows_cols = P->asy_rc;
-    out->fft_points = P->fft_points;
+    const int copies = reported_copies(P);
+    out->n = copies * P->n;
+    out->m = copies * P->m;
+    out->n_local = copies * P->n_loc;
+    out->n_asy = copies * P->n_asy;
+    out->n_direct = copies * P->n_dir;
+    out->direct_entries = copies * P->direct_entries;
+    out->local_rows_cols = copies * P->local_rc;
+    out->asy_rows_cols = copies * P->asy_rc;
+    out->fft_points = copies * P->fft_points;
     out->device_bytes = (int64_t)P->dbytes;
     for (int i = 0; i < 4; ++i) out->plan_ms[i] = P->plan_ms[i];
     return NUHT_OK;
@@ -1787,17 +1792,21 @@ int nuht_get_blocks(nuht_plan_t P, int cls, int64_t* ranges, int64_t cap, int64_
 {
     if (!P || cls < 0 || cls > 2 || !count || cap < 0 || (cap > 0 && !ranges)) return NUHT_ERR_INVALID_ARG;
     const int64_t first = cls == 0 ? 0 : (cls == 1 ? P->n_loc : (int64_t)P->n_loc + P->n_asy);
-    *count = cls == 0 ? P->n_loc : (cls == 1 ? P->n_asy : P->n_dir);
-    const int64_t nc = cap < *count ? cap : *count;
+    const int64_t own = cls == 0 ? P->n_loc : (cls == 1 ? P->n_asy : P->n_dir);
+    *count = reported_copies(P) * own;
+    const int64_t nc = cap < *count ? cap : *count, nown = nc < own ? nc : own;
     if (nc <= 0) return NUHT_OK;
-    std::vector<SubBlk> v((size_t)nc);
-    NUHT_CK(cudaMemcpyAsync(v.data(), P->d_blk + first, sizeof(SubBlk) * nc, cudaMemcpyDeviceToHost, P->stream));
+    std::vector<SubBlk> v((size_t)nown);
+    NUHT_CK(cudaMemcpyAsync(v.data(), P->d_blk + first, sizeof(SubBlk) * nown, cudaMemcpyDeviceToHost, P->stream));
     NUHT_CK(cudaStreamSynchronize(P->stream));
     for (int64_t i = 0; i < nc; ++i) {
-        ranges[4 * i + 0] = v[(size_t)i].k0;
-        ranges[4 * i + 1] = v[(size_t)i].k1;
-        ranges[4 * i + 2] = v[(size_t)i].j0;
-        ranges[4 * i + 3] = v[(size_t)i].j1;
+        // the second copy lies behind the first in both directions
+        const SubBlk& b = v[(size_t)(i % own)];
+        const int64_t dk = i / own * P->m, dj = i / own * P->n;
+        ranges[4 * i + 0] = b.k0 + dk;
+        ranges[4 * i + 1] = b.k1 + dk;
+        ranges[4 * i + 2] = b.j0 + dj;
+        ranges[4 * i + 3] = b.j1 + dj;
     }
     return NUHT_OK;
 }
@@ -1805,10 +1814,14 @@ int nuht_get_blocks(nuht_plan_t P, int cls, int64_t* ranges, int64_t cap, int64_
 int nuht_get_permutations(nuht_plan_t P, int32_t* perm_r, int32_t* perm_omega)
 {
     if (!P) return NUHT_ERR_INVALID_ARG;
-    if (perm_r && P->n)
-        NUHT_CK(cudaMemcpyAsync(perm_r, P->d_pr, sizeof(int32_t) * P->n, cudaMemcpyDeviceToHost, P->stream));
-    if (perm_omega && P->m)
-        NUHT_CK(cudaMemcpyAsync(perm_omega, P->d_pw, sizeof(int32_t) * P->m, cudaMemcpyDeviceToHost, P->stream));
+    for (int64_t k = 0; k < reported_copies(P); ++k) {
+        if (perm_r && P->n)
+            NUHT_CK(cudaMemcpyAsync(perm_r + k * P->n, P->d_pr, sizeof(int32_t) * P->n, cudaMemcpyDeviceToHost,
+                                    P->stream));
+        if (perm_omega && P->m)
+            NUHT_CK(cudaMemcpyAsync(perm_omega + k * P->m, P->d_pw, sizeof(int32_t) * P->m, cudaMemcpyDeviceToHost,
+                                    P->stream));
+    }
     NUHT_CK(cudaStreamSynchronize(P->stream));
     return NUHT_OK;
 }
