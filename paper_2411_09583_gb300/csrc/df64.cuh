@@ -151,6 +151,17 @@ __device__ __forceinline__ double acc_join(acc2 a, acc2 b)
     return f64_of(s) + (f64_of(h) + f64_of(t + u));
 }
 
+// The same and x.
+__device__ __forceinline__ double acc_join(acc2 a, acc2 b, float x)
+{
+    float s, e, h, t, u, v;
+    two_sum(a.s, b.s, s, e);
+    two_sum(a.c, b.c, h, t);
+    two_sum(h, e, h, u);
+    two_sum(h, x, h, v);
+    return f64_of(s) + (f64_of(h) + f64_of(t + (u + v)));
+}
+
 // a += the value of lane ^ off (two-sum through the shuffles), where this lane
 // keeps `keep` and hands over `give`.
 __device__ __forceinline__ acc2 acc_exchange(acc2 keep, acc2 give, int off)

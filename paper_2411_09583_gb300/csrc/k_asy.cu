@@ -405,7 +405,7 @@ __device__ __forceinline__ void spread_moments(const ProbParams& P, const Tile& 
                 }
                 for (; e < L.dpad; ++e) sf = fmaf(ar[e].x, mb[e * Q2].x, sf);
             }
-            const double val = acc_join(s, s1) + f64_of(sf);
+            const double val = acc_join(s, s1, sf);
             if (__double_as_longlong(val) << 1)   // (an integer test: FP64 issues 64 times slower)
                 gv.add(2 * ((int64_t)idx * Q + (qv >> 1)) + (qv & 1), val);
         }
@@ -729,7 +729,7 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
         // (b) M[d][q] = sum_k beta_qk (N[d+k] + N[|d-k|]) / 2 into the row order of Mb;
         // each item forms two consecutive q, so one sum N[d+k] + N[|d-k|]
         // (an unevaluated (hi, lo) pair) serves both
-        // (items of a group of bins in the order of list_items, two rows each,
+        // (items of a group of bins in the order of list_moment_items, two rows each,
         // so that the double-float ones fill warps)
         for (int o = tid; o < gn * L.dpad * (Q >> 1); o += nt) {
             const int row = o / gn, b = o - row * gn;

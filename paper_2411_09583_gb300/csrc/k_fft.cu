@@ -17,6 +17,8 @@
 
 namespace nuht {
 
+int device_sm_count();
+
 namespace {
 
 // Complex double-float values are float4 (re.h, re.l, im.h, im.l).
@@ -685,7 +687,7 @@ cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* bl
     // blocks of up to kFftSmallPts points in small CTAs (8 KiB, many per SM),
     // the larger ones in CTAs sized for the largest
     constexpr int kFftSmallPts = 1024;
-    constexpr int kFftScanCtas = 8 * 152;   // at least eight CTAs per SM look for the larger ones
+    const int scan_ctas = 8 * device_sm_count();   // at least eight CTAs per SM look for the larger ones
     const int ranges[2][2] = {{0, max_pts < kFftSmallPts ? max_pts : kFftSmallPts}, {kFftSmallPts, max_pts}};
     int launched = 0;
     for (int r = 0; r < 2; ++r) {
@@ -700,7 +702,7 @@ cudaError_t launch_asy_fft_block_f32(const ProbParams* probs, const AsyBlock* bl
         cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         int gx = nitems;
-        if (r) gx = std::min(nitems, std::max((nitems + nt - 1) / nt, kFftScanCtas));
+        if (r) gx = std::min(nitems, std::max((nitems + nt - 1) / nt, scan_ctas));
         kern<<<dim3(gx, members), nt, smem, s>>>(probs, blks, items, nitems, tab, src, dst, lo, hi, src_stride,
                                                  dst_stride);
         e = cudaGetLastError();

@@ -167,7 +167,8 @@ struct Tile {
 // A run of tiles: indices first..last of block blk cut into tiles of len.
 // Tile lists are expanded from these on the device (k_expand_lists).  FFT work
 // items are tiles of length one whose start is the item's ordinal in its
-// block (q for single-pass FFTs, q * lines + line for the two-pass passes).
+// block: of a double-float pass's tiles (fft_tile), or in mixed precision q for
+// single-pass FFTs and group of lines * Q + q for the two-pass ones.
 struct Seg {
     int32_t blk, len;
     int64_t first, last;
@@ -319,7 +320,9 @@ cudaError_t launch_staircase(const double* r, const double* w, int64_t m, const 
 // same either way.
 constexpr int kSubGridMax = 1024;
 // up to this many points + frequencies: one CTA, no cooperative launch (levels of
-// up to ~120 blocks there: 52 -> 20 us at 4000 in all, the grid's barriers included)
+// up to ~120 blocks: 52 -> 20 us at 4000 in all, the grid's barriers included; at
+// 32600 in all the two take the same time, 26 to 54 us from min_size 1024 to 1,
+// where levels have thousands of blocks)
 constexpr int64_t kSubOneCta = 32768;
 int subdivide_grid_ctas();
 cudaError_t launch_subdivide(const int32_t* stair, const double* r_s, const double* w_s, const ProbParams* probs,

@@ -76,7 +76,7 @@ struct nuht_plan_s {
     Tile *d_tmom = nullptr, *d_teval = nullptr;
     AsyBlock* d_asy = nullptr;
     Tile *d_tspread = nullptr, *d_tinterp = nullptr;
-    int32_t* d_smode = nullptr;   // path of each spreading tile (k_spread_modes)
+    int32_t* d_smode = nullptr;   // path of each spreading tile (k_expand_lists)
     Tile *d_fblock = nullptr, *d_fsmall = nullptr, *d_fa = nullptr, *d_fb = nullptr;   // FP32 FFTs
     Tile* d_fpass[3] = {nullptr, nullptr, nullptr};   // passes of the double-float FFTs
     DirectBlock* d_dir = nullptr;
@@ -625,7 +625,7 @@ static int build_plan(nuht_plan_t P, const double* r, const double* omega, const
     }
     size_t o_qa = sa.reserve<SubBlk>(qcap), o_qb = sa.reserve<SubBlk>(qcap);
     size_t o_out = sa.reserve<SubBlk>(3 * ocap);
-    // up to kSubOneCta points and frequencies no level outgrows one CTA's walk
+    // up to kSubOneCta points and frequencies one CTA's walk is at least as fast
     const int sub_ctas = n + m <= kSubOneCta ? 0 : subdivide_grid_ctas();
     size_t o_ctot = sa.reserve<int4>(sub_ctas > 0 ? (size_t)sub_ctas : 1), o_gst = sa.reserve<int64_t>(8);
     BuildTemps bt = reserve_build_temps(sa, ocap);
@@ -1312,8 +1312,8 @@ static int apply_forward(nuht_plan_t P, int c0, int ng, cudaStream_t s)
                                   gsb ? P->d_cs2b : nullptr, gsb, P->det ? 1 : 0, ls));
         NUHT_TRY(T.end(NUHT_STAGE_DIRECT, ls));
     }
-    // the asymptotic pipeline, asy_members components per spreading and
-    // interpolation launch (their FFTs one after the other)
+    // the asymptotic pipeline, asy_members components per launch (mixed
+    // precision: the two-pass FFTs one component after the other)
     const bool lowp = P->opt.precision == NUHT_PREC_MIXED;   // FP32 kernels and butterflies
     const int am = P->asy_members;
     for (int v0 = 0; asy && v0 < ng; v0 += am) {
