@@ -220,11 +220,12 @@ __host__ __device__ __forceinline__ MomLayout mom_layout(int nb, int dcs, int Q2
 //    bins share the barriers and one grid update (a cell of both gets one sum);
 //  - the lanes' partial sums are exchanged and halved (8 exchanges for 8 outputs)
 //    instead of each summed by all lanes (24).
-// n = m = 1e6, eps 1e-12 (forward, with the folded tiles): 1.02 -> 0.92 ms;
-// one vector of 16 at 1.5e5 points 0.128 -> 0.108.  Sums of six instructions a
-// product, from an anchor above the tile's largest value, take 2 % off a gradient
-// at eps 1e-10 (8.62 -> 8.47 ms) but round 4 to 75 times coarser there and at
-// 1e-11, up to 1.7e-12 of the result.  Skipping a phase in a
+// n = m = 1e6, eps 1e-12 (forward, with the folded tiles): 1.00 -> 0.93 ms, 1e-10
+// 0.87 -> 0.79; adjoint 1.41 -> 1.21 and 1.19 -> 0.96; one vector of 16 at 1.5e5
+// points 0.130 -> 0.101.  Sums of six instructions a product, from an anchor above
+// the tile's largest value, take 2 % off a gradient at eps 1e-10 (8.62 -> 8.47 ms)
+// but round 4 to 75 times coarser there and at 1e-11, up to 1.7e-12 of the result.
+// Each bin's sums keep a chain of their own in the shared grid update.  Skipping a phase in a
 // timing-only build at eps 1e-12 (0.96 ms then): double-float items 0.11, FP32
 // items 0.11 (before the high parts had a plane of their own), grid update
 // 0.09; of the folded tiles N 0.04, beta 0.02, M 0.06, grid update 0.11.
@@ -856,8 +857,8 @@ __device__ void spread_fold(const AsyBlock& B, const ProbParams& P, const Tile& 
 // ready at a barrier), else it stands from the previous member.
 // FP32 issue and shared reads of the products bound it.  Two binary searches per
 // lane and output and the FP64 (1/64 rate) halves of every output cost more than
-// the products before: 4e6 far-field points (eps 1e-12, half a point a cell) 1.80 ->
-// 1.18 ms, 256 problems of 3e2 to 1e5 points 5.3 -> 4.8 ms.
+// the products before: 4e6 far-field points (eps 1e-12, half a point a cell) 1.86 ->
+// 1.18 ms, their adjoint 1.68 -> 1.33, 256 problems of 3e2 to 1e5 points 5.0 -> 4.3.
 template <class Put>
 __device__ __forceinline__ void tap_cell_sums(const int* l0s, int cnt, int first, int span, int w, int Q,
                                               const float2* taps, const float4* vals, uint16_t* start, int cap,
